@@ -171,6 +171,9 @@ __device__ __forceinline__ int wrapi(int a, int n) {
     return a < 0 ? a + n : a;
 }
 
+// a in [-1, n] (a lattice neighbour's coordinate) into [0, n)
+__device__ __forceinline__ int wrap_step(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
+
 __device__ __forceinline__ int64_t cell_index(const Lattice& L, int x, int y, int z) {
     return (int64_t)x + (int64_t)L.nx * ((int64_t)y + (int64_t)L.ny * (int64_t)z);
 }
@@ -187,7 +190,7 @@ __device__ __forceinline__ void cell_coords(const Lattice& L, int64_t n, int& x,
 // (x,y,z) before a step of parity q.
 __device__ __forceinline__ int64_t read_slot(const Lattice& L, int i, int x, int y, int z, int q) {
     if (q == 0) return (int64_t)i * L.Np + cell_index(L, x, y, z);
-    int xs = wrapi(x - cx(i), L.nx), ys = wrapi(y - cy(i), L.ny), zs = wrapi(z - cz(i), L.nz);
+    const int xs = wrap_step(x - cx(i), L.nx), ys = wrap_step(y - cy(i), L.ny), zs = wrap_step(z - cz(i), L.nz);
     return (int64_t)opp(i) * L.Np + cell_index(L, xs, ys, zs);
 }
 
