@@ -40,39 +40,53 @@
 
 #include "lbsq_internal.cuh"
 #include "psm.cuh"
+#include "sweep_df.cuh"
 
 namespace lbsq {
 
-constexpr int kLB = 128;  // threads of the link kernel
+constexpr int kLB = 128;  // threads of the link kernel (SEG = 8 in block_sum_fixed)
 constexpr int kBB = 256;  // threads of the box kernels
 static_assert(kBB == kPsmChunk, "a chunk of partially saturated cells is one block of the box kernels");
 
 // ---------------------------------------------------------------- reductions
 
-// Sum K doubles over a block of T threads in a fixed order: each value is
-// added once, by many lanes at a time (one FP64 warp instruction costs the
-// pipe the same with 1 or 32 active lanes).  Stage 1: K*8 threads each sum a
-// segment of T/8 values of one component; stage 2: K threads sum the 8
-// segments.  Result in out[K] (shared), valid for all threads on return.
-// Uses the shared buffer sm[K*T + K*8].
-template <int K, int T>
-__device__ __forceinline__ void block_sum_fixed(const double (&v)[K], double* sm, double* out) {
-    constexpr int SEG = 8, LEN = T / SEG;
+// Sum K values per thread over a block of T threads in a fixed order.  Stage
+// 1: K * SEG threads each add LEN values of one component, SEG apart (so that
+// neighbouring threads read neighbouring words of shared memory; runs of
+// consecutive values put a warp's reads on one bank); stage 2: K threads add
+// the SEG partial sums.  Result in out[K] (shared), valid for all threads on
+// return.  Uses the shared buffer sm[K * T + K * SEG].
+//
+// An FP64 add costs its SM sub-partition 64 cycles per warp whatever its
+// active lanes, so sums of FP32 terms are carried as pairs h + l of FP32
+// numbers instead (two_sum: about 48 bits, no FP64 instruction until the
+// totals); V = double or df.
+__device__ __forceinline__ double sum_add(double a, double b) { return a + b; }
+__device__ __forceinline__ df sum_add(df a, df b) { return dadd(a, b); }
+__device__ __forceinline__ double sum_out(double a) { return a; }
+__device__ __forceinline__ double sum_out(df a) { return (double)a.h + (double)a.l; }
+
+template <int K, int T, class V>
+__device__ __forceinline__ void block_sum_fixed(const V (&v)[K], double* smd, double* out) {
+    static_assert(sizeof(V) == sizeof(double), "one word per value");
+    constexpr int LEN = 16, SEG = T / LEN;
+    V* sm = reinterpret_cast<V*>(smd);
 #pragma unroll
     for (int c = 0; c < K; ++c) sm[c * T + threadIdx.x] = v[c];
     __syncthreads();
-    double* sm2 = sm + K * T;
+    V* sm2 = sm + K * T;
     for (int t = threadIdx.x; t < K * SEG; t += T) {
         const int c = t / SEG, sg = t % SEG;
-        double a = 0.0;
-        for (int q = 0; q < LEN; ++q) a += sm[c * T + sg * LEN + q];
+        V a = sm[c * T + sg];
+#pragma unroll 4
+        for (int q = 1; q < LEN; ++q) a = sum_add(a, sm[c * T + q * SEG + sg]);
         sm2[c * SEG + sg] = a;
     }
     __syncthreads();
     if (threadIdx.x < K) {
-        double a = 0.0;
-        for (int sg = 0; sg < SEG; ++sg) a += sm2[threadIdx.x * SEG + sg];
-        out[threadIdx.x] = a;
+        V a = sm2[threadIdx.x * SEG];
+        for (int sg = 1; sg < SEG; ++sg) a = sum_add(a, sm2[threadIdx.x * SEG + sg]);
+        out[threadIdx.x] = sum_out(a);
     }
     __syncthreads();
 }
@@ -148,12 +162,14 @@ __device__ __forceinline__ bool last_block(int* counter, int nblocks, int* flag)
 // The G partials of one body summed in a fixed order, staged in shared memory
 // with cache-global loads (no stale L1 line): K*8 lanes each sum a run of
 // consecutive partials of one component, K lanes then sum the 8 runs.  The
-// grouping depends on G only (a property of the body).  Result in out[K]
-// (shared).  Uses sm[G*K + K*8].
+// grouping depends on G only (a property of the body).  Partials lie `stride`
+// doubles apart, of which the first K are summed.  Result in out[K] (shared).
+// Uses sm[G*K + K*8].
 template <int K>
-__device__ __forceinline__ void ordered_partial_sum(const double* part, int G, double* sm, double* out) {
+__device__ __forceinline__ void ordered_partial_sum(const double* part, int G, double* sm, double* out,
+                                                    int stride = K) {
     constexpr int SEG = 8;
-    for (int t = threadIdx.x; t < G * K; t += blockDim.x) sm[t] = __ldcg(part + t);
+    for (int t = threadIdx.x; t < G * K; t += blockDim.x) sm[t] = __ldcg(part + (t / K) * stride + t % K);
     __syncthreads();
     double* sm2 = sm + G * K;
     const int run = (G + SEG - 1) / SEG;
@@ -328,39 +344,79 @@ __device__ __noinline__ void rot_coeffs(double t2, double& sa, double& c1, doubl
 
 __device__ __noinline__ double inv_sqrt(double x) { return 1.0 / sqrt(x); }
 
-// WCA force on sphere k from the other bodies of its lattice (Eq. "wca").
+// Whether body j may be within the contact range of sphere k, in FP32: false
+// only if the gap is certainly beyond 2^(1/6) sigma, where the force is exactly
+// zero (2e-5 of slack against FP32 errors of a few 1e-7).  Positions enter
+// through one FP64 difference per axis.
+template <int P>
+__device__ __forceinline__ bool wca_near(const Lattice& L, const Bodies& B, int j, const BodyParams& p,
+                                         const BodyState& s) {
+    const BodyParams& q = B.par[j];
+    const float cut = 1.1225f * (float)L.wca_sigma, R = (float)p.R;
+    if (q.kind == BODY_SPHERE) {
+        const double* t = B.state[P][j].pos;
+        const float n3[3] = {(float)L.nx, (float)L.ny, (float)L.nz};
+        float d2 = 0.0f;
+        for (int b = 0; b < 3; ++b) {
+            float d = fabsf((float)(s.pos[b] - t[b]));
+            d = fminf(d, fabsf(n3[b] - d));  // the nearer image
+            d2 += d * d;
+        }
+        const float lim = R + (float)q.R + cut;
+        return !(d2 > lim * lim * 1.00002f + 1e-4f);
+    }
+    if (q.wall_axis < 0) {
+        const float dx = (float)(s.pos[0] - q.tube[0]), dy = (float)(s.pos[1] - q.tube[1]);
+        const float lim = (float)q.tube[2] - 0.5f - R - cut;
+        return !(lim > 0.0f && dx * dx + dy * dy < lim * lim * 0.99998f - 1e-4f);
+    }
+    return true;
+}
+
+// WCA force on sphere k from the other bodies of its lattice (Eq. "wca"), by
+// one whole warp: the lanes rule out the bodies beyond the contact range in
+// FP32 (in FP64, with its square roots and divisions on the GPU's narrow FP64
+// pipe, each body cost about 5 us), lane 0 sums the force of the rest in the
+// order of the bodies.
 template <int P>
 __device__ __noinline__ void wca_sum(const Lattice& L, const Bodies& B, int k, const BodyParams& p,
                                      const BodyState& s, double* fw) {
-    const int n3[3] = {L.nx, L.ny, L.nz};
-    for (int j = L.body_begin; j < L.body_begin + L.body_count; ++j) {
-        if (j == k) continue;
-        const BodyParams& q = B.par[j];
-        const BodyState& t = B.state[P][j];
-        if (q.kind == BODY_SPHERE) {
-            double dd[3];
-            for (int b = 0; b < 3; ++b) dd[b] = min_image(s.pos[b] - t.pos[b], n3[b]);
-            const double dist = sqrt(dd[0] * dd[0] + dd[1] * dd[1] + dd[2] * dd[2]);
-            const double f = wca_force(dist - p.R - q.R, L.wca_sigma, L.wca_eps);
-            if (f != 0.0)
-                for (int b = 0; b < 3; ++b) fw[b] += f * dd[b] / dist;
-        } else if (q.wall_axis < 0) {
-            // round tube: its surface half a cell inside the first solid
-            // radius, as for a plane wall; the force points to the axis
-            const double dx = s.pos[0] - q.tube[0], dy = s.pos[1] - q.tube[1];
-            const double rho = sqrt(dx * dx + dy * dy);
-            const double f = wca_force((q.tube[2] - 0.5) - rho - p.R, L.wca_sigma, L.wca_eps);
-            if (f != 0.0 && rho > 0.0) {
-                fw[0] -= f * dx / rho;
-                fw[1] -= f * dy / rho;
+    const int n3[3] = {L.nx, L.ny, L.nz}, lane = threadIdx.x & 31, jend = L.body_begin + L.body_count;
+    for (int j0 = L.body_begin; j0 < jend; j0 += 32) {
+        const int jl = j0 + lane;
+        unsigned todo = __ballot_sync(0xffffffffu, jl < jend && jl != k && wca_near<P>(L, B, jl, p, s));
+        if (lane != 0) continue;
+        while (todo) {
+            const int j = j0 + __ffs(todo) - 1;
+            todo &= todo - 1;
+            const BodyParams& q = B.par[j];
+            const BodyState& t = B.state[P][j];
+            if (q.kind == BODY_SPHERE) {
+                double dd[3];
+                for (int b = 0; b < 3; ++b) dd[b] = min_image(s.pos[b] - t.pos[b], n3[b]);
+                const double dist = sqrt(dd[0] * dd[0] + dd[1] * dd[1] + dd[2] * dd[2]);
+                const double f = wca_force(dist - p.R - q.R, L.wca_sigma, L.wca_eps);
+                if (f != 0.0)
+                    for (int b = 0; b < 3; ++b) fw[b] += f * dd[b] / dist;
+            } else if (q.wall_axis < 0) {
+                // round tube: its surface half a cell inside the first solid
+                // radius, as for a plane wall; the force points to the axis
+                const double dx = s.pos[0] - q.tube[0], dy = s.pos[1] - q.tube[1];
+                const double rho = sqrt(dx * dx + dy * dy);
+                const double f = wca_force((q.tube[2] - 0.5) - rho - p.R, L.wca_sigma, L.wca_eps);
+                if (f != 0.0 && rho > 0.0) {
+                    fw[0] -= f * dx / rho;
+                    fw[1] -= f * dy / rho;
+                }
+            } else {
+                const int ax = q.wall_axis;
+                const double dd = min_image(s.pos[ax] - (double)q.wall_index, n3[ax]);
+                const double f = wca_force(fabs(dd) - 0.5 - p.R, L.wca_sigma, L.wca_eps);
+                if (f != 0.0) fw[ax] += dd > 0.0 ? f : -f;
             }
-        } else {
-            const int ax = q.wall_axis;
-            const double dd = min_image(s.pos[ax] - (double)q.wall_index, n3[ax]);
-            const double f = wca_force(fabs(dd) - 0.5 - p.R, L.wca_sigma, L.wca_eps);
-            if (f != 0.0) fw[ax] += dd > 0.0 ? f : -f;
         }
     }
+    __syncwarp();
 }
 
 // Sum over lanes 0..2 of a value held per lane, as (x0 + x1) + x2 on every
@@ -374,61 +430,59 @@ __device__ __forceinline__ double sum3(double v) {
 // Component b of a vector held as one component per lane 0..2.
 __device__ __forceinline__ double comp(double v, int b) { return __shfl_sync(0xffffffffu, v, b); }
 
-// Symplectic Euler of body k, by one whole warp (lane a < 3 holds vector
-// component a): applies the momentum exchange of this step plus the
-// conversion force booked by the last remap, writes state[1-P], and decides
-// whether a node can cross the surface.  Splitting the vectors over lanes
-// shortens the serial FP64 chain, which this GPU issues at a low rate.
+// Symplectic Euler of body k: applies the momentum exchange of this step
+// plus the conversion force booked by the last remap, writes state[1-P], and
+// decides whether a node can cross the surface.
+//
+// The update is a serial chain of FP64 instructions, each of which takes its
+// SM sub-partition 64 cycles (one lane or 32), so it is cut in three parts that
+// run on different warps (sub-partitions): update_move (translation, margin
+// test) and update_turn (rotation) side by side, then, after a block barrier,
+// update_stats.  In one warp the whole took 4.5 us at 128^3, alone.  Lane
+// a < 3 holds vector component a.
+//
 // p, s, Ai: the body's parameters, state of this step and accumulators (the
-// tables of B or copies of them); the results go to the tables of B.
-// Results go to *Ao (accumulators) and *So (the state of the next step); if
-// `out` is given, the new state and the re-classification flag are also
-// written there (lane a < 3: components a; lane 0: *out_reclass).  Out of
-// line, with its outputs behind pointers: a call with the outputs pointed at
-// scratch runs the same instructions (see k_body_fused).
+// tables of B or copies of them); the results go to *Ao (accumulators), *So
+// (the state of the next step) and *out (the same, in shared memory); lane 0
+// of update_move writes *flags (shared): kReclass, the body must re-classify,
+// and kHeld, it left the scheme and stays where it is.  Out of line, with the
+// outputs behind pointers: a call with the outputs pointed at scratch runs
+// the same instructions (see k_body_fused).
+constexpr int kReclass = 1, kHeld = 2;
 template <int P>
-__device__ __noinline__ void update_body(const Lattice& L, const Bodies& B, int k, const BodyParams& p,
+__device__ __noinline__ void update_move(const Lattice& L, const Bodies& B, int k, const BodyParams& p,
                                          const BodyState& s, const BodyAcc& Ai, const double* tot, BodyAcc* Ao,
-                                         BodyState* So, BodyState* out = nullptr, int* out_reclass = nullptr) {
+                                         BodyState* So, BodyState* out, int* flags) {
     const int lane = threadIdx.x & 31;
     const int a = lane < 3 ? lane : 0;  // lanes >= 3 shadow component 0 and store nothing
     const bool own = lane < 3;
     BodyAcc& A = *Ao;
     // Ladd's coupling averages the momentum exchange over this step and the
     // last (Sec. III names the option; the paper's runs leave it off).  Ai.Fbb
-    // and Ai.Tbb still hold the last step's values here (0 before a body's
-    // first step).
+    // still holds the last step's value here (0 before a body's first step).
     const double Fh = L.force_avg ? 0.5 * (tot[a] + Ai.Fbb[a]) : tot[a];
-    const double Th = L.force_avg ? 0.5 * (tot[3 + a] + Ai.Tbb[a]) : tot[3 + a];
-    const double Fa = Fh + Ai.Fc[a], Ta = Th + Ai.Tc[a];
-    const double rc = Ai.r_class[a], vs = Ai.vsum[a], ves = Ai.vesum;
-    const long long ns = Ai.nsum;
+    const double Fa = Fh + Ai.Fc[a];
+    const double rc = Ai.r_class[a];
     const unsigned long long mbits = Ai.margin_bits;
-    double v = s.vel[a], w = s.omega[a], x = s.pos[a], e = s.e[a];
+    double v = s.vel[a], x = s.pos[a];
     __syncwarp();
     if (own) {
         A.Fbb[a] = tot[a];
-        A.Tbb[a] = tot[3 + a];
-        A.Sbb[a] = tot[6 + a];
-        A.Sbb[3 + a] = tot[9 + a];
         A.Fapp[a] = Fa;
-        A.Tapp[a] = Ta;
         A.Fc[a] = 0.0;
-        A.Tc[a] = 0.0;
     }
-    int reclass = 0;
+    int reclass = 0, held = 0;
     if (p.kind == BODY_SPHERE && p.mobile) {
         const int n3[3] = {L.nx, L.ny, L.nz};
         double Fw = 0.0;  // WCA contact force, component a
         if (L.wca_eps != 0.0) {
             double fw[3] = {0.0, 0.0, 0.0};
-            if (lane == 0) wca_sum<P>(L, B, k, p, s, fw);
+            wca_sum<P>(L, B, k, p, s, fw);
             const double f0 = __shfl_sync(0xffffffffu, fw[0], 0), f1 = __shfl_sync(0xffffffffu, fw[1], 0),
                          f2 = __shfl_sync(0xffffffffu, fw[2], 0);
             Fw = a == 0 ? f0 : (a == 1 ? f1 : f2);
         }
         v = v + (Fa + Fw) * p.inv_mass;
-        w = w + Ta * p.inv_inertia;
         const double sp = sum3(v * v);
         // The geometry of the next step (node-crossing stencils, the near
         // window) assumes a move of under half a cell.  A body at |v| >= 1/2
@@ -441,8 +495,50 @@ __device__ __noinline__ void update_body(const Lattice& L, const Bodies& B, int 
             else if (x < 0.0) x += (double)n3[a];
         } else {
             v = 0.0;
-            w = 0.0;
+            held = kHeld;
+            if (lane == 0) set_error(L.err, 5);
         }
+        const double dd = min_image(x - rc, n3[a]);
+        const double disp2 = sum3(dd * dd);
+        // Node crossing test: every node of the box kept its side of the surface
+        // if the centre moved less than the distance of the nearest node to the
+        // surface at the last classification (less a 1e-9 guard, far above the
+        // FP64 error of the inside test).
+        const double mg = __longlong_as_double((long long)mbits) - 1e-9;
+        reclass = !(mg > 0.0 && disp2 < mg * mg);
+        __syncwarp();
+        if (reclass && lane == 0) A.margin_bits = (unsigned long long)__double_as_longlong(DBL_MAX);
+    }
+    if (own) {
+        So->pos[a] = out->pos[a] = x;
+        So->vel[a] = out->vel[a] = v;
+    }
+    if (lane == 0) {
+        A.reclass = reclass;
+        *flags = (reclass ? kReclass : 0) | held;
+    }
+    __syncwarp();
+}
+
+__device__ __noinline__ void update_turn(const Lattice& L, const BodyParams& p, const BodyState& s, const BodyAcc& Ai,
+                                         const double* tot, BodyAcc* Ao, BodyState* So, BodyState* out) {
+    const int lane = threadIdx.x & 31;
+    const int a = lane < 3 ? lane : 0;
+    const bool own = lane < 3;
+    BodyAcc& A = *Ao;
+    const double Th = L.force_avg ? 0.5 * (tot[3 + a] + Ai.Tbb[a]) : tot[3 + a];
+    const double Ta = Th + Ai.Tc[a];
+    double w = s.omega[a], e = s.e[a];
+    __syncwarp();
+    if (own) {
+        A.Tbb[a] = tot[3 + a];
+        A.Sbb[a] = tot[6 + a];
+        A.Sbb[3 + a] = tot[9 + a];
+        A.Tapp[a] = Ta;
+        A.Tc[a] = 0.0;
+    }
+    if (p.kind == BODY_SPHERE && p.mobile) {
+        w = w + Ta * p.inv_inertia;
         // Rotation of e about w by the angle th = |w| (Rodrigues), renormalised:
         //   e' = e cos(th) + (w x e) sin(th)/th + w (w.e) (1 - cos(th))/th^2.
         // A body turns by far less than 0.01 rad per step, where the Taylor
@@ -468,43 +564,32 @@ __device__ __noinline__ void update_body(const Lattice& L, const Bodies& B, int 
             const double inr = fabs(n2 - 1.0) < 1e-8 ? 1.5 - 0.5 * n2 : inv_sqrt(n2);
             e = r * inr;
         }
-        const double ve = sum3(v * e);
-        const double dd = min_image(x - rc, n3[a]);
-        const double disp2 = sum3(dd * dd);
-        __syncwarp();
-        if (own) A.vsum[a] = vs + v;
-        if (lane == 0) {
-            A.vesum = ves + ve;
-            A.nsum = ns + 1;
-            if (!ok) set_error(L.err, 5);
-        }
-        // Node crossing test: every node of the box kept its side of the surface
-        // if the centre moved less than the distance of the nearest node to the
-        // surface at the last classification (less a 1e-9 guard, far above the
-        // FP64 error of the inside test).
-        const double mg = __longlong_as_double((long long)mbits) - 1e-9;
-        reclass = !(mg > 0.0 && disp2 < mg * mg);
-        __syncwarp();
-        if (reclass && lane == 0) A.margin_bits = (unsigned long long)__double_as_longlong(DBL_MAX);
     }
-    BodyState& so = *So;
     if (own) {
-        so.pos[a] = x;
-        so.vel[a] = v;
-        so.omega[a] = w;
-        so.e[a] = e;
-        if (out) {
-            out->pos[a] = x;
-            out->vel[a] = v;
-            out->omega[a] = w;
-            out->e[a] = e;
-        }
-    }
-    if (lane == 0) {
-        A.reclass = reclass;
-        if (out_reclass) *out_reclass = reclass;
+        So->omega[a] = out->omega[a] = w;
+        So->e[a] = out->e[a] = e;
     }
     __syncwarp();
+}
+
+// After both and a block barrier, by one warp: the sums over the updates of v
+// and of v.e; a body held in place does not turn either.
+__device__ __forceinline__ void update_stats(const BodyParams& p, const BodyState& s, const BodyAcc& Ai, int flags,
+                                             BodyAcc* Ao, BodyState* So, BodyState* out) {
+    if (!(p.kind == BODY_SPHERE && p.mobile)) return;
+    const int lane = threadIdx.x & 31;
+    const int a = lane < 3 ? lane : 0;
+    if ((flags & kHeld) && lane < 3) {
+        So->omega[a] = out->omega[a] = 0.0;
+        So->e[a] = out->e[a] = s.e[a];
+    }
+    __syncwarp();
+    const double v = out->vel[a], ve = sum3(v * out->e[a]);
+    if (lane < 3) Ao->vsum[a] = Ai.vsum[a] + v;
+    if (lane == 0) {
+        Ao->vesum = Ai.vesum + ve;
+        Ao->nsum = Ai.nsum + 1;
+    }
 }
 
 // ---------------------------------------------------------------- k_links
@@ -547,165 +632,236 @@ __device__ __noinline__ double post_density(const Lattice& L, int64_t n, int x, 
     return L.rho0 + (double)r;
 }
 
-template <int P, bool DP>
-__device__ __forceinline__ void link_terms(const Lattice& L, const BodyParams& p, const BodyState& s, long long cnt,
-                                           const uint32_t* links, int g, int G, double (&acc)[12]) {
+// The g-th of G runs of the body's links, cnt / G each: every block has its
+// share however few links there are (handing whole blocks
+// of threads out first left most blocks of a small sphere idle: at R = 4, 1000
+// links sat on 4 of 15).
+__device__ __forceinline__ void link_range(long long cnt, int g, int G, int& l0, int& l1) {
+    const unsigned c = (unsigned)cnt, q = c / (unsigned)G, r = c % (unsigned)G;
+    l0 = (int)((unsigned)g * q + umin((unsigned)g, r));
+    l1 = l0 + (int)(q + ((unsigned)g < r ? 1u : 0u));
+}
+
+// A link's code taken apart: fluid node n = (x, y, z), direction i and the
+// solid node's cell ns.
+struct Link {
+    int64_t n, ns;
+    int x, y, z, i;
+};
+__device__ __forceinline__ Link link_of(const Lattice& L, uint32_t code) {
+    Link k;
+    k.n = code >> 5;
+    k.i = (int)(code & 31u);
+    cell_coords(L, k.n, k.x, k.y, k.z);
+    k.ns = cell_index(L, step_wrap(k.x, cx(k.i), L.nx), step_wrap(k.y, cy(k.i), L.ny), step_wrap(k.z, cz(k.i), L.nz));
+    return k;
+}
+
+// FP64 links of a sphere (FP64 storage) or a wall (any storage): acc takes
+// force (0..2) and, for a sphere, torque (3..5) and the negated stresslet, its
+// off-diagonal components doubled (6..11; sphere_totals).  A link's dF lies
+// along its direction, c_i sf with c in {-1, 0, 1}, so its nine products
+// d_a dF_b are selected from three; term by term they took twice the FP64
+// instructions.  Block g takes every G-th link: links all over the sphere,
+// whose large rest parts cancel within the block (runs of neighbouring links
+// tripled the rounding error of the stresslet at R = 7); the trace leaves each
+// link for the same reason.
+template <int P, bool SPHERE>
+__device__ __forceinline__ void link_terms64(const Lattice& L, const BodyParams& p, const BodyState& s, long long cnt,
+                                             const uint32_t* links, int g, int G, double (&acc)[12]) {
     const int64_t Np = L.Np;
-    const bool sphere = p.kind == BODY_SPHERE;
+    int ip[3];
+    double fp[3];
+    for (int a = 0; a < 3; ++a) {  // exact: the fraction of a coordinate
+        const double f = floor(s.pos[a]);
+        ip[a] = (int)f;
+        fp[a] = s.pos[a] - f;
+    }
+    const int n3[3] = {L.nx, L.ny, L.nz};
+    for (int l = g + G * (int)threadIdx.x; l < (int)cnt; l += G * (int)blockDim.x) {
+        const Link k = link_of(L, links[l]);
+        const int i = k.i, ib = opp(i);
+        const int ci[3] = {cx(i), cy(i), cz(i)};
+        // where sweep P left f*_i of the fluid node, and where the next sweep
+        // reads the reflected population f_ib of the fluid node
+        const int64_t out_slot = P == 0 ? (int64_t)ib * Np + k.n : (int64_t)i * Np + k.ns;
+        const int64_t in_slot = P == 0 ? (int64_t)i * Np + k.ns : (int64_t)ib * Np + k.n;
+        const double fout = load_abs(L, out_slot, i);
+        double d[3], cv;
+        if (SPHERE) {
+            // link midpoint (or boundary node) relative to the centre (minimum
+            // image: a link lies within R + 2 of it, less than half the box);
+            // rigid motion + slip there, along c: with n = d / |d|,
+            // c.v_b = c.v + w.(d x c) + (B1 + B2 e.n) ((e.n)(c.n) - c.e)
+            const int xi[3] = {k.x, k.y, k.z};
+            const double la = (double)L.link_at;
+            for (int a = 0; a < 3; ++a) {
+                int o = xi[a] - ip[a];
+                if (2 * o > n3[a]) o -= n3[a];
+                else if (2 * o <= -n3[a]) o += n3[a];
+                d[a] = ((double)o + csel(ci[a], la)) - fp[a];
+            }
+            const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+            const double ir = r2 > 0.0 ? rsqrt(r2) : 0.0;
+            const double ct = (s.e[0] * d[0] + s.e[1] * d[1] + s.e[2] * d[2]) * ir;
+            const double cn = (csel(ci[0], d[0]) + csel(ci[1], d[1]) + csel(ci[2], d[2])) * ir;
+            const double ce = csel(ci[0], s.e[0]) + csel(ci[1], s.e[1]) + csel(ci[2], s.e[2]);
+            const double slip = r2 > 0.0 ? (p.B1 + p.B2 * ct) * (ct * cn - ce) : 0.0;
+            const double rot = s.omega[0] * (csel(ci[2], d[1]) - csel(ci[1], d[2])) +
+                               s.omega[1] * (csel(ci[0], d[2]) - csel(ci[2], d[0])) +
+                               s.omega[2] * (csel(ci[1], d[0]) - csel(ci[0], d[1]));
+            cv = csel(ci[0], s.vel[0]) + csel(ci[1], s.vel[1]) + csel(ci[2], s.vel[2]) + (rot + slip);
+        } else {
+            cv = csel(ci[0], p.wall_vel[0]) + csel(ci[1], p.wall_vel[1]) + csel(ci[2], p.wall_vel[2]);
+        }
+        const double rs = L.rho_local ? post_density<P>(L, k.n, k.x, k.y, k.z) : L.rho0;
+        const double fin = fout - 6.0 * rs * wgt(i) * cv;
+        store_abs(L, in_slot, ib, fin);
+        // momentum given to the body, c_i (f_out + f_in)
+        const double sf = fout + fin;
+        const double dF[3] = {csel(ci[0], sf), csel(ci[1], sf), csel(ci[2], sf)};
+        for (int a = 0; a < 3; ++a) acc[a] += dF[a];
+        if (SPHERE) {
+            const double m[3] = {d[0] * sf, d[1] * sf, d[2] * sf};
+            const double tr = (csel(ci[0], m[0]) + csel(ci[1], m[1]) + csel(ci[2], m[2])) * (1.0 / 3.0);
+            for (int a = 0; a < 3; ++a) {
+                acc[6 + a] += csel(ci[a], m[a]) - tr;
+                const int b = a == 2 ? 0 : a + 1;  // (0,1), (1,2), (2,0)
+                const double ab = csel(ci[b], m[a]), ba = csel(ci[a], m[b]);
+                acc[3 + (a == 2 ? 1 : (a == 0 ? 2 : 0))] += ab - ba;  // torque component 2, 0, 1
+                acc[9 + (a == 2 ? 1 : (a == 0 ? 0 : 2))] += ab + ba;  // xy, yz, xz
+            }
+        }
+    }
+}
+
+// Links of a sphere in reduced storage: deviations g = f - w rho0 in FP32,
+// each term of force, torque and stresslet an FP32 number, summed as pairs
+// (block_sum_fixed).
+template <int P>
+__device__ __forceinline__ void link_terms32(const Lattice& L, const BodyParams& p, const BodyState& s, long long cnt,
+                                             const uint32_t* links, int g, int G, df (&acc)[12]) {
+    const int64_t Np = L.Np;
     // body position split into integer and fraction, so that FP32 link
     // offsets keep full precision far from the origin
     int ip[3];
     float fp[3], e32[3], v32[3], w32[3];
-    if (!DP) {
-        for (int a = 0; a < 3; ++a) {
-            ip[a] = (int)floor(s.pos[a]);
-            fp[a] = (float)(s.pos[a] - (double)ip[a]);
-            e32[a] = (float)s.e[a];
-            v32[a] = (float)s.vel[a];
-            w32[a] = (float)s.omega[a];
-        }
+    for (int a = 0; a < 3; ++a) {
+        ip[a] = (int)floor(s.pos[a]);
+        fp[a] = (float)(s.pos[a] - (double)ip[a]);
+        e32[a] = (float)s.e[a];
+        v32[a] = (float)s.vel[a];
+        w32[a] = (float)s.omega[a];
     }
     const float B1f = (float)p.B1, B2f = (float)p.B2, shf0 = (float)(6.0 * L.rho0), lat = L.link_at;
+    int l0, l1;
+    link_range(cnt, g, G, l0, l1);
     // A thread's links are taken kU at a time: the link codes, then the
     // outgoing populations of all kU are loaded before any arithmetic or
     // store, so their memory latencies overlap.
     constexpr int kU = 2;
-    const long long stride = (long long)G * blockDim.x;
-    for (long long l0 = (long long)g * blockDim.x + threadIdx.x; l0 < cnt; l0 += kU * stride) {
-    uint32_t codes[kU];
-    double fouts[kU];
+    const int stride = (int)blockDim.x;
+    for (int lb = l0 + (int)threadIdx.x; lb < l1; lb += kU * stride) {
+    Link lk[kU];
     float gouts[kU];
+    uint32_t codes[kU];
 #pragma unroll
-    for (int u = 0; u < kU; ++u) codes[u] = l0 + u * stride < cnt ? links[l0 + u * stride] : 0u;
+    for (int u = 0; u < kU; ++u) codes[u] = lb + u * stride < l1 ? links[lb + u * stride] : 0u;
 #pragma unroll
     for (int u = 0; u < kU; ++u) {
-        if (l0 + u * stride >= cnt) continue;
-        const int64_t n = codes[u] >> 5;
-        const int i = codes[u] & 31;
-        int x, y, z;
-        cell_coords(L, n, x, y, z);
-        const int64_t ns =
-            cell_index(L, step_wrap(x, cx(i), L.nx), step_wrap(y, cy(i), L.ny), step_wrap(z, cz(i), L.nz));
-        const int64_t out_slot = P == 0 ? (int64_t)opp(i) * Np + n : (int64_t)i * Np + ns;
-        if (DP || !sphere) fouts[u] = load_abs(L, out_slot, i);
-        else gouts[u] = load_dev(L, out_slot);
+        if (lb + u * stride >= l1) continue;
+        lk[u] = link_of(L, codes[u]);
+        const int i = lk[u].i;
+        gouts[u] = load_dev(L, P == 0 ? (int64_t)opp(i) * Np + lk[u].n : (int64_t)i * Np + lk[u].ns);
     }
 #pragma unroll
     for (int u = 0; u < kU; ++u) {
-        if (l0 + u * stride >= cnt) continue;
-        const uint32_t code = codes[u];
-        const int64_t n = code >> 5;
-        const int i = code & 31, ib = opp(i);
+        if (lb + u * stride >= l1) continue;
+        const int64_t n = lk[u].n, ns = lk[u].ns;
+        const int i = lk[u].i, ib = opp(i), x = lk[u].x, y = lk[u].y, z = lk[u].z;
         const int ci[3] = {cx(i), cy(i), cz(i)};
-        int x, y, z;
-        cell_coords(L, n, x, y, z);
-        const int64_t ns =
-            cell_index(L, step_wrap(x, ci[0], L.nx), step_wrap(y, ci[1], L.ny), step_wrap(z, ci[2], L.nz));
-        // where sweep P left f*_i of the fluid node (loaded above), and where
-        // the next sweep reads the reflected population f_ib of the fluid node
         const int64_t in_slot = P == 0 ? (int64_t)i * Np + ns : (int64_t)ib * Np + n;
-        if (DP || !sphere) {
-            const double fout = fouts[u];
-            double vb[3], d[3];
-            if (sphere) {
-                // link midpoint (or boundary node) relative to the centre; rigid motion + slip there
-                const double la = (double)L.link_at;
-                d[0] = min_image(((double)x + la * ci[0]) - s.pos[0], L.nx);
-                d[1] = min_image(((double)y + la * ci[1]) - s.pos[1], L.ny);
-                d[2] = min_image(((double)z + la * ci[2]) - s.pos[2], L.nz);
-                const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-                double sl[3] = {0.0, 0.0, 0.0};
-                if (r2 > 0.0) {
-                    const double ir = 1.0 / sqrt(r2);
-                    const double n0 = d[0] * ir, n1 = d[1] * ir, n2 = d[2] * ir;
-                    const double ct = s.e[0] * n0 + s.e[1] * n1 + s.e[2] * n2;
-                    const double a = p.B1 + p.B2 * ct;
-                    sl[0] = a * (ct * n0 - s.e[0]);
-                    sl[1] = a * (ct * n1 - s.e[1]);
-                    sl[2] = a * (ct * n2 - s.e[2]);
-                }
-                double w[3];
-                cross3(s.omega, d, w);
-                for (int a = 0; a < 3; ++a) vb[a] = s.vel[a] + w[a] + sl[a];
-            } else {
-                for (int a = 0; a < 3; ++a) vb[a] = p.wall_vel[a];
-            }
-            const double cv = csel(ci[0], vb[0]) + csel(ci[1], vb[1]) + csel(ci[2], vb[2]);
-            const double rs = L.rho_local ? post_density<P>(L, n, x, y, z) : L.rho0;
-            const double fin = fout - 6.0 * rs * wgt(i) * cv;
-            store_abs(L, in_slot, ib, fin);
-            // momentum given to the body, c_i (f_out + f_in); torque, stresslet
-            const double sf = fout + fin;
-            const double dF[3] = {csel(ci[0], sf), csel(ci[1], sf), csel(ci[2], sf)};
-            acc[0] += dF[0];
-            acc[1] += dF[1];
-            acc[2] += dF[2];
-            if (sphere) {
-                acc[3] += d[1] * dF[2] - d[2] * dF[1];
-                acc[4] += d[2] * dF[0] - d[0] * dF[2];
-                acc[5] += d[0] * dF[1] - d[1] * dF[0];
-                const double tr = (d[0] * dF[0] + d[1] * dF[1] + d[2] * dF[2]) * (1.0 / 3.0);
-                acc[6] -= d[0] * dF[0] - tr;
-                acc[7] -= d[1] * dF[1] - tr;
-                acc[8] -= d[2] * dF[2] - tr;
-                acc[9] -= 0.5 * (d[0] * dF[1] + d[1] * dF[0]);
-                acc[10] -= 0.5 * (d[0] * dF[2] + d[2] * dF[0]);
-                acc[11] -= 0.5 * (d[1] * dF[2] + d[2] * dF[1]);
-            }
-        } else {
-            // FP32 path (reduced storage, sphere): deviations g = f - w rho0
-            const float gout = gouts[u];
-            float d[3];
-            const int xi[3] = {x, y, z};
-            const int n3[3] = {L.nx, L.ny, L.nz};
-            for (int a = 0; a < 3; ++a) {
-                float t = (float)(xi[a] - ip[a]) + (lat * (float)ci[a] - fp[a]);
-                const float h = 0.5f * (float)n3[a];
-                if (t > h) t -= (float)n3[a];
-                else if (t <= -h) t += (float)n3[a];
-                d[a] = t;
-            }
-            const float r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-            float sl[3] = {0.0f, 0.0f, 0.0f};
-            if (r2 > 0.0f) {
-                const float ir = rsqrtf(r2);
-                const float n0 = d[0] * ir, n1 = d[1] * ir, n2 = d[2] * ir;
-                const float ct = e32[0] * n0 + e32[1] * n1 + e32[2] * n2;
-                const float a = B1f + B2f * ct;
-                sl[0] = a * (ct * n0 - e32[0]);
-                sl[1] = a * (ct * n1 - e32[1]);
-                sl[2] = a * (ct * n2 - e32[2]);
-            }
-            const float vb0 = v32[0] + (w32[1] * d[2] - w32[2] * d[1]) + sl[0];
-            const float vb1 = v32[1] + (w32[2] * d[0] - w32[0] * d[2]) + sl[1];
-            const float vb2 = v32[2] + (w32[0] * d[1] - w32[1] * d[0]) + sl[2];
-            const float cv = (ci[0] > 0 ? vb0 : (ci[0] < 0 ? -vb0 : 0.0f)) +
-                             (ci[1] > 0 ? vb1 : (ci[1] < 0 ? -vb1 : 0.0f)) +
-                             (ci[2] > 0 ? vb2 : (ci[2] < 0 ? -vb2 : 0.0f));
-            const float shf = L.rho_local ? (float)(6.0 * post_density<P>(L, n, x, y, z)) : shf0;
-            const float gin = gout - shf * (float)wgt(i) * cv;
-            store_dev(L, in_slot, gin);
-            const float sf = gout + gin;
-            const float dF[3] = {ci[0] > 0 ? sf : (ci[0] < 0 ? -sf : 0.0f), ci[1] > 0 ? sf : (ci[1] < 0 ? -sf : 0.0f),
-                                 ci[2] > 0 ? sf : (ci[2] < 0 ? -sf : 0.0f)};
-            const float tr = (d[0] * dF[0] + d[1] * dF[1] + d[2] * dF[2]) * (1.0f / 3.0f);
-            const float t12[12] = {dF[0],
-                                   dF[1],
-                                   dF[2],
-                                   d[1] * dF[2] - d[2] * dF[1],
-                                   d[2] * dF[0] - d[0] * dF[2],
-                                   d[0] * dF[1] - d[1] * dF[0],
-                                   -(d[0] * dF[0] - tr),
-                                   -(d[1] * dF[1] - tr),
-                                   -(d[2] * dF[2] - tr),
-                                   -0.5f * (d[0] * dF[1] + d[1] * dF[0]),
-                                   -0.5f * (d[0] * dF[2] + d[2] * dF[0]),
-                                   -0.5f * (d[1] * dF[2] + d[2] * dF[1])};
+        const float gout = gouts[u];
+        float d[3];
+        const int xi[3] = {x, y, z};
+        const int n3[3] = {L.nx, L.ny, L.nz};
+        for (int a = 0; a < 3; ++a) {
+            float t = (float)(xi[a] - ip[a]) + (lat * (float)ci[a] - fp[a]);
+            const float h = 0.5f * (float)n3[a];
+            if (t > h) t -= (float)n3[a];
+            else if (t <= -h) t += (float)n3[a];
+            d[a] = t;
+        }
+        const float r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+        float sl[3] = {0.0f, 0.0f, 0.0f};
+        if (r2 > 0.0f) {
+            const float ir = rsqrtf(r2);
+            const float n0 = d[0] * ir, n1 = d[1] * ir, n2 = d[2] * ir;
+            const float ct = e32[0] * n0 + e32[1] * n1 + e32[2] * n2;
+            const float a = B1f + B2f * ct;
+            sl[0] = a * (ct * n0 - e32[0]);
+            sl[1] = a * (ct * n1 - e32[1]);
+            sl[2] = a * (ct * n2 - e32[2]);
+        }
+        const float vb0 = v32[0] + (w32[1] * d[2] - w32[2] * d[1]) + sl[0];
+        const float vb1 = v32[1] + (w32[2] * d[0] - w32[0] * d[2]) + sl[1];
+        const float vb2 = v32[2] + (w32[0] * d[1] - w32[1] * d[0]) + sl[2];
+        const float cv = (ci[0] > 0 ? vb0 : (ci[0] < 0 ? -vb0 : 0.0f)) +
+                         (ci[1] > 0 ? vb1 : (ci[1] < 0 ? -vb1 : 0.0f)) +
+                         (ci[2] > 0 ? vb2 : (ci[2] < 0 ? -vb2 : 0.0f));
+        const float shf = L.rho_local ? (float)(6.0 * post_density<P>(L, n, x, y, z)) : shf0;
+        const float gin = gout - shf * (float)wgt(i) * cv;
+        store_dev(L, in_slot, gin);
+        const float sf = gout + gin;
+        const float dF[3] = {ci[0] > 0 ? sf : (ci[0] < 0 ? -sf : 0.0f), ci[1] > 0 ? sf : (ci[1] < 0 ? -sf : 0.0f),
+                             ci[2] > 0 ? sf : (ci[2] < 0 ? -sf : 0.0f)};
+        const float tr = (d[0] * dF[0] + d[1] * dF[1] + d[2] * dF[2]) * (1.0f / 3.0f);
+        const float t12[12] = {dF[0],
+                               dF[1],
+                               dF[2],
+                               d[1] * dF[2] - d[2] * dF[1],
+                               d[2] * dF[0] - d[0] * dF[2],
+                               d[0] * dF[1] - d[1] * dF[0],
+                               -(d[0] * dF[0] - tr),
+                               -(d[1] * dF[1] - tr),
+                               -(d[2] * dF[2] - tr),
+                               -0.5f * (d[0] * dF[1] + d[1] * dF[0]),
+                               -0.5f * (d[0] * dF[2] + d[2] * dF[0]),
+                               -0.5f * (d[1] * dF[2] + d[2] * dF[1])};
 #pragma unroll
-            for (int c = 0; c < 12; ++c) acc[c] += (double)t12[c];
+        for (int c = 0; c < 12; ++c) {
+            const df t = two_sum(acc[c].h, t12[c]);
+            acc[c] = {t.h, __fadd_rn(acc[c].l, t.l)};
         }
     }
     }
+}
+
+// A block's share of a sphere's links and the block's sums in tot (shared):
+// force, torque and stresslet, or what link_terms64 sums (FP64 storage).
+// none: the block takes no links (zero sums).
+template <int P, int T>
+__device__ __forceinline__ void sphere_links(const Lattice& L, const BodyParams& p, const BodyState& s, long long cnt,
+                                             const uint32_t* links, int g, int G, bool none, double* sm, double* tot) {
+    if (L.storage == ST_F64) {
+        double acc[12];
+#pragma unroll
+        for (int c = 0; c < 12; ++c) acc[c] = 0.0;
+        if (!none) link_terms64<P, true>(L, p, s, cnt, links, g, G, acc);
+        block_sum_fixed<12, T>(acc, sm, tot);
+    } else {
+        df acc[12];
+#pragma unroll
+        for (int c = 0; c < 12; ++c) acc[c] = {0.0f, 0.0f};
+        if (!none) link_terms32<P>(L, p, s, cnt, links, g, G, acc);
+        block_sum_fixed<12, T>(acc, sm, tot);
+    }
+}
+
+// The body's totals tot[12] from the sums over its blocks, in place, by
+// threads 0..11.
+__device__ __forceinline__ void sphere_totals(const Lattice& L, double* tot) {
+    if (L.storage == ST_F64 && threadIdx.x >= 6) tot[threadIdx.x] *= threadIdx.x < 9 ? -1.0 : -0.5;
 }
 
 // Links of a still body with no force readout: out slot copied to in slot in
@@ -734,6 +890,7 @@ template <int P>
 __global__ void __launch_bounds__(kLB) k_links(const Bodies B) {
     __shared__ double sm[12 * kLB + 12 * 8];
     __shared__ double s_tot[12];
+    __shared__ BodyState s_new;
     __shared__ int s_flag;
     const int nitems = *B.n_link_items;
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
@@ -750,23 +907,36 @@ __global__ void __launch_bounds__(kLB) k_links(const Bodies B) {
             copy_links<P>(L, A.link_count, B.links + p.link_off, g, G);
             continue;
         }
-        double acc[12];
+        const BodyState& s = B.state[P][k];
+        const uint32_t* links = B.links + p.link_off;
+        double* parts = B.part_links + (size_t)k * B.GL * 12;
+        if (p.kind == BODY_SPHERE) {
+            sphere_links<P, kLB>(L, p, s, A.link_count, links, g, G, false, sm, s_tot);
+            if (threadIdx.x < 12) parts[g * 12 + threadIdx.x] = s_tot[threadIdx.x];
+        } else {  // a wall: its force only
+            double acc[12];
 #pragma unroll
-        for (int c = 0; c < 12; ++c) acc[c] = 0.0;
-        if (L.storage == ST_F64)
-            link_terms<P, true>(L, p, B.state[P][k], A.link_count, B.links + p.link_off, g, G, acc);
-        else
-            link_terms<P, false>(L, p, B.state[P][k], A.link_count, B.links + p.link_off, g, G, acc);
-        block_sum_fixed<12, kLB>(acc, sm, s_tot);
-        double* part = B.part_links + ((size_t)k * B.GL + g) * 12;
-        if (threadIdx.x < 12) part[threadIdx.x] = s_tot[threadIdx.x];
+            for (int c = 0; c < 3; ++c) acc[c] = 0.0;
+            link_terms64<P, false>(L, p, s, A.link_count, links, g, G, acc);
+            double F[3] = {acc[0], acc[1], acc[2]};
+            block_sum_fixed<3, kLB>(F, sm, s_tot);
+            if (threadIdx.x < 3) parts[g * 12 + threadIdx.x] = s_tot[threadIdx.x];
+        }
         if (!last_block(&A.counter_links, G, &s_flag)) continue;
-        ordered_partial_sum<12>(B.part_links + (size_t)k * B.GL * 12, G, sm, s_tot);
-        if (threadIdx.x < 32) update_body<P>(L, B, k, p, B.state[P][k], A, s_tot, &A, &B.state[1 - P][k]);
+        if (p.kind == BODY_SPHERE) {
+            ordered_partial_sum<12>(parts, G, sm, s_tot);
+            if (threadIdx.x < 12) sphere_totals(L, s_tot);
+            __syncthreads();
+        } else {
+            ordered_partial_sum<3>(parts, G, sm, s_tot, 12);
+            if (threadIdx.x >= 3 && threadIdx.x < 12) s_tot[threadIdx.x] = 0.0;
+            __syncthreads();
+        }
+        if (threadIdx.x < 32) update_move<P>(L, B, k, p, s, A, s_tot, &A, &B.state[1 - P][k], &s_new, &s_flag);
+        else if (threadIdx.x < 64) update_turn(L, p, s, A, s_tot, &A, &B.state[1 - P][k], &s_new);
         __syncthreads();
-        if (threadIdx.x == 0) s_flag = A.reclass;
-        __syncthreads();
-        if (s_flag) append_items(B.box_items, B.n_box, B.box_cap, k, p.g_box, B.err, (int*)sm);
+        if (threadIdx.x >= 64 && threadIdx.x < 96) update_stats(p, s, A, s_flag, &A, &B.state[1 - P][k], &s_new);
+        if (s_flag & kReclass) append_items(B.box_items, B.n_box, B.box_cap, k, p.g_box, B.err, (int*)sm);
         __syncthreads();
     }
 }
@@ -1098,7 +1268,7 @@ __device__ __noinline__ void refill_cell(const Lattice& L, const BodyState& s, i
 
 template <int P>
 __global__ void __launch_bounds__(kBB) k_convert(const Bodies B) {
-    __shared__ double sm[6 * kBB + 6 * 8];
+    __shared__ double sm[6 * kBB + 6 * 16];
     __shared__ double s_tot[6];
     __shared__ long long sml[kBB];
     __shared__ int s_list[kBB], s_scan[kBB / 32 + 1], s_flag;
@@ -1495,7 +1665,7 @@ __global__ void __launch_bounds__(kFT, 2) k_body_fused(const Bodies B, int cls, 
     const int KC = (int)cl.num_blocks();
     const int rank = (int)cl.block_rank();
     const int cid = blockIdx.x / KC, ncl = gridDim.x / KC;
-    __shared__ double sm[12 * kFT + 12 * 8];
+    __shared__ double sm[12 * kFT + 12 * 16];
     __shared__ double s_tot[12], s_conv[6];
     __shared__ Lattice s_L;
     __shared__ BodyParams s_p;
@@ -1503,7 +1673,7 @@ __global__ void __launch_bounds__(kFT, 2) k_body_fused(const Bodies B, int cls, 
     __shared__ BodyAcc s_A, s_dryA;
     __shared__ BodyState s_dryS, s_dryS2;
     __shared__ double s_zero[12];
-    __shared__ int s_dryMode;
+    __shared__ int s_dryMode, s_flags;
     __shared__ ShellGeo s_geo;
     __shared__ uint32_t s_stc[kStcBuf];
     __shared__ uint32_t s_emask[kStcBuf];  // phase A's link mask of each stencil entry, for phase B
@@ -1514,14 +1684,15 @@ __global__ void __launch_bounds__(kFT, 2) k_body_fused(const Bodies B, int cls, 
     __shared__ int s_scan[kFT / 32 + 1], s_list[kFT], s_mode, s_base;
     __shared__ float s_min[kFT / 32], s_margin;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int i0 = B.fused_first[cls], nitems = B.n_fused[cls];
+    // tail: the lattice holds one sphere and nothing else, item (0, 0)
+    const int i0 = tail ? 0 : B.fused_first[cls], nitems = tail ? 1 : B.n_fused[cls];
     if (threadIdx.x < 12) s_zero[threadIdx.x] = 0.0;
     if (threadIdx.x == 0) s_updated = 0;
     for (int it = cid; it < nitems; it += ncl) {
         // everything of this body and lattice that the step reads, in one go
         // (the sweep streams the whole lattice through L2 between two steps,
         // so these tables come from HBM)
-        const int2 item = B.fused_items[i0 + it];
+        const int2 item = tail ? make_int2(0, 0) : B.fused_items[i0 + it];
         const int k = item.x;
         __syncthreads();  // the previous item's readers of the copies are done
         copy_words(&s_L, B.lats + item.y, sizeof(Lattice));
@@ -1540,22 +1711,17 @@ __global__ void __launch_bounds__(kFT, 2) k_body_fused(const Bodies B, int cls, 
         for (long long b = b0 + threadIdx.x; b < b1 && b < b0 + kStcBuf; b += kFT) s_stc[b - b0] = __ldg(stc + b);
 
         // ---- bounce-back and momentum exchange on the links (as k_links), by
-        // ranks 1 .. KC-1.  Meanwhile warp 0 of rank 0 runs the update once on
-        // scratch: its code is cold every step (the sweep streams the lattice
+        // ranks 1 .. KC-1.  Meanwhile warps 0 and 1 of rank 0 run the update once
+        // on scratch: its code is cold every step (the sweep streams the lattice
         // through L2 between steps), and the real update after the reduction
         // then runs warm.  The scratch call writes only shared memory.
-        double acc[12];
-#pragma unroll
-        for (int c = 0; c < 12; ++c) acc[c] = 0.0;
         if (rank == 0) {
             if (threadIdx.x < 32)
-                update_body<P>(L, B, k, p, s0, s_A, s_zero, &s_dryA, &s_dryS, &s_dryS2, &s_dryMode);
-        } else if (L.storage == ST_F64) {
-            link_terms<P, true>(L, p, s0, s_A.link_count, B.links + p.link_off, rank - 1, KC - 1, acc);
-        } else {
-            link_terms<P, false>(L, p, s0, s_A.link_count, B.links + p.link_off, rank - 1, KC - 1, acc);
+                update_move<P>(L, B, k, p, s0, s_A, s_zero, &s_dryA, &s_dryS, &s_dryS2, &s_dryMode);
+            else if (threadIdx.x < 64)
+                update_turn(L, p, s0, s_A, s_zero, &s_dryA, &s_dryS, &s_dryS2);
         }
-        block_sum_fixed<12, kFT>(acc, sm, s_tot);
+        sphere_links<P, kFT>(L, p, s0, s_A.link_count, B.links + p.link_off, rank - 1, KC - 1, rank == 0, sm, s_tot);
         int near = 0;
         if (rank == 0)
             for (int j = L.body_begin + threadIdx.x; j < L.body_begin + L.body_count; j += kFT)
@@ -1566,17 +1732,30 @@ __global__ void __launch_bounds__(kFT, 2) k_body_fused(const Bodies B, int cls, 
             // the blocks' partial sums, all fetched at once, then summed in rank order
             if (threadIdx.x < 12 * KC) sm[threadIdx.x] = cl.map_shared_rank(s_tot, threadIdx.x / 12)[threadIdx.x % 12];
             __syncthreads();
-            if (threadIdx.x < 12) {
-                double t = 0.0;
-                for (int r = 0; r < KC; ++r) t += sm[r * 12 + threadIdx.x];
+            // four runs of KC / 4 ranks per component, then the four sums
+            const int run = KC / 4;
+            if (threadIdx.x < 48) {
+                const int c = threadIdx.x % 12, r0 = (threadIdx.x / 12) * run;
+                double t = sm[r0 * 12 + c];
+                for (int r = r0 + 1; r < r0 + run; ++r) t += sm[r * 12 + c];
                 sm[12 * KC + threadIdx.x] = t;
             }
             __syncthreads();
-            if (threadIdx.x < 32)
-                update_body<P>(L, B, k, p, s0, s_A, sm + 12 * KC, &B.acc[k], &B.state[1 - P][k], &s_new, &s_mode);
+            if (threadIdx.x < 12) {
+                const double* q4 = sm + 12 * KC + threadIdx.x;
+                s_tot[threadIdx.x] = (q4[0] + q4[12]) + (q4[24] + q4[36]);
+                sphere_totals(L, s_tot);
+            }
             __syncthreads();
+            if (threadIdx.x < 32)
+                update_move<P>(L, B, k, p, s0, s_A, s_tot, &B.acc[k], &B.state[1 - P][k], &s_new, &s_flags);
+            else if (threadIdx.x < 64)
+                update_turn(L, p, s0, s_A, s_tot, &B.acc[k], &B.state[1 - P][k], &s_new);
+            __syncthreads();
+            if (threadIdx.x >= 64 && threadIdx.x < 96)
+                update_stats(p, s0, s_A, s_flags, &B.acc[k], &B.state[1 - P][k], &s_new);
             if (threadIdx.x == 0) {
-                s_mode = s_mode ? (near ? 2 : 1) : 0;
+                s_mode = s_flags & kReclass ? (near ? 2 : 1) : 0;
                 s_updated = 1;
             }
             __syncthreads();
@@ -1946,8 +2125,9 @@ __global__ void __launch_bounds__(kBB) k_psm_clear(const Bodies B, int P) {
 
 template <int P, class V>
 __global__ void __launch_bounds__(kBB, 2) k_psm_cover(const Bodies B) {
-    __shared__ double sm[12 * kBB + 12 * 8];
+    __shared__ double sm[12 * kBB + 12 * 16];
     __shared__ double s_tot[12];
+    __shared__ BodyState s_new;
     __shared__ int s_flag;
     __shared__ int s_w[kBB / 32];
     __shared__ int s_list[kBB];
@@ -2033,7 +2213,10 @@ __global__ void __launch_bounds__(kBB, 2) k_psm_cover(const Bodies B) {
         if (threadIdx.x < 12) B.part_psm[chunk * 12 + threadIdx.x] = s_tot[threadIdx.x];
         if (!last_block(&A.counter_links, psm_chunks(p), &s_flag)) continue;
         ordered_sum_staged<12>(B.part_psm + (p.psm_off / kBB) * 12, psm_chunks(p), sm, s_tot);
-        if (threadIdx.x < 32) update_body<P>(L, B, k, p, s, A, s_tot, &A, &B.state[1 - P][k]);
+        if (threadIdx.x < 32) update_move<P>(L, B, k, p, s, A, s_tot, &A, &B.state[1 - P][k], &s_new, &s_flag);
+        else if (threadIdx.x < 64) update_turn(L, p, s, A, s_tot, &A, &B.state[1 - P][k], &s_new);
+        __syncthreads();
+        if (threadIdx.x < 32) update_stats(p, s, A, s_flag, &A, &B.state[1 - P][k], &s_new);
         __syncthreads();
     }
 }
