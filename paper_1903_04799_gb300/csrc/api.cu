@@ -15,12 +15,11 @@
 
 namespace lbsq {
 void launch_sweep(const Lattice& L, double lambda_e, double lambda_o, int parity, int variant, int zmode,
-                  const int* win, int gz, int gy, cudaStream_t st);
+                  const int* win, int gz, int gy, cudaStream_t st, bool dep = false);
 void launch_body_kernel(int which, const Bodies& B, int parity, int grid_links, int grid_box, long long* step,
-                        cudaStream_t st);
-void launch_body_step(const Bodies& B, int parity, int grid_links, int grid_box, long long* step, cudaStream_t st);
+                        cudaStream_t st, bool dep = false);
 void launch_body_fused(const Bodies& B, int parity, int cls, int clusters, cudaStream_t st, int tail,
-                       cudaEvent_t started = nullptr);
+                       bool dep = false, cudaEvent_t started = nullptr);
 cudaError_t prepare_body_kernels();
 void launch_fill_rest(const Lattice& L, cudaStream_t st);
 void launch_set_eq(const Lattice& L, const double* rho, const double* u, int q, cudaStream_t st);
@@ -124,6 +123,8 @@ struct lb_ctx {
     // the far sweep on `side`, the body kernels on `hi` (highest priority, so
     // that SM slots freed by sweep blocks go to the short body kernels first)
     cudaStream_t side = nullptr, hi = nullptr;
+    cudaStream_t wall = nullptr;  // the link kernel of walls beside the fused kernel (see body_step)
+    cudaEvent_t ev_wall = nullptr, ev_wall2 = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr;
     cudaEvent_t ev_started = nullptr;  // every block of the fused body kernel has begun (see enqueue_unit)
     int* d_win = nullptr;  // [4][4] near-body windows (z0, z length, y0, y length) by step (mod 4)
@@ -705,6 +706,9 @@ lb_status lb_create(const lb_params* p, lb_ctx** out) {
     if (cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi) != cudaSuccess) return bail(LB_ERR_CUDA);
     if (cudaStreamCreateWithPriority(&c->side, cudaStreamNonBlocking, prio_lo) != cudaSuccess ||
         cudaStreamCreateWithPriority(&c->hi, cudaStreamNonBlocking, prio_hi) != cudaSuccess ||
+        cudaStreamCreateWithPriority(&c->wall, cudaStreamNonBlocking, prio_hi) != cudaSuccess ||
+        cudaEventCreateWithFlags(&c->ev_wall, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&c->ev_wall2, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_join2, cudaEventDisableTiming) != cudaSuccess ||
@@ -740,7 +744,9 @@ lb_status lb_destroy(lb_ctx* c) {
     if (c->ev_join) cudaEventDestroy(c->ev_join);
     if (c->ev_join2) cudaEventDestroy(c->ev_join2);
     if (c->ev_started) cudaEventDestroy(c->ev_started);
-    for (cudaStream_t st : {c->side, c->hi})
+    if (c->ev_wall) cudaEventDestroy(c->ev_wall);
+    if (c->ev_wall2) cudaEventDestroy(c->ev_wall2);
+    for (cudaStream_t st : {c->side, c->hi, c->wall})
         if (st) {
             cudaStreamSynchronize(st);
             cudaStreamDestroy(st);
@@ -1049,8 +1055,9 @@ static cudaEvent_t pool_event(lb_ctx* c, size_t k) {
     return c->ev_pool[k];
 }
 
-static void sweep_all(lb_ctx* c, int parity, cudaStream_t st) {
-    launch_sweep(c->L, c->lambda_e, c->lambda_o, parity, c->sweep_variant, 0, nullptr, c->L.nz, c->L.ny, st);
+// dep: the last operation on st is a kernel (see dep_wait).
+static void sweep_all(lb_ctx* c, int parity, cudaStream_t st, bool dep = false) {
+    launch_sweep(c->L, c->lambda_e, c->lambda_o, parity, c->sweep_variant, 0, nullptr, c->L.nz, c->L.ny, st, dep);
 }
 
 // The sweep of a lattice with partially saturated cells: before it the
@@ -1074,22 +1081,46 @@ static int psm_sweep(lb_ctx* c, const Bodies& B, int parity, cudaStream_t st) {
 // another body) and end the step; for a lattice with a single sphere and no
 // other body, the fused kernel alone.  Returns the launch count.
 // started: recorded when every block of the fused kernel has begun (if it is
-// launched: c->solo or c->n_fused > 0).
-static int body_step(lb_ctx* c, const Bodies& B, int parity, cudaStream_t st, cudaEvent_t started = nullptr) {
+// launched: c->solo or c->n_fused > 0).  dep: the last operation on st is a
+// kernel, so the first kernel here may be a dependent launch (see dep_wait);
+// the others follow kernels of this step.
+//
+// The link kernel (walls and still obstacles) and the fused kernel run side by
+// side: links of different bodies touch different slots, and a sphere that
+// converts cells in the fused kernel has no wall within its box grown by two
+// cells (one that has is only queued there, and converts in the kernels that
+// follow both).
+static int body_step(lb_ctx* c, const Bodies& B, int parity, cudaStream_t st, bool dep = false,
+                     cudaEvent_t started = nullptr) {
     if (c->solo) {  // the fused kernel is the whole body step
-        launch_body_fused(B, parity, c->fused_cls, 1, st, 1, started);
+        launch_body_fused(B, parity, c->fused_cls, 1, st, 1, dep, started);
         return 1;
     }
     int n = 0;
+    const bool both = c->n_fused > 0 && c->n_link_items > 0;
+    if (both) {
+        cudaEventRecord(c->ev_wall, st);
+        cudaStreamWaitEvent(c->wall, c->ev_wall, 0);
+    }
     if (c->n_fused > 0) {
-        launch_body_fused(B, parity, c->fused_cls, c->n_fused, st, 0, started);
+        launch_body_fused(B, parity, c->fused_cls, c->n_fused, st, 0, dep, started);
+        dep = true;
         n++;
     }
     if (c->n_link_items > 0) {
-        launch_body_kernel(1, B, parity, c->n_link_items, c->grid_box, nullptr, st);
+        launch_body_kernel(1, B, parity, c->n_link_items, c->grid_box, nullptr, both ? c->wall : st, !both && dep);
+        dep = true;
         n++;
     }
-    for (int which = 2; which <= 4; ++which) launch_body_kernel(which, B, parity, c->n_link_items, c->grid_box, nullptr, st);
+    if (both) {
+        cudaEventRecord(c->ev_wall2, c->wall);
+        cudaStreamWaitEvent(st, c->ev_wall2, 0);
+        dep = false;  // two predecessors
+    }
+    for (int which = 2; which <= 4; ++which) {
+        launch_body_kernel(which, B, parity, c->n_link_items, c->grid_box, nullptr, st, dep);
+        dep = true;
+    }
     return n + 3;
 }
 
@@ -1150,10 +1181,10 @@ static void enqueue_steps(lb_ctx* c, int64_t n) {
         if (c->psm) {
             c->launches += psm_sweep(c, B, parity, c->stream);
         } else {
-            sweep_all(c, parity, c->stream);
+            sweep_all(c, parity, c->stream, k > 0);
             c->launches += 1;
         }
-        if (bodies) c->launches += body_step(c, B, parity, c->stream);
+        if (bodies) c->launches += body_step(c, B, parity, c->stream, !c->psm);
         c->step++;
     }
 }
@@ -1183,7 +1214,8 @@ static void begin_units(lb_ctx* c) {
     cudaEventRecord(c->ev_join2, c->stream);  // "the last near sweep"
 }
 
-static void enqueue_unit(lb_ctx* c) {
+// dep: the last operation on hi is the near sweep of the unit before.
+static void enqueue_unit(lb_ctx* c, bool dep) {
     const int64_t t = c->step - 1;
     const int parity = (int)(t & 1), q = 1 - parity;
     const int* win = win_slot(c, t + 1);
@@ -1191,7 +1223,7 @@ static void enqueue_unit(lb_ctx* c) {
     // first, it would fill every SM, and a cluster waits for SMs of one GPC to
     // drain together
     const bool fused = c->solo || c->n_fused > 0;
-    c->launches += body_step(c, bodies_for_step(c, t), parity, c->hi, fused ? c->ev_started : nullptr);
+    c->launches += body_step(c, bodies_for_step(c, t), parity, c->hi, dep, fused ? c->ev_started : nullptr);
     cudaStreamWaitEvent(c->hi, c->ev_join, 0);  // far(t), before near(t+1)
     if (fused) cudaStreamWaitEvent(c->side, c->ev_started, 0);
     cudaStreamWaitEvent(c->side, c->ev_join2, 0);  // near(t), before far(t+1)
@@ -1225,7 +1257,7 @@ static lb_status build_graph(lb_ctx* c, int which) {
     if (c->split) {
         c->step = 2 + 2 * which;  // 8 units from t = 1 or 3 (the window slots repeat every 4 steps)
         begin_units(c);
-        for (int k = 0; k < kGraphSteps; ++k) enqueue_unit(c);
+        for (int k = 0; k < kGraphSteps; ++k) enqueue_unit(c, k > 0);
         end_units(c);
     } else {
         c->step = 0;  // 8 steps from an even step
@@ -1265,7 +1297,7 @@ lb_status lb_step(lb_ctx* c, int64_t nsteps) {
         }
         if (left > 0 && ((c->step - 1) & 1) == 0) {  // graphs start on a unit of odd t
             begin_units(c);
-            enqueue_unit(c);
+            enqueue_unit(c, false);
             end_units(c);
             left--;
         }
@@ -1289,7 +1321,7 @@ lb_status lb_step(lb_ctx* c, int64_t nsteps) {
     }
     if (c->split && left > 0) {
         begin_units(c);
-        for (; left > 0; --left) enqueue_unit(c);
+        for (bool dep = false; left > 0; --left, dep = true) enqueue_unit(c, dep);
         end_units(c);
     } else if (left > 0) {
         enqueue_steps(c, left);

@@ -888,6 +888,8 @@ __device__ __forceinline__ void copy_links(const Lattice& L, long long cnt, cons
 
 template <int P>
 __global__ void __launch_bounds__(kLB) k_links(const Bodies B) {
+    dep_wait();
+    dep_launch();
     __shared__ double sm[12 * kLB + 12 * 8];
     __shared__ double s_tot[12];
     __shared__ BodyState s_new;
@@ -1091,6 +1093,8 @@ __device__ __forceinline__ uint32_t link_mask(const Lattice& L, int x, int y, in
 
 template <int P>
 __global__ void __launch_bounds__(kBB) k_classify(const Bodies B) {
+    dep_wait();
+    dep_launch();
     __shared__ double smd[kBB / 32];
     __shared__ int s_base, s_scan[kBB / 32 + 1];
     const int nitems = *B.n_box;
@@ -1268,6 +1272,8 @@ __device__ __noinline__ void refill_cell(const Lattice& L, const BodyState& s, i
 
 template <int P>
 __global__ void __launch_bounds__(kBB) k_convert(const Bodies B) {
+    dep_wait();
+    dep_launch();
     __shared__ double sm[6 * kBB + 6 * 16];
     __shared__ double s_tot[6];
     __shared__ long long sml[kBB];
@@ -1421,6 +1427,8 @@ __device__ void near_window(const Bodies& B) {
 
 template <int P>
 __global__ void __launch_bounds__(kBB) k_rebuild(const Bodies B) {
+    dep_wait();
+    dep_launch();
     __shared__ long long sml[kBB];
     __shared__ int s_scan[kBB / 32 + 1], s_flag;
     __shared__ long long s_base;
@@ -1703,12 +1711,19 @@ __global__ void __launch_bounds__(kFT, 2) k_body_fused(const Bodies B, int cls, 
         const Lattice& L = s_L;
         const BodyParams& p = s_p;
         const BodyState& s0 = s_s0;
-        if (!lattice_active(L)) continue;  // the same in every block of the cluster
+        if (!lattice_active(L)) {  // the same in every block of the cluster
+            dep_wait();
+            continue;
+        }
         // this block's share of the shell stencil, fetched while the links run
         const uint32_t* stc = B.stencil + p.st_off;
         long long b0, b1;
         box_range(p.st_count, rank, KC, b0, b1);
         for (long long b = b0 + threadIdx.x; b < b1 && b < b0 + kStcBuf; b += kFT) s_stc[b - b0] = __ldg(stc + b);
+        // the populations follow; everything above was written by kernels
+        // before the sweep this launch may have started beside
+        dep_wait();
+        dep_launch();
 
         // ---- bounce-back and momentum exchange on the links (as k_links), by
         // ranks 1 .. KC-1.  Meanwhile warps 0 and 1 of rank 0 run the update once
@@ -1943,6 +1958,7 @@ __global__ void __launch_bounds__(kFT, 2) k_body_fused(const Bodies B, int cls, 
             base += tot;
         }
     }
+    dep_wait();  // a cluster without an item
     // no block leaves while another may still read its shared memory
     cl.sync();
     // tail != 0: this launch is the lattice's whole body step (one sphere and
@@ -1967,7 +1983,8 @@ __global__ void __launch_bounds__(kFT, 2) k_body_fused(const Bodies B, int cls, 
 
 // which: 1 links, 2 classify, 3 convert, 4 rebuild, 5 tick.  The link kernel
 // gets grid_links blocks over its static item list; the box kernels walk their
-// device-built lists with grid_box blocks.
+// device-built lists with grid_box blocks.  dep: a dependent launch (see
+// dep_wait).
 // ---------------------------------------------------------------- partially saturated cells
 // (psm.cuh).  Per step, before the sweep of parity P: the previous step's
 // solid fractions of each sphere are cleared (its box at the step's position,
@@ -2267,19 +2284,15 @@ void launch_psm_scatter(const Bodies& B, int parity, int grid, cudaStream_t st) 
 }
 
 void launch_body_kernel(int which, const Bodies& B, int parity, int grid_links, int grid_box, long long* step,
-                        cudaStream_t st) {
+                        cudaStream_t st, bool dep) {
     if (which == 1) {
-        if (parity == 0) k_links<0><<<grid_links, kLB, 0, st>>>(B);
-        else k_links<1><<<grid_links, kLB, 0, st>>>(B);
+        launch(parity == 0 ? k_links<0> : k_links<1>, grid_links, kLB, 0, st, dep, B);
     } else if (which == 2) {
-        if (parity == 0) k_classify<0><<<grid_box, kBB, 0, st>>>(B);
-        else k_classify<1><<<grid_box, kBB, 0, st>>>(B);
+        launch(parity == 0 ? k_classify<0> : k_classify<1>, grid_box, kBB, 0, st, dep, B);
     } else if (which == 3) {
-        if (parity == 0) k_convert<0><<<grid_box, kBB, 0, st>>>(B);
-        else k_convert<1><<<grid_box, kBB, 0, st>>>(B);
+        launch(parity == 0 ? k_convert<0> : k_convert<1>, grid_box, kBB, 0, st, dep, B);
     } else if (which == 4) {
-        if (parity == 0) k_rebuild<0><<<grid_box, kBB, 0, st>>>(B);
-        else k_rebuild<1><<<grid_box, kBB, 0, st>>>(B);
+        launch(parity == 0 ? k_rebuild<0> : k_rebuild<1>, grid_box, kBB, 0, st, dep, B);
     } else {
         k_tick<<<1, 1, 0, st>>>(B.n_box, B.n_rel, step);
     }
@@ -2301,8 +2314,8 @@ int fused_cluster(int c) { return c == 0 ? 16 : (c == 1 ? 8 : 4); }
 // started: null, or an event (created with cudaEventDisableTiming) to fire
 // once every block of the launch has begun (a launch-completion event): a
 // stream that waits on it starts after the clusters are placed, not after
-// the kernel ends.
-void launch_body_fused(const Bodies& B, int parity, int cls, int clusters, cudaStream_t st, int tail,
+// the kernel ends.  dep: a dependent launch (see dep_wait).
+void launch_body_fused(const Bodies& B, int parity, int cls, int clusters, cudaStream_t st, int tail, bool dep,
                        cudaEvent_t started) {
     if (clusters <= 0) return;
     const int kc = fused_cluster(cls);
@@ -2310,7 +2323,7 @@ void launch_body_fused(const Bodies& B, int parity, int cls, int clusters, cudaS
     cfg.gridDim = dim3(clusters * kc);
     cfg.blockDim = dim3(kFT);
     cfg.stream = st;
-    cudaLaunchAttribute attr[2];
+    cudaLaunchAttribute attr[3];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = kc;
     attr[0].val.clusterDim.y = 1;
@@ -2323,14 +2336,13 @@ void launch_body_fused(const Bodies& B, int parity, int cls, int clusters, cudaS
         attr[cfg.numAttrs].val.launchCompletionEvent.flags = 0;
         cfg.numAttrs++;
     }
+    if (dep) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+        cfg.numAttrs++;
+    }
     if (parity == 0) cudaLaunchKernelEx(&cfg, k_body_fused<0>, B, cls, tail);
     else cudaLaunchKernelEx(&cfg, k_body_fused<1>, B, cls, tail);
-}
-
-// A step's body kernels: links, classify, convert, rebuild (whose last block
-// empties the work lists).
-void launch_body_step(const Bodies& B, int parity, int grid_links, int grid_box, long long* step, cudaStream_t st) {
-    for (int which = 1; which <= 4; ++which) launch_body_kernel(which, B, parity, grid_links, grid_box, step, st);
 }
 
 }  // namespace lbsq

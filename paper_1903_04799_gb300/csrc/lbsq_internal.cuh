@@ -123,6 +123,37 @@ template <> struct StoreT<ST_BF16> {
 
 inline int storage_bytes(int s) { return s == ST_F64 ? 8 : (s == ST_F32 ? 4 : 2); }
 
+// ---- dependent launches
+//
+// The kernels of a step follow each other in one stream, and a step of a small
+// lattice is as long as their chain, launch gaps (about 2 us each) included.  A
+// kernel launched with `dependent` set may start while its predecessor in the
+// stream still runs: its blocks are placed once every block of the predecessor
+// has called dep_launch (or exited), and wait in dep_wait for the predecessor's
+// end and its writes.  Every kernel launched this way calls dep_wait in every
+// thread before it reads or writes what the predecessor touches, and dep_launch
+// only after dep_wait; so when a block starts, every kernel before its
+// predecessor has ended, and what those wrote may be read at once.  Both
+// calls do nothing in an ordinary launch.
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... KA, class... A>
+inline void launch(void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool dependent,
+                   A&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = dependent ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<KA>(args)...);
+}
+
 // One lattice as seen by kernels (an array of these lives in device memory;
 // a context has one, a server one per resident request).
 struct Lattice {

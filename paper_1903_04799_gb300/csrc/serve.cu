@@ -29,7 +29,7 @@
 
 namespace lbsq {
 void launch_body_kernel(int which, const Bodies& B, int parity, int grid_links, int grid_box, long long* step,
-                        cudaStream_t st);
+                        cudaStream_t st, bool dep = false);
 void launch_fill_rest(const Lattice& L, cudaStream_t st);
 void launch_plane_claim(const Lattice& L, int32_t* own, int axis, int index, int id, cudaStream_t st);
 void launch_set_flags(BodyAcc* acc, int nb, int k, int reclass, cudaStream_t st);

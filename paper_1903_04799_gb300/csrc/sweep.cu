@@ -13,6 +13,8 @@ namespace lbsq {
 
 template <int S, int P, bool NATIVE>
 __global__ void __launch_bounds__(256) k_sweep(const SweepArgs a) {
+    dep_wait();
+    dep_launch();
     const uint32_t skey = S == ST_BF16 ? sr_step_key(a) : 0u;  // before any exit (see sr_step)
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int z = sweep_plane(a);
@@ -27,6 +29,8 @@ __global__ void __launch_bounds__(256) k_sweep(const SweepArgs a) {
 // bandwidth).
 template <int P, bool O32, bool LE1>
 __global__ void __launch_bounds__(256, 3) k_sweep_df(const SweepArgs a) {
+    dep_wait();
+    dep_launch();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int z = sweep_plane(a);
     const int y = z < 0 ? -1 : sweep_row(a, blockIdx.y, z);
@@ -35,13 +39,15 @@ __global__ void __launch_bounds__(256, 3) k_sweep_df(const SweepArgs a) {
 }
 
 template <bool O32, bool LE1>
-static void launch_df(const SweepArgs& a, int parity, const dim3& grid, int bx, cudaStream_t st) {
-    if (parity == 0) k_sweep_df<0, O32, LE1><<<grid, bx, 0, st>>>(a);
-    else k_sweep_df<1, O32, LE1><<<grid, bx, 0, st>>>(a);
+static void launch_df(const SweepArgs& a, int parity, const dim3& grid, int bx, cudaStream_t st, bool dep) {
+    if (parity == 0) launch(k_sweep_df<0, O32, LE1>, grid, bx, 0, st, dep, a);
+    else launch(k_sweep_df<1, O32, LE1>, grid, bx, 0, st, dep, a);
 }
 
 template <int S, int P, bool O32>
 __global__ void __launch_bounds__(256, 2) k_sweep2(const SweepArgs a) {
+    dep_wait();
+    dep_launch();
     const uint32_t skey = S == ST_BF16 ? sr_step_key(a) : 0u;  // before any exit (see sr_step)
     const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     const int z = sweep_plane(a);
@@ -55,6 +61,8 @@ __global__ void __launch_bounds__(256, 2) k_sweep2(const SweepArgs a) {
 // 10 x rows x nx elements on odd steps.
 template <int S, int P, bool O32>
 __global__ void __launch_bounds__(P == 0 ? 256 : 192, 2) k_sweep4r(const SweepArgs a) {
+    dep_wait();
+    dep_launch();
     extern __shared__ unsigned short rowbuf[];
     const uint32_t skey = S == ST_BF16 ? sr_step_key(a) : 0u;  // before any exit (see sr_step)
     const int z = sweep_plane(a);
@@ -69,6 +77,8 @@ __global__ void __launch_bounds__(P == 0 ? 256 : 192, 2) k_sweep4r(const SweepAr
 // spills 72-80 bytes and measured 3-4 % slower).
 template <int S, bool O32>
 __global__ void __launch_bounds__(192, 2) k_sweep4o(const SweepArgs a) {
+    dep_wait();
+    dep_launch();
     const uint32_t skey = S == ST_BF16 ? sr_step_key(a) : 0u;  // before any exit (see sr_step)
     const int x0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
     const int z = sweep_plane(a);
@@ -127,7 +137,7 @@ static int prefetch_ahead16(const SweepArgs& a, const dim3& grid, int extra) {
 }
 
 template <int S>
-static void launch_s(const SweepArgs& a, int parity, int variant, int gz, int gy, cudaStream_t st) {
+static void launch_s(const SweepArgs& a, int parity, int variant, int gz, int gy, cudaStream_t st, bool dep) {
     const bool o32 = 19 * a.Np < (int64_t(1) << 32);  // element offsets fit 32 bits
     if constexpr (S == ST_F64) {
         int bx = ((a.nx + 31) / 32) * 32;
@@ -136,14 +146,14 @@ static void launch_s(const SweepArgs& a, int parity, int variant, int gz, int gy
         SweepArgs b = a;
         b.pf = prefetch_ahead(a, S, grid);
         if (variant == 1) {  // FP64 arithmetic
-            if (parity == 0) k_sweep<S, 0, true><<<grid, bx, 0, st>>>(a);
-            else k_sweep<S, 1, true><<<grid, bx, 0, st>>>(a);
+            if (parity == 0) launch(k_sweep<S, 0, true>, grid, bx, 0, st, dep, a);
+            else launch(k_sweep<S, 1, true>, grid, bx, 0, st, dep, a);
         } else if (o32) {
-            if (a.K.df.le1) launch_df<true, true>(b, parity, grid, bx, st);
-            else launch_df<true, false>(b, parity, grid, bx, st);
+            if (a.K.df.le1) launch_df<true, true>(b, parity, grid, bx, st, dep);
+            else launch_df<true, false>(b, parity, grid, bx, st, dep);
         } else {
-            if (a.K.df.le1) launch_df<false, true>(b, parity, grid, bx, st);
-            else launch_df<false, false>(b, parity, grid, bx, st);
+            if (a.K.df.le1) launch_df<false, true>(b, parity, grid, bx, st, dep);
+            else launch_df<false, false>(b, parity, grid, bx, st, dep);
         }
     } else {
     if constexpr (S == ST_F16 || S == ST_BF16) {
@@ -168,8 +178,8 @@ static void launch_s(const SweepArgs& a, int parity, int variant, int gz, int gy
             dim3 block(bx, by), grid((quads + bx - 1) / bx, (gy + by - 1) / by, gz);
             SweepArgs b = a;
             b.pf = prefetch_ahead16(a, grid, 0);
-            if (o32) k_sweep4o<S, true><<<grid, block, 0, st>>>(b);
-            else k_sweep4o<S, false><<<grid, block, 0, st>>>(b);
+            if (o32) launch(k_sweep4o<S, true>, grid, block, 0, st, dep, b);
+            else launch(k_sweep4o<S, false>, grid, block, 0, st, dep, b);
             return;
         }
         if ((variant == 3 || (variant == 0 && parity == 0)) && rows4) {
@@ -179,12 +189,12 @@ static void launch_s(const SweepArgs& a, int parity, int variant, int gz, int gy
             if (parity == 0) {
                 SweepArgs b = a;
                 b.pf = prefetch_ahead16(a, grid, 2);
-                if (o32) k_sweep4r<S, 0, true><<<grid, block, 0, st>>>(b);
-                else k_sweep4r<S, 0, false><<<grid, block, 0, st>>>(b);
+                if (o32) launch(k_sweep4r<S, 0, true>, grid, block, 0, st, dep, b);
+                else launch(k_sweep4r<S, 0, false>, grid, block, 0, st, dep, b);
             } else {
                 const size_t smem = (size_t)10 * ty * a.nx * sizeof(unsigned short);
-                if (o32) k_sweep4r<S, 1, true><<<grid, block, smem, st>>>(a);
-                else k_sweep4r<S, 1, false><<<grid, block, smem, st>>>(a);
+                if (o32) launch(k_sweep4r<S, 1, true>, grid, block, smem, st, dep, a);
+                else launch(k_sweep4r<S, 1, false>, grid, block, smem, st, dep, a);
             }
             return;
         }
@@ -199,19 +209,19 @@ static void launch_s(const SweepArgs& a, int parity, int variant, int gz, int gy
         b.pf = prefetch_ahead(a, S, grid);
         if (S == ST_F16 || S == ST_BF16) b.pf = parity == 1 ? prefetch_ahead16(a, grid, 0) : 0;
         if (o32) {
-            if (parity == 0) k_sweep2<S, 0, true><<<grid, block, 0, st>>>(b);
-            else k_sweep2<S, 1, true><<<grid, block, 0, st>>>(b);
+            if (parity == 0) launch(k_sweep2<S, 0, true>, grid, block, 0, st, dep, b);
+            else launch(k_sweep2<S, 1, true>, grid, block, 0, st, dep, b);
         } else {
-            if (parity == 0) k_sweep2<S, 0, false><<<grid, block, 0, st>>>(b);
-            else k_sweep2<S, 1, false><<<grid, block, 0, st>>>(b);
+            if (parity == 0) launch(k_sweep2<S, 0, false>, grid, block, 0, st, dep, b);
+            else launch(k_sweep2<S, 1, false>, grid, block, 0, st, dep, b);
         }
         return;
     }
     int bx = ((a.nx + 31) / 32) * 32;
     if (bx > 256) bx = 256;
     dim3 grid((a.nx + bx - 1) / bx, gy, gz);
-    if (parity == 0) k_sweep<S, 0, false><<<grid, bx, 0, st>>>(a);
-    else k_sweep<S, 1, false><<<grid, bx, 0, st>>>(a);
+    if (parity == 0) launch(k_sweep<S, 0, false>, grid, bx, 0, st, dep, a);
+    else launch(k_sweep<S, 1, false>, grid, bx, 0, st, dep, a);
     }
 }
 
@@ -225,9 +235,9 @@ static void launch_s(const SweepArgs& a, int parity, int variant, int gz, int gy
 // zmode / win / gz / gy: cell selection (see SweepArgs); gz and gy = grid
 // planes and rows (nz and ny for modes 0 and 1, upper bounds of the window's
 // z and y lengths for mode 2).  Odd steps sweep the planes in descending
-// order.
+// order.  dep: a dependent launch (see dep_wait).
 void launch_sweep(const Lattice& L, double lambda_e, double lambda_o, int parity, int variant, int zmode,
-                  const int* win, int gz, int gy, cudaStream_t st) {
+                  const int* win, int gz, int gy, cudaStream_t st, bool dep) {
     SweepArgs a = sweep_args(L, lambda_e, lambda_o);
     a.zmode = zmode;
     a.win = win;
@@ -235,10 +245,10 @@ void launch_sweep(const Lattice& L, double lambda_e, double lambda_o, int parity
     a.sr_writer = zmode != 2;  // of a split step's two sweeps, the far one advances the step counter
     if (gz <= 0 || gy <= 0) return;
     switch (L.storage) {
-        case ST_F64: launch_s<ST_F64>(a, parity, variant, gz, gy, st); break;
-        case ST_F32: launch_s<ST_F32>(a, parity, variant, gz, gy, st); break;
-        case ST_F16: launch_s<ST_F16>(a, parity, variant, gz, gy, st); break;
-        default: launch_s<ST_BF16>(a, parity, variant, gz, gy, st); break;
+        case ST_F64: launch_s<ST_F64>(a, parity, variant, gz, gy, st, dep); break;
+        case ST_F32: launch_s<ST_F32>(a, parity, variant, gz, gy, st, dep); break;
+        case ST_F16: launch_s<ST_F16>(a, parity, variant, gz, gy, st, dep); break;
+        default: launch_s<ST_BF16>(a, parity, variant, gz, gy, st, dep); break;
     }
 }
 
