@@ -6,8 +6,7 @@
 // Why: GB300 issues FP64 arithmetic at about 2 lanes per SM and cycle against
 // 128 for FP32.  A TRT update in FP64 is about 130 FP64 instructions per cell,
 // which caps the FP64 sweep near a fifth of its HBM roofline.  The same update
-// in double-float takes about 900 FP32 instructions, which the FP32 pipes
-// retire in a third of the time the populations take to stream.
+// in double-float takes about 900 FP32 operations, issued two at a time.
 //
 // Precision: FP64 storage holds the deviations g_i = f_i - w_i rho0, whose
 // magnitude is that of the flow (|g| ~ 1e-3 here), not of f (~0.05 .. 1/3).
@@ -164,29 +163,81 @@ __device__ __forceinline__ uint2 df_to_bits(df x) {
     return make_uint2(lo, hi);
 }
 
-// Signed sum over the nine pairs of component AX of the pair's first member
-// times d[p] (as pair_moment in sweep_body.cuh, in double-float).
-template <int AX>
-__device__ __forceinline__ df df_pair_moment(const df d[10]) {
-    df acc{0.0f, 0.0f};
-    bool first = true;
-#pragma unroll
-    for (int p = 1; p <= 9; ++p) {
-        const int i = 2 * p - 1;
-        const int c = AX == 0 ? cx(i) : (AX == 1 ? cy(i) : cz(i));
-        if (c == 0) continue;
-        if (first) acc = d[p];
-        else acc = c > 0 ? dadd(acc, d[p]) : dsub(acc, d[p]);
-        first = false;
-    }
-    return acc;
+// ---- two double-float numbers at a time
+//
+// GB300 retires add/mul/fma.f32x2 (two FP32 operations per instruction), and
+// with one operation per instruction the sweep was bound by instruction issue
+// (76 % of the slots busy, FMA pipe 51 %), so the collision carries its
+// direction pairs two by two; every half rounds as the scalar operation would.
+// Whole sweeps on GB300, scalar -> in pairs: 256^3 891 -> 830 us (0.90 of the
+// 6.8 TB/s copy rate), 128^3 107 -> 100 us.
+struct df2 {
+    unsigned long long h, l;
+};
+__device__ __forceinline__ unsigned long long f2_pack(float a, float b) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
 }
-__device__ __forceinline__ df df_pair_dot(int i, df x, df y, df z) {
-    const int a = cx(i), b = cy(i), c = cz(i);
-    if (a != 0 && b != 0) return b > 0 ? dadd(x, y) : dsub(x, y);
-    if (a != 0 && c != 0) return c > 0 ? dadd(x, z) : dsub(x, z);
-    if (b != 0 && c != 0) return c > 0 ? dadd(y, z) : dsub(y, z);
-    return a != 0 ? x : (b != 0 ? y : z);
+__device__ __forceinline__ void f2_unpack(unsigned long long v, float& a, float& b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long f2_sub(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long f2_mul(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b,
+                                                     unsigned long long c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ df2 pack(df a, df b) { return {f2_pack(a.h, b.h), f2_pack(a.l, b.l)}; }
+__device__ __forceinline__ df2 splat(df a) { return pack(a, a); }
+__device__ __forceinline__ void unpack(df2 v, df& a, df& b) {
+    f2_unpack(v.h, a.h, b.h);
+    f2_unpack(v.l, a.l, b.l);
+}
+__device__ __forceinline__ df2 dadd(df2 x, df2 y) {
+    const unsigned long long s = f2_add(x.h, y.h);
+    const unsigned long long bb = f2_sub(s, x.h);
+    const unsigned long long e = f2_add(f2_sub(x.h, f2_sub(s, bb)), f2_sub(y.h, bb));
+    return {s, f2_add(e, f2_add(x.l, y.l))};
+}
+__device__ __forceinline__ df2 dsub(df2 x, df2 y) {
+    const unsigned long long s = f2_sub(x.h, y.h);
+    const unsigned long long bb = f2_sub(s, x.h);
+    const unsigned long long e = f2_sub(f2_sub(x.h, f2_sub(s, bb)), f2_add(y.h, bb));
+    return {s, f2_add(e, f2_sub(x.l, y.l))};
+}
+__device__ __forceinline__ df2 dmul(df2 x, df2 y) {
+    const unsigned long long p = f2_mul(x.h, y.h);
+    unsigned long long e = f2_fma(x.h, y.h, p ^ 0x8000000080000000ull);
+    e = f2_fma(x.h, y.l, e);
+    e = f2_fma(x.l, y.h, e);
+    return {p, e};
+}
+__device__ __forceinline__ df2 dsqr(df2 x) {
+    const unsigned long long p = f2_mul(x.h, x.h);
+    const unsigned long long t = f2_add(x.h, x.h);
+    unsigned long long e = f2_fma(x.h, x.h, p ^ 0x8000000080000000ull);
+    e = f2_fma(t, x.l, e);
+    return {p, e};
+}
+__device__ __forceinline__ df2 dpow2(df2 x, float p2) {
+    const unsigned long long q = f2_pack(p2, p2);
+    return {f2_mul(x.h, q), f2_mul(x.l, q)};
 }
 
 // TRT collision (Sec. III) of one cell on deviations g_i = f_i - w_i rho0, in
@@ -201,19 +252,38 @@ __device__ __forceinline__ df df_pair_dot(int i, df x, df y, df z) {
 //            g_i += E + O,  g_ib += E - O.
 // LE1: le == 1 (K.le1), the form taken.  Returns false when the cell's
 // density or momentum is not finite.
+//
+// The nine direction pairs p (first members 2p - 1) are taken as x alone,
+// (y, z), and the edges as (xy+, xz+), (xy-, xz-), (yz+, yz-): then the momentum
+// and c.j of two pairs come from one operation each,
+//   (jy, jz) = (d_y, d_z) + (d_xy+ - d_xy-, d_xz+ - d_xz-)
+//              + (d_yz+ + d_yz-, d_yz+ - d_yz-),
+//   c.j = jx +- (jy, jz) for the first two edge groups, jy +- jz for the third.
+// first member's index in g of group q's pair k
+__host__ __device__ constexpr int df_i(int q, int k) {
+    return 2 * (q == 0 ? 2 + k : (q == 1 ? 4 + 2 * k : (q == 2 ? 5 + 2 * k : 8 + k))) - 1;
+}
 template <bool LE1>
 __device__ __forceinline__ bool collide_trt_df(df g[Q], const DfK& K, int inc) {
-    df s[10], d[10];
+    df2 s[4], d[4];
 #pragma unroll
-    for (int p = 1; p <= 9; ++p) {
-        s[p] = dadd(g[2 * p - 1], g[2 * p]);
-        d[p] = dsub(g[2 * p - 1], g[2 * p]);
+    for (int q = 0; q < 4; ++q) {
+        const int a = df_i(q, 0), b = df_i(q, 1);
+        const df2 u = pack(g[a], g[b]), v = pack(g[a + 1], g[b + 1]);
+        s[q] = dadd(u, v);
+        d[q] = dsub(u, v);
     }
-    df sum = g[0];
-#pragma unroll
-    for (int p = 1; p <= 9; ++p) sum = dadd(sum, s[p]);
-    sum = dnorm(sum);
-    const df jx = dnorm(df_pair_moment<0>(d)), jy = dnorm(df_pair_moment<1>(d)), jz = dnorm(df_pair_moment<2>(d));
+    const df s1 = dadd(g[1], g[2]), d1 = dsub(g[1], g[2]);
+    df sa, sb;
+    unpack(dadd(dadd(s[0], s[1]), dadd(s[2], s[3])), sa, sb);
+    const df sum = dnorm(dadd(dadd(g[0], s1), dadd(sa, sb)));
+    df xp, xq, e8, e9, jy, jz;
+    unpack(dadd(d[1], d[2]), xp, xq);  // d_xy+ + d_xy-, d_xz+ + d_xz-
+    const df jx = dnorm(dadd(dadd(d1, xp), xq));
+    unpack(d[3], e8, e9);
+    unpack(dadd(dadd(d[0], dsub(d[1], d[2])), dadd(pack(e8, e8), pack(e9, dneg(e9)))), jy, jz);
+    jy = dnorm(jy);
+    jz = dnorm(jz);
     const df j2 = dadd(dadd(dsqr(jx), dsqr(jy)), dsqr(jz));
     const bool ok = fabsf(sum.h) < 0x1p60f && j2.h < 0x1p100f;
     const df inv = inc ? dk(K, DK_IRHO0) : drcp(dnorm(dadd(dk(K, DK_RHO0), sum)));
@@ -221,37 +291,46 @@ __device__ __forceinline__ bool collide_trt_df(df g[Q], const DfK& K, int inc) {
     const df base = dnorm(dsub(sum, dmulf(ju, 1.5f)));  // sigma - 3/2 rho u.u
     const df wb18 = dmul(base, dk(K, DK_W18)), wb36 = dpow2(wb18, 0.5f);
     const df lw18 = dk(K, DK_LW18), lw36 = dk(K, DK_LW36);
+    const df2 jyz = pack(jy, jz), jxx = splat(jx), inv2 = splat(inv);
+    const df2 cj[4] = {jyz, dadd(jxx, jyz), dsub(jxx, jyz), dadd(splat(jy), pack(jz, dneg(jz)))};
+    // ep = w base + 9/2 w (c.j)^2 / rho; 9/2 w = 1/4 (faces), 1/8 (edges)
+    const df ep1 = dadd(dpow2(dmul(dsqr(jx), inv), 0.25f), wb18);
     if constexpr (LE1) {
         g[0] = dmul(base, dk(K, DK_W3));
         const df ch = dk(K, DK_CH);
+        const df2 ch2 = splat(ch), lwf = splat(lw18), lwe = splat(lw36), wbf = splat(wb18), wbe = splat(wb36);
+        const df h1 = dadd(dmul(lw18, jx), dmul(ch, d1));
+        g[1] = dadd(ep1, h1);
+        g[2] = dsub(ep1, h1);
 #pragma unroll
-        for (int p = 1; p <= 9; ++p) {
-            const int i = 2 * p - 1;
-            const bool face = i < 7;
-            const df cj = df_pair_dot(i, jx, jy, jz);
-            const df t = dmul(dsqr(cj), inv);  // (c.j)^2 / rho; 9/2 w = 1/4 (faces), 1/8 (edges)
-            const df ep = dadd(dpow2(t, face ? 0.25f : 0.125f), face ? wb18 : wb36);
-            const df h = dadd(dmul(face ? lw18 : lw36, cj), dmul(ch, d[p]));
-            g[i] = dadd(ep, h);
-            g[i + 1] = dsub(ep, h);
+        for (int q = 0; q < 4; ++q) {
+            const int a = df_i(q, 0), b = df_i(q, 1);
+            const df2 ep = dadd(dpow2(dmul(dsqr(cj[q]), inv2), q == 0 ? 0.25f : 0.125f), q == 0 ? wbf : wbe);
+            const df2 h = dadd(dmul(q == 0 ? lwf : lwe, cj[q]), dmul(ch2, d[q]));
+            unpack(dadd(ep, h), g[a], g[b]);
+            unpack(dsub(ep, h), g[a + 1], g[b + 1]);
         }
         return ok;
     } else {
-    g[0] = dadd(dmul(dk(K, DK_LE3), base), dmul(dk(K, DK_1MLE), g[0]));
-    const df le = dk(K, DK_LE), mhle = dk(K, DK_MHLE), mhlo = dk(K, DK_MHLO);
+        g[0] = dadd(dmul(dk(K, DK_LE3), base), dmul(dk(K, DK_1MLE), g[0]));
+        const df le = dk(K, DK_LE), mhle = dk(K, DK_MHLE), mhlo = dk(K, DK_MHLO);
+        const df2 le2 = splat(le), mhle2 = splat(mhle), mhlo2 = splat(mhlo);
+        const df2 lwf = splat(lw18), lwe = splat(lw36), wbf = splat(wb18), wbe = splat(wb36);
+        {
+            const df E = dadd(dmul(le, ep1), dmul(mhle, s1)), O = dadd(dmul(lw18, jx), dmul(mhlo, d1));
+            g[1] = dadd(g[1], dadd(E, O));
+            g[2] = dadd(g[2], dsub(E, O));
+        }
 #pragma unroll
-    for (int p = 1; p <= 9; ++p) {
-        const int i = 2 * p - 1;
-        const bool face = i < 7;
-        const df cj = df_pair_dot(i, jx, jy, jz);
-        const df t = dmul(dsqr(cj), inv);
-        const df ep = dadd(dpow2(t, face ? 0.25f : 0.125f), face ? wb18 : wb36);
-        const df E = dadd(dmul(le, ep), dmul(mhle, s[p]));
-        const df O = dadd(dmul(face ? lw18 : lw36, cj), dmul(mhlo, d[p]));
-        g[i] = dadd(g[i], dadd(E, O));
-        g[i + 1] = dadd(g[i + 1], dsub(E, O));
-    }
-    return ok;
+        for (int q = 0; q < 4; ++q) {
+            const int a = df_i(q, 0), b = df_i(q, 1);
+            const df2 ep = dadd(dpow2(dmul(dsqr(cj[q]), inv2), q == 0 ? 0.25f : 0.125f), q == 0 ? wbf : wbe);
+            const df2 E = dadd(dmul(le2, ep), dmul(mhle2, s[q]));
+            const df2 O = dadd(dmul(q == 0 ? lwf : lwe, cj[q]), dmul(mhlo2, d[q]));
+            unpack(dadd(pack(g[a], g[b]), dadd(E, O)), g[a], g[b]);
+            unpack(dadd(pack(g[a + 1], g[b + 1]), dsub(E, O)), g[a + 1], g[b + 1]);
+        }
+        return ok;
     }
 }
 
