@@ -7,85 +7,119 @@
 // geometry-free: solid cells are swept too (their slots are private to them,
 // and every slot a fluid cell reads from a solid neighbour is rewritten by the
 // link kernel after the sweep), so no flag field is read.
+#include <algorithm>
+
 #include "sweep_body.cuh"
 
 namespace lbsq {
 
-template <int S, int P, bool NATIVE>
+// Every kernel comes in two forms: NEAR = false over grid rows (modes 0 and
+// 1), NEAR = true over the rows of the window (mode 2).
+template <int S, int P, bool NATIVE, bool NEAR>
 __global__ void __launch_bounds__(256) k_sweep(const SweepArgs a) {
     dep_wait();
     dep_launch();
     const uint32_t skey = S == ST_BF16 ? sr_step_key(a) : 0u;  // before any exit (see sr_step)
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int z = sweep_plane(a);
-    const int y = z < 0 ? -1 : sweep_row(a, blockIdx.y, z);
-    if (x >= a.nx || y < 0) return;
-    sweep_one<S, P, NATIVE>(a, x, y, z, skey);
+    if constexpr (NEAR) {
+        near_rows(a, [&](int y, int z, bool active) {
+            if (active && x < a.nx) sweep_one<S, P, NATIVE>(a, x, y, z, skey);
+        });
+    } else {
+        int y, z;
+        if (!sweep_at(a, blockIdx.y, y, z) || x >= a.nx) return;
+        sweep_one<S, P, NATIVE>(a, x, y, z, skey);
+    }
 }
 
-// FP64 storage, double-float collision (sweep_df.cuh), one cell per thread,
-// three blocks per SM (80 registers, 40 bytes of spill): 24 warps per SM hide
-// the loads better than 16 at 122 registers (256^3: 0.77 -> 0.83 of the copy
-// bandwidth).
-template <int P, bool O32, bool LE1>
-__global__ void __launch_bounds__(256, 3) k_sweep_df(const SweepArgs a) {
+// FP64 storage, double-float collision (sweep_df.cuh), one cell per thread.
+// lambda_e = 1: three blocks per SM (80 registers, 56 bytes of spill): 24 warps
+// per SM hide the loads better than 16.  The general relaxation keeps the pair
+// sums as well; at 80 registers it spilled 240 bytes and 160 x 144 x 130 took
+// 219 us per step against 177 at two blocks per SM.  The near form, with its
+// loop over rows, runs at two blocks too.
+template <int P, bool O32, bool LE1, bool NEAR>
+__global__ void __launch_bounds__(256, NEAR || !LE1 ? 2 : 3) k_sweep_df(const SweepArgs a) {
     dep_wait();
     dep_launch();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int z = sweep_plane(a);
-    const int y = z < 0 ? -1 : sweep_row(a, blockIdx.y, z);
-    if (x >= a.nx || y < 0) return;
-    sweep_one_df<P, O32, LE1>(a, x, y, z);
+    if constexpr (NEAR) {
+        near_rows(a, [&](int y, int z, bool active) {
+            if (active && x < a.nx) sweep_one_df<P, O32, LE1>(a, x, y, z);
+        });
+    } else {
+        int y, z;
+        if (!sweep_at(a, blockIdx.y, y, z) || x >= a.nx) return;
+        sweep_one_df<P, O32, LE1>(a, x, y, z);
+    }
 }
 
-template <bool O32, bool LE1>
-static void launch_df(const SweepArgs& a, int parity, const dim3& grid, int bx, cudaStream_t st, bool dep) {
-    if (parity == 0) launch(k_sweep_df<0, O32, LE1>, grid, bx, 0, st, dep, a);
-    else launch(k_sweep_df<1, O32, LE1>, grid, bx, 0, st, dep, a);
-}
-
-template <int S, int P, bool O32>
+template <int S, int P, bool O32, bool NEAR>
 __global__ void __launch_bounds__(256, 2) k_sweep2(const SweepArgs a) {
     dep_wait();
     dep_launch();
     const uint32_t skey = S == ST_BF16 ? sr_step_key(a) : 0u;  // before any exit (see sr_step)
     const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-    const int z = sweep_plane(a);
-    const int y = z < 0 ? -1 : sweep_row(a, blockIdx.y * blockDim.y + threadIdx.y, z);
-    if (x0 >= a.nx || y < 0) return;
-    sweep_two<S, P, O32>(a, x0, y, z, skey);
+    if constexpr (NEAR) {
+        near_rows(a, [&](int y, int z, bool active) {
+            if (active && x0 < a.nx) sweep_two<S, P, O32>(a, x0, y, z, skey);
+        });
+    } else {
+        int y, z;
+        const bool go = sweep_at(a, blockIdx.y * blockDim.y + threadIdx.y, y, z);
+        if (x0 >= a.nx || y >= a.ny) return;
+        sweep_two<S, P, O32>(a, x0, y, z, skey, go);
+    }
 }
 
 // 16-bit storages with nx % 4 == 0, nx <= 768: blocks of whole rows, four
 // cells per thread (see sweep_four_rows); dynamic shared memory of
 // 10 x rows x nx elements on odd steps.
-template <int S, int P, bool O32>
+template <int S, int P, bool O32, bool NEAR>
 __global__ void __launch_bounds__(P == 0 ? 256 : 192, 2) k_sweep4r(const SweepArgs a) {
     dep_wait();
     dep_launch();
     extern __shared__ unsigned short rowbuf[];
     const uint32_t skey = S == ST_BF16 ? sr_step_key(a) : 0u;  // before any exit (see sr_step)
-    const int z = sweep_plane(a);
-    if (z < 0) return;  // the whole block
-    const int y = sweep_row(a, blockIdx.y * blockDim.y + threadIdx.y, z);
-    sweep_four_rows<S, P, O32>(a, y < 0 ? 0 : y, z, y >= 0, rowbuf, skey);
+    if constexpr (NEAR) {
+        near_rows(a, [&](int y, int z, bool active) {
+            sweep_four_rows<S, P, O32>(a, y, z, active, rowbuf, skey);
+            if (P == 1) __syncthreads();  // the row buffer is reused
+        });
+    } else {
+        int y, z;
+        const bool go = sweep_at(a, blockIdx.y * blockDim.y + threadIdx.y, y, z);
+        sweep_four_rows<S, P, O32>(a, y < a.ny ? y : 0, z, go, rowbuf, skey);
+    }
 }
 
 // 16-bit storages with nx % 4 == 0, odd steps of split sweeps: four cells per
 // thread without shared memory (see sweep_four_odd), blocks of at most 192
 // threads (167 registers, no spill; at 256 threads the 128-register cap
 // spills 72-80 bytes and measured 3-4 % slower).
-template <int S, bool O32>
+template <int S, bool O32, bool NEAR>
 __global__ void __launch_bounds__(192, 2) k_sweep4o(const SweepArgs a) {
     dep_wait();
     dep_launch();
     const uint32_t skey = S == ST_BF16 ? sr_step_key(a) : 0u;  // before any exit (see sr_step)
     const int x0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
-    const int z = sweep_plane(a);
-    const int y = z < 0 ? -1 : sweep_row(a, blockIdx.y * blockDim.y + threadIdx.y, z);
-    if (x0 >= a.nx || y < 0) return;
-    sweep_four_odd<S, O32>(a, x0, y, z, skey);
+    if constexpr (NEAR) {
+        near_rows(a, [&](int y, int z, bool active) {
+            if (active && x0 < a.nx) sweep_four_odd<S, O32>(a, x0, y, z, skey, true);
+        });
+    } else {
+        int y, z;
+        const bool go = sweep_at(a, blockIdx.y * blockDim.y + threadIdx.y, y, z);
+        if (x0 >= a.nx || y >= a.ny) return;
+        sweep_four_odd<S, O32>(a, x0, y, z, skey, go);
+    }
 }
+
+// Shape of a sweep launch: bx x by threads, xblocks blocks along a row, grid
+// planes and rows gz, gy, blocks per SM that reside together.
+struct Rows {
+    int bx, by, xblocks, gz, gy, resident;
+};
 
 static int sm_count() {
     static int n = 0;
@@ -111,10 +145,12 @@ static int sm_count() {
 // sweeps) that evicted their code again (128^3 step 0.050 -> 0.056 ms).  The
 // FP64 sweep is long against its body step, and prefetches in split sweeps
 // too (256^3 pusher, whole step: 13 970 -> 15 830 MLUPS).
-static int prefetch_ahead(const SweepArgs& a, int storage, const dim3& grid) {
-    if (storage == ST_F32 ? a.zmode != 0 : storage != ST_F64) return 0;
-    const long long per_plane = (long long)grid.x * grid.y;
-    const long long resident = (storage == ST_F32 ? 2LL : 3LL) * sm_count();
+// A near sweep prefetches nothing: its window is a few planes deep (250^3 pair
+// in BF16, whole step: 341 -> 334 us without).
+static int prefetch_ahead(const SweepArgs& a, int storage, const Rows& r) {
+    if (a.zmode == 2 || (storage == ST_F32 && a.zmode != 0)) return 0;
+    const long long per_plane = (long long)r.xblocks * ((r.gy + r.by - 1) / r.by);
+    const long long resident = (long long)r.resident * sm_count();
     const int ahead = (int)((resident + per_plane - 1) / per_plane) + (storage == ST_F32 ? 2 : 0);
     return ahead < a.nz ? ahead : 0;
 }
@@ -129,40 +165,66 @@ static int prefetch_ahead(const SweepArgs& a, int storage, const dim3& grid) {
 // 0.2850 ms.  (An earlier measurement of the two-cell form prefetching on both
 // parities, 0.745 -> 0.684, was taken before the sweeps' traffic was marked
 // evict-first.)
-static int prefetch_ahead16(const SweepArgs& a, const dim3& grid, int extra) {
-    const long long per_plane = (long long)grid.x * grid.y;
+static int prefetch_ahead16(const SweepArgs& a, const Rows& r, int extra) {
+    if (a.zmode == 2) return 0;
+    const long long per_plane = (long long)r.xblocks * ((r.gy + r.by - 1) / r.by);
     const long long resident = 2LL * sm_count();
     const int ahead = (int)((resident + per_plane - 1) / per_plane) + extra;
     return ahead < a.nz ? ahead : 0;
 }
 
-template <int S>
-static void launch_s(const SweepArgs& a, int parity, int variant, int gz, int gy, cudaStream_t st, bool dep) {
-    const bool o32 = 19 * a.Np < (int64_t(1) << 32);  // element offsets fit 32 bits
+// Launch of one of the kernels above: bx x by threads, x blocks of bx threads
+// along a row.  Rows of the lattice (modes 0 and 1) take a grid of their own;
+// the near sweep a wave of `resident` blocks per SM that stride over the
+// window, at most one block per by rows of its bound gz x gy.
+template <class K>
+static void launch_rows(K far_kernel, K near_kernel, const SweepArgs& a, const Rows& r, size_t smem, cudaStream_t st,
+                        bool dep) {
+    const dim3 block(r.bx, r.by);
+    if (a.zmode != 2) {
+        launch(far_kernel, dim3(r.xblocks, (r.gy + r.by - 1) / r.by, r.gz), block, smem, st, dep, a);
+        return;
+    }
+    const long long want = ((long long)r.gz * r.gy + r.by - 1) / r.by;
+    const long long wave = std::max(1, r.resident * sm_count() / r.xblocks);
+    launch(near_kernel, dim3(r.xblocks, (unsigned)std::min(want, wave), 1), block, smem, st, dep, a);
+}
+
+template <bool O32, bool LE1>
+static void launch_df(const SweepArgs& a, int parity, const Rows& r, cudaStream_t st, bool dep) {
+    if (parity == 0) launch_rows(k_sweep_df<0, O32, LE1, false>, k_sweep_df<0, O32, LE1, true>, a, r, 0, st, dep);
+    else launch_rows(k_sweep_df<1, O32, LE1, false>, k_sweep_df<1, O32, LE1, true>, a, r, 0, st, dep);
+}
+
+template <int S, bool O32>
+static void launch_o(SweepArgs a, int parity, int variant, int gz, int gy, cudaStream_t st, bool dep) {
+    const int nx = a.nx;
+    auto rows = [&](int cells, int max_bx, int threads, int resident) {
+        const int units = nx / cells;
+        const int bx = std::min(max_bx, (units + 31) / 32 * 32);
+        return Rows{bx, std::max(1, threads / bx), (units + bx - 1) / bx, gz, gy, resident};
+    };
     if constexpr (S == ST_F64) {
-        int bx = ((a.nx + 31) / 32) * 32;
-        if (bx > 256) bx = 256;
-        dim3 grid((a.nx + bx - 1) / bx, gy, gz);
-        SweepArgs b = a;
-        b.pf = prefetch_ahead(a, S, grid);
+        Rows r = rows(1, 256, 1, 3);
         if (variant == 1) {  // FP64 arithmetic
-            if (parity == 0) launch(k_sweep<S, 0, true>, grid, bx, 0, st, dep, a);
-            else launch(k_sweep<S, 1, true>, grid, bx, 0, st, dep, a);
-        } else if (o32) {
-            if (a.K.df.le1) launch_df<true, true>(b, parity, grid, bx, st, dep);
-            else launch_df<true, false>(b, parity, grid, bx, st, dep);
-        } else {
-            if (a.K.df.le1) launch_df<false, true>(b, parity, grid, bx, st, dep);
-            else launch_df<false, false>(b, parity, grid, bx, st, dep);
+            r.resident = 2;
+            if (parity == 0) launch_rows(k_sweep<S, 0, true, false>, k_sweep<S, 0, true, true>, a, r, 0, st, dep);
+            else launch_rows(k_sweep<S, 1, true, false>, k_sweep<S, 1, true, true>, a, r, 0, st, dep);
+            return;
         }
-    } else {
+        if (a.zmode == 2 || !a.K.df.le1) r.resident = 2;
+        a.pf = prefetch_ahead(a, S, r);
+        if (a.K.df.le1) launch_df<O32, true>(a, parity, r, st, dep);
+        else launch_df<O32, false>(a, parity, r, st, dep);
+        return;
+    }
     if constexpr (S == ST_F16 || S == ST_BF16) {
         // default: even steps in whole-row four-cell blocks (aligned 8-byte
         // chunks: 0.86 of the copy bandwidth at 256^3, against 0.74 for two
         // cells), odd steps in the two-cell form (0.63 before the L2
         // prefetch; the whole-row form's odd steps, with their x-shifts
         // through shared memory, measured 0.62), or in split sweeps as below
-        const bool rows4 = a.nx % 4 == 0 && a.nx <= 768;
+        const bool rows4 = nx % 4 == 0 && nx <= 768;
         // odd steps of split sweeps (far and near, mode 1 and 2): four cells per
         // thread.  Measured on GB300, 256^3 pusher, whole step against the
         // two-cell form: FP16 0.242 -> 0.232 ms, BF16 with stochastic rounding
@@ -170,59 +232,44 @@ static void launch_s(const SweepArgs& a, int parity, int variant, int gz, int gy
         // whole-lattice sweeps the two-cell form stays ahead (bare 256^3 step:
         // FP16 0.210 against 0.214 ms, BF16 to nearest 0.211 against 0.223),
         // so they keep it; why the split steps favour four cells is not known.
-        if (variant == 0 && parity == 1 && a.nx % 4 == 0 && a.zmode != 0) {
-            const int quads = a.nx / 4;
-            int bx = ((quads + 31) / 32) * 32;
-            if (bx > 64) bx = 64;
-            const int by = 192 / bx > 0 ? 192 / bx : 1;
-            dim3 block(bx, by), grid((quads + bx - 1) / bx, (gy + by - 1) / by, gz);
-            SweepArgs b = a;
-            b.pf = prefetch_ahead16(a, grid, 0);
-            if (o32) launch(k_sweep4o<S, true>, grid, block, 0, st, dep, b);
-            else launch(k_sweep4o<S, false>, grid, block, 0, st, dep, b);
+        if (variant == 0 && parity == 1 && nx % 4 == 0 && a.zmode != 0) {
+            const Rows r = rows(4, 64, 192, 2);
+            a.pf = prefetch_ahead16(a, r, 0);
+            launch_rows(k_sweep4o<S, O32, false>, k_sweep4o<S, O32, true>, a, r, 0, st, dep);
             return;
         }
         if ((variant == 3 || (variant == 0 && parity == 0)) && rows4) {
             // odd steps (more live values) in blocks of at most 192 threads
-            const int tx = a.nx / 4, ty = (parity == 0 ? 256 : 192) / tx > 0 ? (parity == 0 ? 256 : 192) / tx : 1;
-            dim3 block(tx, ty), grid(1, (gy + ty - 1) / ty, gz);
+            const int tx = nx / 4, ty = std::max(1, (parity == 0 ? 256 : 192) / tx);
+            const Rows r{tx, ty, 1, gz, gy, 2};
             if (parity == 0) {
-                SweepArgs b = a;
-                b.pf = prefetch_ahead16(a, grid, 2);
-                if (o32) launch(k_sweep4r<S, 0, true>, grid, block, 0, st, dep, b);
-                else launch(k_sweep4r<S, 0, false>, grid, block, 0, st, dep, b);
+                a.pf = prefetch_ahead16(a, r, 2);
+                launch_rows(k_sweep4r<S, 0, O32, false>, k_sweep4r<S, 0, O32, true>, a, r, 0, st, dep);
             } else {
-                const size_t smem = (size_t)10 * ty * a.nx * sizeof(unsigned short);
-                if (o32) launch(k_sweep4r<S, 1, true>, grid, block, smem, st, dep, a);
-                else launch(k_sweep4r<S, 1, false>, grid, block, smem, st, dep, a);
+                const size_t smem = (size_t)10 * ty * nx * sizeof(unsigned short);
+                launch_rows(k_sweep4r<S, 1, O32, false>, k_sweep4r<S, 1, O32, true>, a, r, smem, st, dep);
             }
             return;
         }
     }
-    if (variant != 1 && a.nx % 2 == 0) {
-        const int pairs = a.nx / 2;
-        int bx = ((pairs + 31) / 32) * 32;
-        if (bx > 128) bx = 128;
-        const int by = 256 / bx;
-        dim3 block(bx, by), grid((pairs + bx - 1) / bx, (gy + by - 1) / by, gz);
-        SweepArgs b = a;
-        b.pf = prefetch_ahead(a, S, grid);
-        if (S == ST_F16 || S == ST_BF16) b.pf = parity == 1 ? prefetch_ahead16(a, grid, 0) : 0;
-        if (o32) {
-            if (parity == 0) launch(k_sweep2<S, 0, true>, grid, block, 0, st, dep, b);
-            else launch(k_sweep2<S, 1, true>, grid, block, 0, st, dep, b);
-        } else {
-            if (parity == 0) launch(k_sweep2<S, 0, false>, grid, block, 0, st, dep, b);
-            else launch(k_sweep2<S, 1, false>, grid, block, 0, st, dep, b);
+    if constexpr (S != ST_F64) {
+        if (variant != 1 && nx % 2 == 0) {
+            const Rows r = rows(2, 128, 256, 2);
+            if (S == ST_F32) a.pf = prefetch_ahead(a, S, r);
+            else a.pf = parity == 1 ? prefetch_ahead16(a, r, 0) : 0;
+            if (parity == 0) launch_rows(k_sweep2<S, 0, O32, false>, k_sweep2<S, 0, O32, true>, a, r, 0, st, dep);
+            else launch_rows(k_sweep2<S, 1, O32, false>, k_sweep2<S, 1, O32, true>, a, r, 0, st, dep);
+            return;
         }
-        return;
+        const Rows r = rows(1, 256, 1, 4);
+        if (parity == 0) launch_rows(k_sweep<S, 0, false, false>, k_sweep<S, 0, false, true>, a, r, 0, st, dep);
+        else launch_rows(k_sweep<S, 1, false, false>, k_sweep<S, 1, false, true>, a, r, 0, st, dep);
     }
-    int bx = ((a.nx + 31) / 32) * 32;
-    if (bx > 256) bx = 256;
-    dim3 grid((a.nx + bx - 1) / bx, gy, gz);
-    if (parity == 0) launch(k_sweep<S, 0, false>, grid, bx, 0, st, dep, a);
-    else launch(k_sweep<S, 1, false>, grid, bx, 0, st, dep, a);
-    }
+}
+
+template <int S>
+static void launch_s(const SweepArgs& a, int parity, int variant, int gz, int gy, cudaStream_t st, bool dep) {
+    launch_o<S, true>(a, parity, variant, gz, gy, st, dep);
 }
 
 // variant: 0 = default (FP64: double-float collision, one cell per thread;

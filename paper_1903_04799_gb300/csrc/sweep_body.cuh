@@ -57,8 +57,7 @@ struct SweepArgs {
     // near-body window split.  The window is the box of rows win[0..3] =
     // (z0, z length, y0, y length), periodic in both.  Mode 0 sweeps every
     // cell; mode 1 ("far") every cell outside the window; mode 2 ("near") the
-    // cells inside it, blockIdx.z counting planes from z0 and the grid's rows
-    // counting from y0
+    // cells inside it (near_rows)
     TrtK K;  // collision constants (trt_constants)
     int zmode;
     const int* win;
@@ -80,41 +79,43 @@ struct SweepArgs {
     int pf;
 };
 
-// Plane of plane slot bz (grid z index, or a block's k-th plane in the
-// multi-plane form), or -1 if none.  The far sweep leaves out a window plane
-// only when the window spans every row.
-__device__ __forceinline__ int sweep_plane_at(const SweepArgs& a, int bz) {
-    if (a.zmode == 0) return a.reverse ? a.nz - 1 - bz : bz;
-    const int z0 = __ldg(a.win), len = __ldg(a.win + 1);
-    if (a.zmode == 2) {
-        if (bz >= len) return -1;
-        const int z = z0 + (a.reverse ? len - 1 - bz : bz);
-        return z >= a.nz ? z - a.nz : z;
-    }
-    if (a.reverse) bz = a.nz - 1 - bz;
-    const int rel = bz - z0 < 0 ? bz - z0 + a.nz : bz - z0;
-    return rel < len && __ldg(a.win + 3) >= a.ny ? -1 : bz;
+// Row (y, z) of grid row ly of this block in modes 0 and 1, and whether it is
+// swept.  The window comes in one 16-byte load and the row is known without
+// it, so that the two- and four-cell sweeps put the test (a load and about ten
+// instructions) behind their address arithmetic and prefetches: as four
+// separate loads and modulo steps ahead of everything else it cost a far
+// sweep 4 % (256^3: FP64 892 -> 927 us with an empty window, FP16 210 -> 217).
+__device__ __forceinline__ bool sweep_at(const SweepArgs& a, int ly, int& y, int& z) {
+    y = ly;
+    z = a.reverse ? a.nz - 1 - (int)blockIdx.z : (int)blockIdx.z;
+    if (a.zmode == 0) return ly < a.ny;
+    const int4 w = __ldg(reinterpret_cast<const int4*>(a.win));
+    int rz = z - w.x, ry = y - w.z;
+    rz += rz < 0 ? a.nz : 0;
+    ry += ry < 0 ? a.ny : 0;
+    return ly < a.ny && !(rz < w.y && ry < w.w);
 }
 
-// Row swept by grid row ly on plane z (a plane sweep_plane_at returned), or
-// -1 if none.
-__device__ __forceinline__ int sweep_row(const SweepArgs& a, int ly, int z) {
-    if (a.zmode == 0) return ly < a.ny ? ly : -1;
-    const int y0 = __ldg(a.win + 2), ylen = __ldg(a.win + 3);
-    if (a.zmode == 2) {
-        if (ly >= ylen) return -1;
-        const int y = y0 + ly;
-        return y >= a.ny ? y - a.ny : y;
+// Mode 2 (near): f(y, z, active) for the rows of the window, blockDim.y of them
+// at a time per block, strided by the grid (gridDim.y blocks, blockIdx.z = 0).
+// The window's size is known on the device only; a grid over its upper bound
+// cost about 1 us per wave of blocks that only found their row outside
+// (250^3 with two squirmers, whose window's bound is the whole lattice).
+// active is false for the threads past the last row (y, z are in range).
+template <class F>
+__device__ __forceinline__ void near_rows(const SweepArgs& a, F f) {
+    const int4 w = __ldg(reinterpret_cast<const int4*>(a.win));
+    const int rows = w.y * w.w;
+    for (int r0 = blockIdx.y * blockDim.y; r0 < rows; r0 += gridDim.y * blockDim.y) {
+        const bool active = r0 + (int)threadIdx.y < rows;
+        const unsigned r = active ? r0 + threadIdx.y : 0u;
+        const int bz = (int)(r / (unsigned)w.w), ly = (int)(r - (unsigned)bz * (unsigned)w.w);
+        int z = w.x + (a.reverse ? w.y - 1 - bz : bz), y = w.z + ly;
+        z -= z >= a.nz ? a.nz : 0;
+        y -= y >= a.ny ? a.ny : 0;
+        f(y, z, active);
     }
-    if (ly >= a.ny) return -1;
-    const int z0 = __ldg(a.win), zlen = __ldg(a.win + 1);
-    const int rz = z - z0 < 0 ? z - z0 + a.nz : z - z0;
-    const int ry = ly - y0 < 0 ? ly - y0 + a.ny : ly - y0;
-    return rz < zlen && ry < ylen ? -1 : ly;
 }
-
-// Plane swept by this block, or -1 if none.
-__device__ __forceinline__ int sweep_plane(const SweepArgs& a) { return sweep_plane_at(a, blockIdx.z); }
 
 // Arithmetic of the collision with every rounding spelled out (no contraction
 // left to the compiler), so that every sweep form -- one, two or four cells
@@ -480,7 +481,7 @@ __device__ __forceinline__ typename Pair<typename StoreT<S>::T>::V enc2_r(float 
 // O32: element offsets in 32-bit arithmetic (the launch checks 19 Np < 2^32):
 // three instructions an access instead of about seven.
 template <int S, int P, bool O32, bool SR>
-__device__ __forceinline__ void sweep_two_r(const SweepArgs& a, int x0, int y, int z, uint32_t skey) {
+__device__ __forceinline__ void sweep_two_r(const SweepArgs& a, int x0, int y, int z, uint32_t skey, bool go) {
     using Off = typename std::conditional<O32, uint32_t, int64_t>::type;
     using ST = StoreT<S>;
     using T = typename ST::T;
@@ -516,6 +517,7 @@ __device__ __forceinline__ void sweep_two_r(const SweepArgs& a, int x0, int y, i
             }
         }
     }
+    if (!go) return;
     R g0[Q], g1[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
@@ -570,14 +572,15 @@ __device__ __forceinline__ void sweep_two_r(const SweepArgs& a, int x0, int y, i
 // uniform branch per thread instead of a select between two conversions at
 // every store.
 template <int S, int P, bool O32 = false>
-__device__ __forceinline__ void sweep_two(const SweepArgs& a, int x0, int y, int z, uint32_t skey = 0u) {
+__device__ __forceinline__ void sweep_two(const SweepArgs& a, int x0, int y, int z, uint32_t skey = 0u,
+                                          bool go = true) {
     if constexpr (S == ST_BF16) {
         if (a.sr) {
-            sweep_two_r<S, P, O32, true>(a, x0, y, z, skey);
+            sweep_two_r<S, P, O32, true>(a, x0, y, z, skey, go);
             return;
         }
     }
-    sweep_two_r<S, P, O32, false>(a, x0, y, z, skey);
+    sweep_two_r<S, P, O32, false>(a, x0, y, z, skey, go);
 }
 
 template <int S> __device__ __forceinline__ float dec16(unsigned int h, float isc);
@@ -664,7 +667,8 @@ __device__ __forceinline__ void collide_four(uint2 g[Q], const SweepArgs& a, uin
 // aligned source chunks there and read the shifted elements back; stores
 // write the shifted results there and store the aligned chunks.  `buf` holds
 // 10 x blockDim.y x nx elements.  All threads of the block take part in the
-// barriers (`active`: the thread's row exists).
+// barriers (`active`: the thread's row exists and is swept; y, z are in range
+// either way).
 // O32: element offsets in 32-bit arithmetic (the launch checks 19 Np < 2^32).
 template <int S, int P, bool O32 = false>
 __device__ __forceinline__ void sweep_four_rows(const SweepArgs& a, int y, int z, bool active, unsigned short* buf,
@@ -681,7 +685,7 @@ __device__ __forceinline__ void sweep_four_rows(const SweepArgs& a, int y, int z
     const int dstride = blockDim.y * nx;
     auto at = [&](int x) -> int { return x < 0 ? x + nx : (x >= nx ? x - nx : x); };
     // even steps: L2 prefetch of the sources a.pf planes ahead (see sweep_two)
-    if (P == 0 && a.pf && active) {
+    if (P == 0 && a.pf) {
         const int zp = z + (a.reverse ? -a.pf : a.pf);
         if (zp >= 0 && zp < nz) {
 #pragma unroll
@@ -769,7 +773,7 @@ __device__ __forceinline__ void sweep_four_rows(const SweepArgs& a, int y, int z
 // issue four of each; the collision is the same (collide_four), so are the
 // bits.
 template <int S, bool O32 = false>
-__device__ __forceinline__ void sweep_four_odd(const SweepArgs& a, int x0, int y, int z, uint32_t skey) {
+__device__ __forceinline__ void sweep_four_odd(const SweepArgs& a, int x0, int y, int z, uint32_t skey, bool go) {
     using Off = typename std::conditional<O32, uint32_t, int64_t>::type;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
     const int ys[3] = {y == 0 ? ny - 1 : y - 1, y, y == ny - 1 ? 0 : y + 1};
@@ -790,6 +794,7 @@ __device__ __forceinline__ void sweep_four_odd(const SweepArgs& a, int x0, int y
                     F + ((Off)opp(i) * Np + (Off)nx * ((Off)ys[1 - cy(i)] + (Off)ny * (Off)zsp[1 - cz(i)]) + (Off)x0)));
         }
     }
+    if (!go) return;
     // g[i]: cells x0, x0 + 1 in .x, x0 + 2, x0 + 3 in .y (low half first)
     uint2 g[Q];
 #pragma unroll
