@@ -58,11 +58,11 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int4 tile) 
         const int y = (int)(r % ny), z = (int)(r / ny);
         if constexpr (S != ST_F64) {
             if (tile.w) {
-                sweep_two<S, P, true>(a, 2 * xi, y, z, skey);
+                sweep_two<S, P>(a, 2 * xi, y, z, skey);
                 continue;
             }
         }
-        sweep_one<S, P, false, true>(a, xi, y, z, skey);
+        sweep_one<S, P>(a, xi, y, z, skey);
     }
 }
 

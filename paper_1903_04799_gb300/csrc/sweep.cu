@@ -38,23 +38,23 @@ __global__ void __launch_bounds__(256) k_sweep(const SweepArgs a) {
 // sums as well; at 80 registers it spilled 240 bytes and 160 x 144 x 130 took
 // 219 us per step against 177 at two blocks per SM.  The near form, with its
 // loop over rows, runs at two blocks too.
-template <int P, bool O32, bool LE1, bool NEAR>
+template <int P, bool LE1, bool NEAR>
 __global__ void __launch_bounds__(256, NEAR || !LE1 ? 2 : 3) k_sweep_df(const SweepArgs a) {
     dep_wait();
     dep_launch();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if constexpr (NEAR) {
         near_rows(a, [&](int y, int z, bool active) {
-            if (active && x < a.nx) sweep_one_df<P, O32, LE1>(a, x, y, z);
+            if (active && x < a.nx) sweep_one_df<P, LE1>(a, x, y, z);
         });
     } else {
         int y, z;
         if (!sweep_at(a, blockIdx.y, y, z) || x >= a.nx) return;
-        sweep_one_df<P, O32, LE1>(a, x, y, z);
+        sweep_one_df<P, LE1>(a, x, y, z);
     }
 }
 
-template <int S, int P, bool O32, bool NEAR>
+template <int S, int P, bool NEAR>
 __global__ void __launch_bounds__(256, 2) k_sweep2(const SweepArgs a) {
     dep_wait();
     dep_launch();
@@ -62,20 +62,20 @@ __global__ void __launch_bounds__(256, 2) k_sweep2(const SweepArgs a) {
     const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     if constexpr (NEAR) {
         near_rows(a, [&](int y, int z, bool active) {
-            if (active && x0 < a.nx) sweep_two<S, P, O32>(a, x0, y, z, skey);
+            if (active && x0 < a.nx) sweep_two<S, P>(a, x0, y, z, skey);
         });
     } else {
         int y, z;
         const bool go = sweep_at(a, blockIdx.y * blockDim.y + threadIdx.y, y, z);
         if (x0 >= a.nx || y >= a.ny) return;
-        sweep_two<S, P, O32>(a, x0, y, z, skey, go);
+        sweep_two<S, P>(a, x0, y, z, skey, go);
     }
 }
 
 // 16-bit storages with nx % 4 == 0, nx <= 768: blocks of whole rows, four
 // cells per thread (see sweep_four_rows); dynamic shared memory of
 // 10 x rows x nx elements on odd steps.
-template <int S, int P, bool O32, bool NEAR>
+template <int S, int P, bool NEAR>
 __global__ void __launch_bounds__(P == 0 ? 256 : 192, 2) k_sweep4r(const SweepArgs a) {
     dep_wait();
     dep_launch();
@@ -83,13 +83,63 @@ __global__ void __launch_bounds__(P == 0 ? 256 : 192, 2) k_sweep4r(const SweepAr
     const uint32_t skey = S == ST_BF16 ? sr_step_key(a) : 0u;  // before any exit (see sr_step)
     if constexpr (NEAR) {
         near_rows(a, [&](int y, int z, bool active) {
-            sweep_four_rows<S, P, O32>(a, y, z, active, rowbuf, skey);
+            sweep_four_rows<S, P>(a, y, z, active, rowbuf, skey);
             if (P == 1) __syncthreads();  // the row buffer is reused
         });
     } else {
         int y, z;
         const bool go = sweep_at(a, blockIdx.y * blockDim.y + threadIdx.y, y, z);
-        sweep_four_rows<S, P, O32>(a, y < a.ny ? y : 0, z, go, rowbuf, skey);
+        sweep_four_rows<S, P>(a, y < a.ny ? y : 0, z, go, rowbuf, skey);
+    }
+}
+
+// 16-bit storages, even steps (modes 0 and 1), any nx: four consecutive cells
+// per thread (sweep_four_flat), those `ahead` cells further prefetched into L2.  The cells at the
+// lattice's end that fill no chunk of four, and the chunks that the window's
+// border cuts, go one by one.
+template <int S>
+__global__ void __launch_bounds__(256, 2) k_sweep4f(const SweepArgs a, uint32_t ahead) {
+    dep_wait();
+    dep_launch();
+    const uint32_t skey = S == ST_BF16 ? sr_step_key(a) : 0u;  // before any exit (see sr_step)
+    const uint32_t nx = a.nx, ny = a.ny, N = nx * ny * (uint32_t)a.nz;
+    const uint32_t n0 = 4u * (blockIdx.x * blockDim.x + threadIdx.x);
+    if (n0 >= N) return;
+    if (ahead && n0 + ahead < N) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"((const unsigned short*)a.F + ((Off)i * (Off)a.Np + n0 + ahead)));
+    }
+    unsigned take = n0 + 3 < N ? 15u : (1u << (N - n0)) - 1u;  // bit k: cell n0 + k is swept
+    if (a.zmode == 1) {
+        const int4 w = __ldg(reinterpret_cast<const int4*>(a.win));
+        unsigned in = 0;  // cells in the window
+        const uint32_t r0 = n0 / nx, r3 = (n0 + 3u) / nx;
+        uint32_t r = r0, x = n0 - r0 * nx;
+        for (int k = 0; k < 4; ++k) {
+            if (k > 0 && r0 != r3 && ++x >= nx) {
+                x = 0;
+                ++r;
+            }
+            if (k == 0 || x == 0) {
+                int rz = (int)(r / ny) - w.x, ry = (int)(r % ny) - w.z;
+                rz += rz < 0 ? a.nz : 0;
+                ry += ry < 0 ? a.ny : 0;
+                in |= rz < w.y && ry < w.w ? 1u << k : 0u;
+            } else {
+                in |= (in >> (k - 1) & 1u) << k;
+            }
+        }
+        take &= ~in;
+    }
+    if (take == 15u) {
+        sweep_four_flat<S>(a, n0, skey);
+    } else {
+        for (uint32_t k = 0; k < 4; ++k)
+            if (take >> k & 1u) {
+                const uint32_t n = n0 + k, r = n / nx;
+                sweep_one<S, 0>(a, (int)(n - r * nx), (int)(r % ny), (int)(r / ny), skey);
+            }
     }
 }
 
@@ -97,7 +147,7 @@ __global__ void __launch_bounds__(P == 0 ? 256 : 192, 2) k_sweep4r(const SweepAr
 // thread without shared memory (see sweep_four_odd), blocks of at most 192
 // threads (167 registers, no spill; at 256 threads the 128-register cap
 // spills 72-80 bytes and measured 3-4 % slower).
-template <int S, bool O32, bool NEAR>
+template <int S, bool NEAR>
 __global__ void __launch_bounds__(192, 2) k_sweep4o(const SweepArgs a) {
     dep_wait();
     dep_launch();
@@ -105,13 +155,13 @@ __global__ void __launch_bounds__(192, 2) k_sweep4o(const SweepArgs a) {
     const int x0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
     if constexpr (NEAR) {
         near_rows(a, [&](int y, int z, bool active) {
-            if (active && x0 < a.nx) sweep_four_odd<S, O32>(a, x0, y, z, skey, true);
+            if (active && x0 < a.nx) sweep_four_odd<S>(a, x0, y, z, skey, true);
         });
     } else {
         int y, z;
         const bool go = sweep_at(a, blockIdx.y * blockDim.y + threadIdx.y, y, z);
         if (x0 >= a.nx || y >= a.ny) return;
-        sweep_four_odd<S, O32>(a, x0, y, z, skey, go);
+        sweep_four_odd<S>(a, x0, y, z, skey, go);
     }
 }
 
@@ -190,14 +240,14 @@ static void launch_rows(K far_kernel, K near_kernel, const SweepArgs& a, const R
     launch(near_kernel, dim3(r.xblocks, (unsigned)std::min(want, wave), 1), block, smem, st, dep, a);
 }
 
-template <bool O32, bool LE1>
+template <bool LE1>
 static void launch_df(const SweepArgs& a, int parity, const Rows& r, cudaStream_t st, bool dep) {
-    if (parity == 0) launch_rows(k_sweep_df<0, O32, LE1, false>, k_sweep_df<0, O32, LE1, true>, a, r, 0, st, dep);
-    else launch_rows(k_sweep_df<1, O32, LE1, false>, k_sweep_df<1, O32, LE1, true>, a, r, 0, st, dep);
+    if (parity == 0) launch_rows(k_sweep_df<0, LE1, false>, k_sweep_df<0, LE1, true>, a, r, 0, st, dep);
+    else launch_rows(k_sweep_df<1, LE1, false>, k_sweep_df<1, LE1, true>, a, r, 0, st, dep);
 }
 
-template <int S, bool O32>
-static void launch_o(SweepArgs a, int parity, int variant, int gz, int gy, cudaStream_t st, bool dep) {
+template <int S>
+static void launch_s(SweepArgs a, int parity, int variant, int gz, int gy, cudaStream_t st, bool dep) {
     const int nx = a.nx;
     auto rows = [&](int cells, int max_bx, int threads, int resident) {
         const int units = nx / cells;
@@ -214,8 +264,8 @@ static void launch_o(SweepArgs a, int parity, int variant, int gz, int gy, cudaS
         }
         if (a.zmode == 2 || !a.K.df.le1) r.resident = 2;
         a.pf = prefetch_ahead(a, S, r);
-        if (a.K.df.le1) launch_df<O32, true>(a, parity, r, st, dep);
-        else launch_df<O32, false>(a, parity, r, st, dep);
+        if (a.K.df.le1) launch_df<true>(a, parity, r, st, dep);
+        else launch_df<false>(a, parity, r, st, dep);
         return;
     }
     if constexpr (S == ST_F16 || S == ST_BF16) {
@@ -225,6 +275,18 @@ static void launch_o(SweepArgs a, int parity, int variant, int gz, int gy, cudaS
         // prefetch; the whole-row form's odd steps, with their x-shifts
         // through shared memory, measured 0.62), or in split sweeps as below
         const bool rows4 = nx % 4 == 0 && nx <= 768;
+        // even steps of rows that whole-row blocks do not fit: four cells
+        // regardless of rows.  Whole-lattice steps (both parities) against the
+        // one- and two-cell forms: 250^3 FP16 241 -> 207 us, BF16 252 -> 217;
+        // 251^3 FP16 259 -> 217, BF16 375 -> 278.  Where whole rows fit, the two
+        // are equal in bare sweeps (256^3: 204 us) and the rows faster in split
+        // ones (256^3 pusher FP16 222 against 226 us: no divisions for the window)
+        if (variant == 0 && parity == 0 && a.zmode != 2 && !rows4) {
+            const uint32_t N = (uint32_t)nx * a.ny * a.nz, cells = 4 * 256;
+            const uint32_t ahead = 2u * sm_count() * cells + 2u * nx * a.ny;
+            launch(k_sweep4f<S>, (N + cells - 1) / cells, 256, 0, st, dep, a, ahead < N ? ahead : 0u);
+            return;
+        }
         // odd steps of split sweeps (far and near, mode 1 and 2): four cells per
         // thread.  Measured on GB300, 256^3 pusher, whole step against the
         // two-cell form: FP16 0.242 -> 0.232 ms, BF16 with stochastic rounding
@@ -235,7 +297,7 @@ static void launch_o(SweepArgs a, int parity, int variant, int gz, int gy, cudaS
         if (variant == 0 && parity == 1 && nx % 4 == 0 && a.zmode != 0) {
             const Rows r = rows(4, 64, 192, 2);
             a.pf = prefetch_ahead16(a, r, 0);
-            launch_rows(k_sweep4o<S, O32, false>, k_sweep4o<S, O32, true>, a, r, 0, st, dep);
+            launch_rows(k_sweep4o<S, false>, k_sweep4o<S, true>, a, r, 0, st, dep);
             return;
         }
         if ((variant == 3 || (variant == 0 && parity == 0)) && rows4) {
@@ -244,10 +306,10 @@ static void launch_o(SweepArgs a, int parity, int variant, int gz, int gy, cudaS
             const Rows r{tx, ty, 1, gz, gy, 2};
             if (parity == 0) {
                 a.pf = prefetch_ahead16(a, r, 2);
-                launch_rows(k_sweep4r<S, 0, O32, false>, k_sweep4r<S, 0, O32, true>, a, r, 0, st, dep);
+                launch_rows(k_sweep4r<S, 0, false>, k_sweep4r<S, 0, true>, a, r, 0, st, dep);
             } else {
                 const size_t smem = (size_t)10 * ty * nx * sizeof(unsigned short);
-                launch_rows(k_sweep4r<S, 1, O32, false>, k_sweep4r<S, 1, O32, true>, a, r, smem, st, dep);
+                launch_rows(k_sweep4r<S, 1, false>, k_sweep4r<S, 1, true>, a, r, smem, st, dep);
             }
             return;
         }
@@ -257,24 +319,20 @@ static void launch_o(SweepArgs a, int parity, int variant, int gz, int gy, cudaS
             const Rows r = rows(2, 128, 256, 2);
             if (S == ST_F32) a.pf = prefetch_ahead(a, S, r);
             else a.pf = parity == 1 ? prefetch_ahead16(a, r, 0) : 0;
-            if (parity == 0) launch_rows(k_sweep2<S, 0, O32, false>, k_sweep2<S, 0, O32, true>, a, r, 0, st, dep);
-            else launch_rows(k_sweep2<S, 1, O32, false>, k_sweep2<S, 1, O32, true>, a, r, 0, st, dep);
+            if (parity == 0) launch_rows(k_sweep2<S, 0, false>, k_sweep2<S, 0, true>, a, r, 0, st, dep);
+            else launch_rows(k_sweep2<S, 1, false>, k_sweep2<S, 1, true>, a, r, 0, st, dep);
             return;
         }
         const Rows r = rows(1, 256, 1, 4);
+        // (no L2 prefetch: 125 x 99 x 111 FP16 16.9 us per step without, 19.1 with)
         if (parity == 0) launch_rows(k_sweep<S, 0, false, false>, k_sweep<S, 0, false, true>, a, r, 0, st, dep);
         else launch_rows(k_sweep<S, 1, false, false>, k_sweep<S, 1, false, true>, a, r, 0, st, dep);
     }
 }
 
-template <int S>
-static void launch_s(const SweepArgs& a, int parity, int variant, int gz, int gy, cudaStream_t st, bool dep) {
-    launch_o<S, true>(a, parity, variant, gz, gy, st, dep);
-}
-
 // variant: 0 = default (FP64: double-float collision, one cell per thread;
-// FP32: two cells per thread (even nx); FP16 / BF16: even steps as 3, odd
-// steps as 2, or four cells per thread without shared memory in split
+// FP32: two cells per thread (even nx); FP16 / BF16: even steps as 3 or
+// k_sweep4f, odd steps as 2, or four cells per thread without shared memory in split
 // sweeps), 1 = one cell per thread (FP64: FP64 arithmetic), 2 = two
 // cells per thread where possible (not FP64), 3 = FP16 / BF16: four cells per
 // thread in blocks of whole rows on both parities, odd-step x-shifts through

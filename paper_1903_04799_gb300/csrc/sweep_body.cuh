@@ -44,6 +44,11 @@ __host__ __device__ inline TrtK trt_constants(double le, double lo) {
     k.inc = 0;
     return k;
 }
+// Element offset of a population slot.  A lattice holds fewer than 2^27 cells
+// (lb_create, the server's validate), so 19 Np < 2^32: an offset in 32 bits is
+// three instructions an access instead of about seven.
+using Off = uint32_t;
+
 struct SweepArgs {
     void* F;
     int nx, ny, nz;
@@ -322,11 +327,9 @@ __device__ __forceinline__ unsigned short bf16_sr(float v, uint32_t r) {
 __device__ __forceinline__ uint32_t bf16x2_sr(float a, float b, uint32_t w) { return cvt_rs_bf16x2(b, a, w); }
 
 // One cell (x, y, z) with FP64 storage, collided in double-float arithmetic
-// (sweep_df.cuh).  O32: element offsets in 32-bit arithmetic (the launch
-// checks 19 Np < 2^32).
-template <int P, bool O32 = false, bool LE1 = true>
+// (sweep_df.cuh).
+template <int P, bool LE1 = true>
 __device__ __forceinline__ void sweep_one_df(const SweepArgs& a, int x, int y, int z) {
-    using Off = typename std::conditional<O32, uint32_t, int64_t>::type;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
     const int xs[3] = {x == 0 ? nx - 1 : x - 1, x, x == nx - 1 ? 0 : x + 1};
     const int ys[3] = {y == 0 ? ny - 1 : y - 1, y, y == ny - 1 ? 0 : y + 1};
@@ -370,15 +373,11 @@ __device__ __forceinline__ void sweep_one_df(const SweepArgs& a, int x, int y, i
         st_stream(F + (P == 0 ? (Off)opp(i) * Np + cell(0, 0, 0) : (Off)i * Np + cell(cx(i), cy(i), cz(i))), w[i]);
 }
 
-// One cell (x, y, z).  FP64 storage collides in double-float arithmetic
-// unless NATIVE (FP64 arithmetic, the measured reference form); O32 (caller
-// checks 19 Np < 2^32) gives that form 32-bit element offsets.
-template <int S, int P, bool NATIVE = false, bool O32 = false>
-__device__ __forceinline__ void sweep_one(const SweepArgs& a, int x, int y, int z, uint32_t skey = 0u) {
-    if constexpr (S == ST_F64 && !NATIVE) {
-        if (a.K.df.le1) sweep_one_df<P, O32, true>(a, x, y, z);
-        else sweep_one_df<P, O32, false>(a, x, y, z);
-    } else {
+// One cell (x, y, z) in the storage's plain arithmetic; SR: BF16 stores round
+// stochastically (a compile-time branch, as in the two-cell form: 251^3 BF16,
+// whole-lattice step, 430 -> 375 us).
+template <int S, int P, bool SR>
+__device__ __forceinline__ void sweep_one_r(const SweepArgs& a, int x, int y, int z, uint32_t skey) {
     using ST = StoreT<S>;
     using T = typename ST::T;
     using R = typename ST::R;
@@ -387,43 +386,58 @@ __device__ __forceinline__ void sweep_one(const SweepArgs& a, int x, int y, int 
     const int ys[3] = {y == 0 ? ny - 1 : y - 1, y, y == ny - 1 ? 0 : y + 1};
     const int zs[3] = {z == 0 ? nz - 1 : z - 1, z, z == nz - 1 ? 0 : z + 1};
     T* __restrict__ F = (T*)a.F;
-    const int64_t Np = a.Np;
+    const Off Np = (Off)a.Np;
     // 16-bit storages collide in their scaled units (see kScaled)
     const R isc = kScaled<S> ? R(1) : (R)a.inv_scale, sc = kScaled<S> ? R(1) : (R)a.scale;
     const R rho0 = kScaled<S> ? (R)a.rho0s : (std::is_same<R, float>::value ? (R)a.rho0f : (R)a.rho0);
     R g[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-        int64_t off;
+        Off off;
         if (P == 0) {
-            off = (int64_t)i * Np + (x + (int64_t)nx * (y + (int64_t)ny * z));
+            off = (Off)i * Np + (x + (Off)nx * (y + (Off)ny * z));
         } else {
             const int ib = opp(i);
-            off = (int64_t)ib * Np +
-                  (xs[1 - cx(i)] + (int64_t)nx * (ys[1 - cy(i)] + (int64_t)ny * zs[1 - cz(i)]));
+            off = (Off)ib * Np +
+                  (xs[1 - cx(i)] + (Off)nx * (ys[1 - cy(i)] + (Off)ny * zs[1 - cz(i)]));
         }
         g[i] = ST::load(F + off, isc);
     }
     collide_trt<R, ST::dev>(g, a.K, rho0);
     const uint32_t ncell = (uint32_t)(x + nx * (y + ny * z));
-    const uint32_t ck = S == ST_BF16 && a.sr ? sr_pair_key(skey, ncell) : 0u;
+    const uint32_t ck = SR ? sr_pair_key(skey, ncell) : 0u;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-        int64_t off;
+        Off off;
         if (P == 0) {
-            off = (int64_t)opp(i) * Np + (x + (int64_t)nx * (y + (int64_t)ny * z));
+            off = (Off)opp(i) * Np + (x + (Off)nx * (y + (Off)ny * z));
         } else {
-            off = (int64_t)i * Np + (xs[1 + cx(i)] + (int64_t)nx * (ys[1 + cy(i)] + (int64_t)ny * zs[1 + cz(i)]));
+            off = (Off)i * Np + (xs[1 + cx(i)] + (Off)nx * (ys[1 + cy(i)] + (Off)ny * zs[1 + cz(i)]));
         }
-        if constexpr (S == ST_BF16) {
-            if (a.sr) {
-                st_stream(reinterpret_cast<unsigned short*>(F + off), bf16_sr((float)g[i], sr_half(sr_word(ck, i), ncell)));
-                continue;
-            }
+        if constexpr (SR) {
+            st_stream(reinterpret_cast<unsigned short*>(F + off), bf16_sr((float)g[i], sr_half(sr_word(ck, i), ncell)));
+        } else {
+            ST::store(F + off, g[i], sc);
         }
-        ST::store(F + off, g[i], sc);
     }
+}
+
+// One cell (x, y, z).  FP64 storage collides in double-float arithmetic
+// unless NATIVE (FP64 arithmetic, the measured reference form).
+template <int S, int P, bool NATIVE = false>
+__device__ __forceinline__ void sweep_one(const SweepArgs& a, int x, int y, int z, uint32_t skey = 0u) {
+    if constexpr (S == ST_F64 && !NATIVE) {
+        if (a.K.df.le1) sweep_one_df<P, true>(a, x, y, z);
+        else sweep_one_df<P, false>(a, x, y, z);
+        return;
     }
+    if constexpr (S == ST_BF16) {
+        if (a.sr) {
+            sweep_one_r<S, P, true>(a, x, y, z, skey);
+            return;
+        }
+    }
+    if constexpr (S != ST_F64 || NATIVE) sweep_one_r<S, P, false>(a, x, y, z, skey);
 }
 
 // Two-cell pair types: the stored element type T and its 2-vector.
@@ -478,11 +492,8 @@ __device__ __forceinline__ typename Pair<typename StoreT<S>::T>::V enc2_r(float 
 // directions on even steps, the directions with c_x = 0 on odd steps; scalar
 // accesses for the x-shifted slots of odd steps.  Twice the bytes in flight per
 // thread of the one-cell form, for the same arithmetic per cell.
-// O32: element offsets in 32-bit arithmetic (the launch checks 19 Np < 2^32):
-// three instructions an access instead of about seven.
-template <int S, int P, bool O32, bool SR>
+template <int S, int P, bool SR>
 __device__ __forceinline__ void sweep_two_r(const SweepArgs& a, int x0, int y, int z, uint32_t skey, bool go) {
-    using Off = typename std::conditional<O32, uint32_t, int64_t>::type;
     using ST = StoreT<S>;
     using T = typename ST::T;
     using R = typename ST::R;
@@ -571,16 +582,16 @@ __device__ __forceinline__ void sweep_two_r(const SweepArgs& a, int x0, int y, i
 // The rounding mode is a compile-time branch of the two-cell body: one
 // uniform branch per thread instead of a select between two conversions at
 // every store.
-template <int S, int P, bool O32 = false>
+template <int S, int P>
 __device__ __forceinline__ void sweep_two(const SweepArgs& a, int x0, int y, int z, uint32_t skey = 0u,
                                           bool go = true) {
     if constexpr (S == ST_BF16) {
         if (a.sr) {
-            sweep_two_r<S, P, O32, true>(a, x0, y, z, skey, go);
+            sweep_two_r<S, P, true>(a, x0, y, z, skey, go);
             return;
         }
     }
-    sweep_two_r<S, P, O32, false>(a, x0, y, z, skey, go);
+    sweep_two_r<S, P, false>(a, x0, y, z, skey, go);
 }
 
 template <int S> __device__ __forceinline__ float dec16(unsigned int h, float isc);
@@ -613,17 +624,16 @@ template <> __device__ __forceinline__ uint32_t enc16x2<ST_BF16>(float a, float 
     return u;
 }
 
-// Collision of four cells x0 .. x0 + 3 of row (y, z) (x0 and nx multiples of
-// 4) whose 16-bit populations g[i] hold two cells per 32-bit word (cell x0 in
-// the low half of .x), in place: decode, TRT in FP32 in the storage's scaled
+// Collision of four consecutive cells n0 .. n0 + 3 (n0 a multiple of 4) whose
+// 16-bit populations g[i] hold two cells per 32-bit word (cell n0 in the low
+// half of .x), in place: decode, TRT in FP32 in the storage's scaled
 // units (see kScaled), encode (BF16 with stochastic rounding: the four cells
 // are two pairs of the random bits).  Every four-cell form calls this, so they
 // all give the same bits.
 template <int S, bool SR>
-__device__ __forceinline__ void collide_four_r(uint2 g[Q], const SweepArgs& a, uint32_t skey, int x0, int y, int z) {
+__device__ __forceinline__ void collide_four_r(uint2 g[Q], const SweepArgs& a, uint32_t skey, uint32_t n0) {
     constexpr bool sr = SR;
     const float rho0 = a.rho0s;  // scaled units (see kScaled)
-    const uint32_t n0 = (uint32_t)x0 + (uint32_t)a.nx * ((uint32_t)y + (uint32_t)a.ny * (uint32_t)z);
     const uint32_t k01 = sr ? sr_pair_key(skey, n0) : 0u, k23 = sr ? sr_pair_key(skey, n0 + 2u) : 0u;
     // the cells in pairs (x0, x0 + 1) and (x0 + 2, x0 + 3): a pair's word of
     // each population is decoded, both cells collide, and one packed
@@ -649,14 +659,14 @@ __device__ __forceinline__ void collide_four_r(uint2 g[Q], const SweepArgs& a, u
     }
 }
 template <int S>
-__device__ __forceinline__ void collide_four(uint2 g[Q], const SweepArgs& a, uint32_t skey, int x0, int y, int z) {
+__device__ __forceinline__ void collide_four(uint2 g[Q], const SweepArgs& a, uint32_t skey, uint32_t n0) {
     if constexpr (S == ST_BF16) {
         if (a.sr) {
-            collide_four_r<S, true>(g, a, skey, x0, y, z);
+            collide_four_r<S, true>(g, a, skey, n0);
             return;
         }
     }
-    collide_four_r<S, false>(g, a, skey, x0, y, z);
+    collide_four_r<S, false>(g, a, skey, n0);
 }
 
 // 16-bit storages, four cells per thread, blocks of whole rows: a row of nx
@@ -669,8 +679,7 @@ __device__ __forceinline__ void collide_four(uint2 g[Q], const SweepArgs& a, uin
 // 10 x blockDim.y x nx elements.  All threads of the block take part in the
 // barriers (`active`: the thread's row exists and is swept; y, z are in range
 // either way).
-// O32: element offsets in 32-bit arithmetic (the launch checks 19 Np < 2^32).
-template <int S, int P, bool O32 = false>
+template <int S, int P>
 __device__ __forceinline__ void sweep_four_rows(const SweepArgs& a, int y, int z, bool active, unsigned short* buf,
                                                 uint32_t skey = 0u) {
     const int nx = a.nx, ny = a.ny, nz = a.nz;
@@ -678,7 +687,6 @@ __device__ __forceinline__ void sweep_four_rows(const SweepArgs& a, int y, int z
     const int ys[3] = {y == 0 ? ny - 1 : y - 1, y, y >= ny - 1 ? 0 : y + 1};
     const int zs[3] = {z == 0 ? nz - 1 : z - 1, z, z == nz - 1 ? 0 : z + 1};
     unsigned short* F = (unsigned short*)a.F;
-    using Off = typename std::conditional<O32, uint32_t, int64_t>::type;
     const Off Np = (Off)a.Np;
     auto row = [&](int dy, int dz) -> Off { return (Off)nx * ((Off)ys[1 + dy] + (Off)ny * (Off)zs[1 + dz]); };
     unsigned short* rowbuf = buf + (int64_t)threadIdx.y * nx;  // + d * blockDim.y * nx for shifted direction d
@@ -728,7 +736,7 @@ __device__ __forceinline__ void sweep_four_rows(const SweepArgs& a, int y, int z
         }
         __syncthreads();  // the buffer is reused for the stores
     }
-    collide_four<S>(g, a, skey, x0, y, z);
+    collide_four<S>(g, a, skey, (uint32_t)x0 + (uint32_t)nx * ((uint32_t)y + (uint32_t)ny * (uint32_t)z));
     d = 0;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
@@ -763,6 +771,22 @@ __device__ __forceinline__ void sweep_four_rows(const SweepArgs& a, int y, int z
     }
 }
 
+// 16-bit storages, even steps, four consecutive cells n0 .. n0 + 3 per thread
+// (n0 a multiple of 4; planes are padded to 64 cells, so every access is an
+// aligned 8-byte chunk).  An even step reads and writes a cell's own slots
+// only, so rows do not matter: any nx.
+template <int S>
+__device__ __forceinline__ void sweep_four_flat(const SweepArgs& a, Off n0, uint32_t skey) {
+    unsigned short* __restrict__ F = (unsigned short*)a.F;
+    const Off Np = (Off)a.Np;
+    uint2 g[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) g[i] = ld_stream(reinterpret_cast<const uint2*>(F + ((Off)i * Np + n0)));
+    collide_four<S>(g, a, skey, n0);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) st_stream(reinterpret_cast<uint2*>(F + ((Off)opp(i) * Np + n0)), g[i]);
+}
+
 // 16-bit storages, odd steps, four cells x0 .. x0 + 3 per thread (x0 and nx
 // multiples of 4), no shared memory: each direction's four sources are the
 // aligned 8-byte chunk at x0, shifted by one element with the element beyond
@@ -772,9 +796,8 @@ __device__ __forceinline__ void sweep_four_rows(const SweepArgs& a, int y, int z
 // that is two loads and three stores, where two threads of the two-cell form
 // issue four of each; the collision is the same (collide_four), so are the
 // bits.
-template <int S, bool O32 = false>
+template <int S>
 __device__ __forceinline__ void sweep_four_odd(const SweepArgs& a, int x0, int y, int z, uint32_t skey, bool go) {
-    using Off = typename std::conditional<O32, uint32_t, int64_t>::type;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
     const int ys[3] = {y == 0 ? ny - 1 : y - 1, y, y == ny - 1 ? 0 : y + 1};
     const int zs[3] = {z == 0 ? nz - 1 : z - 1, z, z == nz - 1 ? 0 : z + 1};
@@ -811,7 +834,7 @@ __device__ __forceinline__ void sweep_four_odd(const SweepArgs& a, int x0, int y
             g[i] = make_uint2(__byte_perm(c.x, c.y, 0x5432), __byte_perm(c.y, e, 0x5432));
         }
     }
-    collide_four<S>(g, a, skey, x0, y, z);
+    collide_four<S>(g, a, skey, (uint32_t)x0 + (uint32_t)nx * ((uint32_t)y + (uint32_t)ny * (uint32_t)z));
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         unsigned short* base = F + ((Off)i * Np + row(cy(i), cz(i)));

@@ -672,6 +672,26 @@ def test_sweep_variants_bitwise_16bit(storage, nx, lambda_e):
         assert np.array_equal(out[v][1], out[1][1]), v
 
 
+@pytest.mark.parametrize("storage", ["f16dev", "bf16dev"])
+@pytest.mark.parametrize("shape,lambda_e", [((3, 1, 1), 1.0), ((33, 13, 11), 1.0), ((50, 7, 9), 1.3),
+                                            ((45, 6, 10), 1.3), ((772, 3, 5), 1.0)])
+def test_flat_even_steps_bitwise_16bit(storage, shape, lambda_e):
+    """Even steps of rows that fit no whole-row block take four consecutive
+    cells per thread across rows: the same bits as the one-cell form, on cell
+    counts that leave 1, 2 and 3 cells over (3, 4719, 3150), on odd and even
+    rows and on rows too long for whole-row blocks."""
+    w = np.array([1 / 3] + [1 / 18] * 6 + [1 / 36] * 12)
+    f = W.random_populations(int(np.prod(shape)), seed=12, base=w, spread=0.2)
+    out = []
+    for variant in (0, 1):
+        with Lattice(shape, collision="trt", lambda_e=lambda_e, storage=storage) as g:
+            g.set_sweep_variant(variant)
+            g.set_populations(f)
+            g.step(7)
+            out.append(g.populations())
+    assert np.array_equal(out[0], out[1])
+
+
 def test_four_cell_f16_against_oracle():
     """FP16 storage on a 128-wide lattice (the four-cell sweep) against the
     FP64 oracle, with the tolerance of the two-cell FP16 test."""
