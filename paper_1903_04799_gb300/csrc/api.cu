@@ -37,8 +37,9 @@ void launch_tube_overlap(const Lattice& L, const int32_t* own, const int* kind, 
                          cudaStream_t st);
 void launch_tube_claim(const Lattice& L, int32_t* own, const BodyParams& q, int id, cudaStream_t st);
 void launch_set_flags(BodyAcc* acc, int nb, int k, int reclass, cudaStream_t st);
-void launch_psm_cover(const Bodies& B, int parity, int grid, bool f64, cudaStream_t st);
-void launch_psm_scatter(const Bodies& B, int parity, int grid, cudaStream_t st);
+void launch_psm_cover(const Bodies& B, int parity, int grid, bool f64, cudaStream_t st, bool dep = false,
+                      cudaEvent_t started = nullptr);
+void launch_psm_scatter(const Bodies& B, int parity, int grid, cudaStream_t st, bool dep = false);
 }  // namespace lbsq
 
 using namespace lbsq;
@@ -115,7 +116,8 @@ struct lb_ctx {
     std::vector<std::pair<void*, size_t>> allocs;
     // graph of two steps (even then odd)
     // graphs of 8 steps: [0] whole steps, or (split lattices) 8 units from t =
-    // 1 (mod 4); [1] split lattices, 8 units from t = 3 (mod 4)
+    // 1 (mod 4); [1] split lattices, 8 units from t = 3 (mod 4).  Split
+    // partially saturated cells: 8 steps from t = 0 or t = 2 (mod 4)
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     int64_t graph_launches = 0;  // kernel launches in one replay
     int sweep_variant = 0;
@@ -128,7 +130,8 @@ struct lb_ctx {
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr;
     cudaEvent_t ev_started = nullptr;  // every block of the fused body kernel has begun (see enqueue_unit)
     int* d_win = nullptr;  // [4][4] near-body windows (z0, z length, y0, y length) by step (mod 4)
-    bool split = false;    // whether steps are split into far and near sweeps
+    bool split = false;    // whether steps are split into far and near sweeps (link coupling: enqueue_unit)
+    bool psm_split = false;  // the same under partially saturated cells (enqueue_psm_steps)
     int win_max = 0;       // upper bound of the window's z length (planes)
     int ywin_max = 0;      // upper bound of its y length (rows)
     bool pending = false;  // split steps: the body step of step `step - 1` is not issued yet (see settle)
@@ -240,7 +243,7 @@ int* win_slot(const lb_ctx* c, int64_t s) { return c->d_win + 4 * (int)(s & 3); 
 // The view for the body kernels of step t: they write the window of step t + 2.
 Bodies bodies_for_step(const lb_ctx* c, int64_t t) {
     Bodies B = bodies_view(c);
-    if (c->split) B.win = win_slot(c, t + 2);
+    if (c->split || c->psm_split) B.win = win_slot(c, t + 2);
     return B;
 }
 
@@ -495,8 +498,11 @@ lb_status relayout(lb_ctx* c) {
             across = true;
         }
     }
-    // (partially saturated cells: every step sweeps the whole lattice)
-    c->split = !c->psm && !across && nb > 0 && wmax * 5 < 3 * c->L.nz;
+    // (partially saturated cells split only without walls, whose links would
+    // have to follow the scattered results)
+    const bool thin = !across && nb > 0 && wmax * 5 < 3 * c->L.nz;
+    c->split = !c->psm && thin;
+    c->psm_split = c->psm && thin && std::all_of(c->par.begin(), c->par.end(), [](const BodyParams& b) { return b.psm != 0; });
     if (ranges > 1) {
         wmax = c->L.nz;
         ymax = c->L.ny;
@@ -1060,19 +1066,26 @@ static void sweep_all(lb_ctx* c, int parity, cudaStream_t st, bool dep = false) 
     launch_sweep(c->L, c->lambda_e, c->lambda_o, parity, c->sweep_variant, 0, nullptr, c->L.nz, c->L.ny, st, dep);
 }
 
-// The sweep of a lattice with partially saturated cells: before it the
-// solid fractions, the covered cells' collisions and each sphere's force and
-// update (from the populations the step starts from); after it the covered
-// cells' results over the sweep's.  Returns the launch count.
-static int psm_sweep(lb_ctx* c, const Bodies& B, int parity, cudaStream_t st) {
-    if (c->n_psm_items == 0) {
-        sweep_all(c, parity, st);
-        return 1;
+// A step of a lattice with partially saturated cells, on stream st: the solid
+// fractions, the covered cells' collisions and each sphere's force and update
+// (from the populations the step starts from); the sweep; the covered cells'
+// results over the sweep's; the links of walls.  No sphere has links or
+// re-classifies, so nothing else follows.  dep: the last operation on st is a
+// kernel.  Returns the launch count.
+static int psm_step(lb_ctx* c, const Bodies& B, int parity, cudaStream_t st, bool dep) {
+    int n = 1;
+    if (c->n_psm_items > 0) {
+        launch_psm_cover(B, parity, c->grid_psm, c->p.storage == LB_F64, st, dep);
+        dep = true;
+        n += 3;
     }
-    launch_psm_cover(B, parity, c->grid_psm, c->p.storage == LB_F64, st);
-    sweep_all(c, parity, st);
-    launch_psm_scatter(B, parity, c->grid_psm, st);
-    return 4;
+    sweep_all(c, parity, st, dep);
+    if (c->n_psm_items > 0) launch_psm_scatter(B, parity, c->grid_psm, st, true);
+    if (c->n_link_items > 0) {
+        launch_body_kernel(1, B, parity, c->n_link_items, c->grid_box, nullptr, st, true);
+        ++n;
+    }
+    return n;
 }
 
 // The body kernels of one step on stream st: the fused kernel (spheres), the
@@ -1132,7 +1145,7 @@ static void enqueue_traced_step(lb_ctx* c) {
     if (psm) {  // kind 1: solid fractions, covered cells, sphere forces
         const size_t e0 = 2 * c->ev_used.size();
         cudaEventRecord(pool_event(c, e0), c->stream);
-        launch_psm_cover(bodies_view(c), parity, c->grid_psm, c->p.storage == LB_F64, c->stream);
+        launch_psm_cover(bodies_for_step(c, c->step), parity, c->grid_psm, c->p.storage == LB_F64, c->stream);
         c->launches += 2;
         cudaEventRecord(pool_event(c, e0 + 1), c->stream);
         c->ev_used.emplace_back(1, (int)e0);
@@ -1179,12 +1192,12 @@ static void enqueue_steps(lb_ctx* c, int64_t n) {
     for (int64_t k = 0; k < n; ++k) {
         const int parity = (int)(c->step & 1);
         if (c->psm) {
-            c->launches += psm_sweep(c, B, parity, c->stream);
+            c->launches += psm_step(c, B, parity, c->stream, k > 0);
         } else {
             sweep_all(c, parity, c->stream, k > 0);
             c->launches += 1;
+            if (bodies) c->launches += body_step(c, B, parity, c->stream, true);
         }
-        if (bodies) c->launches += body_step(c, B, parity, c->stream, !c->psm);
         c->step++;
     }
 }
@@ -1241,6 +1254,45 @@ static void end_units(lb_ctx* c) {
     cudaStreamWaitEvent(c->stream, c->ev_join2, 0);
 }
 
+// n steps of a lattice of partially saturated spheres that occupy a thin box
+// of rows.  Step t runs its cover kernels, the near sweep (the window) and the
+// scatter on `hi`, and the far sweep on `side`:
+//   - cover(t) reads the populations of the window, which near(t-1) and
+//     scatter(t-1) left (stream order), so it runs beside far(t-1);
+//   - near(t) waits for cover(t) (stream order) and far(t-1);
+//   - far(t) waits for far(t-1) (stream order) and near(t-1): a far cell's
+//     slots are not among those scatter(t-1) writes, whose cells lie two cells
+//     inside the window; and for the blocks of cover(t) to be placed, which
+//     the far sweep would otherwise keep off the SMs until its own last block
+//     is dispatched.
+// Cover(t) advances the spheres and writes the window of step t + 2, which
+// holds what the cover and scatter kernels of steps t + 1 .. t + 3 touch: a
+// sphere moves under half a cell a step, the window has two cells to spare.
+// In one chain the three kernels, whose few blocks leave the GPU idle, took
+// 80 us a step beside a sweep of 368 (256^3, R = 16, FP32).
+static void enqueue_psm_steps(lb_ctx* c, int64_t n) {
+    begin_units(c);
+    for (int64_t k = 0; k < n; ++k) {
+        const int64_t t = c->step;
+        const int parity = (int)(t & 1);
+        const int* win = win_slot(c, t);
+        const Bodies B = bodies_for_step(c, t);
+        launch_psm_cover(B, parity, c->grid_psm, c->p.storage == LB_F64, c->hi, k > 0, c->ev_started);
+        cudaStreamWaitEvent(c->side, c->ev_started, 0);
+        cudaStreamWaitEvent(c->hi, c->ev_join, 0);     // far(t-1), before near(t)
+        cudaStreamWaitEvent(c->side, c->ev_join2, 0);  // near(t-1), before far(t)
+        launch_sweep(c->L, c->lambda_e, c->lambda_o, parity, c->sweep_variant, 1, win, c->L.nz, c->L.ny, c->side);
+        cudaEventRecord(c->ev_join, c->side);
+        launch_sweep(c->L, c->lambda_e, c->lambda_o, parity, c->sweep_variant, 2, win, c->win_max, c->ywin_max, c->hi);
+        cudaEventRecord(c->ev_join2, c->hi);
+        launch_psm_scatter(B, parity, c->grid_psm, c->hi, true);
+        c->launches += 5;
+        c->step++;
+    }
+    cudaEventRecord(c->ev_join2, c->hi);  // the last scatter
+    end_units(c);
+}
+
 // Issue the pending body kernels, if any: the context then holds whole steps.
 static void settle(lb_ctx* c) {
     if (!c->pending) return;
@@ -1259,6 +1311,9 @@ static lb_status build_graph(lb_ctx* c, int which) {
         begin_units(c);
         for (int k = 0; k < kGraphSteps; ++k) enqueue_unit(c, k > 0);
         end_units(c);
+    } else if (c->psm_split) {
+        c->step = 2 * which;  // 8 steps from t = 0 or 2
+        enqueue_psm_steps(c, kGraphSteps);
     } else {
         c->step = 0;  // 8 steps from an even step
         enqueue_steps(c, kGraphSteps);
@@ -1302,12 +1357,14 @@ lb_status lb_step(lb_ctx* c, int64_t nsteps) {
             left--;
         }
     } else if (left > 0 && (c->step & 1)) {  // graphs start on even steps
-        enqueue_steps(c, 1);
+        if (c->psm_split) enqueue_psm_steps(c, 1);
+        else enqueue_steps(c, 1);
         left--;
     }
     if (left >= kGraphSteps) {
         // split lattices: t = step - 1 is odd here; t = 3 (mod 4) takes graph 1
-        const int which = c->split ? (int)(((c->step - 1) >> 1) & 1) : 0;
+        // (split partially saturated cells: t = step, even, 2 (mod 4) takes graph 1)
+        const int which = c->split ? (int)(((c->step - 1) >> 1) & 1) : (c->psm_split ? (int)((c->step >> 1) & 1) : 0);
         if (!c->graph[which]) {
             lb_status s = build_graph(c, which);
             if (s != LB_OK) return s;
@@ -1323,6 +1380,8 @@ lb_status lb_step(lb_ctx* c, int64_t nsteps) {
         begin_units(c);
         for (bool dep = false; left > 0; --left, dep = true) enqueue_unit(c, dep);
         end_units(c);
+    } else if (c->psm_split && left > 0) {
+        enqueue_psm_steps(c, left);
     } else if (left > 0) {
         enqueue_steps(c, left);
     }

@@ -2015,8 +2015,7 @@ __global__ void __launch_bounds__(kFT, 2) k_body_fused(const Bodies B, int cls, 
 // full: the cells to sample are taken one per warp (32 lanes share the 512
 // sample points), and the covered fluid cells one per thread.
 
-// Chunks of sphere p's box (kBB cells each) and the first one's index among
-// all spheres' chunks.
+// Chunks of sphere p's box (kBB cells each).
 __device__ __forceinline__ int psm_chunks(const BodyParams& p) {
     return (int)(((long long)p.box_w[0] * p.box_w[1] * p.box_w[2] + kBB - 1) / kBB);
 }
@@ -2114,6 +2113,8 @@ __device__ __forceinline__ void psm_cell_work(const Lattice& L, const Bodies& B,
 }
 
 __global__ void __launch_bounds__(kBB) k_psm_clear(const Bodies B, int P) {
+    dep_launch();  // before dep_wait: see launch_psm_cover
+    dep_wait();
     for (int it = blockIdx.x; it < B.n_psm_items; it += gridDim.x) {
         const int2 item = B.psm_items[it];
         const int k = item.x, q = item.y;
@@ -2142,6 +2143,8 @@ __global__ void __launch_bounds__(kBB) k_psm_clear(const Bodies B, int P) {
 
 template <int P, class V>
 __global__ void __launch_bounds__(kBB, 2) k_psm_cover(const Bodies B) {
+    dep_launch();  // before dep_wait: see launch_psm_cover
+    dep_wait();
     __shared__ double sm[12 * kBB + 12 * 16];
     __shared__ double s_tot[12];
     __shared__ BodyState s_new;
@@ -2235,11 +2238,23 @@ __global__ void __launch_bounds__(kBB, 2) k_psm_cover(const Bodies B) {
         __syncthreads();
         if (threadIdx.x < 32) update_stats(p, s, A, s_flag, &A, &B.state[1 - P][k], &s_new);
         __syncthreads();
+        // split steps: the last sphere to finish computes the near-body window
+        // of the sweeps two steps later
+        if (B.win && threadIdx.x == 0) {
+            __threadfence();
+            if (atomicAdd(B.fused_done, 1) == L.body_count - 1) {
+                *B.fused_done = 0;
+                __threadfence();
+                near_window<P>(B);
+            }
+        }
     }
 }
 
 template <int P>
 __global__ void __launch_bounds__(kBB) k_psm_scatter(const Bodies B) {
+    dep_launch();  // before dep_wait: see launch_psm_cover
+    dep_wait();
     for (int it = blockIdx.x; it < B.n_psm_items; it += gridDim.x) {
         const int2 item = B.psm_items[it];
         const int k = item.x, q = item.y;
@@ -2265,22 +2280,38 @@ __global__ void __launch_bounds__(kBB) k_psm_scatter(const Bodies B) {
 }
 
 // Before the sweep of a step of parity P: clear and cover (two launches);
-// f64: the lattice stores FP64 populations.
-void launch_psm_cover(const Bodies& B, int parity, int grid, bool f64, cudaStream_t st) {
-    k_psm_clear<<<grid, kBB, 0, st>>>(B, parity);
-    if (f64) {
-        if (parity == 0) k_psm_cover<0, double><<<grid, kBB, 0, st>>>(B);
-        else k_psm_cover<1, double><<<grid, kBB, 0, st>>>(B);
-    } else {
-        if (parity == 0) k_psm_cover<0, float><<<grid, kBB, 0, st>>>(B);
-        else k_psm_cover<1, float><<<grid, kBB, 0, st>>>(B);
+// f64: the lattice stores FP64 populations.  dep: the first is a dependent
+// launch (see dep_wait).  started: null, or an event to fire once every block
+// of the cover kernel is placed.  The three kernels release their dependents
+// before they wait themselves, so that scatter, clear and cover are all placed
+// while the near sweep before them drains, each waiting for the one before; a
+// far sweep that waits for `started` finds them on the SMs and cannot fill
+// these first.  (None of them reads anything before dep_wait.)
+void launch_psm_cover(const Bodies& B, int parity, int grid, bool f64, cudaStream_t st, bool dep,
+                      cudaEvent_t started) {
+    launch(k_psm_clear, grid, kBB, 0, st, dep, B, parity);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kBB);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (started) {
+        attr[1].id = cudaLaunchAttributeLaunchCompletionEvent;
+        attr[1].val.launchCompletionEvent.event = started;
+        attr[1].val.launchCompletionEvent.flags = 0;
+        cfg.numAttrs = 2;
     }
+    if (f64) cudaLaunchKernelEx(&cfg, parity == 0 ? k_psm_cover<0, double> : k_psm_cover<1, double>, B);
+    else cudaLaunchKernelEx(&cfg, parity == 0 ? k_psm_cover<0, float> : k_psm_cover<1, float>, B);
 }
 
 // After the sweep: the covered cells' results (one launch).
-void launch_psm_scatter(const Bodies& B, int parity, int grid, cudaStream_t st) {
-    if (parity == 0) k_psm_scatter<0><<<grid, kBB, 0, st>>>(B);
-    else k_psm_scatter<1><<<grid, kBB, 0, st>>>(B);
+void launch_psm_scatter(const Bodies& B, int parity, int grid, cudaStream_t st, bool dep) {
+    launch(parity == 0 ? k_psm_scatter<0> : k_psm_scatter<1>, grid, kBB, 0, st, dep, B);
 }
 
 void launch_body_kernel(int which, const Bodies& B, int parity, int grid_links, int grid_box, long long* step,

@@ -369,7 +369,7 @@ struct Bodies {
     const int* fused_first;  // [3]
     const int* n_fused;      // [3]
     const uint32_t* stencil; // shell stencils of those spheres
-    int* fused_done;         // clusters of a solo fused launch that finished (self-resetting)
+    int* fused_done;         // clusters of a solo fused launch, or spheres of k_psm_cover, that finished (self-resetting)
     // spheres coupled by partially saturated cells: items (body, block) of
     // their boxes, and per-block partial sums [body][GB][12]
     const int2* psm_items;

@@ -246,3 +246,37 @@ def test_psm_coupling_rules_and_tracing():
     assert (runs[0][0] == runs[1][0]).all()
     for a, b in zip(runs[0][1], runs[1][1]):
         assert (a == b).all()
+
+
+@pytest.mark.parametrize("storage", ["f64", "f32", "f16dev", "bf16dev"])
+@pytest.mark.parametrize("spheres", [1, 2])
+def test_split_steps_bitwise(storage, spheres):
+    """Split steps (the far sweep beside the cover kernels, the near sweep of
+    the window, the scatter) against whole-lattice sweeps (the traced mode
+    never splits): the same bits for every population, state, force and solid
+    fraction.  The first sphere sits across the periodic faces in y and z, so
+    the window wraps; the second one, 30 planes away, makes it span the gap.
+    Eager steps of both parities, both graphs (steps 0 and 2 mod 4) and reads
+    in between."""
+    shape = (50, 45, 130)
+    runs = []
+    for traced in (False, True):
+        g = Lattice(shape, collision="trt", storage=storage)
+        g.set_coupling("psm")
+        ids = [g.add_squirmer((24.3, 1.7, 128.9), (0.3, 0.5, 1.0), 4.3, 0.05, -3.0, mobile=True)]
+        if spheres == 2:
+            ids.append(g.add_squirmer((20.1, 40.2, 30.4), (0.1, -0.2, -1.0), 3.6, 0.05, 2.0, mobile=True))
+        if traced:
+            g.profile_begin()
+        seen = []
+        for n, read in ((5, False), (16, True), (3, False), (9, True), (1, True), (10, False), (8, False)):
+            g.step(n)
+            if read:
+                seen.append([*g.state(ids[0]), *g.force_torque(ids[0])])
+        if traced:
+            g.profile_end()
+        runs.append([g.populations(), g.solid_fraction(), *[x for i in ids for x in (*g.state(i), g.stresslet(i))],
+                     *[x for r in seen for x in r]])
+        g.close()
+    for a, b in zip(*runs):
+        assert np.array_equal(a, b)
