@@ -335,6 +335,13 @@ lb_status ensure_body_capacity(lb_ctx* c, int n) {
     return LB_OK;
 }
 
+// Whether a lattice is large enough for split steps: they hide the sweep
+// behind the body step at the price of one more kernel in the chain.  Measured
+// on GB300, one squirmer R = 3 (us per step, whole against split): FP64 32^3
+// 14.9 / 16.6, 40^3 24.5 / 24.2, 56^3 29.6 / 25.5; FP32 40^3 18.7 / 20.4, 64^3
+// 22.2 / 23.3, 80^3 28.4 / 24.5; FP16 64^3 22.1 / 22.6, 80^3 27.3 / 24.4.
+bool worth_splitting(const lb_ctx* c) { return c->L.N >= (c->p.storage == LB_F64 ? 64000 : 350000); }
+
 // After the body set changed: assign link segments, size the partial-sum
 // buffers and work lists, and upload the body parameters.
 lb_status relayout(lb_ctx* c) {
@@ -500,7 +507,7 @@ lb_status relayout(lb_ctx* c) {
     }
     // (partially saturated cells split only without walls, whose links would
     // have to follow the scattered results)
-    const bool thin = !across && nb > 0 && wmax * 5 < 3 * c->L.nz;
+    const bool thin = !across && nb > 0 && wmax * 5 < 3 * c->L.nz && worth_splitting(c);
     c->split = !c->psm && thin;
     c->psm_split = c->psm && thin && std::all_of(c->par.begin(), c->par.end(), [](const BodyParams& b) { return b.psm != 0; });
     if (ranges > 1) {
