@@ -93,53 +93,55 @@ __global__ void __launch_bounds__(P == 0 ? 256 : 192, 2) k_sweep4r(const SweepAr
     }
 }
 
-// 16-bit storages, even steps (modes 0 and 1), any nx: four consecutive cells
-// per thread (sweep_four_flat), those `ahead` cells further prefetched into L2.  The cells at the
-// lattice's end that fill no chunk of four, and the chunks that the window's
-// border cuts, go one by one.
+// Which of the `count` consecutive cells from n0 on are swept, as a bit mask
+// (modes 0 and 1).
+__device__ __forceinline__ unsigned cells_swept(const SweepArgs& a, uint32_t n0, uint32_t count) {
+    const unsigned all = (1u << count) - 1u;
+    if (a.zmode == 0) return all;
+    const int4 w = __ldg(reinterpret_cast<const int4*>(a.win));
+    const uint32_t nx = a.nx, ny = a.ny;
+    uint32_t r = n0 / nx, x = n0 - r * nx;
+    unsigned in = 0;  // cells in the window
+    for (uint32_t k = 0; k < count;) {
+        const uint32_t run = umin(count - k, nx - x);  // cells of row r
+        int rz = (int)(r / ny) - w.x, ry = (int)(r % ny) - w.z;
+        rz += rz < 0 ? a.nz : 0;
+        ry += ry < 0 ? a.ny : 0;
+        if (rz < w.y && ry < w.w) in |= ((1u << run) - 1u) << k;
+        k += run;
+        x = 0;
+        ++r;
+    }
+    return all & ~in;
+}
+
+// Even steps (modes 0 and 1) of rows that the forms above do not fit: four
+// consecutive cells per thread in 16 bits (sweep_four_flat), two in FP32, those
+// `ahead` cells further prefetched into L2.  The cells at the lattice's end
+// that fill no chunk, and the chunks that the window's border cuts, go one by
+// one.
 template <int S>
-__global__ void __launch_bounds__(256, 2) k_sweep4f(const SweepArgs a, uint32_t ahead) {
+__global__ void __launch_bounds__(256, 2) k_sweep_flat(const SweepArgs a, uint32_t ahead) {
     dep_wait();
     dep_launch();
     const uint32_t skey = S == ST_BF16 ? sr_step_key(a) : 0u;  // before any exit (see sr_step)
-    const uint32_t nx = a.nx, ny = a.ny, N = nx * ny * (uint32_t)a.nz;
-    const uint32_t n0 = 4u * (blockIdx.x * blockDim.x + threadIdx.x);
+    using T = typename StoreT<S>::T;
+    constexpr uint32_t W = S == ST_F32 ? 2 : 4;
+    const uint32_t N = (uint32_t)a.nx * (uint32_t)a.ny * (uint32_t)a.nz;
+    const uint32_t n0 = W * (blockIdx.x * blockDim.x + threadIdx.x);
     if (n0 >= N) return;
     if (ahead && n0 + ahead < N) {
 #pragma unroll
         for (int i = 0; i < Q; ++i)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"((const unsigned short*)a.F + ((Off)i * (Off)a.Np + n0 + ahead)));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"((const T*)a.F + ((Off)i * (Off)a.Np + n0 + ahead)));
     }
-    unsigned take = n0 + 3 < N ? 15u : (1u << (N - n0)) - 1u;  // bit k: cell n0 + k is swept
-    if (a.zmode == 1) {
-        const int4 w = __ldg(reinterpret_cast<const int4*>(a.win));
-        unsigned in = 0;  // cells in the window
-        const uint32_t r0 = n0 / nx, r3 = (n0 + 3u) / nx;
-        uint32_t r = r0, x = n0 - r0 * nx;
-        for (int k = 0; k < 4; ++k) {
-            if (k > 0 && r0 != r3 && ++x >= nx) {
-                x = 0;
-                ++r;
-            }
-            if (k == 0 || x == 0) {
-                int rz = (int)(r / ny) - w.x, ry = (int)(r % ny) - w.z;
-                rz += rz < 0 ? a.nz : 0;
-                ry += ry < 0 ? a.ny : 0;
-                in |= rz < w.y && ry < w.w ? 1u << k : 0u;
-            } else {
-                in |= (in >> (k - 1) & 1u) << k;
-            }
-        }
-        take &= ~in;
-    }
-    if (take == 15u) {
-        sweep_four_flat<S>(a, n0, skey);
+    const unsigned take = cells_swept(a, n0, umin(W, N - n0));
+    if (take == (1u << W) - 1u) {
+        if constexpr (S == ST_F32) sweep_two_flat(a, n0);
+        else sweep_four_flat<S>(a, n0, skey);
     } else {
-        for (uint32_t k = 0; k < 4; ++k)
-            if (take >> k & 1u) {
-                const uint32_t n = n0 + k, r = n / nx;
-                sweep_one<S, 0>(a, (int)(n - r * nx), (int)(r % ny), (int)(r / ny), skey);
-            }
+        for (uint32_t k = 0; k < W; ++k)
+            if (take >> k & 1u) sweep_one_call<S, 0>(a, (int)(n0 + k), 0, 0, skey);  // own slots only: any cell as x
     }
 }
 
@@ -246,6 +248,16 @@ static void launch_df(const SweepArgs& a, int parity, const Rows& r, cudaStream_
     else launch_rows(k_sweep_df<1, LE1, false>, k_sweep_df<1, LE1, true>, a, r, 0, st, dep);
 }
 
+// k_sweep_flat.  Whole-lattice steps (both parities) against the one- and
+// two-cell forms: 250^3 FP16 241 -> 207 us, BF16 252 -> 217; 251^3 FP16 259 ->
+// 217, BF16 375 -> 278; without the prefetch 250^3 FP16 215, BF16 227.
+template <int S>
+static void launch_flat(const SweepArgs& a, cudaStream_t st, bool dep) {
+    const uint32_t N = (uint32_t)a.nx * a.ny * a.nz, cells = (S == ST_F32 ? 2 : 4) * 256;
+    const uint32_t ahead = 2u * sm_count() * cells + 2u * a.nx * a.ny;
+    launch(k_sweep_flat<S>, (N + cells - 1) / cells, 256, 0, st, dep, a, ahead < N ? ahead : 0u);
+}
+
 template <int S>
 static void launch_s(SweepArgs a, int parity, int variant, int gz, int gy, cudaStream_t st, bool dep) {
     const int nx = a.nx;
@@ -281,10 +293,12 @@ static void launch_s(SweepArgs a, int parity, int variant, int gz, int gy, cudaS
         // 251^3 FP16 259 -> 217, BF16 375 -> 278.  Where whole rows fit, the two
         // are equal in bare sweeps (256^3: 204 us) and the rows faster in split
         // ones (256^3 pusher FP16 222 against 226 us: no divisions for the window)
+        // even steps of rows that whole-row blocks do not fit: four cells
+        // regardless of rows.  Where whole rows fit, the two are equal in bare
+        // sweeps (256^3: 204 us) and the rows faster in split ones (256^3 pusher
+        // FP16 222 against 226 us: no divisions for the window)
         if (variant == 0 && parity == 0 && a.zmode != 2 && !rows4) {
-            const uint32_t N = (uint32_t)nx * a.ny * a.nz, cells = 4 * 256;
-            const uint32_t ahead = 2u * sm_count() * cells + 2u * nx * a.ny;
-            launch(k_sweep4f<S>, (N + cells - 1) / cells, 256, 0, st, dep, a, ahead < N ? ahead : 0u);
+            launch_flat<S>(a, st, dep);
             return;
         }
         // odd steps of split sweeps (far and near, mode 1 and 2): four cells per
@@ -321,6 +335,15 @@ static void launch_s(SweepArgs a, int parity, int variant, int gz, int gy, cudaS
             else a.pf = parity == 1 ? prefetch_ahead16(a, r, 0) : 0;
             if (parity == 0) launch_rows(k_sweep2<S, 0, false>, k_sweep2<S, 0, true>, a, r, 0, st, dep);
             else launch_rows(k_sweep2<S, 1, false>, k_sweep2<S, 1, true>, a, r, 0, st, dep);
+            return;
+        }
+        // FP32 with odd nx, even steps: two cells regardless of rows (whole-lattice
+        // steps: 251^3 382 -> 361 us, 125 x 99 x 111 25.6 -> 25.1).  Odd steps keep
+        // one cell: pairs across odd rows, every access scalar and every second
+        // element left to another instruction, took 408 us.  In split steps of
+        // small lattices the window's divisions cost what the pairs gain.
+        if (S == ST_F32 && variant == 0 && parity == 0 && (a.zmode == 0 || (a.zmode == 1 && 19 * a.Np * 4 > (128 << 20)))) {
+            launch_flat<S>(a, st, dep);
             return;
         }
         const Rows r = rows(1, 256, 1, 4);

@@ -440,6 +440,13 @@ __device__ __forceinline__ void sweep_one(const SweepArgs& a, int x, int y, int 
     if constexpr (S != ST_F64 || NATIVE) sweep_one_r<S, P, false>(a, x, y, z, skey);
 }
 
+// sweep_one out of line, for kernels that take it beside a wider form (its
+// registers would add to theirs).
+template <int S, int P>
+__device__ __noinline__ void sweep_one_call(const SweepArgs& a, int x, int y, int z, uint32_t skey) {
+    sweep_one<S, P>(a, x, y, z, skey);
+}
+
 // Two-cell pair types: the stored element type T and its 2-vector.
 template <class T> struct Pair;
 template <> struct Pair<double> { using V = double2; __device__ static double lo(V v) { return v.x; } __device__ static double hi(V v) { return v.y; } __device__ static V make(double a, double b) { return make_double2(a, b); } };
@@ -769,6 +776,25 @@ __device__ __forceinline__ void sweep_four_rows(const SweepArgs& a, int y, int z
                           *reinterpret_cast<const uint2*>(r + x0));
         }
     }
+}
+
+// FP32, even steps, two consecutive cells n0, n0 + 1 per thread (n0 even): as
+// sweep_four_flat.
+__device__ __forceinline__ void sweep_two_flat(const SweepArgs& a, Off n0) {
+    float* __restrict__ F = (float*)a.F;
+    const Off Np = (Off)a.Np;
+    float g0[Q], g1[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const float2 v = ld_stream(reinterpret_cast<const float2*>(F + ((Off)i * Np + n0)));
+        g0[i] = v.x;
+        g1[i] = v.y;
+    }
+    collide_trt<float, true>(g0, a.K, a.rho0f);
+    collide_trt<float, true>(g1, a.K, a.rho0f);
+#pragma unroll
+    for (int i = 0; i < Q; ++i)
+        st_stream(reinterpret_cast<float2*>(F + ((Off)opp(i) * Np + n0)), make_float2(g0[i], g1[i]));
 }
 
 // 16-bit storages, even steps, four consecutive cells n0 .. n0 + 3 per thread
