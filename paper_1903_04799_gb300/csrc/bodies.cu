@@ -678,15 +678,33 @@ __device__ __forceinline__ void link_terms64(const Lattice& L, const BodyParams&
         fp[a] = s.pos[a] - f;
     }
     const int n3[3] = {L.nx, L.ny, L.nz};
-    for (int l = g + G * (int)threadIdx.x; l < (int)cnt; l += G * (int)blockDim.x) {
-        const Link k = link_of(L, links[l]);
+    // A wall's threads hold several links each: kU codes, then their outgoing
+    // populations, are loaded before any arithmetic or store (tube run: 80 000
+    // links on 128 blocks).
+    constexpr int kU = SPHERE ? 1 : 4;
+    const int stride = G * (int)blockDim.x;
+    for (int lb = g + G * (int)threadIdx.x; lb < (int)cnt; lb += kU * stride) {
+    uint32_t codes[kU];
+    Link lk[kU];
+    double fouts[kU];
+#pragma unroll
+    for (int q = 0; q < kU; ++q) codes[q] = lb + q * stride < (int)cnt ? links[lb + q * stride] : 0u;
+#pragma unroll
+    for (int q = 0; q < kU; ++q) {
+        if (lb + q * stride >= (int)cnt) continue;
+        lk[q] = link_of(L, codes[q]);
+        // where sweep P left f*_i of the fluid node
+        fouts[q] = load_abs(L, P == 0 ? (int64_t)opp(lk[q].i) * Np + lk[q].n : (int64_t)lk[q].i * Np + lk[q].ns, lk[q].i);
+    }
+#pragma unroll
+    for (int q = 0; q < kU; ++q) {
+        if (lb + q * stride >= (int)cnt) continue;
+        const Link k = lk[q];
         const int i = k.i, ib = opp(i);
         const int ci[3] = {cx(i), cy(i), cz(i)};
-        // where sweep P left f*_i of the fluid node, and where the next sweep
-        // reads the reflected population f_ib of the fluid node
-        const int64_t out_slot = P == 0 ? (int64_t)ib * Np + k.n : (int64_t)i * Np + k.ns;
+        // where the next sweep reads the reflected population f_ib of the fluid node
         const int64_t in_slot = P == 0 ? (int64_t)i * Np + k.ns : (int64_t)ib * Np + k.n;
-        const double fout = load_abs(L, out_slot, i);
+        const double fout = fouts[q];
         double d[3], cv;
         if (SPHERE) {
             // link midpoint (or boundary node) relative to the centre (minimum
@@ -732,6 +750,7 @@ __device__ __forceinline__ void link_terms64(const Lattice& L, const BodyParams&
                 acc[9 + (a == 2 ? 1 : (a == 0 ? 0 : 2))] += ab + ba;  // xy, yz, xz
             }
         }
+    }
     }
 }
 
@@ -865,25 +884,38 @@ __device__ __forceinline__ void sphere_totals(const Lattice& L, double* tot) {
 }
 
 // Links of a still body with no force readout: out slot copied to in slot in
-// the storage format (f_in = f_out when the wall velocity is zero).
+// the storage format T (f_in = f_out when the wall velocity is zero), kU links
+// at a time per thread so that their latencies overlap.
+template <int P, class T>
+__device__ __forceinline__ void copy_links_t(const Lattice& L, int cnt, const uint32_t* links, int g, int G) {
+    constexpr int kU = 4;
+    const int64_t Np = L.Np;
+    T* F = (T*)L.F;
+    const int stride = G * (int)blockDim.x;
+    for (int l0 = g * (int)blockDim.x + (int)threadIdx.x; l0 < cnt; l0 += kU * stride) {
+        uint32_t code[kU];
+        int64_t to[kU];
+        T v[kU];
+#pragma unroll
+        for (int q = 0; q < kU; ++q) code[q] = l0 + q * stride < cnt ? links[l0 + q * stride] : 0u;
+#pragma unroll
+        for (int q = 0; q < kU; ++q) {
+            if (l0 + q * stride >= cnt) continue;
+            const Link k = link_of(L, code[q]);
+            const int64_t a = (int64_t)opp(k.i) * Np + k.n, b = (int64_t)k.i * Np + k.ns;
+            to[q] = P == 0 ? b : a;
+            v[q] = F[P == 0 ? a : b];
+        }
+#pragma unroll
+        for (int q = 0; q < kU; ++q)
+            if (l0 + q * stride < cnt) F[to[q]] = v[q];
+    }
+}
 template <int P>
 __device__ __forceinline__ void copy_links(const Lattice& L, long long cnt, const uint32_t* links, int g, int G) {
-    const int64_t Np = L.Np;
-    const int bytes = L.storage == ST_F64 ? 8 : (L.storage == ST_F32 ? 4 : 2);
-    for (long long l = (long long)g * blockDim.x + threadIdx.x; l < cnt; l += (long long)G * blockDim.x) {
-        const uint32_t code = links[l];
-        const int64_t n = code >> 5;
-        const int i = code & 31, ib = opp(i);
-        int x, y, z;
-        cell_coords(L, n, x, y, z);
-        const int64_t ns =
-            cell_index(L, step_wrap(x, cx(i), L.nx), step_wrap(y, cy(i), L.ny), step_wrap(z, cz(i), L.nz));
-        const int64_t out_slot = P == 0 ? (int64_t)ib * Np + n : (int64_t)i * Np + ns;
-        const int64_t in_slot = P == 0 ? (int64_t)i * Np + ns : (int64_t)ib * Np + n;
-        if (bytes == 8) ((double*)L.F)[in_slot] = ((const double*)L.F)[out_slot];
-        else if (bytes == 4) ((float*)L.F)[in_slot] = ((const float*)L.F)[out_slot];
-        else ((unsigned short*)L.F)[in_slot] = ((const unsigned short*)L.F)[out_slot];
-    }
+    if (L.storage == ST_F64) copy_links_t<P, double>(L, (int)cnt, links, g, G);
+    else if (L.storage == ST_F32) copy_links_t<P, float>(L, (int)cnt, links, g, G);
+    else copy_links_t<P, unsigned short>(L, (int)cnt, links, g, G);
 }
 
 template <int P>
