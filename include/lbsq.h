@@ -405,7 +405,7 @@ typedef struct {
                                 owners, boundary links); allocated at creation */
     int32_t max_resident;    /* lattice slots, 1..256 */
     int32_t round_steps;     /* steps per scheduling round (even, >= 2) */
-    int32_t tile_units;      /* cells (or cell pairs) per sweep tile; 0 = pick by timing at creation */
+    int32_t tile_units;      /* cell pairs per sweep tile; 0 = pick by timing at creation */
     const lb_allocator* allocator; /* NULL = cudaMalloc / cudaFree */
 } lb_server_params;
 

@@ -8,10 +8,13 @@
 // memory and one captured CUDA graph (a round of steps) serves any mix of
 // resident requests.
 //
-// A step: k_sweep_tiles (persistent; each block walks the packed list of
-// z-slab tiles of all active lattices, branching per tile on the lattice's
-// storage), then the body kernels of bodies.cu over all bodies (work lists),
-// the last of which advances the device step counter.  A request admitted at
+// The resident lattices form two groups (kGroups), each a chain of its own:
+// while one chain is in its body kernels, which are bound by latency and leave
+// most of the GPU idle, the other sweeps.  A request joins the group that holds
+// fewer population bytes.  A step of a group: k_sweep_tiles (persistent; each
+// block walks the packed list of tiles of the group's active lattices of one
+// storage), then the body kernels of bodies.cu over the group's bodies (work
+// lists), the last of which advances the group's device step counter.  A request admitted at
 // global step s0 with n steps is active while s0 <= step < s0 + n, so it stops
 // inside a round at its own step; every round starts on an even step, which
 // keeps all resident lattices on the same streaming parity.
@@ -39,31 +42,62 @@ void launch_set_flags(BodyAcc* acc, int nb, int k, int reclass, cudaStream_t st)
 struct TileArgs {
     const Lattice* lats;
     const SweepArgs* sargs;  // per slot, built on the host at admission (collision constants included)
-    const int4* tiles;  // (lattice, first unit, end unit, paired), sorted by storage
-    const int* n_tiles; // [5]: tiles of storage S are [n_tiles[S], n_tiles[S+1])
+    const int4* tiles;  // (lattice, first cell, end cell, nx even), sorted by group and storage
+    const int* n_tiles; // [5], of the group: tiles of storage S are [n_tiles[S], n_tiles[S+1])
 };
 
-// A tile is the unit range [tile.y, tile.z) of one lattice, a unit being a cell
-// pair (paired tiles, nx even) or a cell, numbered x-fastest over the lattice.
-// A request holds fewer than 2^27 cells (validate), so every population index
-// of its lattice, below 19 x 2^27 < 2^32, fits the sweeps' 32-bit offsets.
+// A tile is the range [tile.y, tile.z) of cells of one lattice, x-fastest
+// (tile.y a multiple of 4; tile.w: nx is even).  A request holds fewer than
+// 2^27 cells (validate), so every population index of its lattice fits the
+// sweeps' 32-bit offsets.
+//
+// Even steps work on a cell's own slots, so a tile is a flat range: four cells
+// per thread in 16 bits, two in FP32, as aligned 8-byte chunks.  Odd steps take
+// a pair of neighbours per thread where nx is even, else one cell.  (Measured on
+// 24 requests, half of them with odd nx: pairs with scalar accesses for odd nx
+// 3 % slower, two cells a block apart per thread the same within 0.3 %; an
+// L2 prefetch of the thread's next unit 2 % slower.)
+template <int S>
+__device__ __forceinline__ void sweep_tile_even(const SweepArgs& a, const int4 tile, uint32_t skey) {
+    constexpr unsigned W = S == ST_F64 ? 1u : (S == ST_F32 ? 2u : 4u);
+    const unsigned end = (unsigned)tile.z, step = W * blockDim.x;
+    for (unsigned n = (unsigned)tile.y + W * threadIdx.x; n < end; n += step) {
+        if (n + W > end) {  // the lattice's last cells
+            for (unsigned m = n; m < end; ++m) sweep_one_call<S, 0>(a, (int)m, 0, 0, skey);
+        } else if constexpr (S == ST_F64) {
+            sweep_one<S, 0>(a, (int)n, 0, 0, skey);
+        } else if constexpr (S == ST_F32) {
+            sweep_two_flat(a, n);
+        } else {
+            sweep_four_flat<S>(a, n, skey);
+        }
+    }
+}
+
+template <int S>
+__device__ __forceinline__ void sweep_tile_odd(const SweepArgs& a, const int4 tile, uint32_t skey) {
+    const unsigned nx = (unsigned)a.nx, ny = (unsigned)a.ny, end = (unsigned)tile.z;
+    if (S == ST_F64 || tile.w) {
+        constexpr unsigned W = S == ST_F64 ? 1u : 2u;
+        for (unsigned n = (unsigned)tile.y + W * threadIdx.x; n < end; n += W * blockDim.x) {
+            const unsigned r = n / nx, z = r / ny;
+            const int x = (int)(n - r * nx), y = (int)(r - z * ny);
+            if constexpr (S == ST_F64) sweep_one<S, 1>(a, x, y, (int)z, skey);
+            else sweep_two<S, 1>(a, x, y, (int)z, skey);
+        }
+    } else if constexpr (S != ST_F64) {
+        for (unsigned n = (unsigned)tile.y + threadIdx.x; n < end; n += blockDim.x) {
+            const unsigned r = n / nx, z = r / ny;
+            sweep_one<S, 1>(a, (int)(n - r * nx), (int)(r - z * ny), (int)z, skey);
+        }
+    }
+}
+
 template <int P, int S>
 __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int4 tile) {
     const uint32_t skey = S == ST_BF16 ? sr_step_key(a) : 0u;  // the lattice's own step (global - start)
-    const unsigned nx = (unsigned)a.nx, ny = (unsigned)a.ny;
-    const unsigned per_row = tile.w ? nx / 2 : nx;
-    for (unsigned u = (unsigned)tile.y + threadIdx.x; u < (unsigned)tile.z; u += blockDim.x) {
-        const unsigned r = u / per_row;
-        const int xi = (int)(u - r * per_row);
-        const int y = (int)(r % ny), z = (int)(r / ny);
-        if constexpr (S != ST_F64) {
-            if (tile.w) {
-                sweep_two<S, P>(a, 2 * xi, y, z, skey);
-                continue;
-            }
-        }
-        sweep_one<S, P>(a, xi, y, z, skey);
-    }
+    if constexpr (P == 0) sweep_tile_even<S>(a, tile, skey);
+    else sweep_tile_odd<S>(a, tile, skey);
 }
 
 // One kernel per storage, so that none pays for another's registers; the
@@ -75,8 +109,10 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, const int4 tile) 
 // is swept, so that their dependent loads (tile, lattice, step counter) do not
 // stall the block between tiles.
 template <int P, int S>
-__global__ void __launch_bounds__(256, S == ST_F64 ? 1 : 2) k_sweep_tiles(const TileArgs T) {
+__global__ void __launch_bounds__(256, 2) k_sweep_tiles(const TileArgs T) {
     __shared__ __align__(16) SweepArgs s_a;
+    dep_wait();
+    dep_launch();
     const int t0 = T.n_tiles[S], t1 = T.n_tiles[S + 1];
     int cur = -1;
     int t = t0 + blockIdx.x;
@@ -111,17 +147,22 @@ __global__ void __launch_bounds__(256, S == ST_F64 ? 1 : 2) k_sweep_tiles(const 
     }
 }
 
+// The tile kernels of the storages in `mask` (bit S), one after the other;
+// dep: the first is a dependent launch (see dep_wait).
 template <int P>
-static void launch_tiles_p(const TileArgs& T, int grid, cudaStream_t st) {
-    k_sweep_tiles<P, ST_F64><<<grid, 256, 0, st>>>(T);
-    k_sweep_tiles<P, ST_F32><<<grid, 256, 0, st>>>(T);
-    k_sweep_tiles<P, ST_F16><<<grid, 256, 0, st>>>(T);
-    k_sweep_tiles<P, ST_BF16><<<grid, 256, 0, st>>>(T);
+static void launch_tiles_p(const TileArgs& T, unsigned mask, int grid, cudaStream_t st, bool dep) {
+    void (*k[4])(TileArgs) = {k_sweep_tiles<P, ST_F64>, k_sweep_tiles<P, ST_F32>, k_sweep_tiles<P, ST_F16>,
+                              k_sweep_tiles<P, ST_BF16>};
+    for (int s = 0; s < 4; ++s) {
+        if (!(mask >> s & 1u)) continue;
+        launch(k[s], grid, 256, 0, st, dep, T);
+        dep = true;
+    }
 }
 
-static void launch_tiles(const TileArgs& T, int parity, int grid, cudaStream_t st) {
-    if (parity == 0) launch_tiles_p<0>(T, grid, st);
-    else launch_tiles_p<1>(T, grid, st);
+static void launch_tiles(const TileArgs& T, int parity, unsigned mask, int grid, cudaStream_t st, bool dep) {
+    if (parity == 0) launch_tiles_p<0>(T, mask, grid, st, dep);
+    else launch_tiles_p<1>(T, mask, grid, st, dep);
 }
 
 }  // namespace lbsq
@@ -134,6 +175,7 @@ constexpr int kBodiesPerSlot = 5;  // squirmer + up to four walls (or an obstacl
 constexpr int kMaxGL = 128, kMaxGB = 256;
 constexpr size_t kAlign = 256;
 constexpr int kMaxSkips = 4;
+constexpr int kGroups = 2;  // chains of lattices stepped side by side
 
 // First-fit allocator over one device block.
 struct Arena {
@@ -197,6 +239,7 @@ struct Slot {
     std::vector<std::pair<size_t, size_t>> blocks;  // arena (offset, size)
     int nbodies = 0;
     int squirmer = -1;  // global body index
+    int group = 0;
     int64_t start = 0, stop = 0, half = 0;
     bool half_taken = false;
     double ve_half = 0.0;
@@ -230,7 +273,7 @@ struct lb_server {
     int2* d_link_items = nullptr;
     int2* d_box_items = nullptr;
     int2* d_rel_items = nullptr;
-    int* d_counts = nullptr;  // link items, box items, relink items, rebuild blocks done
+    int* d_counts = nullptr;  // per group: link items, box items, relink items, rebuild blocks done
     SweepArgs* d_sargs = nullptr;  // sweep arguments per slot
     int4* d_tiles = nullptr;
     int* d_ntiles = nullptr;
@@ -247,6 +290,9 @@ struct lb_server {
     double cell_updates = 0.0;
     int tile_units = 2048, blocks_per_sm = 2;
     cudaGraphExec_t graph = nullptr;
+    unsigned storages = 0;  // storages a request has had so far (bit lb_storage): the tile kernels of a step
+    cudaStream_t chain = nullptr;  // the second group's chain
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     std::string msg;
 };
 
@@ -296,20 +342,22 @@ std::vector<TableSpec> tables(lb_server* s) {
         {(void**)&s->d_part_links, sizeof(double) * B * kMaxGL * 12},
         {(void**)&s->d_part_conv, sizeof(double) * B * kMaxGB * 6},
         {(void**)&s->d_part_count, sizeof(int) * B * kMaxGB},
-        {(void**)&s->d_link_items, sizeof(int2) * s->list_cap},
-        {(void**)&s->d_box_items, sizeof(int2) * s->list_cap},
-        {(void**)&s->d_rel_items, sizeof(int2) * s->list_cap},
-        {(void**)&s->d_counts, sizeof(int) * 4},
+        {(void**)&s->d_link_items, sizeof(int2) * s->list_cap * kGroups},
+        {(void**)&s->d_box_items, sizeof(int2) * s->list_cap * kGroups},
+        {(void**)&s->d_rel_items, sizeof(int2) * s->list_cap * kGroups},
+        {(void**)&s->d_counts, sizeof(int) * 4 * kGroups},
         {(void**)&s->d_sargs, sizeof(SweepArgs) * s->cap_slots},
         {(void**)&s->d_tiles, sizeof(int4) * s->tile_cap},
-        {(void**)&s->d_ntiles, sizeof(int) * 5},
-        {(void**)&s->d_gstep, sizeof(long long)},
+        {(void**)&s->d_ntiles, sizeof(int) * 5 * kGroups},
+        {(void**)&s->d_gstep, sizeof(long long) * kGroups},
         {(void**)&s->d_errs, sizeof(int) * s->cap_slots},
     };
 }
 
-Bodies bodies_view(lb_server* s, bool step) {
-    Bodies B;
+Bodies bodies_view(lb_server* s, int group, bool step) {
+    Bodies B{};
+    int* counts = s->d_counts + 4 * group;
+    const size_t items = (size_t)s->list_cap * group;
     B.lats = s->d_lats;
     B.par = s->d_par;
     B.state[0] = s->d_state[0];
@@ -321,18 +369,18 @@ Bodies bodies_view(lb_server* s, bool step) {
     B.part_count = s->d_part_count;
     B.GL = kMaxGL;
     B.GB = kMaxGB;
-    B.link_items = s->d_link_items;
-    B.n_link_items = s->d_counts;
-    B.box_items = s->d_box_items;
-    B.n_box = s->d_counts + 1;
+    B.link_items = s->d_link_items + items;
+    B.n_link_items = counts;
+    B.box_items = s->d_box_items + items;
+    B.n_box = counts + 1;
     B.box_cap = s->list_cap;
-    B.rel_items = s->d_rel_items;
-    B.n_rel = s->d_counts + 2;
+    B.rel_items = s->d_rel_items + items;
+    B.n_rel = counts + 2;
     B.rel_cap = s->list_cap;
-    B.done = s->d_counts + 3;
+    B.done = counts + 3;
     B.err = s->d_errs;  // list overflow is reported on slot 0's word
     B.win = nullptr;
-    B.gstep = step ? s->d_gstep : nullptr;
+    B.gstep = step ? s->d_gstep + group : nullptr;
     // every body takes the multi-kernel path: the fused cluster kernel for the
     // squirmers measured no faster on the serving mix (28.78k against 28.75k
     // MLUPS with 8-block clusters, slower with 16)
@@ -342,7 +390,9 @@ Bodies bodies_view(lb_server* s, bool step) {
     return B;
 }
 
-TileArgs tile_args(lb_server* s) { return TileArgs{s->d_lats, s->d_sargs, s->d_tiles, s->d_ntiles}; }
+TileArgs tile_args(lb_server* s, int group) {
+    return TileArgs{s->d_lats, s->d_sargs, s->d_tiles, s->d_ntiles + 5 * group};
+}
 
 int storage_bytes_of(int st) { return st == LB_F64 ? 8 : (st == LB_F32 ? 4 : 2); }
 
@@ -457,6 +507,11 @@ lb_status admit(lb_server* s, int l, const Queued& q) {
         blocks.emplace_back(off, n);
     }
     const int64_t N = (int64_t)r.nx * r.ny * r.nz;
+    // the group with fewer population bytes
+    size_t held[kGroups] = {};
+    for (const Slot& o : s->slots)
+        if (o.used) held[o.group] += o.blocks[0].second;
+    const int group = (int)(std::min_element(held, held + kGroups) - held);
     Lattice L{};
     L.F = s->arena.base + blocks[0].first;
     L.nx = r.nx;
@@ -477,7 +532,7 @@ lb_status admit(lb_server* s, int l, const Queued& q) {
     L.wca_eps = r.wca_eps > 0.0 ? r.wca_eps : 0.0;
     L.body_begin = l * kBodiesPerSlot;
     L.active = 0;  // not stepped until set up
-    L.gstep = s->d_gstep;
+    L.gstep = s->d_gstep + group;
     L.stop_step = s->gstep + r.steps;
     L.start_step = s->gstep;
     L.rho_local = 0;
@@ -506,7 +561,8 @@ lb_status admit(lb_server* s, int l, const Queued& q) {
     SCK(cudaMemsetAsync(L.own_prev, 0, sizeof(int32_t) * N, str));
     SCK(cudaMemsetAsync(L.err, 0, sizeof(int), str));
     launch_fill_rest(L, str);
-    const Bodies B = bodies_view(s, false);
+    const Bodies B = bodies_view(s, group, false);
+    int* counts = s->d_counts + 4 * group;
     // parity of the next step is that of gstep (even); set-up passes run "after
     // a step of the other parity"
     const int P = 1 - (int)(s->gstep & 1);
@@ -517,10 +573,9 @@ lb_status admit(lb_server* s, int l, const Queued& q) {
         } else {
             std::vector<int2> items;
             for (int g = 0; g < bodies[j].g_box; ++g) items.push_back(make_int2(k, g));
-            SCK(cudaMemcpyAsync(s->d_box_items, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice,
-                                str));
+            SCK(cudaMemcpyAsync(B.box_items, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice, str));
             const int cnt[3] = {0, (int)items.size(), 0};
-            SCK(cudaMemcpyAsync(s->d_counts + 1, cnt + 1, sizeof(int) * 2, cudaMemcpyHostToDevice, str));
+            SCK(cudaMemcpyAsync(counts + 1, cnt + 1, sizeof(int) * 2, cudaMemcpyHostToDevice, str));
             launch_set_flags(s->d_acc, s->cap_bodies, k, 2, str);  // whole box
             launch_body_kernel(2, B, P, 1, std::max(1, std::min((int)items.size(), 4 * s->n_sm)), nullptr, str);
             SCK(cudaStreamSynchronize(str));  // item vector is transient
@@ -530,9 +585,9 @@ lb_status admit(lb_server* s, int l, const Queued& q) {
     std::vector<int2> items;
     for (size_t j = 0; j < bodies.size(); ++j)
         for (int g = 0; g < bodies[j].g_box; ++g) items.push_back(make_int2(L.body_begin + (int)j, g));
-    SCK(cudaMemcpyAsync(s->d_rel_items, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice, str));
+    SCK(cudaMemcpyAsync(B.rel_items, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice, str));
     const int cnt[2] = {0, (int)items.size()};
-    SCK(cudaMemcpyAsync(s->d_counts + 1, cnt, sizeof(int) * 2, cudaMemcpyHostToDevice, str));
+    SCK(cudaMemcpyAsync(counts + 1, cnt, sizeof(int) * 2, cudaMemcpyHostToDevice, str));
     for (size_t j = 0; j < bodies.size(); ++j) launch_set_flags(s->d_acc, s->cap_bodies, L.body_begin + (int)j, 0, str);
     const int gb = std::max(1, std::min((int)items.size(), 4 * s->n_sm));
     launch_body_kernel(3, B, P, 1, gb, nullptr, str);
@@ -552,6 +607,12 @@ lb_status admit(lb_server* s, int l, const Queued& q) {
     sl.L = L;
     sl.blocks = blocks;
     sl.nbodies = (int)bodies.size();
+    sl.group = group;
+    if (!(s->storages >> r.storage & 1u)) {  // a step gets another tile kernel
+        s->storages |= 1u << r.storage;
+        if (s->graph) cudaGraphExecDestroy(s->graph);
+        s->graph = nullptr;
+    }
     sl.squirmer = L.body_begin + (int)bodies.size() - 1;
     sl.start = s->gstep;
     sl.stop = L.stop_step;
@@ -598,61 +659,77 @@ lb_status fill_result(lb_server* s, int l, lb_result* out) {
     return LB_OK;
 }
 
-// Upload the static work of the resident mix: link items and sweep tiles.
+// Cells of a sweep tile of `units` cell pairs: a multiple of 4 (see sweep_tile).
+int64_t tile_cells(int units) { return (2 * (int64_t)units + 3) / 4 * 4; }
+
+// Upload the static work of the resident mix: each group's link items and
+// sweep tiles.
 lb_status upload_mix(lb_server* s) {
-    std::vector<int2> items;
+    std::vector<int2> items[kGroups];
     std::vector<int4> tiles;
-    int bounds[5] = {0, 0, 0, 0, 0};
+    int bounds[5 * kGroups];
     for (int l = 0; l < s->cap_slots; ++l) {
         const Slot& sl = s->slots[l];
         if (!sl.used) continue;
         for (int j = 0; j < sl.nbodies; ++j) {
             const int k = sl.L.body_begin + j;
-            for (int g = 0; g < s->par[k].g_links; ++g) items.push_back(make_int2(k, g));
+            for (int g = 0; g < s->par[k].g_links; ++g) items[sl.group].push_back(make_int2(k, g));
         }
     }
-    for (int st = 0; st < 4; ++st) {  // tiles sorted by storage
-        bounds[st] = (int)tiles.size();
-        for (int l = 0; l < s->cap_slots; ++l) {
-            const Slot& sl = s->slots[l];
-            if (!sl.used || sl.L.storage != st) continue;
-            const int paired = (sl.L.nx % 2 == 0 && st != LB_F64) ? 1 : 0;
-            const int64_t units = paired ? sl.L.N / 2 : sl.L.N;
-            for (int64_t u0 = 0; u0 < units; u0 += s->tile_units)
-                tiles.push_back(make_int4(l, (int)u0, (int)std::min<int64_t>(units, u0 + s->tile_units), paired));
+    for (int g = 0; g < kGroups; ++g) {
+        for (int st = 0; st < 4; ++st) {  // a group's tiles sorted by storage
+            bounds[5 * g + st] = (int)tiles.size();
+            for (int l = 0; l < s->cap_slots; ++l) {
+                const Slot& sl = s->slots[l];
+                if (!sl.used || sl.group != g || sl.L.storage != st) continue;
+                const int64_t cells = tile_cells(s->tile_units);
+                for (int64_t n0 = 0; n0 < sl.L.N; n0 += cells)
+                    tiles.push_back(make_int4(l, (int)n0, (int)std::min(sl.L.N, n0 + cells), sl.L.nx % 2 == 0));
+            }
         }
+        bounds[5 * g + 4] = (int)tiles.size();
+        if ((int)items[g].size() > s->list_cap) return sfail(s, LB_ERR_CAPACITY, "work lists of the resident mix");
     }
-    bounds[4] = (int)tiles.size();
-    if ((int)items.size() > s->list_cap || (int)tiles.size() > s->tile_cap)
-        return sfail(s, LB_ERR_CAPACITY, "work lists of the resident mix");
-    if (!items.empty())
-        SCK(cudaMemcpyAsync(s->d_link_items, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice,
-                            s->stream));
+    if ((int)tiles.size() > s->tile_cap) return sfail(s, LB_ERR_CAPACITY, "work lists of the resident mix");
+    int ni[kGroups];
+    for (int g = 0; g < kGroups; ++g) {
+        ni[g] = (int)items[g].size();
+        if (ni[g])
+            SCK(cudaMemcpyAsync(s->d_link_items + (size_t)s->list_cap * g, items[g].data(), sizeof(int2) * ni[g],
+                                cudaMemcpyHostToDevice, s->stream));
+        SCK(cudaMemcpyAsync(s->d_counts + 4 * g, &ni[g], sizeof(int), cudaMemcpyHostToDevice, s->stream));
+    }
     if (!tiles.empty())
         SCK(cudaMemcpyAsync(s->d_tiles, tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice, s->stream));
-    const int ni = (int)items.size();
-    SCK(cudaMemcpyAsync(s->d_counts, &ni, sizeof(int), cudaMemcpyHostToDevice, s->stream));
     SCK(cudaMemcpyAsync(s->d_ntiles, bounds, sizeof(bounds), cudaMemcpyHostToDevice, s->stream));
     SCK(cudaStreamSynchronize(s->stream));
     return LB_OK;
 }
 
-void enqueue_round(lb_server* s, cudaStream_t st) {
-    const Bodies B = bodies_view(s, true);
-    const TileArgs T = tile_args(s);
+// A round: each group's steps on a chain of its own.
+void enqueue_round(lb_server* s) {
     const int grid = s->blocks_per_sm * s->n_sm;
     const int glinks = 8 * s->n_sm, gbox = 4 * s->n_sm;  // latency-bound: many blocks
-    for (int k = 0; k < s->p.round_steps; ++k) {
-        const int P = k & 1;  // rounds start on even steps
-        launch_tiles(T, P, grid, st);
-        for (int w = 1; w <= 4; ++w) launch_body_kernel(w, B, P, glinks, gbox, nullptr, st);
+    cudaEventRecord(s->ev_fork, s->stream);
+    cudaStreamWaitEvent(s->chain, s->ev_fork, 0);
+    for (int g = 0; g < kGroups; ++g) {
+        const cudaStream_t st = g == 0 ? s->stream : s->chain;
+        const Bodies B = bodies_view(s, g, true);
+        const TileArgs T = tile_args(s, g);
+        for (int k = 0; k < s->p.round_steps; ++k) {
+            const int P = k & 1;  // rounds start on even steps
+            launch_tiles(T, P, s->storages, grid, st, k > 0);
+            for (int w = 1; w <= 4; ++w) launch_body_kernel(w, B, P, glinks, gbox, nullptr, st, true);
+        }
     }
+    cudaEventRecord(s->ev_join, s->chain);
+    cudaStreamWaitEvent(s->stream, s->ev_join, 0);
 }
 
 lb_status build_graph(lb_server* s) {
     cudaGraph_t g = nullptr;
     SCK(cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal));
-    enqueue_round(s, s->stream);
+    enqueue_round(s);
     cudaError_t e = cudaStreamEndCapture(s->stream, &g);
     if (e != cudaSuccess) return sfail(s, LB_ERR_CUDA, std::string("capture: ") + cudaGetErrorString(e));
     e = cudaGraphInstantiate(&s->graph, g, 0);
@@ -664,11 +741,12 @@ lb_status build_graph(lb_server* s) {
     return LB_OK;
 }
 
-// Tile-shape autotuner: time the tile sweep on two synthetic lattices (96^3
-// FP32 and FP16) for each candidate (planes per tile, blocks per SM) and keep
-// the fastest.  Uses arena memory that is free at creation.
+// Tile-shape autotuner: time the tile sweep on two synthetic lattices (128^3
+// FP32 and FP16: as many tiles as a group of requests has; on 96^3 the smallest
+// tiles won by their even tail, and served 24 requests 6 % slower) for each
+// candidate (cell pairs per tile, blocks per SM) and keep the fastest.  Uses arena memory that is free at creation.
 lb_status autotune(lb_server* s) {
-    const int n = 96;
+    const int n = 128;
     Lattice Ls[2];
     std::vector<std::pair<size_t, size_t>> blocks;
     const int storages[2] = {LB_F32, LB_F16DEV};
@@ -705,23 +783,24 @@ lb_status autotune(lb_server* s) {
     SCK(cudaEventCreate(&e1));
     float best = 1e30f;
     int best_tu = s->tile_units, best_b = s->blocks_per_sm;
-    const int tu_cand[4] = {512, 1024, 2048, 4096}, b_cand[2] = {2, 4};
+    const int tu_cand[2] = {1024, 2048}, b_cand[2] = {2, 4};  // 512 and 4096 pairs: 3-6 % slower on 24 requests
     for (int tu : tu_cand)
         for (int bps : b_cand) {
             // lattice 0 is FP32, lattice 1 FP16: tiles [0, m) and [m, 2m)
             std::vector<int4> tiles;
-            const int units = n * n * n / 2;
+            const int N = n * n * n, cells = (int)tile_cells(tu);
             for (int i = 0; i < 2; ++i)
-                for (int u0 = 0; u0 < units; u0 += tu) tiles.push_back(make_int4(i, u0, std::min(units, u0 + tu), 1));
+                for (int n0 = 0; n0 < N; n0 += cells) tiles.push_back(make_int4(i, n0, std::min(N, n0 + cells), 1));
             const int m = (int)tiles.size() / 2;
             const int bounds[5] = {0, 0, m, 2 * m, 2 * m};
             SCK(cudaMemcpyAsync(s->d_tiles, tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice,
                                 s->stream));
             SCK(cudaMemcpyAsync(s->d_ntiles, bounds, sizeof(bounds), cudaMemcpyHostToDevice, s->stream));
-            const TileArgs T = tile_args(s);
-            for (int w = 0; w < 2; ++w) launch_tiles(T, w & 1, bps * s->n_sm, s->stream);
+            const TileArgs T = tile_args(s, 0);
+            const unsigned both = 1u << LB_F32 | 1u << LB_F16DEV;
+            for (int w = 0; w < 2; ++w) launch_tiles(T, w & 1, both, bps * s->n_sm, s->stream, false);
             SCK(cudaEventRecord(e0, s->stream));
-            for (int w = 0; w < 6; ++w) launch_tiles(T, w & 1, bps * s->n_sm, s->stream);
+            for (int w = 0; w < 4; ++w) launch_tiles(T, w & 1, both, bps * s->n_sm, s->stream, false);
             SCK(cudaEventRecord(e1, s->stream));
             SCK(cudaEventSynchronize(e1));
             float ms = 0.0f;
@@ -778,6 +857,10 @@ lb_status lb_server_create(const lb_server_params* p, lb_server** out) {
         if (cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking) != cudaSuccess) return bail(LB_ERR_CUDA);
         s->own_stream = true;
     }
+    if (cudaStreamCreateWithFlags(&s->chain, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&s->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&s->ev_join, cudaEventDisableTiming) != cudaSuccess)
+        return bail(LB_ERR_CUDA);
     cudaDeviceGetAttribute(&s->n_sm, cudaDevAttrMultiProcessorCount, p->device);
     s->cap_slots = p->max_resident;
     s->cap_bodies = s->cap_slots * kBodiesPerSlot;
@@ -804,6 +887,9 @@ lb_status lb_server_destroy(lb_server* s) {
     if (!s) return LB_OK;
     if (s->stream) cudaStreamSynchronize(s->stream);
     if (s->graph) cudaGraphExecDestroy(s->graph);
+    if (s->ev_fork) cudaEventDestroy(s->ev_fork);
+    if (s->ev_join) cudaEventDestroy(s->ev_join);
+    if (s->chain) cudaStreamDestroy(s->chain);
     for (auto& t : tables(s)) sv_free(s, *t.ptr, t.bytes);
     sv_free(s, s->arena_mem, s->p.hbm_budget_bytes);
     if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);
@@ -882,7 +968,9 @@ lb_status lb_server_advance(lb_server* s, int32_t* running, int32_t* queued) {
             lb_status st = build_graph(s);
             if (st != LB_OK) return st;
         }
-        SCK(cudaMemcpyAsync(s->d_gstep, &s->gstep, sizeof(long long), cudaMemcpyHostToDevice, s->stream));
+        long long gs[kGroups];
+        std::fill(gs, gs + kGroups, (long long)s->gstep);
+        SCK(cudaMemcpyAsync(s->d_gstep, gs, sizeof(gs), cudaMemcpyHostToDevice, s->stream));
         SCK(cudaGraphLaunch(s->graph, s->stream));
         for (auto& sl : s->slots)
             if (sl.used) {
