@@ -356,7 +356,19 @@ __global__ void k_set_flags(BodyAcc* acc, int nb, int k, int reclass) {
     if (reclass) acc[j].margin_bits = (unsigned long long)__double_as_longlong(DBL_MAX);
 }
 
+// A read-out of a few hundred bytes: `words` 64-bit words of src after the
+// device error word, so that the host gets both in one copy.
+__global__ void k_gather(const int* err, const unsigned long long* src, int words, unsigned long long* dst) {
+    const int t = threadIdx.x;
+    if (t == 0) dst[0] = (unsigned long long)(unsigned)*err;
+    for (int w = t; w < words; w += blockDim.x) dst[1 + w] = src[w];
+}
+
 // ---------------------------------------------------------------- launchers
+
+void launch_gather(const int* err, const void* src, int words, void* dst, cudaStream_t st) {
+    k_gather<<<1, 64, 0, st>>>(err, (const unsigned long long*)src, words, (unsigned long long*)dst);
+}
 
 // f(storage, parity) with both as compile-time constants.
 template <class Fn>
