@@ -657,6 +657,38 @@ __device__ __forceinline__ Link link_of(const Lattice& L, uint32_t code) {
     return k;
 }
 
+// What the links of a sphere take of its state, converted once per block by a
+// few lanes of different warps (every thread for itself, the 20 or so FP64
+// conversions took a block of 256 threads 1.3 us): position split into integer
+// and fraction, so that link offsets keep full precision far from the origin
+// (fd: the fraction in FP64, exact), and the FP32 copies.
+struct SphereF {
+    int ip[3];
+    float fp[3], e[3], v[3], w[3], B1, B2, sh;
+    double fd[3];
+};
+__device__ __forceinline__ void load_sphere(const Lattice& L, const BodyParams& p, const BodyState& s, SphereF& o) {
+    const int warp = threadIdx.x >> 5, a = threadIdx.x & 31;
+    if (a < 3) {
+        if (warp == 0) {
+            const double f = floor(s.pos[a]), d = s.pos[a] - f;
+            o.ip[a] = (int)f;
+            o.fd[a] = d;
+            o.fp[a] = (float)d;
+        } else if (warp == 1) {
+            o.e[a] = (float)s.e[a];
+            o.v[a] = (float)s.vel[a];
+        } else if (warp == 2) {
+            o.w[a] = (float)s.omega[a];
+        } else if (warp == 3) {
+            if (a == 0) o.sh = (float)(6.0 * L.rho0);
+            else if (a == 1) o.B1 = (float)p.B1;
+            else o.B2 = (float)p.B2;
+        }
+    }
+    __syncthreads();
+}
+
 // FP64 links of a sphere (FP64 storage) or a wall (any storage): acc takes
 // force (0..2) and, for a sphere, torque (3..5) and the negated stresslet, its
 // off-diagonal components doubled (6..11; sphere_totals).  A link's dF lies
@@ -667,16 +699,12 @@ __device__ __forceinline__ Link link_of(const Lattice& L, uint32_t code) {
 // tripled the rounding error of the stresslet at R = 7); the trace leaves each
 // link for the same reason.
 template <int P, bool SPHERE>
-__device__ __forceinline__ void link_terms64(const Lattice& L, const BodyParams& p, const BodyState& s, long long cnt,
-                                             const uint32_t* links, int g, int G, double (&acc)[12]) {
+__device__ __forceinline__ void link_terms64(const Lattice& L, const BodyParams& p, const BodyState& s,
+                                             const SphereF& sp, long long cnt, const uint32_t* links, int g, int G,
+                                             double (&acc)[12]) {
     const int64_t Np = L.Np;
-    int ip[3];
-    double fp[3];
-    for (int a = 0; a < 3; ++a) {  // exact: the fraction of a coordinate
-        const double f = floor(s.pos[a]);
-        ip[a] = (int)f;
-        fp[a] = s.pos[a] - f;
-    }
+    const int* ip = sp.ip;
+    const double* fp = sp.fd;
     const int n3[3] = {L.nx, L.ny, L.nz};
     // A wall's threads hold several links each: kU codes, then their outgoing
     // populations, are loaded before any arithmetic or store (tube run: 80 000
@@ -758,21 +786,19 @@ __device__ __forceinline__ void link_terms64(const Lattice& L, const BodyParams&
 // each term of force, torque and stresslet an FP32 number, summed as pairs
 // (block_sum_fixed).
 template <int P>
-__device__ __forceinline__ void link_terms32(const Lattice& L, const BodyParams& p, const BodyState& s, long long cnt,
+__device__ __forceinline__ void link_terms32(const Lattice& L, const SphereF& sf, long long cnt,
                                              const uint32_t* links, int g, int G, df (&acc)[12]) {
     const int64_t Np = L.Np;
-    // body position split into integer and fraction, so that FP32 link
-    // offsets keep full precision far from the origin
     int ip[3];
     float fp[3], e32[3], v32[3], w32[3];
     for (int a = 0; a < 3; ++a) {
-        ip[a] = (int)floor(s.pos[a]);
-        fp[a] = (float)(s.pos[a] - (double)ip[a]);
-        e32[a] = (float)s.e[a];
-        v32[a] = (float)s.vel[a];
-        w32[a] = (float)s.omega[a];
+        ip[a] = sf.ip[a];
+        fp[a] = sf.fp[a];
+        e32[a] = sf.e[a];
+        v32[a] = sf.v[a];
+        w32[a] = sf.w[a];
     }
-    const float B1f = (float)p.B1, B2f = (float)p.B2, shf0 = (float)(6.0 * L.rho0), lat = L.link_at;
+    const float B1f = sf.B1, B2f = sf.B2, shf0 = sf.sh, lat = L.link_at;
     int l0, l1;
     link_range(cnt, g, G, l0, l1);
     // A thread's links are taken kU at a time: the link codes, then the
@@ -831,9 +857,9 @@ __device__ __forceinline__ void link_terms32(const Lattice& L, const BodyParams&
         const float shf = L.rho_local ? (float)(6.0 * post_density<P>(L, n, x, y, z)) : shf0;
         const float gin = gout - shf * (float)wgt(i) * cv;
         store_dev(L, in_slot, gin);
-        const float sf = gout + gin;
-        const float dF[3] = {ci[0] > 0 ? sf : (ci[0] < 0 ? -sf : 0.0f), ci[1] > 0 ? sf : (ci[1] < 0 ? -sf : 0.0f),
-                             ci[2] > 0 ? sf : (ci[2] < 0 ? -sf : 0.0f)};
+        const float sg = gout + gin;
+        const float dF[3] = {ci[0] > 0 ? sg : (ci[0] < 0 ? -sg : 0.0f), ci[1] > 0 ? sg : (ci[1] < 0 ? -sg : 0.0f),
+                             ci[2] > 0 ? sg : (ci[2] < 0 ? -sg : 0.0f)};
         const float tr = (d[0] * dF[0] + d[1] * dF[1] + d[2] * dF[2]) * (1.0f / 3.0f);
         const float t12[12] = {dF[0],
                                dF[1],
@@ -860,19 +886,20 @@ __device__ __forceinline__ void link_terms32(const Lattice& L, const BodyParams&
 // force, torque and stresslet, or what link_terms64 sums (FP64 storage).
 // none: the block takes no links (zero sums).
 template <int P, int T>
-__device__ __forceinline__ void sphere_links(const Lattice& L, const BodyParams& p, const BodyState& s, long long cnt,
-                                             const uint32_t* links, int g, int G, bool none, double* sm, double* tot) {
+__device__ __forceinline__ void sphere_links(const Lattice& L, const BodyParams& p, const BodyState& s,
+                                             const SphereF& sf, long long cnt, const uint32_t* links, int g, int G,
+                                             bool none, double* sm, double* tot) {
     if (L.storage == ST_F64) {
         double acc[12];
 #pragma unroll
         for (int c = 0; c < 12; ++c) acc[c] = 0.0;
-        if (!none) link_terms64<P, true>(L, p, s, cnt, links, g, G, acc);
+        if (!none) link_terms64<P, true>(L, p, s, sf, cnt, links, g, G, acc);
         block_sum_fixed<12, T>(acc, sm, tot);
     } else {
         df acc[12];
 #pragma unroll
         for (int c = 0; c < 12; ++c) acc[c] = {0.0f, 0.0f};
-        if (!none) link_terms32<P>(L, p, s, cnt, links, g, G, acc);
+        if (!none) link_terms32<P>(L, sf, cnt, links, g, G, acc);
         block_sum_fixed<12, T>(acc, sm, tot);
     }
 }
@@ -925,6 +952,7 @@ __global__ void __launch_bounds__(kLB) k_links(const Bodies B) {
     __shared__ double sm[12 * kLB + 12 * 8];
     __shared__ double s_tot[12];
     __shared__ BodyState s_new;
+    __shared__ SphereF s_sf;
     __shared__ int s_flag;
     const int nitems = *B.n_link_items;
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
@@ -945,13 +973,14 @@ __global__ void __launch_bounds__(kLB) k_links(const Bodies B) {
         const uint32_t* links = B.links + p.link_off;
         double* parts = B.part_links + (size_t)k * B.GL * 12;
         if (p.kind == BODY_SPHERE) {
-            sphere_links<P, kLB>(L, p, s, A.link_count, links, g, G, false, sm, s_tot);
+            load_sphere(L, p, s, s_sf);
+            sphere_links<P, kLB>(L, p, s, s_sf, A.link_count, links, g, G, false, sm, s_tot);
             if (threadIdx.x < 12) parts[g * 12 + threadIdx.x] = s_tot[threadIdx.x];
         } else {  // a wall: its force only
             double acc[12];
 #pragma unroll
             for (int c = 0; c < 3; ++c) acc[c] = 0.0;
-            link_terms64<P, false>(L, p, s, A.link_count, links, g, G, acc);
+            link_terms64<P, false>(L, p, s, s_sf, A.link_count, links, g, G, acc);
             double F[3] = {acc[0], acc[1], acc[2]};
             block_sum_fixed<3, kLB>(F, sm, s_tot);
             if (threadIdx.x < 3) parts[g * 12 + threadIdx.x] = s_tot[threadIdx.x];
@@ -1262,17 +1291,17 @@ __device__ __noinline__ void refill_finish(const Lattice& L, const BodyState& s,
     cross3(s.omega, d, wd);
     const double u[3] = {s.vel[0] + wd[0], s.vel[1] + wd[1], s.vel[2] + wd[2]};
     const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    double fi = 0.0;
     if (lane < Q) {
         const double cu = cx(lane) * u[0] + cy(lane) * u[1] + cz(lane) * u[2];
-        fi = L.inc ? wgt(lane) * (rb + L.rho0 * (3.0 * cu + 4.5 * cu * cu - 1.5 * uu))
-                   : wgt(lane) * rb * (1.0 + 3.0 * cu + 4.5 * cu * cu - 1.5 * uu);
+        const double fi = L.inc ? wgt(lane) * (rb + L.rho0 * (3.0 * cu + 4.5 * cu * cu - 1.5 * uu))
+                                : wgt(lane) * rb * (1.0 + 3.0 * cu + 4.5 * cu * cu - 1.5 * uu);
         store_abs(L, read_slot(L, lane, x, y, z, q), lane, fi);
     }
-    // created momentum sum_l c_l f_l: lane l holds its term (zero beyond Q)
-    const double m[3] = {warp_tree_sum(lane < Q ? fi * cx(lane) : 0.0), warp_tree_sum(lane < Q ? fi * cy(lane) : 0.0),
-                         warp_tree_sum(lane < Q ? fi * cz(lane) : 0.0)};
+    // created momentum sum_l c_l f_l of the equilibrium: rho u (incompressible:
+    // rho0 u); summed over the lanes, it took 18 more FP64 instructions
     if (lane == 0) {
+        const double rm = L.inc ? L.rho0 : rb;
+        const double m[3] = {rm * u[0], rm * u[1], rm * u[2]};
         double t[3];
         cross3(d, m, t);
         for (int a = 0; a < 3; ++a) {
@@ -1715,14 +1744,15 @@ __global__ void __launch_bounds__(kFT, 2) k_body_fused(const Bodies B, int cls, 
     __shared__ double s_zero[12];
     __shared__ int s_dryMode, s_flags;
     __shared__ ShellGeo s_geo;
+    __shared__ SphereF s_sf;
     __shared__ uint32_t s_stc[kStcBuf];
     __shared__ uint32_t s_emask[kStcBuf];  // phase A's link mask of each stencil entry, for phase B
     __shared__ int s_updated;              // rank 0: s_new holds this launch's new state
     __shared__ int s_lo[3];
-    __shared__ long long sml[kFT / 32];
-    __shared__ long long s_count, s_before;
-    __shared__ int s_scan[kFT / 32 + 1], s_list[kFT], s_mode, s_base;
-    __shared__ float s_min[kFT / 32], s_margin;
+    __shared__ uint32_t s_unc[kStcBuf / 32];  // the entries that were uncovered, a bit each (32 entries a word)
+    __shared__ int s_wcnt[kStcBuf / 32];       // links of each 32 entries
+    __shared__ int s_count, s_before, s_mode, s_base;
+    __shared__ int s_margin;  // FP32 bits, not negative: ordered as integers
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // tail: the lattice holds one sphere and nothing else, item (0, 0)
     const int i0 = tail ? 0 : B.fused_first[cls], nitems = tail ? 1 : B.n_fused[cls];
@@ -1752,6 +1782,7 @@ __global__ void __launch_bounds__(kFT, 2) k_body_fused(const Bodies B, int cls, 
         long long b0, b1;
         box_range(p.st_count, rank, KC, b0, b1);
         for (long long b = b0 + threadIdx.x; b < b1 && b < b0 + kStcBuf; b += kFT) s_stc[b - b0] = __ldg(stc + b);
+        load_sphere(L, p, s0, s_sf);
         // the populations follow; everything above was written by kernels
         // before the sweep this launch may have started beside
         dep_wait();
@@ -1768,7 +1799,8 @@ __global__ void __launch_bounds__(kFT, 2) k_body_fused(const Bodies B, int cls, 
             else if (threadIdx.x < 64)
                 update_turn(L, p, s0, s_A, s_zero, &s_dryA, &s_dryS, &s_dryS2);
         }
-        sphere_links<P, kFT>(L, p, s0, s_A.link_count, B.links + p.link_off, rank - 1, KC - 1, rank == 0, sm, s_tot);
+        sphere_links<P, kFT>(L, p, s0, s_sf, s_A.link_count, B.links + p.link_off, rank - 1, KC - 1, rank == 0, sm,
+                             s_tot);
         int near = 0;
         if (rank == 0)
             for (int j = L.body_begin + threadIdx.x; j < L.body_begin + L.body_count; j += kFT)
@@ -1809,6 +1841,9 @@ __global__ void __launch_bounds__(kFT, 2) k_body_fused(const Bodies B, int cls, 
             if (s_mode == 2) append_items(B.box_items, B.n_box, B.box_cap, k, p.g_box, B.err, &s_base);
         }
         cl.sync();
+        // one sphere and nothing else (see the end): the window from the state
+        // just computed, beside what follows
+        if (tail && ncl == 1 && B.win && rank == 0 && threadIdx.x == kFT - 32) sphere_window(L, p, s_new.pos, B.win);
         if (*cl.map_shared_rank(&s_mode, 0) != 1) continue;
         BodyAcc& A = B.acc[k];
 
@@ -1854,51 +1889,72 @@ __global__ void __launch_bounds__(kFT, 2) k_body_fused(const Bodies B, int cls, 
         // stencil entry b of this block's share (shared memory up to kStcBuf)
         auto entry = [&](long long b) -> uint32_t { return b - b0 < kStcBuf ? s_stc[b - b0] : __ldg(stc + b); };
         const int q = 1 - P;
+        if (threadIdx.x == 0) {
+            s_count = 0;
+            s_margin = __float_as_int(FLT_MAX);
+        }
+        __syncthreads();
         float mloc = FLT_MAX;
         double cacc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-        long long lcount = 0;
-        for (long long r0 = b0; r0 < b1; r0 += kFT) {
-            const long long b = r0 + threadIdx.x;
-            int uncover = 0, ox = 0, oy = 0, oz = 0;
-            uint32_t emask = 0;
-            float s32;
-            if (b < b1) decode_off(entry(b), ox, oy, oz);
-            if (b < b1 && geo_take(G, ox, oy, oz, s32)) {
-                const bool now = geo_inside(G, s32, G.pos, ox, oy, oz);
-                const bool was =
-                    geo_inside(G, d2_off(ox + G.sh[0], oy + G.sh[1], oz + G.sh[2], G.fo), G.old, ox, oy, oz);
-                mloc = fminf(mloc, fmaxf(fabsf(sqrtf(s32) - G.Rf) - 1e-3f, 0.0f));
-                if (now != was) {
-                    int x, y, z;
-                    const int64_t n = geo_cell(L, G, ox, oy, oz, x, y, z);
-                    // the owner, committed at once: nothing of this step reads it
-                    L.own[n] = now ? id : 0;
-                    L.own_prev[n] = now ? id : 0;
-                    if (now) covered_momentum<true>(L, s, x, y, z, q, cacc);  // fluid -> solid: to the body
-                    else uncover = 1;
+        int lcount = 0;
+        // kStcBuf entries at a time (one pass but for the largest spheres): every
+        // entry is classified, with a barrier at the end only; then the uncovered
+        // nodes, in entry order, are refilled one per warp
+        for (long long p0 = b0; p0 < b1; p0 += kStcBuf) {
+            const int np = (int)(b1 - p0 < kStcBuf ? b1 - p0 : kStcBuf);
+            for (int r0 = 0; r0 < np; r0 += kFT) {
+                const int j = r0 + (int)threadIdx.x;
+                const bool have = j < np;
+                int uncover = 0, ox = 0, oy = 0, oz = 0;
+                uint32_t emask = 0;
+                float s32;
+                if (have) decode_off(entry(p0 + j), ox, oy, oz);
+                if (have && geo_take(G, ox, oy, oz, s32)) {
+                    const bool now = geo_inside(G, s32, G.pos, ox, oy, oz);
+                    const bool was =
+                        geo_inside(G, d2_off(ox + G.sh[0], oy + G.sh[1], oz + G.sh[2], G.fo), G.old, ox, oy, oz);
+                    mloc = fminf(mloc, fmaxf(fabsf(sqrtf(s32) - G.Rf) - 1e-3f, 0.0f));
+                    if (now != was) {
+                        int x, y, z;
+                        const int64_t n = geo_cell(L, G, ox, oy, oz, x, y, z);
+                        // the owner, committed at once: nothing of this step reads it
+                        L.own[n] = now ? id : 0;
+                        L.own_prev[n] = now ? id : 0;
+                        if (now) covered_momentum<true>(L, s, x, y, z, q, cacc);  // fluid -> solid: to the body
+                        else uncover = 1;
+                    }
+                    if (!now) {
+                        emask = geo_mask(G, ox, oy, oz);
+                        lcount += __popc(emask);
+                    }
                 }
-                if (!now) {
-                    emask = geo_mask(G, ox, oy, oz);
-                    lcount += __popc(emask);
+                // each thread reads back only its own entries in phase B
+                if (have && p0 == b0) s_emask[j] = emask;
+                const uint32_t ub = __ballot_sync(0xffffffffu, uncover);
+                if (lane == 0) s_unc[j / 32] = ub;
+            }
+            __syncthreads();
+            int u = 0;  // uncovered nodes so far, in entry order
+            for (int w0 = 0; 32 * w0 < np; w0 += 32) {
+                const uint32_t mine = 32 * (w0 + lane) < np ? s_unc[w0 + lane] : 0u;
+                for (uint32_t any = __ballot_sync(0xffffffffu, mine != 0); any; any &= any - 1) {
+                    const int w = __ffs(any) - 1;
+                    for (uint32_t m = __shfl_sync(0xffffffffu, mine, w); m; m &= m - 1, ++u) {
+                        if (u % (kFT / 32) != warp) continue;
+                        int ux, uy, uz;
+                        decode_off(entry(p0 + 32 * (w0 + w) + __ffs(m) - 1), ux, uy, uz);
+                        geo_refill(L, G, s, ux, uy, uz, q, cacc);
+                    }
                 }
             }
-            // each thread reads back only its own entries in phase B
-            if (b - b0 < kStcBuf) s_emask[b - b0] = emask;
-            // uncovered nodes of this round, refilled one per warp
-            int nu;
-            const int pos = block_scan<kFT>(uncover, &nu, s_scan);
-            if (uncover) s_list[pos] = (int)(b - r0);
-            __syncthreads();
-            for (int u = warp; u < nu; u += kFT / 32) {
-                int ux, uy, uz;
-                decode_off(entry(r0 + s_list[u]), ux, uy, uz);
-                geo_refill(L, G, s, ux, uy, uz, q, cacc);
-            }
-            __syncthreads();
+            if (p0 + kStcBuf < b1) __syncthreads();  // s_unc is written again
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mloc = fminf(mloc, __shfl_down_sync(0xffffffffu, mloc, o));
-        if (lane == 0) s_min[warp] = mloc;
+        lcount = __reduce_add_sync(0xffffffffu, lcount);
+        const int mbits = __reduce_min_sync(0xffffffffu, __float_as_int(mloc));
+        if (lane == 0) {
+            atomicAdd(&s_count, lcount);
+            atomicMin(&s_margin, mbits);
+        }
         const int had = cacc[0] != 0.0 || cacc[1] != 0.0 || cacc[2] != 0.0 || cacc[3] != 0.0 || cacc[4] != 0.0 ||
                         cacc[5] != 0.0;
         if (__syncthreads_or(had)) {
@@ -1906,28 +1962,17 @@ __global__ void __launch_bounds__(kFT, 2) k_body_fused(const Bodies B, int cls, 
         } else if (threadIdx.x < 6) {
             s_conv[threadIdx.x] = 0.0;
         }
-        lcount = block_sum_ll<kFT>(lcount, sml);
-        if (threadIdx.x == 0) {
-            s_count = lcount;
-            float m = FLT_MAX;
-            for (int r = 0; r < kFT / 32; ++r) m = fminf(m, s_min[r]);
-            s_margin = m;
-        }
         cl.sync();
 
         // ---- phase B: link list compaction, commit of the owners (as k_rebuild)
         // link counts and node margins of all blocks: lane r of warp 0 reads
         // block r's (integer sums and a minimum: any order gives the same)
         if (warp == 0) {
-            const long long v = lane < KC ? *cl.map_shared_rank(&s_count, lane) : 0;
-            float m = lane < KC ? *cl.map_shared_rank(&s_margin, lane) : FLT_MAX;
-            long long all = v, bef = lane < rank ? v : 0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                all += __shfl_xor_sync(0xffffffffu, all, o);
-                bef += __shfl_xor_sync(0xffffffffu, bef, o);
-                m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
-            }
+            const int v = lane < KC ? *cl.map_shared_rank(&s_count, lane) : 0;
+            const int mb = lane < KC ? *cl.map_shared_rank(&s_margin, lane) : __float_as_int(FLT_MAX);
+            const int all = __reduce_add_sync(0xffffffffu, v);
+            const int bef = __reduce_add_sync(0xffffffffu, lane < rank ? v : 0);
+            const float m = __int_as_float(__reduce_min_sync(0xffffffffu, mb));
             if (lane == 0) {
                 s_before = bef;
                 if (rank == 0) {
@@ -1957,37 +2002,66 @@ __global__ void __launch_bounds__(kFT, 2) k_body_fused(const Bodies B, int cls, 
             if (c < 3) A.Fc[c] = t;
             else A.Tc[c - 3] = t;
         }
-        const long long before = s_before;
         uint32_t* links = B.links + p.link_off;
         const long long cap = p.link_cap;
-        long long base = before;
-        for (long long r0 = b0; r0 < b1; r0 += kFT) {
-            const long long b = r0 + threadIdx.x;
-            uint32_t mask = 0;
-            int64_t n = 0;
-            if (b < b1) {
-                int ox, oy, oz;
-                decode_off(entry(b), ox, oy, oz);
-                if (b - b0 < kStcBuf) {
-                    mask = s_emask[b - b0];
-                } else {  // beyond the buffer: as phase A computed it
-                    float s32;
-                    if (geo_take(G, ox, oy, oz, s32) && !geo_inside(G, s32, G.pos, ox, oy, oz))
-                        mask = geo_mask(G, ox, oy, oz);
+        long long base = s_before;
+        for (long long p0 = b0; p0 < b1; p0 += kStcBuf) {
+            const int np = (int)(b1 - p0 < kStcBuf ? b1 - p0 : kStcBuf);
+            // links of each 32 entries (beyond the first pass the masks again, as
+            // phase A computed them), then every warp's place: one barrier a pass
+            for (int r0 = 0; r0 < np; r0 += kFT) {
+                const int j = r0 + (int)threadIdx.x;
+                uint32_t mask = 0;
+                if (j < np) {
+                    if (p0 == b0) {
+                        mask = s_emask[j];
+                    } else {
+                        int ox, oy, oz;
+                        float s32;
+                        decode_off(entry(p0 + j), ox, oy, oz);
+                        if (geo_take(G, ox, oy, oz, s32) && !geo_inside(G, s32, G.pos, ox, oy, oz))
+                            mask = geo_mask(G, ox, oy, oz);
+                        s_emask[j] = mask;
+                    }
                 }
-                int x, y, z;
-                if (mask) n = geo_cell(L, G, ox, oy, oz, x, y, z);
+                const int c = __reduce_add_sync(0xffffffffu, __popc(mask));
+                if (lane == 0) s_wcnt[j / 32] = c;
             }
-            int tot;
-            const int off = block_scan<kFT>(__popc(mask), &tot, s_scan);
-            long long pos = base + off;
-            while (mask) {
-                const int i = __ffs(mask) - 1;
-                mask &= mask - 1;
-                if (pos < cap) links[pos] = (uint32_t)(n * 32 + i);
-                pos++;
+            __syncthreads();
+            int done = 0;  // links of the entries before this warp's next 32
+            int from = 0;  // in units of 32 entries
+            for (int r0 = 0; r0 < np; r0 += kFT) {
+                const int j = r0 + (int)threadIdx.x, word = r0 / 32 + warp;
+                int c = 0;
+                for (int w = from + lane; w < word; w += 32) c += s_wcnt[w];
+                done += __reduce_add_sync(0xffffffffu, c);
+                from = word;
+                uint32_t mask = j < np ? s_emask[j] : 0u;
+                int inc = __popc(mask);
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int t = __shfl_up_sync(0xffffffffu, inc, o);
+                    if (lane >= o) inc += t;
+                }
+                if (mask) {
+                    int ox, oy, oz, x, y, z;
+                    decode_off(entry(p0 + j), ox, oy, oz);
+                    const int64_t n = geo_cell(L, G, ox, oy, oz, x, y, z);
+                    long long pos = base + done + inc - __popc(mask);
+                    while (mask) {
+                        const int i = __ffs(mask) - 1;
+                        mask &= mask - 1;
+                        if (pos < cap) links[pos] = (uint32_t)(n * 32 + i);
+                        pos++;
+                    }
+                }
             }
-            base += tot;
+            if (p0 + kStcBuf < b1) {  // the next pass starts after this one's links
+                int c = 0;
+                for (int w = lane; 32 * w < np; w += 32) c += s_wcnt[w];
+                base += __reduce_add_sync(0xffffffffu, c);
+                __syncthreads();  // s_wcnt and s_emask are written again
+            }
         }
     }
     dep_wait();  // a cluster without an item
@@ -1998,10 +2072,7 @@ __global__ void __launch_bounds__(kFT, 2) k_body_fused(const Bodies B, int cls, 
     // cluster to finish computes the near-body window of the coming sweeps,
     // as the rebuild kernel does otherwise.
     if (tail && B.win && rank == 0 && threadIdx.x == 0) {
-        if (ncl == 1 && s_updated) {  // one cluster: the window from the state it holds
-            sphere_window(s_L, s_p, s_new.pos, B.win);
-            return;
-        }
+        if (ncl == 1 && s_updated) return;  // one cluster: written above
         __threadfence();
         if (atomicAdd(B.fused_done, 1) == ncl - 1) {
             *B.fused_done = 0;
