@@ -41,8 +41,7 @@ enum DfIdx : int {
     DK_LE,       // le
     DK_LE3,      // le / 3
     DK_1MLE,     // 1 - le
-    DK_MHLE,     // -le / 2
-    DK_MHLO,     // -lo / 2
+    DK_CS,       // (1 - le) / 2
     DK_RHO0,     // rho0
     DK_IRHO0,    // 1 / rho0
     DK_N
@@ -57,7 +56,7 @@ __host__ __device__ inline void df_split(double v, float& h, float& l) {
 }
 __host__ __device__ inline DfK df_constants(double le, double lo, double rho0) {
     const double v[DK_N] = {1.0 / 18.0, 1.0 / 3.0, 3.0 * lo / 18.0, 3.0 * lo / 36.0, 0.5 * (1.0 - lo), le,
-                            le / 3.0,   1.0 - le,  -0.5 * le,       -0.5 * lo,       rho0,             1.0 / rho0};
+                            le / 3.0,   1.0 - le,  0.5 * (1.0 - le), rho0,            1.0 / rho0};
     DfK k;
     for (int i = 0; i < DK_N; ++i) df_split(v[i], k.h[i], k.l[i]);
     k.le1 = (1.0 - le) == 0.0;
@@ -245,11 +244,11 @@ __device__ __forceinline__ df2 dpow2(df2 x, float p2) {
 // d = g_i - g_ib for the nine pairs, sigma = sum g, rho = rho0 + sigma,
 //   base = sigma - 3/2 |j|^2 / rho   (incompressible: / rho0),
 //   ep   = w base + 9/2 w (c.j)^2 / rho,
-//   le = 1:  g_0 = base / 3,  g_i = ep + h,  g_ib = ep - h,
-//            h = 3 lo w c.j + (1 - lo)/2 d;
-//   else:    g_0 += le (base / 3 - g_0),
-//            E = le ep - le/2 s,  O = 3 lo w c.j - lo/2 d,
-//            g_i += E + O,  g_ib += E - O.
+//   g_0 += le (base / 3 - g_0),  g_i = q + h,  g_ib = q - h,
+//   q = le ep + (1 - le)/2 s,  h = 3 lo w c.j + (1 - lo)/2 d
+// (g_i + E + O with g_i = (s + d)/2 and the relaxations E = le (ep - s/2),
+// O = 3 lo w c.j - lo/2 d).  le = 1: g_0 = base / 3, q = ep, and s is only
+// summed.
 // LE1: le == 1 (K.le1), the form taken.  Returns false when the cell's
 // density or momentum is not finite.
 //
@@ -295,43 +294,24 @@ __device__ __forceinline__ bool collide_trt_df(df g[Q], const DfK& K, int inc) {
     const df2 cj[4] = {jyz, dadd(jxx, jyz), dsub(jxx, jyz), dadd(splat(jy), pack(jz, dneg(jz)))};
     // ep = w base + 9/2 w (c.j)^2 / rho; 9/2 w = 1/4 (faces), 1/8 (edges)
     const df ep1 = dadd(dpow2(dmul(dsqr(jx), inv), 0.25f), wb18);
-    if constexpr (LE1) {
-        g[0] = dmul(base, dk(K, DK_W3));
-        const df ch = dk(K, DK_CH);
-        const df2 ch2 = splat(ch), lwf = splat(lw18), lwe = splat(lw36), wbf = splat(wb18), wbe = splat(wb36);
-        const df h1 = dadd(dmul(lw18, jx), dmul(ch, d1));
-        g[1] = dadd(ep1, h1);
-        g[2] = dsub(ep1, h1);
+    if constexpr (LE1) g[0] = dmul(base, dk(K, DK_W3));
+    else g[0] = dadd(dmul(dk(K, DK_LE3), base), dmul(dk(K, DK_1MLE), g[0]));
+    const df ch = dk(K, DK_CH), le = dk(K, DK_LE), cs = dk(K, DK_CS);
+    const df2 ch2 = splat(ch), lwf = splat(lw18), lwe = splat(lw36), wbf = splat(wb18), wbe = splat(wb36);
+    const df h1 = dadd(dmul(lw18, jx), dmul(ch, d1));
+    const df q1 = LE1 ? ep1 : dadd(dmul(le, ep1), dmul(cs, s1));
+    g[1] = dadd(q1, h1);
+    g[2] = dsub(q1, h1);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int a = df_i(q, 0), b = df_i(q, 1);
-            const df2 ep = dadd(dpow2(dmul(dsqr(cj[q]), inv2), q == 0 ? 0.25f : 0.125f), q == 0 ? wbf : wbe);
-            const df2 h = dadd(dmul(q == 0 ? lwf : lwe, cj[q]), dmul(ch2, d[q]));
-            unpack(dadd(ep, h), g[a], g[b]);
-            unpack(dsub(ep, h), g[a + 1], g[b + 1]);
-        }
-        return ok;
-    } else {
-        g[0] = dadd(dmul(dk(K, DK_LE3), base), dmul(dk(K, DK_1MLE), g[0]));
-        const df le = dk(K, DK_LE), mhle = dk(K, DK_MHLE), mhlo = dk(K, DK_MHLO);
-        const df2 le2 = splat(le), mhle2 = splat(mhle), mhlo2 = splat(mhlo);
-        const df2 lwf = splat(lw18), lwe = splat(lw36), wbf = splat(wb18), wbe = splat(wb36);
-        {
-            const df E = dadd(dmul(le, ep1), dmul(mhle, s1)), O = dadd(dmul(lw18, jx), dmul(mhlo, d1));
-            g[1] = dadd(g[1], dadd(E, O));
-            g[2] = dadd(g[2], dsub(E, O));
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int a = df_i(q, 0), b = df_i(q, 1);
-            const df2 ep = dadd(dpow2(dmul(dsqr(cj[q]), inv2), q == 0 ? 0.25f : 0.125f), q == 0 ? wbf : wbe);
-            const df2 E = dadd(dmul(le2, ep), dmul(mhle2, s[q]));
-            const df2 O = dadd(dmul(q == 0 ? lwf : lwe, cj[q]), dmul(mhlo2, d[q]));
-            unpack(dadd(pack(g[a], g[b]), dadd(E, O)), g[a], g[b]);
-            unpack(dadd(pack(g[a + 1], g[b + 1]), dsub(E, O)), g[a + 1], g[b + 1]);
-        }
-        return ok;
+    for (int q = 0; q < 4; ++q) {
+        const int a = df_i(q, 0), b = df_i(q, 1);
+        df2 e = dadd(dpow2(dmul(dsqr(cj[q]), inv2), q == 0 ? 0.25f : 0.125f), q == 0 ? wbf : wbe);
+        if constexpr (!LE1) e = dadd(dmul(splat(le), e), dmul(splat(cs), s[q]));
+        const df2 h = dadd(dmul(q == 0 ? lwf : lwe, cj[q]), dmul(ch2, d[q]));
+        unpack(dadd(e, h), g[a], g[b]);
+        unpack(dsub(e, h), g[a + 1], g[b + 1]);
     }
+    return ok;
 }
 
 }  // namespace lbsq
