@@ -67,7 +67,7 @@ __device__ __forceinline__ double sum_out(double a) { return a; }
 __device__ __forceinline__ double sum_out(df a) { return (double)a.h + (double)a.l; }
 
 template <int K, int T, class V>
-__device__ __forceinline__ void block_sum_fixed(const V (&v)[K], double* smd, double* out) {
+__device__ __forceinline__ void block_sum_fixed(const V (&v)[K], double* smd, double* out, int active = T) {
     static_assert(sizeof(V) == sizeof(double), "one word per value");
     constexpr int LEN = 16, SEG = T / LEN;
     V* sm = reinterpret_cast<V*>(smd);
@@ -79,7 +79,7 @@ __device__ __forceinline__ void block_sum_fixed(const V (&v)[K], double* smd, do
         const int c = t / SEG, sg = t % SEG;
         V a = sm[c * T + sg];
 #pragma unroll 4
-        for (int q = 1; q < LEN; ++q) a = sum_add(a, sm[c * T + q * SEG + sg]);
+        for (int q = 1; q < LEN && q * SEG < active; ++q) a = sum_add(a, sm[c * T + q * SEG + sg]);
         sm2[c * SEG + sg] = a;
     }
     __syncthreads();
@@ -884,23 +884,22 @@ __device__ __forceinline__ void link_terms32(const Lattice& L, const SphereF& sf
 
 // A block's share of a sphere's links and the block's sums in tot (shared):
 // force, torque and stresslet, or what link_terms64 sums (FP64 storage).
-// none: the block takes no links (zero sums).
 template <int P, int T>
 __device__ __forceinline__ void sphere_links(const Lattice& L, const BodyParams& p, const BodyState& s,
                                              const SphereF& sf, long long cnt, const uint32_t* links, int g, int G,
-                                             bool none, double* sm, double* tot) {
+                                             double* sm, double* tot) {
     if (L.storage == ST_F64) {
         double acc[12];
 #pragma unroll
         for (int c = 0; c < 12; ++c) acc[c] = 0.0;
-        if (!none) link_terms64<P, true>(L, p, s, sf, cnt, links, g, G, acc);
-        block_sum_fixed<12, T>(acc, sm, tot);
+        link_terms64<P, true>(L, p, s, sf, cnt, links, g, G, acc);
+        block_sum_fixed<12, T>(acc, sm, tot, (int)min((long long)T, (cnt + G - 1) / G));
     } else {
         df acc[12];
 #pragma unroll
         for (int c = 0; c < 12; ++c) acc[c] = {0.0f, 0.0f};
-        if (!none) link_terms32<P>(L, sf, cnt, links, g, G, acc);
-        block_sum_fixed<12, T>(acc, sm, tot);
+        link_terms32<P>(L, sf, cnt, links, g, G, acc);
+        block_sum_fixed<12, T>(acc, sm, tot, (int)min((long long)T, (cnt + G - 1) / G));
     }
 }
 
@@ -974,7 +973,7 @@ __global__ void __launch_bounds__(kLB) k_links(const Bodies B) {
         double* parts = B.part_links + (size_t)k * B.GL * 12;
         if (p.kind == BODY_SPHERE) {
             load_sphere(L, p, s, s_sf);
-            sphere_links<P, kLB>(L, p, s, s_sf, A.link_count, links, g, G, false, sm, s_tot);
+            sphere_links<P, kLB>(L, p, s, s_sf, A.link_count, links, g, G, sm, s_tot);
             if (threadIdx.x < 12) parts[g * 12 + threadIdx.x] = s_tot[threadIdx.x];
         } else {  // a wall: its force only
             double acc[12];
@@ -1789,23 +1788,26 @@ __global__ void __launch_bounds__(kFT, 2) k_body_fused(const Bodies B, int cls, 
         dep_launch();
 
         // ---- bounce-back and momentum exchange on the links (as k_links), by
-        // ranks 1 .. KC-1.  Meanwhile warps 0 and 1 of rank 0 run the update once
-        // on scratch: its code is cold every step (the sweep streams the lattice
-        // through L2 between steps), and the real update after the reduction
-        // then runs warm.  The scratch call writes only shared memory.
-        if (rank == 0) {
-            if (threadIdx.x < 32)
-                update_move<P>(L, B, k, p, s0, s_A, s_zero, &s_dryA, &s_dryS, &s_dryS2, &s_dryMode);
-            else if (threadIdx.x < 64)
-                update_turn(L, p, s0, s_A, s_zero, &s_dryA, &s_dryS, &s_dryS2);
-        }
-        sphere_links<P, kFT>(L, p, s0, s_sf, s_A.link_count, B.links + p.link_off, rank - 1, KC - 1, rank == 0, sm,
-                             s_tot);
+        // ranks 1 .. KC-1.  Meanwhile rank 0, which takes none, runs the update
+        // once on scratch (warps 0 and 1: its code is cold every step, the sweep
+        // streams the lattice through L2 between steps, and the real update after
+        // the reduction then runs warm; the scratch call writes only shared
+        // memory) and looks for bodies near this one (the other warps).
         int near = 0;
-        if (rank == 0)
-            for (int j = L.body_begin + threadIdx.x; j < L.body_begin + L.body_count; j += kFT)
-                if (j != k && boxes_near(L, p, s0, B.par[j], B.state[P][j])) near = 1;
-        near = __syncthreads_or(near);
+        if (rank == 0) {
+            if (threadIdx.x < 32) {
+                update_move<P>(L, B, k, p, s0, s_A, s_zero, &s_dryA, &s_dryS, &s_dryS2, &s_dryMode);
+            } else if (threadIdx.x < 64) {
+                update_turn(L, p, s0, s_A, s_zero, &s_dryA, &s_dryS, &s_dryS2);
+            } else {
+                for (int j = L.body_begin + (int)threadIdx.x - 64; j < L.body_begin + L.body_count; j += kFT - 64)
+                    if (j != k && boxes_near(L, p, s0, B.par[j], B.state[P][j])) near = 1;
+            }
+            if (threadIdx.x < 12) s_tot[threadIdx.x] = 0.0;
+            near = __syncthreads_or(near);
+        } else {
+            sphere_links<P, kFT>(L, p, s0, s_sf, s_A.link_count, B.links + p.link_off, rank - 1, KC - 1, sm, s_tot);
+        }
         cl.sync();
         if (rank == 0) {
             // the blocks' partial sums, all fetched at once, then summed in rank order
