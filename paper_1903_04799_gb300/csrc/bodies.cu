@@ -1229,6 +1229,19 @@ __global__ void __launch_bounds__(kBB) k_classify(const Bodies B) {
     }
 }
 
+// Whether node (x, y) can hold a boundary link of wall q: always but for a
+// round tube, whose links leave nodes less than sqrt(2) from its wall nodes in
+// the cross-section, so at r - sqrt(2) or more from the axis (FP32, with slack
+// for its errors: 0.08 and 4e-7 of the lattice's width).  The tube's scan box
+// is the whole lattice; three quarters of its fluid nodes fail here, before
+// their 18 neighbours are read.
+__device__ __forceinline__ bool wall_links_at(const Lattice& L, const BodyParams& q, int x, int y) {
+    if (q.wall_axis >= 0) return true;
+    const float lim = (float)q.tube[2] - 1.5f - 4e-7f * (float)(L.nx + L.ny);
+    const float dx = (float)x - (float)q.tube[0], dy = (float)y - (float)q.tube[1];
+    return !(lim > 0.0f && dx * dx + dy * dy < lim * lim);
+}
+
 // ---------------------------------------------------------------- k_convert
 
 // Sum of one double per lane over the warp, in a fixed tree order (lane 0
@@ -1365,7 +1378,7 @@ __global__ void __launch_bounds__(kBB) k_convert(const Bodies B) {
             bool take = b < b1;
             if (take) {
                 box_cell(L, lo, w, b, x, y, z);
-                if (sphere) take = in_shell(dist2_f(L, cf, x, y, z), Rf);
+                take = sphere ? in_shell(dist2_f(L, cf, x, y, z), Rf) : wall_links_at(L, p, x, y);
             }
             if (take) uncover = convert_cell<false>(L, s, id, x, y, z, q, conv, acc, lcount);
             // solid -> fluid cells of this round, in thread order, refilled by warps
@@ -1542,7 +1555,7 @@ __global__ void __launch_bounds__(kBB) k_rebuild(const Bodies B) {
                 box_cell(L, lo, w, b, x, y, z);
                 // same predicate as the count in k_convert (only shell nodes can
                 // hold links; only they changed owner)
-                if (sphere) take = in_shell(dist2_f(L, cf, x, y, z), Rf);
+                take = sphere ? in_shell(dist2_f(L, cf, x, y, z), Rf) : wall_links_at(L, p, x, y);
             }
             if (take) {
                 n = cell_index(L, x, y, z);

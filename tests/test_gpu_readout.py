@@ -67,3 +67,29 @@ def test_fields_and_totals(storage, shape, rho0, inc, spread):
         _check(g, rho0, inc)  # even parity
         g.step(1)
         _check(g, rho0, inc)  # odd parity
+
+
+@pytest.mark.parametrize("offset", [0, 8, 72])
+def test_large_read_out_into_fresh_and_existing_pages(offset):
+    """A read-out of 23 MB (five blocks and a part, no whole number of pages) into
+    a buffer whose pages do not exist yet, at several alignments, against one
+    into a buffer that has been written: the same bytes, and none outside."""
+    import mmap
+
+    from paper_1903_04799_gb300 import lbsq
+
+    shape = (61, 47, 53)
+    n = math.prod(shape)
+    f = W[:, None] * (1.0 + 0.05 * np.random.default_rng(3).uniform(-1, 1, (19, n)))
+    with Lattice(shape, storage="f64") as g:
+        g.set_populations(f)
+        lib = lbsq.load()
+        warm = np.ones(19 * n)
+        lbsq._check(g.ctx, lib.lb_get_populations(g.ctx, lbsq._dp(warm)), "lb_get_populations")
+        m = mmap.mmap(-1, 19 * n * 8 + (1 << 20))
+        fresh = np.frombuffer(m, dtype=np.float64, count=19 * n, offset=offset)
+        lbsq._check(g.ctx, lib.lb_get_populations(g.ctx, lbsq._dp(fresh)), "lb_get_populations")
+        assert np.array_equal(fresh, warm)
+        rest = np.frombuffer(m, dtype=np.uint8)
+        assert not rest[:offset].any() and not rest[offset + 19 * n * 8:].any()
+        assert np.abs(warm.reshape(19, n) - f).max() < 1e-16  # two roundings of at most 2^-54

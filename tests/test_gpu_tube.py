@@ -77,3 +77,26 @@ def test_tube_centred_start_stays_on_the_axis():
     assert np.abs(uy + uy[:, ::-1, :]).max() < 1e-12 * scale
     assert np.abs(ux - ux[:, ::-1, :]).max() < 1e-12 * scale
     g.close()
+
+
+@pytest.mark.parametrize("shape,axis,radius", [((23, 21, 5), (11.0, 10.0), 9.3), ((30, 31, 3), (14.6, 15.2), 13.0),
+                                               ((12, 12, 4), (5.5, 5.5), 1.4), ((40, 17, 3), (30.2, 8.1), 7.7)])
+def test_tube_links_brute_force(shape, axis, radius):
+    """The tube's link list, built from the nodes near its wall only, against
+    every fluid node with a wall neighbour: wide and narrow tubes (radius below
+    the margin: every node is looked at) and an axis off the box's centre."""
+    from paper_1903_04799_gb300 import Lattice
+
+    nx, ny, nz = shape
+    with Lattice(shape, storage="f32") as g:
+        tube = g.add_round_tube(*axis, radius)
+        links = set(g.links(tube).tolist())
+        wall = (g.owner() == tube).reshape(nz, ny, nx)
+    c = np.array([[0, 1, -1, 0, 0, 0, 0, 1, -1, 1, -1, 1, -1, 1, -1, 0, 0, 0, 0],
+                  [0, 0, 0, 1, -1, 0, 0, 1, -1, -1, 1, 0, 0, 0, 0, 1, -1, 1, -1],
+                  [0, 0, 0, 0, 0, 1, -1, 0, 0, 0, 0, 1, -1, -1, 1, 1, -1, -1, 1]])
+    want = set()
+    for i in range(1, 19):
+        near = np.roll(wall, (-c[2, i], -c[1, i], -c[0, i]), (0, 1, 2))
+        want |= {32 * int(n) + i for n in np.flatnonzero((~wall & near).reshape(-1))}
+    assert links == want and len(links) > 0
