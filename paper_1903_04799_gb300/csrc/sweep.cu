@@ -192,15 +192,18 @@ static int sm_count() {
 //   FP64 (double-float form): 256^3 0.65 -> 0.75 at 1 or 2 planes ahead,
 //     0.66 at 4, 0.60 at 5; 192^3 0.56 -> 0.72; 128^3 0.64 -> 0.78;
 //   16-bit sweeps: see prefetch_ahead16.
-// FP32 prefetches in whole-lattice sweeps only: a prefetch installs its lines
-// in L2 at normal priority, and beside the body kernels of a split step (far
-// sweeps) that evicted their code again (128^3 step 0.050 -> 0.056 ms).  The
-// FP64 sweep is long against its body step, and prefetches in split sweeps
-// too (256^3 pusher, whole step: 13 970 -> 15 830 MLUPS).
+// In the far sweeps of split steps FP32 prefetches from 200 MB of populations
+// on.  Below, the step is as long as its body kernels' chain, whose code the
+// prefetched lines, which enter L2 at normal priority, evict (128^3, 159 MB, one
+// squirmer: 45 us per step without, 56 with); above, the far sweep sets the
+// pace (us per step without / with: 144^3 82 / 76, 160^3 106 / 94, 192^3 169 /
+// 155, 250^3 371 / 355, 256^3 377 / 375; partially saturated cells 160^3 120 /
+// 109, 256^3 420 / 414).  The FP64 sweep is long against its body step, and
+// prefetches in every split sweep.
 // A near sweep prefetches nothing: its window is a few planes deep (250^3 pair
 // in BF16, whole step: 341 -> 334 us without).
 static int prefetch_ahead(const SweepArgs& a, int storage, const Rows& r) {
-    if (a.zmode == 2 || (storage == ST_F32 && a.zmode != 0)) return 0;
+    if (a.zmode == 2 || (storage == ST_F32 && a.zmode != 0 && 19 * a.Np * 4 < 200000000)) return 0;
     const long long per_plane = (long long)r.xblocks * ((r.gy + r.by - 1) / r.by);
     const long long resident = (long long)r.resident * sm_count();
     const int ahead = (int)((resident + per_plane - 1) / per_plane) + (storage == ST_F32 ? 2 : 0);
