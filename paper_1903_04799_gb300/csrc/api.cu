@@ -23,7 +23,7 @@ void launch_sweep(const Lattice& L, double lambda_e, double lambda_o, int parity
                   const int* win, int gz, int gy, cudaStream_t st, bool dep = false);
 void launch_body_kernel(int which, const Bodies& B, int parity, int grid_links, int grid_box, long long* step,
                         cudaStream_t st, bool dep = false);
-void launch_body_fused(const Bodies& B, int parity, int cls, int clusters, cudaStream_t st, int tail,
+void launch_body_fused(const Bodies& B, int parity, int cls, int clusters, bool f64, cudaStream_t st, int tail,
                        bool dep = false, cudaEvent_t started = nullptr);
 cudaError_t prepare_body_kernels();
 void launch_fill_rest(const Lattice& L, cudaStream_t st);
@@ -1183,7 +1183,7 @@ static int psm_step(lb_ctx* c, const Bodies& B, int parity, cudaStream_t st, boo
 static int body_step(lb_ctx* c, const Bodies& B, int parity, cudaStream_t st, bool dep = false,
                      cudaEvent_t started = nullptr) {
     if (c->solo) {  // the fused kernel is the whole body step
-        launch_body_fused(B, parity, c->fused_cls, 1, st, 1, dep, started);
+        launch_body_fused(B, parity, c->fused_cls, 1, c->p.storage == LB_F64, st, 1, dep, started);
         return 1;
     }
     int n = 0;
@@ -1193,7 +1193,7 @@ static int body_step(lb_ctx* c, const Bodies& B, int parity, cudaStream_t st, bo
         cudaStreamWaitEvent(c->wall, c->ev_wall, 0);
     }
     if (c->n_fused > 0) {
-        launch_body_fused(B, parity, c->fused_cls, c->n_fused, st, 0, dep, started);
+        launch_body_fused(B, parity, c->fused_cls, c->n_fused, c->p.storage == LB_F64, st, 0, dep, started);
         dep = true;
         n++;
     }
@@ -1244,7 +1244,7 @@ static void enqueue_traced_step(lb_ctx* c) {
         } else if (k == 1) {
             const Bodies B = bodies_for_step(c, c->step);
             if (c->n_fused > 0) {
-                launch_body_fused(B, parity, c->fused_cls, c->n_fused, c->stream, 0);
+                launch_body_fused(B, parity, c->fused_cls, c->n_fused, c->p.storage == LB_F64, c->stream, 0);
                 c->launches += 1;
             }
             if (c->n_link_items > 0) {

@@ -884,11 +884,11 @@ __device__ __forceinline__ void link_terms32(const Lattice& L, const SphereF& sf
 
 // A block's share of a sphere's links and the block's sums in tot (shared):
 // force, torque and stresslet, or what link_terms64 sums (FP64 storage).
-template <int P, int T>
+template <int P, int T, bool REDUCED = false>
 __device__ __forceinline__ void sphere_links(const Lattice& L, const BodyParams& p, const BodyState& s,
                                              const SphereF& sf, long long cnt, const uint32_t* links, int g, int G,
                                              double* sm, double* tot) {
-    if (L.storage == ST_F64) {
+    if (!REDUCED && L.storage == ST_F64) {
         double acc[12];
 #pragma unroll
         for (int c = 0; c < 12; ++c) acc[c] = 0.0;
@@ -1740,8 +1740,13 @@ __device__ __forceinline__ void copy_words(void* dst, const void* src, int n) {
 
 constexpr int kStcBuf = 2048;  // stencil entries a block keeps in shared memory
 
-template <int P>
-__global__ void __launch_bounds__(kFT, 2) k_body_fused(const Bodies B, int cls, int tail) {
+// MANY: reduced storages in the clusters of 4 blocks that many spheres get.
+// Their blocks come in waves and wait on each other's serial phases, so three
+// per SM (without the FP64 links; 300 bytes of spill) beat two: 200 spheres of R
+// = 6, 471 -> 465 us per step.  With a few spheres there is one wave, and the
+// spills cost (128^3, one sphere: 45.7 -> 48.6 us).
+template <int P, bool MANY>
+__global__ void __launch_bounds__(kFT, MANY ? 3 : 2) k_body_fused(const Bodies B, int cls, int tail) {
     cg::cluster_group cl = cg::this_cluster();
     const int KC = (int)cl.num_blocks();
     const int rank = (int)cl.block_rank();
@@ -1819,7 +1824,7 @@ __global__ void __launch_bounds__(kFT, 2) k_body_fused(const Bodies B, int cls, 
             if (threadIdx.x < 12) s_tot[threadIdx.x] = 0.0;
             near = __syncthreads_or(near);
         } else {
-            sphere_links<P, kFT>(L, p, s0, s_sf, s_A.link_count, B.links + p.link_off, rank - 1, KC - 1, sm, s_tot);
+            sphere_links<P, kFT, MANY>(L, p, s0, s_sf, s_A.link_count, B.links + p.link_off, rank - 1, KC - 1, sm, s_tot);
         }
         cl.sync();
         if (rank == 0) {
@@ -2450,8 +2455,9 @@ void launch_body_kernel(int which, const Bodies& B, int parity, int grid_links, 
 // Once per process and device, before the first launch of k_body_fused:
 // allow clusters of 16 blocks (above the portable maximum of 8).
 cudaError_t prepare_body_kernels() {
-    cudaError_t e = cudaFuncSetAttribute(k_body_fused<0>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_body_fused<1>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaError_t e = cudaFuncSetAttribute(k_body_fused<0, false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_body_fused<1, false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;
 }
 
@@ -2464,8 +2470,8 @@ int fused_cluster(int c) { return c == 0 ? 16 : (c == 1 ? 8 : 4); }
 // once every block of the launch has begun (a launch-completion event): a
 // stream that waits on it starts after the clusters are placed, not after
 // the kernel ends.  dep: a dependent launch (see dep_wait).
-void launch_body_fused(const Bodies& B, int parity, int cls, int clusters, cudaStream_t st, int tail, bool dep,
-                       cudaEvent_t started) {
+void launch_body_fused(const Bodies& B, int parity, int cls, int clusters, bool f64, cudaStream_t st, int tail,
+                       bool dep, cudaEvent_t started) {
     if (clusters <= 0) return;
     const int kc = fused_cluster(cls);
     cudaLaunchConfig_t cfg = {};
@@ -2490,8 +2496,10 @@ void launch_body_fused(const Bodies& B, int parity, int cls, int clusters, cudaS
         attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
         cfg.numAttrs++;
     }
-    if (parity == 0) cudaLaunchKernelEx(&cfg, k_body_fused<0>, B, cls, tail);
-    else cudaLaunchKernelEx(&cfg, k_body_fused<1>, B, cls, tail);
+    if (cls == 2 && !f64)
+        cudaLaunchKernelEx(&cfg, parity == 0 ? k_body_fused<0, true> : k_body_fused<1, true>, B, cls, tail);
+    else
+        cudaLaunchKernelEx(&cfg, parity == 0 ? k_body_fused<0, false> : k_body_fused<1, false>, B, cls, tail);
 }
 
 }  // namespace lbsq
