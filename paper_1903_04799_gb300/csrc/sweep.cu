@@ -192,18 +192,24 @@ static int sm_count() {
 //   FP64 (double-float form): 256^3 0.65 -> 0.75 at 1 or 2 planes ahead,
 //     0.66 at 4, 0.60 at 5; 192^3 0.56 -> 0.72; 128^3 0.64 -> 0.78;
 //   16-bit sweeps: see prefetch_ahead16.
-// In the far sweeps of split steps FP32 prefetches from 200 MB of populations
-// on.  Below, the step is as long as its body kernels' chain, whose code the
-// prefetched lines, which enter L2 at normal priority, evict (128^3, 159 MB, one
-// squirmer: 45 us per step without, 56 with); above, the far sweep sets the
-// pace (us per step without / with: 144^3 82 / 76, 160^3 106 / 94, 192^3 169 /
-// 155, 250^3 371 / 355, 256^3 377 / 375; partially saturated cells 160^3 120 /
-// 109, 256^3 420 / 414).  The FP64 sweep is long against its body step, and
-// prefetches in every split sweep.
+// Far sweeps of split steps prefetch from 200 MB of populations on
+// (far_prefetch).  Below, the step is as long as its body kernels' chain, whose
+// code the prefetched lines, which enter L2 at normal priority, evict; above,
+// the far sweep sets the pace.  One squirmer, us per step without / with:
+//   FP32 128^3 (159 MB) 45 / 56, 144^3 (227 MB) 82 / 76, 160^3 106 / 94, 192^3
+//   169 / 155, 250^3 371 / 355, 256^3 377 / 375; partially saturated cells
+//   160^3 120 / 109, 256^3 420 / 414;
+//   FP64 96^3 (134 MB) 48.1 / 51.2, 112^3 (213 MB) 82.7 / 83.9, 128^3 109 / 108,
+//   144^3 188 / 170, 160^3 236 / 210, 250^3 916 / 825;
+//   FP16 96^3 24.2 / 24.5, 160^3 (156 MB) 69.3 / 70.1, 192^3 (269 MB) 110 / 105,
+//   250^3 225 / 221; BF16 160^3 76.6 / 77.0, 192^3 121 / 114.
+static bool far_prefetch(const SweepArgs& a, int storage) {
+    return a.zmode != 1 || 19 * a.Np * storage_bytes(storage) >= 200000000;
+}
 // A near sweep prefetches nothing: its window is a few planes deep (250^3 pair
 // in BF16, whole step: 341 -> 334 us without).
 static int prefetch_ahead(const SweepArgs& a, int storage, const Rows& r) {
-    if (a.zmode == 2 || (storage == ST_F32 && a.zmode != 0 && 19 * a.Np * 4 < 200000000)) return 0;
+    if (a.zmode == 2 || !far_prefetch(a, storage)) return 0;
     const long long per_plane = (long long)r.xblocks * ((r.gy + r.by - 1) / r.by);
     const long long resident = (long long)r.resident * sm_count();
     const int ahead = (int)((resident + per_plane - 1) / per_plane) + (storage == ST_F32 ? 2 : 0);
@@ -221,7 +227,7 @@ static int prefetch_ahead(const SweepArgs& a, int storage, const Rows& r) {
 // parities, 0.745 -> 0.684, was taken before the sweeps' traffic was marked
 // evict-first.)
 static int prefetch_ahead16(const SweepArgs& a, const Rows& r, int extra) {
-    if (a.zmode == 2) return 0;
+    if (a.zmode == 2 || !far_prefetch(a, ST_F16)) return 0;
     const long long per_plane = (long long)r.xblocks * ((r.gy + r.by - 1) / r.by);
     const long long resident = 2LL * sm_count();
     const int ahead = (int)((resident + per_plane - 1) / per_plane) + extra;
@@ -258,7 +264,7 @@ template <int S>
 static void launch_flat(const SweepArgs& a, cudaStream_t st, bool dep) {
     const uint32_t N = (uint32_t)a.nx * a.ny * a.nz, cells = (S == ST_F32 ? 2 : 4) * 256;
     const uint32_t ahead = 2u * sm_count() * cells + 2u * a.nx * a.ny;
-    launch(k_sweep_flat<S>, (N + cells - 1) / cells, 256, 0, st, dep, a, ahead < N ? ahead : 0u);
+    launch(k_sweep_flat<S>, (N + cells - 1) / cells, 256, 0, st, dep, a, ahead < N && far_prefetch(a, S) ? ahead : 0u);
 }
 
 template <int S>
