@@ -347,7 +347,7 @@ __device__ __noinline__ double inv_sqrt(double x) { return 1.0 / sqrt(x); }
 // Whether body j may be within the contact range of sphere k, in FP32: false
 // only if the gap is certainly beyond 2^(1/6) sigma, where the force is exactly
 // zero (2e-5 of slack against FP32 errors of a few 1e-7).  Positions enter
-// through one FP64 difference per axis.
+// through their FP64 difference per axis.
 template <int P>
 __device__ __forceinline__ bool wca_near(const Lattice& L, const Bodies& B, int j, const BodyParams& p,
                                          const BodyState& s) {
@@ -355,11 +355,11 @@ __device__ __forceinline__ bool wca_near(const Lattice& L, const Bodies& B, int 
     const float cut = 1.1225f * (float)L.wca_sigma, R = (float)p.R;
     if (q.kind == BODY_SPHERE) {
         const double* t = B.state[P][j].pos;
-        const float n3[3] = {(float)L.nx, (float)L.ny, (float)L.nz};
+        const int n3[3] = {L.nx, L.ny, L.nz};
         float d2 = 0.0f;
         for (int b = 0; b < 3; ++b) {
-            float d = fabsf((float)(s.pos[b] - t[b]));
-            d = fminf(d, fabsf(n3[b] - d));  // the nearer image
+            // wrapped in FP64: 2^-24 of a long axis would not be a small error
+            const float d = (float)min_image(s.pos[b] - t[b], n3[b]);
             d2 += d * d;
         }
         const float lim = R + (float)q.R + cut;
