@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <string>
 #include <thread>
@@ -341,7 +342,8 @@ cudaError_t copy_out(lb_ctx* c, void* dst, const void* src, size_t bytes) {
     char* const last = (char*)(((uintptr_t)d + bytes) / page * page) - page;
     if (mincore(last, page, &there) != 0 || (there & 1)) return plain(0, bytes);
     const size_t nb = (bytes + kBlock - 1) / kBlock;
-    std::vector<std::atomic<int>> made(nb);
+    const std::unique_ptr<std::atomic<int>[]> made(new (std::nothrow) std::atomic<int>[nb]());
+    if (!made) return plain(0, bytes);
     std::atomic<size_t> next{0};
     auto work = [&] {
         for (size_t b; (b = next.fetch_add(1)) < nb;) {
@@ -575,7 +577,8 @@ lb_status relayout(lb_ctx* c) {
     // have to follow the scattered results)
     const bool thin = !across && nb > 0 && wmax * 5 < 3 * c->L.nz && worth_splitting(c);
     c->split = !c->psm && thin;
-    c->psm_split = c->psm && thin && std::all_of(c->par.begin(), c->par.end(), [](const BodyParams& b) { return b.psm != 0; });
+    c->psm_split = c->psm && thin &&
+                   std::all_of(c->par.begin(), c->par.end(), [](const BodyParams& b) { return b.psm != 0; });
     if (ranges > 1) {
         wmax = c->L.nz;
         ymax = c->L.ny;

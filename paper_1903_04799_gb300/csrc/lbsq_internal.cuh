@@ -133,8 +133,10 @@ inline int storage_bytes(int s) { return s == ST_F64 ? 8 : (s == ST_F32 ? 4 : 2)
 // end and its writes.  Every kernel launched this way calls dep_wait in every
 // thread before it reads or writes what the predecessor touches, and dep_launch
 // only after dep_wait; so when a block starts, every kernel before its
-// predecessor has ended, and what those wrote may be read at once.  Both
-// calls do nothing in an ordinary launch.
+// predecessor has ended, and what those wrote may be read at once.  (The
+// kernels of partially saturated cells call dep_launch first, so neither they
+// nor their successors read anything before dep_wait.)  Both calls do nothing
+// in an ordinary launch.
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -34,10 +34,10 @@ __global__ void __launch_bounds__(256) k_sweep(const SweepArgs a) {
 
 // FP64 storage, double-float collision (sweep_df.cuh), one cell per thread.
 // lambda_e = 1: three blocks per SM (80 registers, 56 bytes of spill): 24 warps
-// per SM hide the loads better than 16.  The general relaxation keeps the pair
-// sums as well; at 80 registers it spilled 240 bytes and 160 x 144 x 130 took
-// 219 us per step against 177 at two blocks per SM.  The near form, with its
-// loop over rows, runs at two blocks too.
+// per SM hide the loads better than 16.  The general relaxation has more live
+// values; at 80 registers it spills 128 bytes, and 160 x 144 x 130 takes 161 us
+// per step against 159 at two blocks per SM.  The near form, with its loop over
+// rows, runs at two blocks too.
 template <int P, bool LE1, bool NEAR>
 __global__ void __launch_bounds__(256, NEAR || !LE1 ? 2 : 3) k_sweep_df(const SweepArgs a) {
     dep_wait();
@@ -302,10 +302,6 @@ static void launch_s(SweepArgs a, int parity, int variant, int gz, int gy, cudaS
         // 251^3 FP16 259 -> 217, BF16 375 -> 278.  Where whole rows fit, the two
         // are equal in bare sweeps (256^3: 204 us) and the rows faster in split
         // ones (256^3 pusher FP16 222 against 226 us: no divisions for the window)
-        // even steps of rows that whole-row blocks do not fit: four cells
-        // regardless of rows.  Where whole rows fit, the two are equal in bare
-        // sweeps (256^3: 204 us) and the rows faster in split ones (256^3 pusher
-        // FP16 222 against 226 us: no divisions for the window)
         if (variant == 0 && parity == 0 && a.zmode != 2 && !rows4) {
             launch_flat<S>(a, st, dep);
             return;
@@ -351,7 +347,8 @@ static void launch_s(SweepArgs a, int parity, int variant, int gz, int gy, cudaS
         // one cell: pairs across odd rows, every access scalar and every second
         // element left to another instruction, took 408 us.  In split steps of
         // small lattices the window's divisions cost what the pairs gain.
-        if (S == ST_F32 && variant == 0 && parity == 0 && (a.zmode == 0 || (a.zmode == 1 && 19 * a.Np * 4 > (128 << 20)))) {
+        if (S == ST_F32 && variant == 0 && parity == 0 &&
+            (a.zmode == 0 || (a.zmode == 1 && 19 * a.Np * 4 > (128 << 20)))) {
             launch_flat<S>(a, st, dep);
             return;
         }
