@@ -692,12 +692,17 @@ __device__ __forceinline__ void load_sphere(const Lattice& L, const BodyParams& 
 // FP64 links of a sphere (FP64 storage) or a wall (any storage): acc takes
 // force (0..2) and, for a sphere, torque (3..5) and the negated stresslet, its
 // off-diagonal components doubled (6..11; sphere_totals).  A link's dF lies
-// along its direction, c_i sf with c in {-1, 0, 1}, so its nine products
-// d_a dF_b are selected from three; term by term they took twice the FP64
-// instructions.  Block g takes every G-th link: links all over the sphere,
-// whose large rest parts cancel within the block (runs of neighbouring links
-// tripled the rounding error of the stresslet at R = 7); the trace leaves each
-// link for the same reason.
+// along its direction, c_i sf with c in {-1, 0, 1}, so the stresslet's nine
+// products d_a dF_b are selected from three, and the torque takes the d x c of
+// the rotation's boundary velocity; term by term they took twice the FP64
+// instructions.  Block g takes every G-th run of kRun links.  Links all over
+// the sphere, because their large rest parts then cancel within the block
+// (one stretch of neighbouring links per block tripled the rounding error of
+// the stresslet at R = 7); the trace leaves each link for the same reason.  In
+// runs, because the rest torques of one node's links cancel (single links:
+// rms error of the torque 10 % larger at R = 16).
+constexpr int kRun = 8;
+
 template <int P, bool SPHERE>
 __device__ __forceinline__ void link_terms64(const Lattice& L, const BodyParams& p, const BodyState& s,
                                              const SphereF& sp, long long cnt, const uint32_t* links, int g, int G,
@@ -711,7 +716,8 @@ __device__ __forceinline__ void link_terms64(const Lattice& L, const BodyParams&
     // links on 128 blocks).
     constexpr int kU = SPHERE ? 1 : 4;
     const int stride = G * (int)blockDim.x;
-    for (int lb = g + G * (int)threadIdx.x; lb < (int)cnt; lb += kU * stride) {
+    const int t = (int)threadIdx.x, l0 = (t / kRun * G + g) * kRun + t % kRun;
+    for (int lb = l0; lb < (int)cnt; lb += kU * stride) {
     uint32_t codes[kU];
     Link lk[kU];
     double fouts[kU];
@@ -733,7 +739,7 @@ __device__ __forceinline__ void link_terms64(const Lattice& L, const BodyParams&
         // where the next sweep reads the reflected population f_ib of the fluid node
         const int64_t in_slot = P == 0 ? (int64_t)i * Np + k.ns : (int64_t)ib * Np + k.n;
         const double fout = fouts[q];
-        double d[3], cv;
+        double d[3], arm[3], cv;  // arm = d x c, cv = c.v_b
         if (SPHERE) {
             // link midpoint (or boundary node) relative to the centre (minimum
             // image: a link lies within R + 2 of it, less than half the box);
@@ -753,9 +759,10 @@ __device__ __forceinline__ void link_terms64(const Lattice& L, const BodyParams&
             const double cn = (csel(ci[0], d[0]) + csel(ci[1], d[1]) + csel(ci[2], d[2])) * ir;
             const double ce = csel(ci[0], s.e[0]) + csel(ci[1], s.e[1]) + csel(ci[2], s.e[2]);
             const double slip = r2 > 0.0 ? (p.B1 + p.B2 * ct) * (ct * cn - ce) : 0.0;
-            const double rot = s.omega[0] * (csel(ci[2], d[1]) - csel(ci[1], d[2])) +
-                               s.omega[1] * (csel(ci[0], d[2]) - csel(ci[2], d[0])) +
-                               s.omega[2] * (csel(ci[1], d[0]) - csel(ci[0], d[1]));
+            arm[0] = csel(ci[2], d[1]) - csel(ci[1], d[2]);
+            arm[1] = csel(ci[0], d[2]) - csel(ci[2], d[0]);
+            arm[2] = csel(ci[1], d[0]) - csel(ci[0], d[1]);
+            const double rot = s.omega[0] * arm[0] + s.omega[1] * arm[1] + s.omega[2] * arm[2];
             cv = csel(ci[0], s.vel[0]) + csel(ci[1], s.vel[1]) + csel(ci[2], s.vel[2]) + (rot + slip);
         } else {
             cv = csel(ci[0], p.wall_vel[0]) + csel(ci[1], p.wall_vel[1]) + csel(ci[2], p.wall_vel[2]);
@@ -771,11 +778,10 @@ __device__ __forceinline__ void link_terms64(const Lattice& L, const BodyParams&
             const double m[3] = {d[0] * sf, d[1] * sf, d[2] * sf};
             const double tr = (csel(ci[0], m[0]) + csel(ci[1], m[1]) + csel(ci[2], m[2])) * (1.0 / 3.0);
             for (int a = 0; a < 3; ++a) {
+                acc[3 + a] = fma(arm[a], sf, acc[3 + a]);
                 acc[6 + a] += csel(ci[a], m[a]) - tr;
-                const int b = a == 2 ? 0 : a + 1;  // (0,1), (1,2), (2,0)
-                const double ab = csel(ci[b], m[a]), ba = csel(ci[a], m[b]);
-                acc[3 + (a == 2 ? 1 : (a == 0 ? 2 : 0))] += ab - ba;  // torque component 2, 0, 1
-                acc[9 + (a == 2 ? 1 : (a == 0 ? 0 : 2))] += ab + ba;  // xy, yz, xz
+                const int b = a == 2 ? 0 : a + 1;  // (0,1), (1,2), (2,0): xy, yz, xz
+                acc[9 + (a == 2 ? 1 : (a == 0 ? 0 : 2))] += csel(ci[b], m[a]) + csel(ci[a], m[b]);
             }
         }
     }
@@ -893,7 +899,8 @@ __device__ __forceinline__ void sphere_links(const Lattice& L, const BodyParams&
 #pragma unroll
         for (int c = 0; c < 12; ++c) acc[c] = 0.0;
         link_terms64<P, true>(L, p, s, sf, cnt, links, g, G, acc);
-        block_sum_fixed<12, T>(acc, sm, tot, (int)min((long long)T, (cnt + G - 1) / G));
+        // threads that hold links: those of full runs
+        block_sum_fixed<12, T>(acc, sm, tot, (int)min((long long)T, (cnt + kRun * G - 1) / (kRun * G) * kRun));
     } else {
         df acc[12];
 #pragma unroll
