@@ -224,9 +224,17 @@ __device__ __forceinline__ bool axis_overlap(int a, int wa, int b, int wb, int n
 // node that neighbours a wall node of round tube q: nodes at distance r or
 // more from the axis are wall, their lattice neighbours lie at r - sqrt(2) or
 // more (in the cross-section), so a box whose corners (grown) all lie within
-// r - 2 - g of the axis holds none.  Conservative: a box across the periodic
-// edge of the cross-section lies in the wall anyway.
-__device__ __forceinline__ bool box_meets_tube(const BodyParams& q, const int lo[3], const int w[3], int g) {
+// r - 2 - g of the axis holds none.  That holds for neighbours that lie next to
+// a node; a node at the edge of the cross-section also neighbours those across
+// the periodic edge, which are wall or not however near the axis it lies, so a
+// box that reaches the edge (lo, w unwrapped, the centre inside the box) counts
+// as one that may.  For a tube that ends inside the box, whose edge nodes are
+// wall, the corners say the same.
+__device__ __forceinline__ bool box_meets_tube(const Lattice& L, const BodyParams& q, const int lo[3],
+                                               const int w[3], int g) {
+    const int n2[2] = {L.nx, L.ny};
+    for (int a = 0; a < 2; ++a)
+        if (lo[a] - g <= 0 || lo[a] + w[a] - 1 + g >= n2[a] - 1) return true;
     double far2 = 0.0;
     for (int i = 0; i < 2; ++i)
         for (int j = 0; j < 2; ++j) {
@@ -245,8 +253,8 @@ __device__ __forceinline__ bool boxes_intersect(const Lattice& L, const BodyPara
     body_box(L, pa, sa, la, wa);
     body_box(L, pb, sb, lb, wb);
     // a round tube's box is the whole lattice; its links sit along its wall
-    if (round_tube(pb) && !round_tube(pa)) return box_meets_tube(pb, la, wa, 0);
-    if (round_tube(pa) && !round_tube(pb)) return box_meets_tube(pa, lb, wb, 0);
+    if (round_tube(pb) && !round_tube(pa)) return box_meets_tube(L, pb, la, wa, 0);
+    if (round_tube(pa) && !round_tube(pb)) return box_meets_tube(L, pa, lb, wb, 0);
     return axis_overlap(la[0], wa[0], lb[0], wb[0], L.nx) && axis_overlap(la[1], wa[1], lb[1], wb[1], L.ny) &&
            axis_overlap(la[2], wa[2], lb[2], wb[2], L.nz);
 }
@@ -1239,11 +1247,12 @@ __global__ void __launch_bounds__(kBB) k_classify(const Bodies B) {
 // Whether node (x, y) can hold a boundary link of wall q: always but for a
 // round tube, whose links leave nodes less than sqrt(2) from its wall nodes in
 // the cross-section, so at r - sqrt(2) or more from the axis (FP32, with slack
-// for its errors: 0.08 and 4e-7 of the lattice's width).  The tube's scan box
-// is the whole lattice; three quarters of its fluid nodes fail here, before
-// their 18 neighbours are read.
+// for its errors: 0.08 and 4e-7 of the lattice's width), or nodes at the edge
+// of the cross-section, which also neighbour the nodes across it.  The tube's
+// scan box is the whole lattice; three quarters of its fluid nodes fail here,
+// before their 18 neighbours are read.
 __device__ __forceinline__ bool wall_links_at(const Lattice& L, const BodyParams& q, int x, int y) {
-    if (q.wall_axis >= 0) return true;
+    if (q.wall_axis >= 0 || x == 0 || y == 0 || x == L.nx - 1 || y == L.ny - 1) return true;
     const float lim = (float)q.tube[2] - 1.5f - 4e-7f * (float)(L.nx + L.ny);
     const float dx = (float)x - (float)q.tube[0], dy = (float)y - (float)q.tube[1];
     return !(lim > 0.0f && dx * dx + dy * dy < lim * lim);
@@ -1631,8 +1640,8 @@ __device__ __forceinline__ bool boxes_near(const Lattice& L, const BodyParams& p
     int la[3], wa[3], lb[3], wb[3];
     body_box(L, pa, sa, la, wa);
     body_box(L, pb, sb, lb, wb);
-    if (round_tube(pb) && !round_tube(pa)) return box_meets_tube(pb, la, wa, 2);
-    if (round_tube(pa) && !round_tube(pb)) return box_meets_tube(pa, lb, wb, 2);
+    if (round_tube(pb) && !round_tube(pa)) return box_meets_tube(L, pb, la, wa, 2);
+    if (round_tube(pa) && !round_tube(pb)) return box_meets_tube(L, pa, lb, wb, 2);
     const int n3[3] = {L.nx, L.ny, L.nz};
     for (int a = 0; a < 3; ++a)
         if (!axis_overlap(la[a] - 1, wa[a] + 2, lb[a] - 1, wb[a] + 2, n3[a])) return false;

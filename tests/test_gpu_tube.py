@@ -100,3 +100,62 @@ def test_tube_links_brute_force(shape, axis, radius):
         near = np.roll(wall, (-c[2, i], -c[1, i], -c[0, i]), (0, 1, 2))
         want |= {32 * int(n) + i for n in np.flatnonzero((~wall & near).reshape(-1))}
     assert links == want and len(links) > 0
+
+
+@pytest.mark.parametrize("shape,axis,radius", [((32, 32, 4), (4.0, 16.0), 10.0), ((32, 32, 4), (0.0, 16.0), 10.0),
+                                               ((64, 64, 4), (34.0, 32.0), 33.0), ((20, 26, 3), (19.0, 25.0), 8.5)])
+def test_tube_links_across_the_periodic_edge(shape, axis, radius):
+    """Tubes whose cross-section the box's periodic edge cuts: a fluid node at
+    the edge has the nodes across it as neighbours, and those may be wall
+    however near the axis the first lies.  The link list against every fluid
+    node with a wall neighbour, in cell and direction order."""
+    from paper_1903_04799_gb300 import Lattice
+
+    nx, ny, nz = shape
+    with Lattice(shape, storage="f32") as g:
+        tube = g.add_round_tube(*axis, radius)
+        links = g.links(tube).tolist()
+        wall = (g.owner() == tube).reshape(nz, ny, nx)
+    c = np.array([[0, 1, -1, 0, 0, 0, 0, 1, -1, 1, -1, 1, -1, 1, -1, 0, 0, 0, 0],
+                  [0, 0, 0, 1, -1, 0, 0, 1, -1, -1, 1, 0, 0, 0, 0, 1, -1, 1, -1],
+                  [0, 0, 0, 0, 0, 1, -1, 0, 0, 0, 0, 1, -1, -1, 1, 1, -1, -1, 1]])
+    edge = ~wall & (np.hypot(np.arange(nx)[None, None, :] - axis[0], np.arange(ny)[None, :, None] - axis[1])
+                    < radius - 1.5)
+    want, crossing = [], 0
+    for i in range(1, 19):
+        near = ~wall & np.roll(wall, (-c[2, i], -c[1, i], -c[0, i]), (0, 1, 2))
+        want += [32 * int(n) + i for n in np.flatnonzero(near.reshape(-1))]
+        crossing += int((near & edge).sum())
+    assert links == sorted(want) and crossing > 0
+
+
+@pytest.mark.parametrize("axis,r,pos,e", [((4.0, 16.0), 10.0, (3.4, 15.7, 12.2), (-1.0, 0.1, 0.2)),
+                                          ((15.0, 27.0), 10.0, (15.2, 27.6, 11.8), (0.1, 1.0, -0.2)),
+                                          ((0.0, 16.0), 20.0, (3.4, 15.7, 12.2), (-1.0, 0.1, 0.2))])
+def test_swimmer_at_the_cut_edge_of_a_tube_matches_oracle(axis, r, pos, e):
+    """A squirmer that swims at the periodic edge cutting its tube and covers
+    nodes whose neighbours across the edge are wall (30 steps, FP64): owners
+    and link lists as the oracle's, populations and states within 1e-12."""
+    shape, R = (32, 32, 24), 3.0
+    g = Lattice(shape, collision="trt")
+    o = OracleSim(*shape, lambda_e=1.0, collision="trt")
+    g.add_round_tube(*axis, r)
+    o.add_tube(*axis, r)
+    gi = g.add_squirmer(pos, e, R, 0.05, 0.0, mobile=True)
+    oi = o.add_sphere(pos, e, R, 0.05, 0.0, mobile=True)
+    first = g.owner()
+    edge = np.zeros((24, 32, 32), bool)
+    edge[:, :, 0] = edge[:, 31, :] = True
+    covered = False
+    for _ in range(6):
+        g.step(5)
+        o.step(5)
+        own = g.owner()
+        assert (own == o.owner()).all()
+        covered |= bool(((own != first) & edge.reshape(-1)).any())
+        fluid = own == 0  # solid cells hold nothing in the oracle
+        assert _rel(g.populations()[:, fluid], o.populations()[:, fluid]) < 1e-12
+        for a, c in zip(g.state(gi), o.state(oi)):
+            assert np.abs(a - c).max() < 1e-12
+    assert covered  # nodes of the edge changed hands
+    g.close()
