@@ -504,7 +504,6 @@ __device__ __noinline__ void update_move(const Lattice& L, const Bodies& B, int 
         } else {
             v = 0.0;
             held = kHeld;
-            if (lane == 0) set_error(L.err, 5);
         }
         const double dd = min_image(x - rc, n3[a]);
         const double disp2 = sum3(dd * dd);
@@ -581,8 +580,11 @@ __device__ __noinline__ void update_turn(const Lattice& L, const BodyParams& p, 
 }
 
 // After both and a block barrier, by one warp: the sums over the updates of v
-// and of v.e; a body held in place does not turn either.
-__device__ __forceinline__ void update_stats(const BodyParams& p, const BodyState& s, const BodyAcc& Ai, int flags,
+// and of v.e; a body held in place does not turn either, and its lattice's
+// error word says so (here and not in update_move, which k_body_fused also
+// runs on scratch without the links' force, where a body may seem to leave the
+// scheme that does not).
+__device__ __forceinline__ void update_stats(const Lattice& L, const BodyParams& p, const BodyState& s, const BodyAcc& Ai, int flags,
                                              BodyAcc* Ao, BodyState* So, BodyState* out) {
     if (!(p.kind == BODY_SPHERE && p.mobile)) return;
     const int lane = threadIdx.x & 31;
@@ -591,6 +593,7 @@ __device__ __forceinline__ void update_stats(const BodyParams& p, const BodyStat
         So->omega[a] = out->omega[a] = 0.0;
         So->e[a] = out->e[a] = s.e[a];
     }
+    if ((flags & kHeld) && lane == 0) set_error(L.err, 5);
     __syncwarp();
     const double v = out->vel[a], ve = sum3(v * out->e[a]);
     if (lane < 3) Ao->vsum[a] = Ai.vsum[a] + v;
@@ -1012,7 +1015,7 @@ __global__ void __launch_bounds__(kLB) k_links(const Bodies B) {
         if (threadIdx.x < 32) update_move<P>(L, B, k, p, s, A, s_tot, &A, &B.state[1 - P][k], &s_new, &s_flag);
         else if (threadIdx.x < 64) update_turn(L, p, s, A, s_tot, &A, &B.state[1 - P][k], &s_new);
         __syncthreads();
-        if (threadIdx.x >= 64 && threadIdx.x < 96) update_stats(p, s, A, s_flag, &A, &B.state[1 - P][k], &s_new);
+        if (threadIdx.x >= 64 && threadIdx.x < 96) update_stats(L, p, s, A, s_flag, &A, &B.state[1 - P][k], &s_new);
         if (s_flag & kReclass) append_items(B.box_items, B.n_box, B.box_cap, k, p.g_box, B.err, (int*)sm);
         __syncthreads();
     }
@@ -1868,7 +1871,7 @@ __global__ void __launch_bounds__(kFT, MANY ? 3 : 2) k_body_fused(const Bodies B
                 update_turn(L, p, s0, s_A, s_tot, &B.acc[k], &B.state[1 - P][k], &s_new);
             __syncthreads();
             if (threadIdx.x >= 64 && threadIdx.x < 96)
-                update_stats(p, s0, s_A, s_flags, &B.acc[k], &B.state[1 - P][k], &s_new);
+                update_stats(L, p, s0, s_A, s_flags, &B.acc[k], &B.state[1 - P][k], &s_new);
             if (threadIdx.x == 0) {
                 s_mode = s_flags & kReclass ? (near ? 2 : 1) : 0;
                 s_updated = 1;
@@ -2375,7 +2378,7 @@ __global__ void __launch_bounds__(kBB, 2) k_psm_cover(const Bodies B) {
         if (threadIdx.x < 32) update_move<P>(L, B, k, p, s, A, s_tot, &A, &B.state[1 - P][k], &s_new, &s_flag);
         else if (threadIdx.x < 64) update_turn(L, p, s, A, s_tot, &A, &B.state[1 - P][k], &s_new);
         __syncthreads();
-        if (threadIdx.x < 32) update_stats(p, s, A, s_flag, &A, &B.state[1 - P][k], &s_new);
+        if (threadIdx.x < 32) update_stats(L, p, s, A, s_flag, &A, &B.state[1 - P][k], &s_new);
         __syncthreads();
         // split steps: the last sphere to finish computes the near-body window
         // of the sweeps two steps later
