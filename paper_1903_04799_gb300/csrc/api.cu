@@ -45,7 +45,7 @@ void launch_tube_claim(const Lattice& L, int32_t* own, const BodyParams& q, int 
 void launch_gather(const int* err, const void* src, int words, void* dst, cudaStream_t st);
 void launch_set_flags(BodyAcc* acc, int nb, int k, int reclass, cudaStream_t st);
 void launch_psm_cover(const Bodies& B, int parity, int grid, bool f64, cudaStream_t st, bool dep = false,
-                      cudaEvent_t started = nullptr);
+                      bool early = false, cudaEvent_t started = nullptr);
 void launch_psm_scatter(const Bodies& B, int parity, int grid, cudaStream_t st, bool dep = false);
 }  // namespace lbsq
 
@@ -409,6 +409,14 @@ lb_status ensure_body_capacity(lb_ctx* c, int n) {
 // 14.9 / 16.6, 40^3 24.5 / 24.2, 56^3 29.6 / 25.5; FP32 40^3 18.7 / 20.4, 64^3
 // 22.2 / 23.3, 80^3 28.4 / 24.5; FP16 64^3 22.1 / 22.6, 80^3 27.3 / 24.4.
 bool worth_splitting(const lb_ctx* c) { return c->L.N >= (c->p.storage == LB_F64 ? 64000 : 350000); }
+
+// Whether the cover kernel of a split step is placed ahead of time (see
+// launch_psm_cover).  One sphere, us per step, early / ordinary: FP64 96^3, R =
+// 8 106 / 95, 112^3 118 / 117, 128^3, R = 3 120 / 128, R = 16 156 / 155, 160^3,
+// R = 8 218 / 236; FP32 96^3, R = 8 71 / 66, 128^3 77 / 75, 144^3 93 / 96,
+// 256^3, R = 16 414 / 417; FP16 128^3, R = 8 82 / 73, 144^3 83.4 / 84.4, 256^3
+// 232 / 248.
+bool psm_early(const lb_ctx* c) { return c->L.N >= (c->p.storage == LB_F64 ? 1800000 : 2500000); }
 
 // After the body set changed: assign link segments, size the partial-sum
 // buffers and work lists, and upload the body parameters.
@@ -1344,7 +1352,7 @@ static void end_units(lb_ctx* c) {
 //     slots are not among those scatter(t-1) writes, whose cells lie two cells
 //     inside the window; and for the blocks of cover(t) to be placed, which
 //     the far sweep would otherwise keep off the SMs until its own last block
-//     is dispatched.
+//     is dispatched (in large lattices ahead of time: psm_early).
 // Cover(t) advances the spheres and writes the window of step t + 2, which
 // holds what the cover and scatter kernels of steps t + 1 .. t + 3 touch: a
 // sphere moves under half a cell a step, the window has two cells to spare.
@@ -1357,7 +1365,7 @@ static void enqueue_psm_steps(lb_ctx* c, int64_t n) {
         const int parity = (int)(t & 1);
         const int* win = win_slot(c, t);
         const Bodies B = bodies_for_step(c, t);
-        launch_psm_cover(B, parity, c->grid_psm, c->p.storage == LB_F64, c->hi, k > 0, c->ev_started);
+        launch_psm_cover(B, parity, c->grid_psm, c->p.storage == LB_F64, c->hi, k > 0, psm_early(c), c->ev_started);
         cudaStreamWaitEvent(c->side, c->ev_started, 0);
         cudaStreamWaitEvent(c->hi, c->ev_join, 0);     // far(t-1), before near(t)
         cudaStreamWaitEvent(c->side, c->ev_join2, 0);  // near(t-1), before far(t)

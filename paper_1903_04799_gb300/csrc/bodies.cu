@@ -2422,14 +2422,21 @@ __global__ void __launch_bounds__(kBB) k_psm_scatter(const Bodies B) {
 }
 
 // Before the sweep of a step of parity P: clear and cover (two launches);
-// f64: the lattice stores FP64 populations.  dep: the first is a dependent
-// launch (see dep_wait).  started: null, or an event to fire once every block
-// of the cover kernel is placed.  The three kernels release their dependents
-// before they wait themselves, so that scatter, clear and cover are all placed
-// while the near sweep before them drains, each waiting for the one before; a
-// far sweep that waits for `started` finds them on the SMs and cannot fill
-// these first.  (None of them reads anything before dep_wait.)
-void launch_psm_cover(const Bodies& B, int parity, int grid, bool f64, cudaStream_t st, bool dep,
+// f64: the lattice stores FP64 populations.  dep: clear is a dependent launch
+// (see dep_wait).  early: cover is one too.  The kernels here release their
+// dependents before they wait themselves, so scatter, clear and an early cover
+// are all placed while the near sweep before them drains, each waiting for the
+// one before; a far sweep that waits for `started` (null, or an event to fire
+// once every block of the cover kernel is placed) finds them on the SMs and
+// cannot fill these first.  (None of them reads anything before dep_wait.)
+//
+// The price of early: blocks placed beside waiting ones land two on one SM and
+// share its FP64 pipe, where an ordinary launch spreads them.  So only a far
+// sweep long enough to hide that is worth it (psm_early in api.cu); before a
+// whole sweep cover is an ordinary launch (us per step, early / ordinary: FP64
+// 32 x 32 x 62, R = 12 108 / 79, 96^3, two of R = 8 134 / 119; FP32 64^3, R =
+// 12 73.3 / 64.4).
+void launch_psm_cover(const Bodies& B, int parity, int grid, bool f64, cudaStream_t st, bool dep, bool early,
                       cudaEvent_t started) {
     launch(k_psm_clear, grid, kBB, 0, st, dep, B, parity);
     cudaLaunchConfig_t cfg = {};
@@ -2437,15 +2444,18 @@ void launch_psm_cover(const Bodies& B, int parity, int grid, bool f64, cudaStrea
     cfg.blockDim = dim3(kBB);
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 0;
+    if (early) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+        cfg.numAttrs++;
+    }
     if (started) {
-        attr[1].id = cudaLaunchAttributeLaunchCompletionEvent;
-        attr[1].val.launchCompletionEvent.event = started;
-        attr[1].val.launchCompletionEvent.flags = 0;
-        cfg.numAttrs = 2;
+        attr[cfg.numAttrs].id = cudaLaunchAttributeLaunchCompletionEvent;
+        attr[cfg.numAttrs].val.launchCompletionEvent.event = started;
+        attr[cfg.numAttrs].val.launchCompletionEvent.flags = 0;
+        cfg.numAttrs++;
     }
     if (f64) cudaLaunchKernelEx(&cfg, parity == 0 ? k_psm_cover<0, double> : k_psm_cover<1, double>, B);
     else cudaLaunchKernelEx(&cfg, parity == 0 ? k_psm_cover<0, float> : k_psm_cover<1, float>, B);

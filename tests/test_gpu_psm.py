@@ -280,3 +280,35 @@ def test_split_steps_bitwise(storage, spheres):
         g.close()
     for a, b in zip(*runs):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("storage,shape", [("f64", (50, 45, 60)), ("f32", (66, 60, 96)), ("f16dev", (66, 60, 96)),
+                                           ("bf16dev", (66, 60, 96)), ("f32", (45, 100, 90)),
+                                           ("f16dev", (45, 100, 90)), ("f32", (136, 140, 136))])
+def test_split_steps_of_every_storage_bitwise(storage, shape):
+    """As test_split_steps_bitwise for one sphere, on lattices that every storage
+    splits, which the launch counts show (clear, cover, near and far sweep and
+    scatter: five a step, against four with one sweep).  Odd rows take the flat
+    even steps, whose chunks the window's border cuts; the last lattice is large
+    enough for cover kernels placed ahead of time."""
+    nx, ny, nz = shape
+    runs = []
+    for traced in (False, True):
+        g = Lattice(shape, collision="trt", storage=storage)
+        g.set_coupling("psm")
+        i = g.add_squirmer((24.3, 1.7, nz - 1.1), (0.3, 0.5, 1.0), 4.3, 0.05, -3.0, mobile=True)
+        if traced:
+            g.profile_begin()
+        seen, before = [], g.launches
+        for n, read in ((5, False), (16, True), (3, False), (9, True), (10, False)):
+            g.step(n)
+            if read:
+                seen.append([*g.state(i), *g.force_torque(i)])
+        if traced:
+            g.profile_end()
+        else:
+            assert g.launches - before >= 5 * 43
+        runs.append([g.populations(), g.solid_fraction(), *g.state(i), g.stresslet(i), *[x for r in seen for x in r]])
+        g.close()
+    for a, b in zip(*runs):
+        assert np.array_equal(a, b)
