@@ -581,12 +581,17 @@ lb_status relayout(lb_ctx* c) {
             across = true;
         }
     }
-    // (partially saturated cells split only without walls, whose links would
-    // have to follow the scattered results)
+    // Partially saturated cells split for a single sphere only.  Walls' links
+    // would have to follow the scattered results; and the window of several
+    // spheres may come to span the lattice, where the near sweep, behind the
+    // cover kernel and in its slower form, is all there is: two spheres half a
+    // box apart, whole against split, FP64 128^3 173 / 232 us, FP32 144^3 128 /
+    // 166, FP16 160^3 122 / 137 (before the steps were split: 188, 139, 132).
+    // One sphere, whole / split: FP64 48^3, R = 3 71 / 69, R = 8 79.8 / 80.8,
+    // 96^3, R = 8 117 / 95; FP32 72^3 67 / 64, FP16 72^3 71.7 / 70.0.
     const bool thin = !across && nb > 0 && wmax * 5 < 3 * c->L.nz && worth_splitting(c);
     c->split = !c->psm && thin;
-    c->psm_split = c->psm && thin &&
-                   std::all_of(c->par.begin(), c->par.end(), [](const BodyParams& b) { return b.psm != 0; });
+    c->psm_split = c->psm && thin && nb == 1 && c->par[0].psm != 0;
     if (ranges > 1) {
         wmax = c->L.nz;
         ymax = c->L.ny;
@@ -1342,8 +1347,8 @@ static void end_units(lb_ctx* c) {
     cudaStreamWaitEvent(c->stream, c->ev_join2, 0);
 }
 
-// n steps of a lattice of partially saturated spheres that occupy a thin box
-// of rows.  Step t runs its cover kernels, the near sweep (the window) and the
+// n steps of a lattice with one partially saturated sphere, in a thin box of
+// rows.  Step t runs its cover kernels, the near sweep (the window) and the
 // scatter on `hi`, and the far sweep on `side`:
 //   - cover(t) reads the populations of the window, which near(t-1) and
 //     scatter(t-1) left (stream order), so it runs beside far(t-1);
@@ -1353,9 +1358,9 @@ static void end_units(lb_ctx* c) {
 //     inside the window; and for the blocks of cover(t) to be placed, which
 //     the far sweep would otherwise keep off the SMs until its own last block
 //     is dispatched (in large lattices ahead of time: psm_early).
-// Cover(t) advances the spheres and writes the window of step t + 2, which
-// holds what the cover and scatter kernels of steps t + 1 .. t + 3 touch: a
-// sphere moves under half a cell a step, the window has two cells to spare.
+// Cover(t) advances the sphere and writes the window of step t + 2, which
+// holds what the cover and scatter kernels of steps t + 1 .. t + 3 touch: it
+// moves under half a cell a step, the window has two cells to spare.
 // In one chain the three kernels, whose few blocks leave the GPU idle, took
 // 80 us a step beside a sweep of 368 (256^3, R = 16, FP32).
 static void enqueue_psm_steps(lb_ctx* c, int64_t n) {

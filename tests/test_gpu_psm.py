@@ -312,3 +312,16 @@ def test_split_steps_of_every_storage_bitwise(storage, shape):
         g.close()
     for a, b in zip(*runs):
         assert np.array_equal(a, b)
+
+
+def test_several_spheres_step_whole_lattices():
+    """Several partially saturated spheres: one sweep a step (four launches, and
+    one more per read-out)."""
+    g = Lattice((66, 60, 96), collision="trt", storage="f32")
+    g.set_coupling("psm")
+    for z in (20.2, 60.7):
+        g.add_squirmer((30.3, 29.7, z), (0.3, 0.5, 1.0), 4.3, 0.05, -3.0, mobile=True)
+    before = g.launches
+    g.step(40)
+    assert g.launches - before == 4 * 40
+    g.close()
