@@ -504,7 +504,7 @@ lb_status relayout(lb_ctx* c) {
     dfree(c, c->d_part_links);
     dfree(c, c->d_part_conv);
     dfree(c, c->d_part_count);
-    c->d_part_links = dalloc_t<double>(c, (size_t)nb * c->G_links * 12);
+    c->d_part_links = dalloc_t<double>(c, (size_t)nb * c->G_links * kLinkPart);
     c->d_part_conv = dalloc_t<double>(c, (size_t)nb * c->G_box * 6);
     c->d_part_count = dalloc_t<int>(c, (size_t)nb * c->G_box);
     if (!c->d_part_links || !c->d_part_conv || !c->d_part_count) return fail(c, LB_ERR_OOM, "partials");

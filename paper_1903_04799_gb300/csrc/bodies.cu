@@ -700,102 +700,127 @@ __device__ __forceinline__ void load_sphere(const Lattice& L, const BodyParams& 
     __syncthreads();
 }
 
-// FP64 links of a sphere (FP64 storage) or a wall (any storage): acc takes
-// force (0..2) and, for a sphere, torque (3..5) and the negated stresslet, its
-// off-diagonal components doubled (6..11; sphere_totals).  A link's dF lies
-// along its direction, c_i sf with c in {-1, 0, 1}, so the stresslet's nine
-// products d_a dF_b are selected from three, and the torque takes the d x c of
-// the rotation's boundary velocity; term by term they took twice the FP64
-// instructions.  Block g takes every G-th run of kRun links.  Links all over
-// the sphere, because their large rest parts then cancel within the block
-// (one stretch of neighbouring links per block tripled the rounding error of
-// the stresslet at R = 7); the trace leaves each link for the same reason.  In
-// runs, because the rest torques of one node's links cancel (single links:
-// rms error of the torque 10 % larger at R = 16).
+// Links of a wall (any storage): acc takes its force.  A thread holds several
+// links: kU codes, then their outgoing populations, are loaded before any
+// arithmetic or store (tube run: 80 000 links on 128 blocks).
+template <int P>
+__device__ __forceinline__ void wall_terms(const Lattice& L, const BodyParams& p, long long cnt,
+                                           const uint32_t* links, int g, int G, double (&acc)[3]) {
+    constexpr int kU = 4;
+    const int64_t Np = L.Np;
+    const int stride = G * (int)blockDim.x, end = (int)cnt;
+    for (int l0 = g * (int)blockDim.x + (int)threadIdx.x; l0 < end; l0 += kU * stride) {
+        uint32_t codes[kU];
+        Link lk[kU];
+        double fouts[kU];
+#pragma unroll
+        for (int q = 0; q < kU; ++q) codes[q] = l0 + q * stride < end ? links[l0 + q * stride] : 0u;
+#pragma unroll
+        for (int q = 0; q < kU; ++q) {
+            if (l0 + q * stride >= end) continue;
+            const Link k = lk[q] = link_of(L, codes[q]);
+            // where sweep P left f*_i of the fluid node
+            fouts[q] = load_abs(L, P == 0 ? (int64_t)opp(k.i) * Np + k.n : (int64_t)k.i * Np + k.ns, k.i);
+        }
+#pragma unroll
+        for (int q = 0; q < kU; ++q) {
+            if (l0 + q * stride >= end) continue;
+            const Link k = lk[q];
+            const int i = k.i, ib = opp(i);
+            const int ci[3] = {cx(i), cy(i), cz(i)};
+            const double cv = csel(ci[0], p.wall_vel[0]) + csel(ci[1], p.wall_vel[1]) + csel(ci[2], p.wall_vel[2]);
+            const double rs = L.rho_local ? post_density<P>(L, k.n, k.x, k.y, k.z) : L.rho0;
+            const double fin = fouts[q] - 6.0 * rs * wgt(i) * cv;
+            // where the next sweep reads the reflected population f_ib of the fluid node
+            store_abs(L, P == 0 ? (int64_t)i * Np + k.ns : (int64_t)ib * Np + k.n, ib, fin);
+            // momentum given to the body, c_i (f_out + f_in)
+            const double sf = fouts[q] + fin;
+            for (int a = 0; a < 3; ++a) acc[a] += csel(ci[a], sf);
+        }
+    }
+}
+
+// Links of a sphere in FP64 storage: the deviations' part of force (acc[0..2])
+// and torque (3..5), the rest part of both in integers (rest), which
+// sphere_totals puts together, and the negated stresslet, its off-diagonal
+// components doubled (6..11).  A link's dF lies along its direction, c_i sf
+// with c in {-1, 0, 1}, so the stresslet's nine products d_a dF_b are selected
+// from three, and the torque takes the d x c of the rotation's boundary
+// velocity.
+//
+// sf = sg + 2 w_i rho0, sg the sum of the two deviations.  The rest part is
+// some hundred times the deviations' and cancels over the closed surface, and
+// its rounding was the torque's error, larger or smaller by which links a block
+// took.  With d = o + link_at c - frac, o the integer offset of the fluid node
+// from floor(centre), it is made of integer sums over the links (36 w_i = 2 or
+// 1) and of frac, which is the body's.  rms torque error over 60 states, FP64
+// sums of f in contiguous stretches / in runs of eight links / now: R = 5.2 4.8
+// / 4.4 / 3.9e-15, 9.1 1.46 / 1.63 / 1.26e-14, 13.7 3.5 / 3.9 / 3.0e-14, 16 4.5 /
+// 4.6 / 3.6e-14 (the reference's own rounding, in FP64 sums of f, is most of
+// what is left); the force's error fell too, and the stresslet's is the same.
+// 32^3, R = 4, free: 20.8 us per step before, 19.7 now.
+//
+// Block g takes every G-th run of kRun links: links all over the sphere,
+// because the stresslet's large rest parts then cancel within the block (one
+// stretch of neighbouring links per block tripled its rounding error at R = 7);
+// the trace leaves each link for the same reason.
 constexpr int kRun = 8;
 
-template <int P, bool SPHERE>
+template <int P>
 __device__ __forceinline__ void link_terms64(const Lattice& L, const BodyParams& p, const BodyState& s,
                                              const SphereF& sp, long long cnt, const uint32_t* links, int g, int G,
-                                             double (&acc)[12]) {
+                                             double (&acc)[12], int (&rest)[6]) {
     const int64_t Np = L.Np;
-    const int* ip = sp.ip;
-    const double* fp = sp.fd;
+    double* F = (double*)L.F;
     const int n3[3] = {L.nx, L.ny, L.nz};
-    // A wall's threads hold several links each: kU codes, then their outgoing
-    // populations, are loaded before any arithmetic or store (tube run: 80 000
-    // links on 128 blocks).
-    constexpr int kU = SPHERE ? 1 : 4;
-    const int stride = G * (int)blockDim.x;
+    const double la = (double)L.link_at;
     const int t = (int)threadIdx.x, l0 = (t / kRun * G + g) * kRun + t % kRun;
-    for (int lb = l0; lb < (int)cnt; lb += kU * stride) {
-    uint32_t codes[kU];
-    Link lk[kU];
-    double fouts[kU];
-#pragma unroll
-    for (int q = 0; q < kU; ++q) codes[q] = lb + q * stride < (int)cnt ? links[lb + q * stride] : 0u;
-#pragma unroll
-    for (int q = 0; q < kU; ++q) {
-        if (lb + q * stride >= (int)cnt) continue;
-        lk[q] = link_of(L, codes[q]);
-        // where sweep P left f*_i of the fluid node
-        fouts[q] = load_abs(L, P == 0 ? (int64_t)opp(lk[q].i) * Np + lk[q].n : (int64_t)lk[q].i * Np + lk[q].ns, lk[q].i);
-    }
-#pragma unroll
-    for (int q = 0; q < kU; ++q) {
-        if (lb + q * stride >= (int)cnt) continue;
-        const Link k = lk[q];
-        const int i = k.i, ib = opp(i);
-        const int ci[3] = {cx(i), cy(i), cz(i)};
-        // where the next sweep reads the reflected population f_ib of the fluid node
-        const int64_t in_slot = P == 0 ? (int64_t)i * Np + k.ns : (int64_t)ib * Np + k.n;
-        const double fout = fouts[q];
-        double d[3], arm[3], cv;  // arm = d x c, cv = c.v_b
-        if (SPHERE) {
-            // link midpoint (or boundary node) relative to the centre (minimum
-            // image: a link lies within R + 2 of it, less than half the box);
-            // rigid motion + slip there, along c: with n = d / |d|,
-            // c.v_b = c.v + w.(d x c) + (B1 + B2 e.n) ((e.n)(c.n) - c.e)
-            const int xi[3] = {k.x, k.y, k.z};
-            const double la = (double)L.link_at;
-            for (int a = 0; a < 3; ++a) {
-                int o = xi[a] - ip[a];
-                if (2 * o > n3[a]) o -= n3[a];
-                else if (2 * o <= -n3[a]) o += n3[a];
-                d[a] = ((double)o + csel(ci[a], la)) - fp[a];
-            }
-            const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-            const double ir = r2 > 0.0 ? rsqrt(r2) : 0.0;
-            const double ct = (s.e[0] * d[0] + s.e[1] * d[1] + s.e[2] * d[2]) * ir;
-            const double cn = (csel(ci[0], d[0]) + csel(ci[1], d[1]) + csel(ci[2], d[2])) * ir;
-            const double ce = csel(ci[0], s.e[0]) + csel(ci[1], s.e[1]) + csel(ci[2], s.e[2]);
-            const double slip = r2 > 0.0 ? (p.B1 + p.B2 * ct) * (ct * cn - ce) : 0.0;
-            arm[0] = csel(ci[2], d[1]) - csel(ci[1], d[2]);
-            arm[1] = csel(ci[0], d[2]) - csel(ci[2], d[0]);
-            arm[2] = csel(ci[1], d[0]) - csel(ci[0], d[1]);
-            const double rot = s.omega[0] * arm[0] + s.omega[1] * arm[1] + s.omega[2] * arm[2];
-            cv = csel(ci[0], s.vel[0]) + csel(ci[1], s.vel[1]) + csel(ci[2], s.vel[2]) + (rot + slip);
-        } else {
-            cv = csel(ci[0], p.wall_vel[0]) + csel(ci[1], p.wall_vel[1]) + csel(ci[2], p.wall_vel[2]);
+    for (int l = l0; l < (int)cnt; l += G * (int)blockDim.x) {
+        const Link k = link_of(L, links[l]);
+        const int i = k.i, ib = opp(i), w = i < 7 ? 2 : 1;
+        const int ci[3] = {cx(i), cy(i), cz(i)}, xi[3] = {k.x, k.y, k.z};
+        // where sweep P left g*_i of the fluid node
+        const double gout = F[P == 0 ? (int64_t)ib * Np + k.n : (int64_t)i * Np + k.ns];
+        // link midpoint (or boundary node) relative to the centre (minimum
+        // image: a link lies within R + 2 of it, less than half the box); rigid
+        // motion + slip there, along c: with n = d / |d|,
+        // c.v_b = c.v + w.(d x c) + (B1 + B2 e.n) ((e.n)(c.n) - c.e)
+        int o[3];
+        double d[3], arm[3];  // arm = d x c
+        for (int a = 0; a < 3; ++a) {
+            o[a] = xi[a] - sp.ip[a];
+            if (2 * o[a] > n3[a]) o[a] -= n3[a];
+            else if (2 * o[a] <= -n3[a]) o[a] += n3[a];
+            d[a] = ((double)o[a] + csel(ci[a], la)) - sp.fd[a];
         }
+        const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+        const double ir = r2 > 0.0 ? rsqrt(r2) : 0.0;
+        const double ct = (s.e[0] * d[0] + s.e[1] * d[1] + s.e[2] * d[2]) * ir;
+        const double cn = (csel(ci[0], d[0]) + csel(ci[1], d[1]) + csel(ci[2], d[2])) * ir;
+        const double ce = csel(ci[0], s.e[0]) + csel(ci[1], s.e[1]) + csel(ci[2], s.e[2]);
+        const double slip = r2 > 0.0 ? (p.B1 + p.B2 * ct) * (ct * cn - ce) : 0.0;
+        arm[0] = csel(ci[2], d[1]) - csel(ci[1], d[2]);
+        arm[1] = csel(ci[0], d[2]) - csel(ci[2], d[0]);
+        arm[2] = csel(ci[1], d[0]) - csel(ci[0], d[1]);
+        const double rot = s.omega[0] * arm[0] + s.omega[1] * arm[1] + s.omega[2] * arm[2];
+        const double cv = csel(ci[0], s.vel[0]) + csel(ci[1], s.vel[1]) + csel(ci[2], s.vel[2]) + (rot + slip);
         const double rs = L.rho_local ? post_density<P>(L, k.n, k.x, k.y, k.z) : L.rho0;
-        const double fin = fout - 6.0 * rs * wgt(i) * cv;
-        store_abs(L, in_slot, ib, fin);
-        // momentum given to the body, c_i (f_out + f_in)
-        const double sf = fout + fin;
-        const double dF[3] = {csel(ci[0], sf), csel(ci[1], sf), csel(ci[2], sf)};
-        for (int a = 0; a < 3; ++a) acc[a] += dF[a];
-        if (SPHERE) {
-            const double m[3] = {d[0] * sf, d[1] * sf, d[2] * sf};
-            const double tr = (csel(ci[0], m[0]) + csel(ci[1], m[1]) + csel(ci[2], m[2])) * (1.0 / 3.0);
-            for (int a = 0; a < 3; ++a) {
-                acc[3 + a] = fma(arm[a], sf, acc[3 + a]);
-                acc[6 + a] += csel(ci[a], m[a]) - tr;
-                const int b = a == 2 ? 0 : a + 1;  // (0,1), (1,2), (2,0): xy, yz, xz
-                acc[9 + (a == 2 ? 1 : (a == 0 ? 0 : 2))] += csel(ci[b], m[a]) + csel(ci[a], m[b]);
-            }
+        const double gin = gout - 6.0 * rs * wgt(i) * cv;
+        // where the next sweep reads the reflected population of the fluid node
+        F[P == 0 ? (int64_t)i * Np + k.ns : (int64_t)ib * Np + k.n] = gin;
+        // momentum given to the body, c_i (f_out + f_in): deviations, and whole
+        const double sg = gout + gin, sf = fma(2.0 * wgt(i), L.rho0, sg);
+        const double m[3] = {d[0] * sf, d[1] * sf, d[2] * sf};
+        const double tr = (csel(ci[0], m[0]) + csel(ci[1], m[1]) + csel(ci[2], m[2])) * (1.0 / 3.0);
+        for (int a = 0; a < 3; ++a) {
+            const int b = (a + 1) % 3, e = (a + 2) % 3;
+            acc[a] += csel(ci[a], sg);
+            acc[3 + a] = fma(arm[a], sg, acc[3 + a]);
+            acc[6 + a] += csel(ci[a], m[a]) - tr;
+            acc[9 + (a == 2 ? 1 : (a == 0 ? 0 : 2))] += csel(ci[b], m[a]) + csel(ci[a], m[b]);  // xy, yz, xz
+            rest[a] += w * ci[a];
+            rest[3 + a] += w * (o[b] * ci[e] - o[e] * ci[b]);
         }
-    }
     }
 }
 
@@ -900,18 +925,30 @@ __device__ __forceinline__ void link_terms32(const Lattice& L, const SphereF& sf
 }
 
 // A block's share of a sphere's links and the block's sums in tot (shared):
-// force, torque and stresslet, or what link_terms64 sums (FP64 storage).
-template <int P, int T, bool REDUCED = false>
+// force, torque and stresslet, or what link_terms64 sums (F64: FP64 storage;
+// its integers are added to rest, shared, which the caller has zeroed).
+template <int P, int T, bool F64>
 __device__ __forceinline__ void sphere_links(const Lattice& L, const BodyParams& p, const BodyState& s,
                                              const SphereF& sf, long long cnt, const uint32_t* links, int g, int G,
-                                             double* sm, double* tot) {
-    if (!REDUCED && L.storage == ST_F64) {
+                                             double* sm, double* tot, int* rest) {
+    if constexpr (F64) {
         double acc[12];
+        int ri[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll
         for (int c = 0; c < 12; ++c) acc[c] = 0.0;
-        link_terms64<P, true>(L, p, s, sf, cnt, links, g, G, acc);
+        link_terms64<P>(L, p, s, sf, cnt, links, g, G, acc, ri);
         // threads that hold links: those of full runs
-        block_sum_fixed<12, T>(acc, sm, tot, (int)min((long long)T, (cnt + kRun * G - 1) / (kRun * G) * kRun));
+        const int active = (int)min((long long)T, (cnt + kRun * G - 1) / (kRun * G) * kRun);
+        if ((int)(threadIdx.x & ~31u) < active) {
+            int mine = 0;  // lane c < 6: component c
+#pragma unroll
+            for (int c = 0; c < 6; ++c) {
+                const int r = __reduce_add_sync(0xffffffffu, ri[c]);
+                if ((threadIdx.x & 31) == c) mine = r;
+            }
+            if ((threadIdx.x & 31) < 6) atomicAdd(&rest[threadIdx.x & 31], mine);
+        }
+        block_sum_fixed<12, T>(acc, sm, tot, active);
     } else {
         df acc[12];
 #pragma unroll
@@ -921,10 +958,20 @@ __device__ __forceinline__ void sphere_links(const Lattice& L, const BodyParams&
     }
 }
 
-// The body's totals tot[12] from the sums over its blocks, in place, by
-// threads 0..11.
-__device__ __forceinline__ void sphere_totals(const Lattice& L, double* tot) {
-    if (L.storage == ST_F64 && threadIdx.x >= 6) tot[threadIdx.x] *= threadIdx.x < 9 ? -1.0 : -0.5;
+// FP64 storage: the body's force, torque and stresslet in tot[12] from the sums
+// over its blocks, in place, by threads 0..11; force and torque get the rest
+// part from the integers I (see link_terms64).  They are zero for a sphere
+// that touches no other solid: every lattice line through it crosses its
+// surface in pairs of links, whose rest parts cancel.
+__device__ __forceinline__ void sphere_totals(const Lattice& L, const SphereF& sp, const int* I, double* tot) {
+    const int c = threadIdx.x;
+    if (c >= 6) {
+        tot[c] *= c < 9 ? -1.0 : -0.5;
+    } else if ((I[0] | I[1] | I[2] | I[3] | I[4] | I[5]) != 0) {
+        const int a = c % 3, b = (a + 1) % 3, e = (a + 2) % 3;
+        const double arm = c < 3 ? 0.0 : sp.fd[b] * (double)I[e] - sp.fd[e] * (double)I[b];
+        tot[c] += L.rho0 * (1.0 / 18.0) * ((double)I[c] - arm);  // 2 rho0 / 36
+    }
 }
 
 // Links of a still body with no force readout: out slot copied to in slot in
@@ -970,7 +1017,7 @@ __global__ void __launch_bounds__(kLB) k_links(const Bodies B) {
     __shared__ double s_tot[12];
     __shared__ BodyState s_new;
     __shared__ SphereF s_sf;
-    __shared__ int s_flag;
+    __shared__ int s_flag, s_rest[6];
     const int nitems = *B.n_link_items;
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const int2 item = B.link_items[it];
@@ -988,27 +1035,37 @@ __global__ void __launch_bounds__(kLB) k_links(const Bodies B) {
         }
         const BodyState& s = B.state[P][k];
         const uint32_t* links = B.links + p.link_off;
-        double* parts = B.part_links + (size_t)k * B.GL * 12;
+        double* parts = B.part_links + (size_t)k * B.GL * kLinkPart;
+        double* part = parts + (size_t)g * kLinkPart;
         if (p.kind == BODY_SPHERE) {
+            if (threadIdx.x < 6) s_rest[threadIdx.x] = 0;
             load_sphere(L, p, s, s_sf);
-            sphere_links<P, kLB>(L, p, s, s_sf, A.link_count, links, g, G, sm, s_tot);
-            if (threadIdx.x < 12) parts[g * 12 + threadIdx.x] = s_tot[threadIdx.x];
+            if (L.storage == ST_F64)
+                sphere_links<P, kLB, true>(L, p, s, s_sf, A.link_count, links, g, G, sm, s_tot, s_rest);
+            else
+                sphere_links<P, kLB, false>(L, p, s, s_sf, A.link_count, links, g, G, sm, s_tot, s_rest);
+            if (threadIdx.x < 12) part[threadIdx.x] = s_tot[threadIdx.x];
+            if (threadIdx.x < 6) reinterpret_cast<int*>(part + 12)[threadIdx.x] = s_rest[threadIdx.x];
         } else {  // a wall: its force only
-            double acc[12];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) acc[c] = 0.0;
-            link_terms64<P, false>(L, p, s, s_sf, A.link_count, links, g, G, acc);
-            double F[3] = {acc[0], acc[1], acc[2]};
+            double F[3] = {0.0, 0.0, 0.0};
+            wall_terms<P>(L, p, A.link_count, links, g, G, F);
             block_sum_fixed<3, kLB>(F, sm, s_tot);
-            if (threadIdx.x < 3) parts[g * 12 + threadIdx.x] = s_tot[threadIdx.x];
+            if (threadIdx.x < 3) part[threadIdx.x] = s_tot[threadIdx.x];
         }
         if (!last_block(&A.counter_links, G, &s_flag)) continue;
         if (p.kind == BODY_SPHERE) {
-            ordered_partial_sum<12>(parts, G, sm, s_tot);
-            if (threadIdx.x < 12) sphere_totals(L, s_tot);
+            if (threadIdx.x < 6) s_rest[threadIdx.x] = 0;
+            ordered_partial_sum<12>(parts, G, sm, s_tot, kLinkPart);
+            if (L.storage == ST_F64) {
+                for (int q = threadIdx.x; q < 6 * G; q += blockDim.x)
+                    atomicAdd(&s_rest[q % 6],
+                              __ldcg(reinterpret_cast<const int*>(parts + (size_t)(q / 6) * kLinkPart + 12) + q % 6));
+                __syncthreads();
+                if (threadIdx.x < 12) sphere_totals(L, s_sf, s_rest, s_tot);
+            }
             __syncthreads();
         } else {
-            ordered_partial_sum<3>(parts, G, sm, s_tot, 12);
+            ordered_partial_sum<3>(parts, G, sm, s_tot, kLinkPart);
             if (threadIdx.x >= 3 && threadIdx.x < 12) s_tot[threadIdx.x] = 0.0;
             __syncthreads();
         }
@@ -1764,7 +1821,9 @@ constexpr int kStcBuf = 2048;  // stencil entries a block keeps in shared memory
 // per SM (without the FP64 links; 300 bytes of spill) beat two: 200 spheres of R
 // = 6, 471 -> 465 us per step.  With a few spheres there is one wave, and the
 // spills cost (128^3, one sphere: 45.7 -> 48.6 us).
-template <int P, bool MANY>
+// F64: FP64 storage, whose links take FP64 arithmetic and integers for the rest
+// part (link_terms64); each form holds the links of its own storages only.
+template <int P, bool F64, bool MANY>
 __global__ void __launch_bounds__(kFT, MANY ? 3 : 2) k_body_fused(const Bodies B, int cls, int tail) {
     cg::cluster_group cl = cg::this_cluster();
     const int KC = (int)cl.num_blocks();
@@ -1781,6 +1840,7 @@ __global__ void __launch_bounds__(kFT, MANY ? 3 : 2) k_body_fused(const Bodies B
     __shared__ int s_dryMode, s_flags;
     __shared__ ShellGeo s_geo;
     __shared__ SphereF s_sf;
+    __shared__ int s_rest[6], s_rests[6 * 16];  // integers of link_terms64, rank 0: of every rank
     __shared__ uint32_t s_stc[kStcBuf];
     __shared__ uint32_t s_emask[kStcBuf];  // phase A's link mask of each stencil entry, for phase B
     __shared__ int s_updated;              // rank 0: s_new holds this launch's new state
@@ -1818,6 +1878,7 @@ __global__ void __launch_bounds__(kFT, MANY ? 3 : 2) k_body_fused(const Bodies B
         long long b0, b1;
         box_range(p.st_count, rank, KC, b0, b1);
         for (long long b = b0 + threadIdx.x; b < b1 && b < b0 + kStcBuf; b += kFT) s_stc[b - b0] = __ldg(stc + b);
+        if (F64 && threadIdx.x < 6) s_rest[threadIdx.x] = 0;
         load_sphere(L, p, s0, s_sf);
         // the populations follow; everything above was written by kernels
         // before the sweep this launch may have started beside
@@ -1843,12 +1904,15 @@ __global__ void __launch_bounds__(kFT, MANY ? 3 : 2) k_body_fused(const Bodies B
             if (threadIdx.x < 12) s_tot[threadIdx.x] = 0.0;
             near = __syncthreads_or(near);
         } else {
-            sphere_links<P, kFT, MANY>(L, p, s0, s_sf, s_A.link_count, B.links + p.link_off, rank - 1, KC - 1, sm, s_tot);
+            sphere_links<P, kFT, F64>(L, p, s0, s_sf, s_A.link_count, B.links + p.link_off, rank - 1, KC - 1, sm,
+                                       s_tot, s_rest);
         }
         cl.sync();
         if (rank == 0) {
             // the blocks' partial sums, all fetched at once, then summed in rank order
             if (threadIdx.x < 12 * KC) sm[threadIdx.x] = cl.map_shared_rank(s_tot, threadIdx.x / 12)[threadIdx.x % 12];
+            if (F64 && threadIdx.x < 6 * KC)
+                s_rests[threadIdx.x] = cl.map_shared_rank(s_rest, threadIdx.x / 6)[threadIdx.x % 6];
             __syncthreads();
             // four runs of KC / 4 ranks per component, then the four sums
             const int run = KC / 4;
@@ -1858,11 +1922,17 @@ __global__ void __launch_bounds__(kFT, MANY ? 3 : 2) k_body_fused(const Bodies B
                 for (int r = r0 + 1; r < r0 + run; ++r) t += sm[r * 12 + c];
                 sm[12 * KC + threadIdx.x] = t;
             }
+            if (F64 && threadIdx.x >= 64 && threadIdx.x < 70) {
+                const int c = threadIdx.x - 64;
+                int t = 0;
+                for (int r = 0; r < KC; ++r) t += s_rests[6 * r + c];
+                s_rest[c] = t;
+            }
             __syncthreads();
             if (threadIdx.x < 12) {
                 const double* q4 = sm + 12 * KC + threadIdx.x;
                 s_tot[threadIdx.x] = (q4[0] + q4[12]) + (q4[24] + q4[36]);
-                sphere_totals(L, s_tot);
+                if (F64) sphere_totals(L, s_sf, s_rest, s_tot);
             }
             __syncthreads();
             if (threadIdx.x < 32)
@@ -2484,10 +2554,12 @@ void launch_body_kernel(int which, const Bodies& B, int parity, int grid_links, 
 // Once per process and device, before the first launch of k_body_fused:
 // allow clusters of 16 blocks (above the portable maximum of 8).
 cudaError_t prepare_body_kernels() {
-    cudaError_t e = cudaFuncSetAttribute(k_body_fused<0, false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_body_fused<1, false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    return e;
+    for (auto k : {k_body_fused<0, true, false>, k_body_fused<1, true, false>, k_body_fused<0, false, false>,
+                   k_body_fused<1, false, false>}) {
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // Blocks per cluster of fused-kernel class c (see fused_class).
@@ -2525,10 +2597,11 @@ void launch_body_fused(const Bodies& B, int parity, int cls, int clusters, bool 
         attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
         cfg.numAttrs++;
     }
-    if (cls == 2 && !f64)
-        cudaLaunchKernelEx(&cfg, parity == 0 ? k_body_fused<0, true> : k_body_fused<1, true>, B, cls, tail);
-    else
-        cudaLaunchKernelEx(&cfg, parity == 0 ? k_body_fused<0, false> : k_body_fused<1, false>, B, cls, tail);
+    void (*k)(Bodies, int, int) =
+        f64        ? (parity == 0 ? k_body_fused<0, true, false> : k_body_fused<1, true, false>)
+        : cls == 2 ? (parity == 0 ? k_body_fused<0, false, true> : k_body_fused<1, false, true>)
+                   : (parity == 0 ? k_body_fused<0, false, false> : k_body_fused<1, false, false>);
+    cudaLaunchKernelEx(&cfg, k, B, cls, tail);
 }
 
 }  // namespace lbsq

@@ -343,13 +343,17 @@ struct BodyAcc {
 // classification appends the items of every body whose links must be rebuilt.
 std::vector<uint32_t> shell_stencil(double R);
 
+// 64-bit words of a block's partial sums over a body's links: 12 doubles, then
+// 6 integers (see link_terms64).
+constexpr int kLinkPart = 15;
+
 struct Bodies {
     const Lattice* lats;
     const BodyParams* par;
     BodyState* state[2];
     BodyAcc* acc;
     uint32_t* links;       // code = cell * 32 + i
-    double* part_links;    // [body][GL][12]
+    double* part_links;    // [body][GL][kLinkPart]
     double* part_conv;     // [body][GB][6]
     int* part_count;       // [body][GB]
     int GL, GB;            // strides of the partial arrays

@@ -339,7 +339,7 @@ std::vector<TableSpec> tables(lb_server* s) {
         {(void**)&s->d_state[0], sizeof(BodyState) * B},
         {(void**)&s->d_state[1], sizeof(BodyState) * B},
         {(void**)&s->d_acc, sizeof(BodyAcc) * B},
-        {(void**)&s->d_part_links, sizeof(double) * B * kMaxGL * 12},
+        {(void**)&s->d_part_links, sizeof(double) * B * kMaxGL * kLinkPart},
         {(void**)&s->d_part_conv, sizeof(double) * B * kMaxGB * 6},
         {(void**)&s->d_part_count, sizeof(int) * B * kMaxGB},
         {(void**)&s->d_link_items, sizeof(int2) * s->list_cap * kGroups},

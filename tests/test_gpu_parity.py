@@ -782,3 +782,75 @@ def test_c3_full_size_parity(storage, tol):
     assert rel(ug[:, both], uo[:, both]) < tol
     vg, vo = g.state(gi)[1], o.state(oi)[1]
     assert np.abs(vg - vo).max() < tol * np.abs(vo).max()
+
+
+@pytest.mark.parametrize("R,shape", [(5.2, (18, 17, 19)), (9.1, (26, 25, 27)), (13.7, (35, 36, 34))])
+def test_torque_rounding_f64(R, shape):
+    """The torque of a sphere at rest without slip (f_in = f_out, so it follows
+    from the exported populations) against exact sums, FP64 storage.  The rest
+    density's part of the torque is exactly zero (every lattice line crosses the
+    surface in pairs of links), so the reference sums deviations f - w, exact
+    differences, with math.fsum; what it does not know is the rounding of the
+    exported f, ulp(f) / sqrt(12) each.  The library's own rounding has to stay
+    within that: over eight states, an rms error of less than twice the
+    expected one (24 samples, an rms of 1 +- 0.15 if there were no other)."""
+    import math
+
+    c = np.array([[0, 1, -1, 0, 0, 0, 0, 1, -1, 1, -1, 1, -1, 1, -1, 0, 0, 0, 0],
+                  [0, 0, 0, 1, -1, 0, 0, 1, -1, -1, 1, 0, 0, 0, 0, 1, -1, 1, -1],
+                  [0, 0, 0, 0, 0, 1, -1, 0, 0, 0, 0, 1, -1, -1, 1, 1, -1, -1, 1]]).T
+    w = np.array([1 / 3] + [1 / 18] * 6 + [1 / 36] * 12)
+    opp = np.array([0] + [i + 1 if i % 2 else i - 1 for i in range(1, 19)])
+    n3 = np.array(shape)
+    pos = n3 / 2 + np.array([0.21, -0.37, 0.13])
+    ratio = []
+    for seed in range(8):
+        with Lattice(shape, collision="trt", storage="f64") as g:
+            k = g.add_squirmer(pos, (0.0, 0.0, 1.0), R, 0.0, 0.0, mobile=False)
+            g.set_fields(*W.smooth_fields(shape, seed))
+            g.step(1 + seed % 2)
+            codes, f = g.links(k).astype(np.int64), g.populations()
+            T = g.force_torque(k)[1]
+        n, i = codes // 32, codes % 32
+        x = np.stack([n % n3[0], n // n3[0] % n3[1], n // (n3[0] * n3[1])], 1)
+        d = x + 0.5 * c[i] - pos
+        d -= n3 * np.round(d / n3)
+        arm = np.cross(d, c[i])
+        fin = f[opp[i], n]
+        for a in range(3):
+            want = math.fsum(arm[:, a] * (2.0 * (fin - w[i])))
+            sigma = np.sqrt(np.sum((2.0 * arm[:, a] * np.spacing(fin)) ** 2) / 12.0)
+            ratio.append((T[a] - want) / sigma)
+    assert np.sqrt(np.mean(np.square(ratio))) < 2.0
+
+
+@pytest.mark.parametrize("wall", [False, True])
+def test_forces_of_touching_solids_f64(wall):
+    """Two spheres 0.3 cells apart, the first also 0.3 cells from a plane wall:
+    lattice lines pass from one solid into the next without a fluid node, so
+    the rest density's part of force and torque does not cancel.  Forces,
+    torques, stresslets and states against the oracle over six steps."""
+    shape, R = (32, 30, 44), 4.3
+    g, o = make_pair(shape, "trt", 1.0)
+    at = np.array([14.3, 13.8, 5.4 + R + 0.3])
+    to = np.array([0.3, -0.2, 1.0])
+    beside = at + to / np.linalg.norm(to) * (2 * R + 0.3)
+    if wall:
+        g.add_plane_wall(2, 5)
+        o.add_plane_wall(2, 5)
+    put = [(at, (0.2, 0.1, 1.0), False), (beside, (0.0, 0.3, 1.0), True)]
+    gids = [g.add_squirmer(p, e, R, 0.02, -2.0, mobile=m) for p, e, m in put]
+    oids = [o.add_sphere(p, e, R, 0.02, -2.0, mobile=m) for p, e, m in put]
+    c = np.array([[0, 1, -1, 0, 0, 0, 0, 1, -1, 1, -1, 1, -1, 1, -1, 0, 0, 0, 0],
+                  [0, 0, 0, 1, -1, 0, 0, 1, -1, -1, 1, 0, 0, 0, 0, 1, -1, 1, -1],
+                  [0, 0, 0, 0, 0, 1, -1, 0, 0, 0, 0, 1, -1, -1, 1, 1, -1, -1, 1]]).T
+    for a in gids:  # 36 sum w c over the links: the rest part does not cancel
+        i = g.links(a).astype(np.int64) % 32
+        assert (np.where(i < 7, 2, 1)[:, None] * c[i]).sum(0).any()
+    for _ in range(6):
+        g.step(1)
+        o.step(1)
+        for a, b in zip(gids, oids):
+            for x, y in zip((*g.force_torque(a), g.stresslet(a), *g.state(a)),
+                            (*o.force_torque(b), o.stresslet(b), *o.state(b))):
+                assert np.abs(x - y).max() < 1e-11

@@ -168,3 +168,23 @@ def test_ragged_request_against_a_lattice(storage, shape):
         pos, vel, e, omega = g.state(k)
     for got, want in ((r.pos, pos), (r.e, e), (r.vel, vel), (r.omega, omega)):
         assert np.abs(np.array(got) - want).max() < 1e-9 * max(1e-3, np.abs(want).max())
+
+
+def test_request_touching_its_obstacle_f64():
+    """A squirmer 0.3 cells from its obstacle, whose force and torque keep a part
+    of the rest density, in FP64: the server's link kernel against the fused
+    kernel of a lattice of its own."""
+    shape, R, centre = (34, 32, 40), 4.3, np.array([16.2, 15.7, 12.1])
+    to = np.array([0.3, -0.2, 1.0])
+    pos = centre + to / np.linalg.norm(to) * (2 * R + 0.3)
+    for steps in (1, 6):
+        req = make_request(2, shape, "f64", pos=tuple(pos), e=(0.0, 0.3, 1.0), R=R, B1=0.02, beta=-2.0,
+                           obstacle=(*centre, R), steps=steps)
+        res = run_server([req], [0], round_steps=2)[0]
+        with Lattice(shape, collision="trt", storage="f64") as g:
+            g.add_obstacle(tuple(centre), R)
+            k = g.add_squirmer(tuple(pos), (0.0, 0.3, 1.0), R, 0.02, -2.0, True)
+            g.step(steps)
+            want = [*g.state(k), *g.force_torque(k)]
+        for x, y in zip((res.pos, res.vel, res.e, res.omega, res.F, res.T), want):
+            assert np.abs(np.array(x) - y).max() < 1e-11
