@@ -854,3 +854,106 @@ def test_forces_of_touching_solids_f64(wall):
             for x, y in zip((*g.force_torque(a), g.stresslet(a), *g.state(a)),
                             (*o.force_torque(b), o.stresslet(b), *o.state(b))):
                 assert np.abs(x - y).max() < 1e-11
+
+
+def _split_against_traced(shape, storage, body, steps=(3, 40)):
+    """A run with split steps and the same run traced, which never splits: the
+    populations, owners and state of both, and that the first did split (a lone
+    sphere: body kernel, far and near sweep, three launches a step but for the
+    first sweep and the body step left pending; whole steps launch two)."""
+    runs = []
+    for traced in (False, True):
+        g = Lattice(shape, collision="trt", storage=storage)
+        gi = g.add_squirmer(*body, mobile=True)
+        before = g.launches
+        if traced:
+            g.profile_begin()
+        for n in steps:
+            g.step(n)
+        if traced:
+            g.profile_end()
+        else:
+            assert g.launches - before > 2.5 * sum(steps)
+        runs.append((g.populations(), g.owner(), *g.state(gi)))
+        g.close()
+    return runs
+
+
+@pytest.mark.parametrize("storage", ["f16dev", "bf16dev"])
+@pytest.mark.parametrize("shape", [(16, 152, 150), (36, 100, 100), (45, 90, 90), (50, 84, 86), (772, 32, 32)])
+def test_split_steps_of_large_lattices_bitwise_16bit(storage, shape):
+    """test_split_odd_steps_narrow_rows_bitwise on lattices large enough to be
+    split: rows of 4 and 9 four-cell groups with the swimmer across the x faces,
+    and rows that no whole-row block fits (45, 50 and 772 cells), whose even steps
+    take four consecutive cells per thread, those at the window's border one by
+    one.  The swimmer also sits across the y and z faces, so the window wraps."""
+    body = ((0.6, 1.3, shape[2] - 1.8), (0.6, 0.2, 1.0), 3.0, 0.05, -2.0)
+    for a, b in zip(*_split_against_traced(shape, storage, body)):
+        assert np.array_equal(a, b)
+
+
+def test_split_steps_of_odd_rows_bitwise_f32():
+    """Odd rows in FP32, more than 128 MB of populations: the far sweep's even
+    steps take two consecutive cells per thread across rows."""
+    shape = (121, 122, 123)
+    body = ((0.6, 1.3, 121.2), (0.6, 0.2, 1.0), 6.0, 0.05, -2.0)
+    for a, b in zip(*_split_against_traced(shape, "f32", body, (3, 20))):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("shape,lambda_e", [((1, 1, 1), 1.0), ((3, 1, 1), 1.0), ((33, 13, 11), 1.0),
+                                            ((45, 6, 10), 1.3), ((257, 3, 5), 1.0)])
+def test_flat_even_steps_bitwise_f32(shape, lambda_e):
+    """Even steps of odd rows in FP32, two consecutive cells per thread across
+    rows, against the one-cell form: the same bits, on cell counts with and
+    without one left over."""
+    w = np.array([1 / 3] + [1 / 18] * 6 + [1 / 36] * 12)
+    f = W.random_populations(int(np.prod(shape)), seed=12, base=w, spread=0.2)
+    out = []
+    for variant in (0, 1):
+        with Lattice(shape, collision="trt", lambda_e=lambda_e, storage="f32") as g:
+            g.set_sweep_variant(variant)
+            g.set_populations(f)
+            g.step(7)
+            out.append(g.populations())
+    assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16dev"])
+def test_many_spheres_reduced_storage(storage):
+    """160 mobile squirmers in reduced storage against the FP64 oracle: the body
+    kernel's form for many spheres (clusters of four blocks in two waves, three
+    blocks per SM), some with boxes that meet.  FP32: owners equal; the field's
+    rms error within sqrt(40) 2^-24 of max|u| (40 steps, each rounding a
+    population once), velocities within 2e-6 of the largest, the bound of
+    test_reduced_storage_free_swimmer.  FP16: positions err by some 1e-5, so a
+    node may change hands a step early or late; at most one solid cell in a
+    thousand, the field's rms error within that test's 2e-3 of max|u|, and
+    velocities within 2 % (one of a sphere's 74 cells converted a step late
+    carries 1/74 of its momentum)."""
+    rng = np.random.default_rng(160)
+    bodies = _random_spheres(rng, (96, 80, 72), 160, 2.6, 7.7)
+    g = Lattice((96, 80, 72), collision="trt", storage=storage)
+    o = OracleSim(96, 80, 72, lambda_e=1.0, collision="trt")
+    gids = [g.add_squirmer(*b, mobile=True) for b in bodies]
+    oids = [o.add_sphere(*b, mobile=True) for b in bodies]
+    start = o.owner()
+    g.step(40)
+    o.step(40)
+    own, want = g.owner(), o.owner()
+    assert (want != start).sum() > 100  # cells were converted
+    _, ug = g.fields()
+    _, uo = o.fields()
+    vg = np.array([g.state(i)[1] for i in gids])
+    vo = np.array([o.state(i)[1] for i in oids])
+    scale, vmax = np.abs(uo).max(), np.abs(vo).max()
+    if storage == "f32":
+        assert (own == want).all()
+        assert np.sqrt(np.mean((ug - uo) ** 2)) < np.sqrt(40.0) * 2.0 ** -24 * scale
+        assert np.abs(vg - vo).max() < 2e-6 * vmax
+    else:
+        assert (own != want).sum() <= 1e-3 * (want != 0).sum()
+        both = (own == 0) & (want == 0)
+        assert np.sqrt(np.mean((ug - uo)[:, both] ** 2)) < 2e-3 * scale
+        assert np.abs(vg - vo).max() < 2e-2 * vmax
+    g.close()
