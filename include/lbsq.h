@@ -405,7 +405,8 @@ typedef struct {
                                 owners, boundary links); allocated at creation */
     int32_t max_resident;    /* lattice slots, 1..256 */
     int32_t round_steps;     /* steps per scheduling round (even, >= 2) */
-    int32_t tile_units;      /* cell pairs per sweep tile; 0 = pick by timing at creation */
+    int32_t tile_units;      /* cell pairs per sweep tile; 0 = pick by timing at creation (smaller
+                                ones, down to 128, for sweeps of few cells) */
     const lb_allocator* allocator; /* NULL = cudaMalloc / cudaFree */
 } lb_server_params;
 
@@ -455,7 +456,7 @@ lb_status lb_server_advance(lb_server* s, int32_t* running, int32_t* queued);
 /* State and (when done) results of a request; a done request is forgotten
  * after it has been polled once.  LB_ERR_INVALID for an unknown ticket. */
 lb_status lb_server_poll(lb_server* s, int64_t ticket, lb_result* out);
-/* Sweep tile size in use (picked by timing when tile_units = 0), persistent
+/* Largest sweep tile size in use (picked by timing when tile_units = 0), persistent
  * blocks per SM, device memory in use and total cell updates done. */
 lb_status lb_server_info(const lb_server* s, int32_t* tile_units, int32_t* blocks_per_sm, size_t* bytes_used,
                          double* cell_updates);

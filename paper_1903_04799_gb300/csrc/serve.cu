@@ -662,6 +662,21 @@ lb_status fill_result(lb_server* s, int l, lb_result* out) {
 // Cells of a sweep tile of `units` cell pairs: a multiple of 4 (see sweep_tile).
 int64_t tile_cells(int units) { return (2 * (int64_t)units + 3) / 4 * 4; }
 
+// Cell pairs per tile for a tile kernel with `cells` cells in all.  A tile is one
+// block's work, so a kernel of few cells needs small tiles to occupy the GPU:
+// the largest power of two with 256 tiles or more, from 128 up to the tuned
+// size.  us per step, tuned size (1024 or 2048) / by this rule, one request: FP64
+// 32^3 86 / 56, 64^3 92 / 69, FP32 32^3 52 / 47, 96^3 65 / 63; three of 33^3
+// FP32, 40^3 FP16, 48^3 FP64 111 / 76.  (Larger tiles, fixed: 64^3 FP64 at 128
+// pairs 72, 256 70, 512 71, 1024 81; 128^3 FP32 at 256 110, 512 104, 2048 101.)
+// A size given by the caller (lb_server_params) stays.
+int group_tile_units(const lb_server* s, int64_t cells) {
+    if (s->p.tile_units > 0) return s->tile_units;
+    int u = 128;
+    while (2 * u <= s->tile_units && 4 * u <= cells / 256) u *= 2;
+    return u;
+}
+
 // Upload the static work of the resident mix: each group's link items and
 // sweep tiles.
 lb_status upload_mix(lb_server* s) {
@@ -679,10 +694,13 @@ lb_status upload_mix(lb_server* s) {
     for (int g = 0; g < kGroups; ++g) {
         for (int st = 0; st < 4; ++st) {  // a group's tiles sorted by storage
             bounds[5 * g + st] = (int)tiles.size();
+            int64_t total = 0;
+            for (const Slot& sl : s->slots)
+                if (sl.used && sl.group == g && sl.L.storage == st) total += sl.L.N;
+            const int64_t cells = tile_cells(group_tile_units(s, total));
             for (int l = 0; l < s->cap_slots; ++l) {
                 const Slot& sl = s->slots[l];
                 if (!sl.used || sl.group != g || sl.L.storage != st) continue;
-                const int64_t cells = tile_cells(s->tile_units);
                 for (int64_t n0 = 0; n0 < sl.L.N; n0 += cells)
                     tiles.push_back(make_int4(l, (int)n0, (int)std::min(sl.L.N, n0 + cells), sl.L.nx % 2 == 0));
             }

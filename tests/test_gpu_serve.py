@@ -188,3 +188,23 @@ def test_request_touching_its_obstacle_f64():
             want = [*g.state(k), *g.force_torque(k)]
         for x, y in zip((res.pos, res.vel, res.e, res.omega, res.F, res.T), want):
             assert np.abs(np.array(x) - y).max() < 1e-11
+
+
+def test_small_groups_tiles_give_the_same_bits():
+    """Without a given tile size, sweeps of few cells take smaller tiles (cells /
+    512 pairs, a power of two from 128): groups at the smallest tile, between two
+    sizes and with several storages, with cell counts that end inside a tile,
+    against fixed tiles that hold whole lattices."""
+    reqs = [make_request(0, (21, 19, 23), "f64", pos=(10.2, 9.7, 11.1), e=(0.3, -0.4, 1.0), R=3.5, B1=0.03,
+                         beta=-2.0, steps=40),
+            make_request(0, (53, 47, 51), "f32", pos=(26.2, 22.7, 25.1), e=(0.3, -0.4, 1.0), R=4.5, B1=0.03,
+                         beta=-2.0, steps=33),
+            make_request(0, (64, 63, 66), "f16dev", pos=(30.2, 32.7, 31.1), e=(0.3, 0.4, 1.0), R=4.5, B1=0.03,
+                         beta=2.0, steps=40),
+            make_request(0, (33, 35, 37), "bf16dev", pos=(16.2, 17.7, 18.1), e=(0.3, 0.4, -1.0), R=4.5, B1=0.03,
+                         beta=2.0, steps=40)]
+    small = run_server(reqs, [0, 0, 1, 2], budget=128 << 20, tile_units=0)
+    fixed = run_server(reqs, [0, 0, 1, 2], budget=128 << 20, tile_units=1 << 18)
+    for i in range(len(reqs)):
+        assert small[i].state == lbsq.LB_REQ_DONE
+        assert np.array_equal(as_array(small[i]), as_array(fixed[i])), i
