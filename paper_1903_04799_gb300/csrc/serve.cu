@@ -289,7 +289,9 @@ struct lb_server {
     int64_t gstep = 0;
     double cell_updates = 0.0;
     int tile_units = 2048, blocks_per_sm = 2;
-    cudaGraphExec_t graph = nullptr;
+    // a round's graph by the set of groups that hold requests (bit per group): a
+    // chain without requests launches nothing
+    cudaGraphExec_t graph[1 << kGroups] = {};
     unsigned storages = 0;  // storages a request has had so far (bit lb_storage): the tile kernels of a step
     cudaStream_t chain = nullptr;  // the second group's chain
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -490,6 +492,13 @@ lb_status validate(const lb_request& r) {
     return LB_OK;
 }
 
+void drop_graphs(lb_server* s) {
+    for (cudaGraphExec_t& g : s->graph) {
+        if (g) cudaGraphExecDestroy(g);
+        g = nullptr;
+    }
+}
+
 // Set up a request in slot l: memory, populations at rest, walls, spheres
 // (classification with the same kernels as a step), links, committed owners.
 lb_status admit(lb_server* s, int l, const Queued& q) {
@@ -610,8 +619,7 @@ lb_status admit(lb_server* s, int l, const Queued& q) {
     sl.group = group;
     if (!(s->storages >> r.storage & 1u)) {  // a step gets another tile kernel
         s->storages |= 1u << r.storage;
-        if (s->graph) cudaGraphExecDestroy(s->graph);
-        s->graph = nullptr;
+        drop_graphs(s);
     }
     sl.squirmer = L.body_begin + (int)bodies.size() - 1;
     sl.start = s->gstep;
@@ -724,14 +732,18 @@ lb_status upload_mix(lb_server* s) {
     return LB_OK;
 }
 
-// A round: each group's steps on a chain of its own.
-void enqueue_round(lb_server* s) {
+// A round of the groups in `mask`: each one's steps on a chain of its own.
+void enqueue_round(lb_server* s, unsigned mask) {
     const int grid = s->blocks_per_sm * s->n_sm;
     const int glinks = 8 * s->n_sm, gbox = 4 * s->n_sm;  // latency-bound: many blocks
-    cudaEventRecord(s->ev_fork, s->stream);
-    cudaStreamWaitEvent(s->chain, s->ev_fork, 0);
+    const bool fork = (mask & (mask - 1)) != 0;
+    if (fork) {
+        cudaEventRecord(s->ev_fork, s->stream);
+        cudaStreamWaitEvent(s->chain, s->ev_fork, 0);
+    }
     for (int g = 0; g < kGroups; ++g) {
-        const cudaStream_t st = g == 0 ? s->stream : s->chain;
+        if (!(mask >> g & 1u)) continue;
+        const cudaStream_t st = fork && g > 0 ? s->chain : s->stream;
         const Bodies B = bodies_view(s, g, true);
         const TileArgs T = tile_args(s, g);
         for (int k = 0; k < s->p.round_steps; ++k) {
@@ -740,20 +752,22 @@ void enqueue_round(lb_server* s) {
             for (int w = 1; w <= 4; ++w) launch_body_kernel(w, B, P, glinks, gbox, nullptr, st, true);
         }
     }
-    cudaEventRecord(s->ev_join, s->chain);
-    cudaStreamWaitEvent(s->stream, s->ev_join, 0);
+    if (fork) {
+        cudaEventRecord(s->ev_join, s->chain);
+        cudaStreamWaitEvent(s->stream, s->ev_join, 0);
+    }
 }
 
-lb_status build_graph(lb_server* s) {
+lb_status build_graph(lb_server* s, unsigned mask) {
     cudaGraph_t g = nullptr;
     SCK(cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal));
-    enqueue_round(s);
+    enqueue_round(s, mask);
     cudaError_t e = cudaStreamEndCapture(s->stream, &g);
     if (e != cudaSuccess) return sfail(s, LB_ERR_CUDA, std::string("capture: ") + cudaGetErrorString(e));
-    e = cudaGraphInstantiate(&s->graph, g, 0);
+    e = cudaGraphInstantiate(&s->graph[mask], g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) {
-        s->graph = nullptr;
+        s->graph[mask] = nullptr;
         return sfail(s, LB_ERR_CUDA, std::string("instantiate: ") + cudaGetErrorString(e));
     }
     return LB_OK;
@@ -904,7 +918,7 @@ lb_status lb_server_create(const lb_server_params* p, lb_server** out) {
 lb_status lb_server_destroy(lb_server* s) {
     if (!s) return LB_OK;
     if (s->stream) cudaStreamSynchronize(s->stream);
-    if (s->graph) cudaGraphExecDestroy(s->graph);
+    drop_graphs(s);
     if (s->ev_fork) cudaEventDestroy(s->ev_fork);
     if (s->ev_join) cudaEventDestroy(s->ev_join);
     if (s->chain) cudaStreamDestroy(s->chain);
@@ -980,16 +994,21 @@ lb_status lb_server_advance(lb_server* s, int32_t* running, int32_t* queued) {
     }
     // 3. one round for every resident request
     int n_run = 0;
-    for (auto& sl : s->slots) n_run += sl.used ? 1 : 0;
+    unsigned mask = 0;  // groups that hold requests
+    for (auto& sl : s->slots)
+        if (sl.used) {
+            ++n_run;
+            mask |= 1u << sl.group;
+        }
     if (n_run > 0) {
-        if (!s->graph) {
-            lb_status st = build_graph(s);
+        if (!s->graph[mask]) {
+            lb_status st = build_graph(s, mask);
             if (st != LB_OK) return st;
         }
         long long gs[kGroups];
         std::fill(gs, gs + kGroups, (long long)s->gstep);
         SCK(cudaMemcpyAsync(s->d_gstep, gs, sizeof(gs), cudaMemcpyHostToDevice, s->stream));
-        SCK(cudaGraphLaunch(s->graph, s->stream));
+        SCK(cudaGraphLaunch(s->graph[mask], s->stream));
         for (auto& sl : s->slots)
             if (sl.used) {
                 const int64_t a = std::max(s->gstep, sl.start), b = std::min(s->gstep + s->p.round_steps, sl.stop);
