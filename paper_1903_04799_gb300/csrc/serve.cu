@@ -774,11 +774,13 @@ lb_status build_graph(lb_server* s, unsigned mask) {
 }
 
 // Tile-shape autotuner: time the tile sweep on two synthetic lattices (128^3
-// FP32 and FP16: as many tiles as a group of requests has; on 96^3 the smallest
-// tiles won by their even tail, and served 24 requests 6 % slower) for each
-// candidate (cell pairs per tile, blocks per SM) and keep the fastest.  Uses arena memory that is free at creation.
+// FP32 and FP16: as many tiles as a group of requests has; 96^3 where the budget
+// does not hold those) for each candidate (cell pairs per tile, blocks per SM)
+// and keep the fastest.  What it finds holds for groups of many cells
+// (group_tile_units).  Uses arena memory that is free at creation.
 lb_status autotune(lb_server* s) {
-    const int n = 128;
+    const size_t N128 = (size_t)128 * 128 * 128;
+    const int n = s->arena.fits({19 * N128 * 4, 19 * N128 * 2}) ? 128 : 96;
     Lattice Ls[2];
     std::vector<std::pair<size_t, size_t>> blocks;
     const int storages[2] = {LB_F32, LB_F16DEV};
