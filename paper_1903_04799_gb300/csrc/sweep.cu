@@ -27,7 +27,7 @@ __global__ void __launch_bounds__(256) k_sweep(const SweepArgs a) {
         });
     } else {
         int y, z;
-        if (!sweep_at(a, blockIdx.y, y, z) || x >= a.nx) return;
+        if (!sweep_at(a, blockIdx.y * blockDim.y + threadIdx.y, y, z) || x >= a.nx) return;
         sweep_one<S, P, NATIVE>(a, x, y, z, skey);
     }
 }
@@ -260,6 +260,17 @@ static void launch_df(const SweepArgs& a, int parity, const Rows& r, cudaStream_
 // k_sweep_flat.  Whole-lattice steps (both parities) against the one- and
 // two-cell forms: 250^3 FP16 241 -> 207 us, BF16 252 -> 217; 251^3 FP16 259 ->
 // 217, BF16 375 -> 278; without the prefetch 250^3 FP16 215, BF16 227.
+//
+// Small lattices keep those forms, whose more numerous threads hide more
+// latency; what counts is their threads, the cells with rows padded to whole
+// warps.  One-cell / flat, whole-lattice steps: FP16 33^3 2.6 / 3.1 us, 45^3 3.4
+// / 4.0, 59^3 4.4 / 4.9, 61^3 4.9 / 4.9, 65^3 6.2 / 5.4, 5 x 100 x 100 4.8 / 4.1;
+// BF16 51^3 4.4 / 5.1, 65^3 8.2 / 6.7; FP32 33^3 2.6 / 3.0, 45^3 3.6 / 3.6, 51^3
+// 4.1 / 3.9, 65^3 7.0 / 6.7, 7 x 50 x 60 2.3 / 2.7.
+static bool flat_pays(const SweepArgs& a, int storage) {
+    const int64_t threads = (int64_t)(a.nx + 31) / 32 * 32 * a.ny * a.nz;
+    return threads >= (storage == ST_F32 ? 130000 : 240000);
+}
 template <int S>
 static void launch_flat(const SweepArgs& a, cudaStream_t st, bool dep) {
     const uint32_t N = (uint32_t)a.nx * a.ny * a.nz, cells = (S == ST_F32 ? 2 : 4) * 256;
@@ -302,7 +313,7 @@ static void launch_s(SweepArgs a, int parity, int variant, int gz, int gy, cudaS
         // 251^3 FP16 259 -> 217, BF16 375 -> 278.  Where whole rows fit, the two
         // are equal in bare sweeps (256^3: 204 us) and the rows faster in split
         // ones (256^3 pusher FP16 222 against 226 us: no divisions for the window)
-        if (variant == 0 && parity == 0 && a.zmode != 2 && !rows4) {
+        if (variant == 0 && parity == 0 && a.zmode != 2 && !rows4 && flat_pays(a, S)) {
             launch_flat<S>(a, st, dep);
             return;
         }
@@ -346,13 +357,19 @@ static void launch_s(SweepArgs a, int parity, int variant, int gz, int gy, cudaS
         // steps: 251^3 382 -> 361 us, 125 x 99 x 111 25.6 -> 25.1).  Odd steps keep
         // one cell: pairs across odd rows, every access scalar and every second
         // element left to another instruction, took 408 us.  In split steps of
-        // small lattices the window's divisions cost what the pairs gain.
-        if (S == ST_F32 && variant == 0 && parity == 0 &&
+        // lattices that fit L2 the window's divisions cost what the pairs gain
+        // (one squirmer, one cell / flat: 99^3 25.5 / 25.3, 111 x 111 x 112, 105 MB,
+        // 31.8 / 31.3, 121 x 121 x 122, 136 MB, 40.1 / 39.3, 131^3 57.6 / 53.4, 161^3
+        // 105 / 97, 201^3 214 / 195).
+        if (S == ST_F32 && variant == 0 && parity == 0 && flat_pays(a, S) &&
             (a.zmode == 0 || (a.zmode == 1 && 19 * a.Np * 4 > (128 << 20)))) {
             launch_flat<S>(a, st, dep);
             return;
         }
-        const Rows r = rows(1, 256, 1, 4);
+        // Blocks of 128 threads: one row of few cells per block left the GPU
+        // starting blocks (one about every nanosecond: 7 x 200 x 300, 60 000 rows,
+        // FP32 35 -> 14 us per step, FP16 34 -> 14; 5 x 100 x 100 6.9 -> 4.1).
+        const Rows r = rows(1, 256, 128, 4);
         // (no L2 prefetch: 125 x 99 x 111 FP16 16.9 us per step without, 19.1 with)
         if (parity == 0) launch_rows(k_sweep<S, 0, false, false>, k_sweep<S, 0, false, true>, a, r, 0, st, dep);
         else launch_rows(k_sweep<S, 1, false, false>, k_sweep<S, 1, false, true>, a, r, 0, st, dep);
@@ -361,7 +378,7 @@ static void launch_s(SweepArgs a, int parity, int variant, int gz, int gy, cudaS
 
 // variant: 0 = default (FP64: double-float collision, one cell per thread;
 // FP32: two cells per thread (even nx); FP16 / BF16: even steps as 3 or
-// k_sweep4f, odd steps as 2, or four cells per thread without shared memory in split
+// k_sweep_flat, odd steps as 2, or four cells per thread without shared memory in split
 // sweeps), 1 = one cell per thread (FP64: FP64 arithmetic), 2 = two
 // cells per thread where possible (not FP64), 3 = FP16 / BF16: four cells per
 // thread in blocks of whole rows on both parities, odd-step x-shifts through

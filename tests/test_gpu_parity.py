@@ -901,22 +901,47 @@ def test_split_steps_of_odd_rows_bitwise_f32():
         assert np.array_equal(a, b)
 
 
-@pytest.mark.parametrize("shape,lambda_e", [((1, 1, 1), 1.0), ((3, 1, 1), 1.0), ((33, 13, 11), 1.0),
-                                            ((45, 6, 10), 1.3), ((257, 3, 5), 1.0)])
-def test_flat_even_steps_bitwise_f32(shape, lambda_e):
-    """Even steps of odd rows in FP32, two consecutive cells per thread across
-    rows, against the one-cell form: the same bits, on cell counts with and
-    without one left over."""
+@pytest.mark.parametrize("storage,shape,lambda_e", [
+    ("f32", (45, 49, 51), 1.0), ("f32", (257, 23, 29), 1.3), ("f32", (3, 73, 75), 1.0), ("f32", (1, 65, 63), 1.0),
+    ("f16dev", (65, 63, 61), 1.0), ("f16dev", (50, 71, 73), 1.3), ("f16dev", (773, 17, 19), 1.0),
+    ("f16dev", (3, 83, 95), 1.0), ("bf16dev", (65, 63, 61), 1.0), ("bf16dev", (50, 71, 73), 1.3),
+    ("bf16dev", (773, 17, 19), 1.0), ("bf16dev", (1, 91, 93), 1.0)])
+def test_flat_even_steps_of_large_lattices_bitwise(storage, shape, lambda_e):
+    """Even steps over consecutive cells, two per thread in FP32 and four in 16
+    bits, on lattices large enough to take them (rows padded to whole warps:
+    130 000 cells in FP32, 240 000 in 16 bits), against the one-cell form: the
+    same bits, on cell counts that leave 1, 2 and 3 cells over."""
+    cells = int(np.prod(shape))
+    assert -(-shape[0] // 32) * 32 * shape[1] * shape[2] >= (130000 if storage == "f32" else 240000)
     w = np.array([1 / 3] + [1 / 18] * 6 + [1 / 36] * 12)
-    f = W.random_populations(int(np.prod(shape)), seed=12, base=w, spread=0.2)
+    f = W.random_populations(cells, seed=12, base=w, spread=0.2)
     out = []
     for variant in (0, 1):
-        with Lattice(shape, collision="trt", lambda_e=lambda_e, storage="f32") as g:
+        with Lattice(shape, collision="trt", lambda_e=lambda_e, storage=storage) as g:
             g.set_sweep_variant(variant)
             g.set_populations(f)
             g.step(7)
             out.append(g.populations())
     assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("storage,tol", [("f32", 1e-6), ("f16dev", 4e-3), ("bf16dev", 3e-2)])
+@pytest.mark.parametrize("shape", [(7, 13, 9), (1, 6, 5), (33, 5, 3), (31, 9, 4), (65, 3, 7), (97, 5, 3)])
+def test_rows_that_share_a_block(storage, tol, shape):
+    """The one-cell form takes as many rows per block as 128 threads hold, the
+    last block with rows to spare: against FP64 storage, both parities.  Four
+    steps, each rounding a deviation to 2^-24, 2^-11 (FP16) or 2^-8 (BF16) of
+    itself: twice that per step, of the largest deviation."""
+    w = np.array([1 / 3] + [1 / 18] * 6 + [1 / 36] * 12)
+    f = W.random_populations(int(np.prod(shape)), seed=5, base=w, spread=0.1)
+    out = []
+    for s in ("f64", storage):
+        with Lattice(shape, collision="trt", storage=s) as g:
+            g.set_sweep_variant(1 if s != "f64" else 0)
+            g.set_populations(f)
+            g.step(4)
+            out.append(g.populations())
+    assert np.abs(out[0] - out[1]).max() < tol * np.abs(f - w[:, None]).max()
 
 
 @pytest.mark.parametrize("storage", ["f32", "f16dev"])
