@@ -1154,6 +1154,22 @@ static cudaEvent_t pool_event(lb_ctx* c, size_t k) {
     return c->ev_pool[k];
 }
 
+// Whether the FP64 sweeps of a lattice without bodies may follow each other as
+// dependent launches.  These sweeps are bound by instruction issue, and a grid
+// that fills about half to 0.8 of the block slots leaves the next one's blocks
+// crowded on the SMs with room to spare (smaller grids fit beside each other,
+// larger ones come in waves).  us per step, dependent / ordinary: 100 x 20 x 25
+// (0.55 of the slots) 6.9 / 5.9, 33^3 (0.60) 6.9 / 5.9, 36^3 (0.71) 7.2 / 6.9, 7 x
+// 50 x 60 (0.79) 7.2 / 6.9; 20 x 30 x 60 (0.47) 4.9 / 5.4, 39^3 (0.83) 7.4 / 7.5,
+// 64^3 (2.2) 14.9 / 15.2.
+static bool sweeps_overlap(const lb_ctx* c) {
+    if (c->p.storage != LB_F64 || c->lambda_e != 1.0 || c->sweep_variant == 1) return true;
+    const int64_t bx = std::min(256, (c->L.nx + 31) / 32 * 32);
+    const int64_t slots = std::min<int64_t>(32, 65536 / (80 * bx)) * c->n_sm;  // 80 registers a thread
+    const int64_t blocks = (c->L.nx + bx - 1) / bx * c->L.ny * c->L.nz;
+    return blocks * 100 < 48 * slots || blocks * 5 > 4 * slots;
+}
+
 // dep: the last operation on st is a kernel (see dep_wait).
 static void sweep_all(lb_ctx* c, int parity, cudaStream_t st, bool dep = false) {
     launch_sweep(c->L, c->lambda_e, c->lambda_o, parity, c->sweep_variant, 0, nullptr, c->L.nz, c->L.ny, st, dep);
@@ -1287,7 +1303,7 @@ static void enqueue_steps(lb_ctx* c, int64_t n) {
         if (c->psm) {
             c->launches += psm_step(c, B, parity, c->stream, k > 0);
         } else {
-            sweep_all(c, parity, c->stream, k > 0);
+            sweep_all(c, parity, c->stream, k > 0 && (bodies || sweeps_overlap(c)));
             c->launches += 1;
             if (bodies) c->launches += body_step(c, B, parity, c->stream, true);
         }
