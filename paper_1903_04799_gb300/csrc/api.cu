@@ -328,7 +328,8 @@ lb_status read_checked(lb_ctx* c, const void* src, size_t bytes, void* dst) {
 // (335 MB: 12 ms against 1.8 ms into pages that exist), so a few threads touch
 // the pages, block by block ahead of the copies.  A page is touched at its
 // first byte, by the thread of the block that holds this byte and before this
-// block is copied.  Call it when nothing but the copy itself can fail any more.
+// block is copied.  Call it when nothing but the copy itself can still fail (a
+// device error found after it leaves the buffer filled all the same).
 cudaError_t copy_out(lb_ctx* c, void* dst, const void* src, size_t bytes) {
     constexpr size_t kBlock = 4 << 20;
     const size_t page = (size_t)sysconf(_SC_PAGESIZE);
@@ -1138,11 +1139,8 @@ lb_status lb_get_populations(lb_ctx* c, double* f) {
     launch_get_pop(c->L, c->d_pop, (int)(c->step & 1), c->stream);
     c->launches += 1;
     CK(cudaGetLastError());
-    s = sync_checked(c);
-    if (s != LB_OK) return s;
     CK(copy_out(c, f, c->d_pop, Q * N * sizeof(double)));
-    CK(cudaStreamSynchronize(c->stream));
-    return LB_OK;
+    return sync_checked(c);
 }
 
 static cudaEvent_t pool_event(lb_ctx* c, size_t k) {
