@@ -65,14 +65,17 @@ __global__ void k_get_pop(const Lattice L, double* f, int q) {
 
 // ---- density and momentum of a cell
 //
-// rho = rho0 + sum g_i and j = sum g_i c_i of the stored deviations, summed
-// exactly in 64-bit fixed point (unit 2^(k0 - 60), k0 the exponent of rho0).
+// rho = rho0 + sum g_i and j = sum g_i c_i of the stored deviations, summed in
+// 64-bit fixed point (unit 2^(k0 - 60), k0 the exponent of rho0).  The integer
+// sums are exact; what rounds is the conversion, which cuts a deviation off at
+// the unit, 2^-60 rho0 or less (to_fx: FP64 below 2^-8 rho0, FP32 below 2^-37;
+// 19 terms err by less than an ulp of rho, where FP64 sums erred by several).
 // What bounds a read-out kernel is this GPU's FP64 rate, not memory: one FP64
 // warp instruction takes the SM's pipe 16 cycles, the issue slots of 64
 // others, and the sums in FP64 took about 100 per cell (256^3: 4.7 ms on even
 // steps, 7.2 ms on odd ones, 3 % of the DRAM bandwidth).  A deviation becomes
 // a fixed-point number in about 10 integer instructions, a 64-bit add takes
-// two, and no sum rounds.  256^3 after: FP64 0.50 / 0.58 ms (even / odd steps,
+// two.  256^3 after: FP64 0.50 / 0.58 ms (even / odd steps,
 // 0.46 ms at the copy rate), FP32 and 16 bits 0.43 ms.
 // Cells with a deviation outside 0.15 rho0 (NaN and Inf included) or a
 // density that is not positive take the FP64 sums of moments_general.

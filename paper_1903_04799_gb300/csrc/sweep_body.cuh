@@ -449,25 +449,18 @@ __device__ __noinline__ void sweep_one_call(const SweepArgs& a, int x, int y, in
 
 // Two-cell pair types: the stored element type T and its 2-vector.
 template <class T> struct Pair;
-template <> struct Pair<double> { using V = double2; __device__ static double lo(V v) { return v.x; } __device__ static double hi(V v) { return v.y; } __device__ static V make(double a, double b) { return make_double2(a, b); } };
-template <> struct Pair<float> { using V = float2; __device__ static float lo(V v) { return v.x; } __device__ static float hi(V v) { return v.y; } __device__ static V make(float a, float b) { return make_float2(a, b); } };
-template <> struct Pair<__half> { using V = __half2; __device__ static __half lo(V v) { return __low2half(v); } __device__ static __half hi(V v) { return __high2half(v); } __device__ static V make(__half a, __half b) { return __halves2half2(a, b); } };
-template <> struct Pair<__nv_bfloat16> { using V = __nv_bfloat162; __device__ static __nv_bfloat16 lo(V v) { return __low2bfloat16(v); } __device__ static __nv_bfloat16 hi(V v) { return __high2bfloat16(v); } __device__ static V make(__nv_bfloat16 a, __nv_bfloat16 b) { return __halves2bfloat162(a, b); } };
+template <> struct Pair<float> { using V = float2; __device__ static float lo(V v) { return v.x; } __device__ static float hi(V v) { return v.y; } };
+template <> struct Pair<__half> { using V = __half2; __device__ static __half lo(V v) { return __low2half(v); } __device__ static __half hi(V v) { return __high2half(v); } };
+template <> struct Pair<__nv_bfloat16> { using V = __nv_bfloat162; __device__ static __nv_bfloat16 lo(V v) { return __low2bfloat16(v); } __device__ static __nv_bfloat16 hi(V v) { return __high2bfloat16(v); } };
 
-// Decode / encode one stored element (same arithmetic as StoreT::load / store).
+// Decode one stored element (same arithmetic as StoreT::load).
 template <int S> __device__ __forceinline__ typename StoreT<S>::R dec(typename StoreT<S>::T v, float isc);
-template <> __device__ __forceinline__ double dec<ST_F64>(double v, float) { return v; }
 template <> __device__ __forceinline__ float dec<ST_F32>(float v, float) { return v; }
 template <> __device__ __forceinline__ float dec<ST_F16>(__half v, float isc) { return __half2float(v) * isc; }
 template <> __device__ __forceinline__ float dec<ST_BF16>(__nv_bfloat16 v, float isc) { return __bfloat162float(v) * isc; }
-template <int S> __device__ __forceinline__ typename StoreT<S>::T enc(typename StoreT<S>::R v, float sc);
-template <> __device__ __forceinline__ double enc<ST_F64>(double v, float) { return v; }
-template <> __device__ __forceinline__ float enc<ST_F32>(float v, float) { return v; }
-template <> __device__ __forceinline__ __half enc<ST_F16>(float v, float sc) { return __float2half_rn(v * sc); }
-template <> __device__ __forceinline__ __nv_bfloat16 enc<ST_BF16>(float v, float sc) { return __float2bfloat16_rn(v * sc); }
 
 // Encode two values into the storage's pair type (one packed conversion for
-// the 16-bit storages; each half rounds as enc would).
+// the 16-bit storages; each half rounds as StoreT::store would).
 template <int S> __device__ __forceinline__ typename Pair<typename StoreT<S>::T>::V enc2(float a, float b, float sc);
 template <> __device__ __forceinline__ float2 enc2<ST_F32>(float a, float b, float) { return make_float2(a, b); }
 template <> __device__ __forceinline__ __half2 enc2<ST_F16>(float a, float b, float sc) {
@@ -476,7 +469,6 @@ template <> __device__ __forceinline__ __half2 enc2<ST_F16>(float a, float b, fl
 template <> __device__ __forceinline__ __nv_bfloat162 enc2<ST_BF16>(float a, float b, float sc) {
     return __floats2bfloat162_rn(a * sc, b * sc);
 }
-template <> __device__ __forceinline__ double2 enc2<ST_F64>(float, float, float) { return make_double2(0.0, 0.0); }
 
 // enc2 with the stochastic rounding of BF16 stores when sr is set (random
 // bits w from sr_word)
