@@ -212,13 +212,14 @@ def test_small_groups_tiles_give_the_same_bits():
 
 def test_a_chain_without_requests():
     """Only the chains that hold requests run: two requests, of which the first
-    ends early, so that the second chain runs by itself, then a third, which
-    joins the first chain again.  Each gives the bits it gives alone."""
+    ends early, so that the second chain runs by itself (20 rounds with the
+    graph of both, then with its own), then a third, which joins the first chain
+    again.  Each gives the bits it gives alone."""
     args = dict(e=(0.3, -0.4, 1.0), R=4.5, B1=0.03, beta=-2.0)
     reqs = [make_request(0, (30, 26, 28), "f32", pos=(14.2, 12.7, 13.1), steps=30, **args),
-            make_request(0, (36, 32, 34), "bf16dev", pos=(17.5, 15.5, 16.5), steps=150, **args),
+            make_request(0, (36, 32, 34), "bf16dev", pos=(17.5, 15.5, 16.5), steps=505, **args),
             make_request(0, (28, 30, 26), "f64", pos=(13.2, 14.7, 12.1), steps=60, **args)]
-    mix = run_server(reqs, [0, 0, 4])
+    mix = run_server(reqs, [0, 0, 28])
     for i, r in enumerate(reqs):
         alone = run_server([r], [0])[0]
         assert mix[i].state == lbsq.LB_REQ_DONE
