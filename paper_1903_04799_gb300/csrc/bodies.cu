@@ -585,8 +585,9 @@ __device__ __noinline__ void update_turn(const Lattice& L, const BodyParams& p, 
 // error word says so (here and not in update_move, which k_body_fused also
 // runs on scratch without the links' force, where a body may seem to leave the
 // scheme that does not).
-__device__ __forceinline__ void update_stats(const Lattice& L, const BodyParams& p, const BodyState& s, const BodyAcc& Ai, int flags,
-                                             BodyAcc* Ao, BodyState* So, BodyState* out) {
+__device__ __forceinline__ void update_stats(const Lattice& L, const BodyParams& p, const BodyState& s,
+                                             const BodyAcc& Ai, int flags, BodyAcc* Ao, BodyState* So,
+                                             BodyState* out) {
     if (!(p.kind == BODY_SPHERE && p.mobile)) return;
     const int lane = threadIdx.x & 31;
     const int a = lane < 3 ? lane : 0;

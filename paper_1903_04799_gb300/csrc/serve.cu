@@ -680,7 +680,7 @@ int64_t tile_cells(int units) { return (2 * (int64_t)units + 3) / 4 * 4; }
 // the largest power of two with 256 tiles or more, from 128 up to the tuned
 // size.  us per step, tuned size (1024 or 2048) / by this rule, one request: FP64
 // 32^3 86 / 56, 64^3 92 / 69, FP32 32^3 52 / 47, 96^3 65 / 63; three of 33^3
-// FP32, 40^3 FP16, 48^3 FP64 111 / 76.  (Larger tiles, fixed: 64^3 FP64 at 128
+// FP32, 40^3 FP16, 48^3 FP64 111 / 76.  (Fixed sizes: 64^3 FP64 at 128
 // pairs 72, 256 70, 512 71, 1024 81; 128^3 FP32 at 256 110, 512 104, 2048 101.)
 // A size given by the caller (lb_server_params) stays.
 int group_tile_units(const lb_server* s, int64_t cells) {
